@@ -33,10 +33,57 @@ constexpr int kFoldThreads = 320;  // folded-tap forward: producer, MMA issuer a
 // (about four tiles per HBM round trip) whatever else it did; with five the loads run as far ahead as the operand stages.
 constexpr int kYSlots = 5;
 
+// Division by a number that is fixed for a launch, as a multiplication (exact for dividends below 2^31).  The role loops decode
+// a tile number per tile; a 32-bit division by a run-time value costs a single thread about 100 cycles of dependent instructions.
+struct FDiv {
+  uint32_t d, mul, shift;
+};
+FDiv fdiv_of(uint32_t d) {
+  FDiv f{d, 0, 0};
+  if (d == 1) return f;
+  uint32_t lg = 0;
+  while ((1ull << lg) < d) ++lg;
+  f.mul = (uint32_t)(((1ull << (31 + lg)) + d - 1) / d);
+  f.shift = lg - 1;
+  return f;
+}
+__device__ __forceinline__ uint32_t fdiv(uint32_t n, const FDiv& f, uint32_t* rem) {
+  const uint32_t q = f.d == 1 ? n : __umulhi(n, f.mul) >> f.shift;
+  *rem = n - q * f.d;
+  return q;
+}
+
+// First pixel and image (group) of pixel tile m: tiles run along the width, then the height, then the images
+struct TileGrid {
+  FDiv nt, tw, th;  // channel tiles, tile columns, tile rows
+};
+TileGrid tile_grid(int n_tiles, int tiles_w, int tiles_h) { return {fdiv_of(n_tiles), fdiv_of(tiles_w), fdiv_of(tiles_h)}; }
+struct TileAt {
+  uint32_t nt, w, h, n;
+};
+__device__ __forceinline__ TileAt tile_at(uint32_t t, const TileGrid& g) {
+  TileAt a;
+  const uint32_t m = fdiv(t, g.nt, &a.nt), r = fdiv(m, g.tw, &a.w);
+  a.n = fdiv(r, g.th, &a.h);
+  return a;
+}
+
+// Position in a ring of `stages` buffers: index and the parity a waiter for "full" expects in this round
+struct Ring {
+  uint32_t s = 0, ph = 0;
+  __device__ __forceinline__ void next(uint32_t stages) {
+    if (++s == stages) {
+      s = 0;
+      ph ^= 1;
+    }
+  }
+};
+
 struct FwdParams {
   int N, H, W, Cin, Cout;
   int BW, BH, tiles_w, tiles_h, n_tiles, total_tiles, kchunks, stages;
   int stride, BI;     // PT mode: conv stride and images per tile (BW*BH*BI = 128)
+  TileGrid tg;
   int stats;
   float* red;         // [grid * parts][2][Cout] channel partials (pre-zeroed)
   int32_t* status;    // device status word
@@ -95,7 +142,6 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   volatile int* epi_go = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ksteps = (PT ? 9 : 3) * p.kchunks;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -126,108 +172,110 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    // ---------------- producer: one TMA box of activations + three weight tiles per k-step
-    uint32_t it = 0;
-    bool ok = true;
-    if constexpr (RW) {
-      if (lane == 0 && blockIdx.x < p.total_tiles) {
-        ptx::mbar_expect_tx(wfull, (uint32_t)w_bytes);
+    // ---------------- producer: one TMA box of activations + three weight tiles per k-step.  One thread runs the whole loop:
+    // with a warp vote, a ring index by division and a reconvergence per step the producer and the issuer each spent about
+    // 650 cycles per step whatever its size (measured with clock counters), more than a 256-wide step's arithmetic (512).
+    if (ptx::elect_one()) {
+      if constexpr (RW) {
+        if (blockIdx.x < p.total_tiles) {
+          ptx::mbar_expect_tx(wfull, (uint32_t)w_bytes);
 #pragma unroll
-        for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(wres + kw * 3 * BN * 128, &tm_w, wfull, 0, (blockIdx.x % p.n_tiles) * BN, kw, 0);
+          for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(wres + kw * 3 * BN * 128, &tm_w, wfull, 0, (blockIdx.x % p.n_tiles) * BN, kw, 0);
+        }
       }
-      __syncwarp();
-    }
-    uint32_t ptl = 0;
-    for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++ptl) {
-      const int nt = t % p.n_tiles, m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * p.BW, h0 = ((m / p.tiles_w) % p.tiles_h) * p.BH, n = (m / (p.tiles_w * p.tiles_h)) * p.BI;
-      for (int ks = 0; ks < ksteps; ++ks, ++it) {
-        const int s = it % p.stages;
-        const uint32_t ph = (it / p.stages) & 1;
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag))) { ok = false; break; }
-        if (lane == 0) {
-          uint8_t* a_s = smem + (size_t)s * stage_bytes;
-          ptx::mbar_expect_tx(&full[s], (uint32_t)(a_bytes + b_bytes));
-          if constexpr (PT) {
-            const int tap = ks % 9, ck = ks / 9, kh = tap / 3, kw = tap % 3;
-            ptx::tma_load_4d(a_s, &tm_x, &full[s], ck * KC, p.stride * w0 + kw - 1, p.stride * h0 + kh - 1, n);
-            if constexpr (BMN) {
+      Ring rg;
+      uint32_t ptl = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++ptl) {
+        const TileAt at = tile_at(t, p.tg);
+        const int co0 = at.nt * BN, w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
+        for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
-              for (int hf = 0; hf < BN / 64; ++hf)  // [half][KC rows of f][64 channels], both taps mirrored
-                ptx::tma_load_4d(a_s + a_stride + hf * KC * 128, &tm_w, &full[s], nt * BN + hf * 64, 0, 2 - kw, 2 - kh);
+          for (int tap = 0; tap < (PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+            if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) { ok = false; break; }
+            uint64_t* fb = &full[rg.s];
+            uint8_t* a_s = smem + (size_t)rg.s * stage_bytes;
+            ptx::mbar_expect_tx(fb, (uint32_t)(a_bytes + b_bytes));
+            if constexpr (PT) {
+              const int kh = tap / 3, kw = tap % 3;
+              ptx::tma_load_4d(a_s, &tm_x, fb, ck * KC, p.stride * w0 + kw - 1, p.stride * h0 + kh - 1, n);
+              if constexpr (BMN) {
+#pragma unroll
+                for (int hf = 0; hf < BN / 64; ++hf)  // [half][KC rows of f][64 channels], both taps mirrored
+                  ptx::tma_load_4d(a_s + a_stride + hf * KC * 128, &tm_w, fb, co0 + hf * 64, 0, 2 - kw, 2 - kh);
+              } else {
+                ptx::tma_load_4d(a_s + a_stride, &tm_w, fb, ck * 64, co0, kw, kh);
+              }
             } else {
-              ptx::tma_load_4d(a_s + a_stride, &tm_w, &full[s], ck * 64, nt * BN, kw, kh);
-            }
-          } else {
-            const int kw = ks % 3, ck = ks / 3;
-            ptx::tma_load_4d(a_s, &tm_x, &full[s], ck * KC, w0 + kw - 1, h0 - 1, n);
-            if constexpr (BMN) {
+              ptx::tma_load_4d(a_s, &tm_x, fb, ck * KC, w0 + tap - 1, h0 - 1, n);
+              if constexpr (BMN) {
 #pragma unroll
-              for (int hf = 0; hf < BN / 64; ++hf)  // [half][kh][KC rows of f][64 channels], mirrored column tap
-                ptx::tma_load_4d(a_s + a_stride + hf * 3 * KC * 128, &tm_w, &full[s], nt * BN + hf * 64, 0, 2 - kw, 0);
-            } else if constexpr (!RW) {
-              ptx::tma_load_4d(a_s + a_stride, &tm_w, &full[s], ck * 64, nt * BN, kw, 0);
+                for (int hf = 0; hf < BN / 64; ++hf)  // [half][kh][KC rows of f][64 channels], mirrored column tap
+                  ptx::tma_load_4d(a_s + a_stride + hf * 3 * KC * 128, &tm_w, fb, co0 + hf * 64, 0, 2 - tap, 0);
+              } else if constexpr (!RW) {
+                ptx::tma_load_4d(a_s + a_stride, &tm_w, fb, ck * 64, co0, tap, 0);
+              }
             }
           }
         }
-        __syncwarp();
-      }
-      if constexpr (EPI == 0) {
-        // the y2 tile of this output tile goes out after its operand loads: the single buffer is free once the epilogue
-        // has finished the statistics of the previous tile, which it does while this tile is being multiplied
-        if (ok && p.stats == 2) {
-          if (!__all_sync(0xffffffffu, ptx::mbar_wait(yempty, (ptl & 1) ^ 1, abort_flag))) break;
-          if (lane == 0) {
+        if constexpr (EPI == 0) {
+          // the y2 tile of this output tile goes out after its operand loads: the single buffer is free once the epilogue
+          // has finished the statistics of the previous tile, which it does while this tile is being multiplied
+          if (ok && p.stats == 2) {
+            if (!ptx::mbar_wait(yempty, (ptl & 1) ^ 1, abort_flag)) break;
             ptx::mbar_expect_tx(yfull, (uint32_t)(kSub * 16384));
 #pragma unroll
-            for (int sb = 0; sb < kSub; ++sb) ptx::tma_load_4d(ybuf + sb * 16384, &p.tm_y2, yfull, nt * BN + sb * 64, w0, h0, n);
+            for (int sb = 0; sb < kSub; ++sb) ptx::tma_load_4d(ybuf + sb * 16384, &p.tm_y2, yfull, co0 + sb * 64, w0, h0, n);
           }
-          __syncwarp();
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
-    // ---------------- MMA issuer
+    // ---------------- MMA issuer (one thread, as above)
     constexpr uint32_t idesc = ptx::idesc_bf16(128, BN, 0, BMN);
-    uint32_t it = 0, tl = 0;
-    bool ok = true;
     // descriptors differ only in their 14-bit address field: constant upper parts, address added per use
     const uint64_t a_hi = ptx::sdesc(0, 16, 8 * kARow, kALayout);
     const uint64_t b_hi = BMN ? ptx::sdesc(0, (PT ? 1 : 3) * KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
     const uint32_t a_row16 = (uint32_t)(p.BW * kARow) >> 4;  // one image row of the box, in 16-byte units
-    if constexpr (RW) {
-      if (blockIdx.x < p.total_tiles) ok = __all_sync(0xffffffffu, ptx::mbar_wait(wfull, 0, abort_flag));
-    }
-    for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
-      const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag))) break;
-      ptx::tc_fence_after();
-      const uint32_t d = tmem_base + acc * BN;
-      for (int ks = 0; ks < ksteps; ++ks, ++it) {
-        const int s = it % p.stages;
-        const uint32_t ph = (it / p.stages) & 1;
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph, abort_flag))) { ok = false; break; }
-        ptx::tc_fence_after();
-        if (lane == 0) {
-          const uint32_t a_base = ptx::smem_u32(smem + (size_t)s * stage_bytes);
-          const uint32_t a16 = a_base >> 4;
-          const uint32_t b16 = RW ? (ptx::smem_u32(wres) + (ks % 3) * 3 * BN * 128) >> 4 : (a_base + a_stride) >> 4;
-#pragma unroll
-          for (int kh = 0; kh < (PT ? 1 : 3); ++kh)
-#pragma unroll
-            for (int k = 0; k < KC / 16; ++k) {
-              const uint64_t ad = a_hi | (uint64_t)(a16 + kh * a_row16 + k * 2);
-              const uint64_t bd = b_hi | (uint64_t)(BMN ? b16 + (((PT ? 0 : (2 - kh) * KC * 128) + k * 16 * 128) >> 4)
-                                                        : b16 + ((kh * BN * 128 + k * 32) >> 4));
-              ptx::mma_f16(d, ad, bd, idesc, (ks | kh | k) != 0);
-            }
-          ptx::mma_commit(&empty[s]);
-        }
-        __syncwarp();
+    if (ptx::elect_one()) {
+      Ring rg;
+      uint32_t tl = 0;
+      bool ok = true;
+      if constexpr (RW) {
+        if (blockIdx.x < p.total_tiles) ok = ptx::mbar_wait(wfull, 0, abort_flag);
       }
-      if (ok && lane == 0) ptx::mma_commit(&tfull[acc]);
-      __syncwarp();
+      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
+        const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
+        if (!ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag)) break;
+        ptx::tc_fence_after();
+        const uint32_t d = tmem_base + acc * BN;
+        uint32_t accumulate = 0;
+        for (int ck = 0; ok && ck < p.kchunks; ++ck) {
+#pragma unroll
+          for (int tap = 0; tap < (PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+            if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
+            ptx::tc_fence_after();
+            const uint32_t a_base = ptx::smem_u32(smem) + rg.s * stage_bytes;
+            const uint32_t a16 = a_base >> 4;
+            const uint32_t b16 = RW ? (ptx::smem_u32(wres) + tap * 3 * BN * 128) >> 4 : (a_base + a_stride) >> 4;
+#pragma unroll
+            for (int kh = 0; kh < (PT ? 1 : 3); ++kh)
+#pragma unroll
+              for (int k = 0; k < KC / 16; ++k) {
+                const uint64_t ad = a_hi | (uint64_t)(a16 + kh * a_row16 + k * 2);
+                const uint64_t bd = b_hi | (uint64_t)(BMN ? b16 + (((PT ? 0 : (2 - kh) * KC * 128) + k * 16 * 128) >> 4)
+                                                          : b16 + ((kh * BN * 128 + k * 32) >> 4));
+                ptx::mma_f16(d, ad, bd, idesc, accumulate);
+                accumulate = 1;
+              }
+            ptx::mma_commit(&empty[rg.s]);
+          }
+        }
+        if (ok) ptx::mma_commit(&tfull[acc]);
+      }
     }
+    __syncwarp();
   } else {
     // ---------------- epilogue: 128 threads, thread <-> output pixel (TMEM lane)
     if constexpr (EPI == 0) {
@@ -251,8 +299,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
     }
     for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
-      const int nt = t % p.n_tiles, m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * p.BW, h0 = ((m / p.tiles_w) % p.tiles_h) * p.BH, n = (m / (p.tiles_w * p.tiles_h)) * p.BI;
+      const TileAt at = tile_at(t, p.tg);
+      const int nt = at.nt, w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
       const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
       ptx::mbar_wait(&tfull[acc], aph, abort_flag);  // sets the abort flag itself when it gives up
       ptx::tc_fence_after();
@@ -359,8 +407,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const int r = lg * 32 + lane;
       uint32_t tl = 0;
       for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
-        const int m = t / p.n_tiles;
-        const int w0 = (m % p.tiles_w) * p.BW, h0 = ((m / p.tiles_w) % p.tiles_h) * p.BH, n = (m / (p.tiles_w * p.tiles_h)) * p.BI;
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
         const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
         ptx::mbar_wait(&tfull[acc], aph, abort_flag);
         ptx::tc_fence_after();
@@ -467,6 +515,7 @@ __device__ __forceinline__ void fold_group_partial(float (&s1)[8], float (&s2)[8
 
 struct FoldParams {
   int N, H, W, Cout, kchunks, n_tiles, tiles_w, tiles_h, total_tiles, stages, stats;
+  TileGrid tg;
   float* red;         // EPI 0, stats != 0: [grid / n_tiles * 8][2][Cout]
   int32_t* status;
   const float *bn_scale, *bn_shift, *bn_mu, *bn_invstd;  // stats >= 2
@@ -589,68 +638,60 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0 && blockIdx.x < p.total_tiles) {
-      ptx::mbar_expect_tx(wfull, (uint32_t)w_bytes);
-      for (int ck = 0; ck < p.kchunks; ++ck)
+    if (ptx::elect_one()) {  // one thread runs the whole loop, as in the generic kernel
+      if (blockIdx.x < p.total_tiles) {
+        ptx::mbar_expect_tx(wfull, (uint32_t)w_bytes);
+        for (int ck = 0; ck < p.kchunks; ++ck)
 #pragma unroll
-        for (int kh = 0; kh < 3; ++kh)
-          ptx::tma_load_4d(wres + (ck * 3 + kh) * kWTile, &tm_w, wfull, MIR ? (int)(blockIdx.x % p.n_tiles) * 64 : ck * 64, 0, 0, kh);
+          for (int kh = 0; kh < 3; ++kh)
+            ptx::tma_load_4d(wres + (ck * 3 + kh) * kWTile, &tm_w, wfull, MIR ? (int)(blockIdx.x % p.n_tiles) * 64 : ck * 64, 0, 0, kh);
+      }
+      Ring rg, yr;
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * kTW, h0 = at.h * kTH, n = at.n;
+        for (int ck = 0; ck < p.kchunks; ++ck, rg.next(p.stages)) {
+          if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) { ok = false; break; }
+          uint64_t* fb = &full[rg.s];
+          uint8_t* st = smem + (size_t)rg.s * kABytes;
+          ptx::mbar_expect_tx(fb, (uint32_t)(UF == 2 ? kBox : kABytes));
+          if constexpr (UF == 1) {
+#pragma unroll
+            for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(st + kw * kBox, &tm_x, fb, ck * KC, w0 - 1 + kw, h0 - 1, n);
+          } else {
+            ptx::tma_load_4d(st, &tm_x, fb, ck * KC, w0 - 1, h0 - 1, n);
+          }
+        }
+        if constexpr (EPI == 0) {
+          if (ok && p.stats >= 2) {  // the y2 tile of this output tile, for the epilogue group that owns it
+            if (!ptx::mbar_wait(&yempty[yr.s], yr.ph ^ 1, abort_flag)) break;
+            ptx::mbar_expect_tx(&yfull[yr.s], kTW * kTH * 128);
+            ptx::tma_load_4d(ybuf + yr.s * 16384, &tm_y2, &yfull[yr.s], (int)at.nt * 64, w0, h0, n);
+            yr.next(kYSlots);
+          }
+        }
+      }
     }
     __syncwarp();
-    uint32_t it = 0, tl = 0;
-    bool ok = true;
-    for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
-      const int m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * kTW, h0 = ((m / p.tiles_w) % p.tiles_h) * kTH, n = m / (p.tiles_w * p.tiles_h);
-      for (int ck = 0; ck < p.kchunks; ++ck, ++it) {
-        const int s = it % p.stages;
-        const uint32_t ph = (it / p.stages) & 1;
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag))) { ok = false; break; }
-        if (lane == 0) {
-          ptx::mbar_expect_tx(&full[s], (uint32_t)(UF == 2 ? kBox : kABytes));
-          if constexpr (UF == 2) {
-            ptx::tma_load_4d(smem + (size_t)s * kABytes, &tm_x, &full[s], ck * KC, w0 - 1, h0 - 1, n);
-          } else if constexpr (UF) {
-#pragma unroll
-            for (int kw = 0; kw < 3; ++kw)
-              ptx::tma_load_4d(smem + (size_t)s * kABytes + kw * kBox, &tm_x, &full[s], ck * KC, w0 - 1 + kw, h0 - 1, n);
-          } else {
-            ptx::tma_load_4d(smem + (size_t)s * kABytes, &tm_x, &full[s], ck * KC, w0 - 1, h0 - 1, n);
-          }
-        }
-        __syncwarp();
-      }
-      if constexpr (EPI == 0) {
-        if (ok && p.stats >= 2) {  // the y2 tile of this output tile, for the epilogue group that owns it
-          const uint32_t slot = tl % kYSlots;
-          if (!__all_sync(0xffffffffu, ptx::mbar_wait(&yempty[slot], ((tl / kYSlots) & 1) ^ 1, abort_flag))) break;
-          if (lane == 0) {
-            ptx::mbar_expect_tx(&yfull[slot], kTW * kTH * 128);
-            ptx::tma_load_4d(ybuf + slot * 16384, &tm_y2, &yfull[slot], (t % p.n_tiles) * 64, w0, h0, n);
-          }
-          __syncwarp();
-        }
-      }
-    }
   } else if (warp == 1) {
     constexpr uint32_t idesc = ptx::idesc_bf16(128, UF ? G : 3 * G, 0, MIR);
     const uint64_t a_hi = ptx::sdesc(0, 16, (UF == 2 ? 10 : 8) * kARow, kALayout);  // UF 2: next 8-pixel group = next box row
     const uint64_t b_hi = MIR ? ptx::sdesc(0, KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
     const uint32_t w16 = ptx::smem_u32(wres) >> 4;
-    uint32_t it = 0, tl = 0;
-    bool ok = blockIdx.x >= p.total_tiles || __all_sync(0xffffffffu, ptx::mbar_wait(wfull, 0, abort_flag));
-    for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
-      const uint32_t acc = tl % kAccs, aph = (tl / kAccs) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag))) break;
-      ptx::tc_fence_after();
-      const uint32_t d = tmem_base + acc * kAccStride;
-      for (int ck = 0; ck < p.kchunks; ++ck, ++it) {
-        const int s = it % p.stages;
-        const uint32_t ph = (it / p.stages) & 1;
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(XF ? &xfull[s] : &full[s], ph, abort_flag))) { ok = false; break; }
+    if (ptx::elect_one()) {
+      Ring rg;
+      uint32_t tl = 0;
+      bool ok = blockIdx.x >= p.total_tiles || ptx::mbar_wait(wfull, 0, abort_flag);
+      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
+        const uint32_t acc = tl % kAccs, aph = (tl / kAccs) & 1;
+        if (!ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag)) break;
         ptx::tc_fence_after();
-        if (lane == 0) {
-          const uint32_t a16 = ptx::smem_u32(smem + (size_t)s * kABytes) >> 4;
+        const uint32_t d = tmem_base + acc * kAccStride;
+        for (int ck = 0; ck < p.kchunks; ++ck, rg.next(p.stages)) {
+          if (!ptx::mbar_wait(XF ? &xfull[rg.s] : &full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
+          ptx::tc_fence_after();
+          const uint32_t a16 = (ptx::smem_u32(smem) + rg.s * kABytes) >> 4;
           if constexpr (UF) {  // one instruction per tap and 16 input channels; tap (kh, kw) reads the mirrored weight tile
 #pragma unroll
             for (int kh = 0; kh < 3; ++kh)
@@ -663,23 +704,23 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
                   const uint64_t bd = b_hi | (uint64_t)(w16 + (2 - kh) * (kWTile >> 4) + (2 - kw) * (KC * 128 >> 4) + k * 128);
                   ptx::mma_f16(d, ad, bd, idesc, (kh | kw | k) != 0);
                 }
-          } else
+          } else {
 #pragma unroll
-          for (int kh = 0; kh < 3; ++kh)
+            for (int kh = 0; kh < 3; ++kh)
 #pragma unroll
-            for (int k = 0; k < KC / 16; ++k) {
-              const uint64_t ad = a_hi | (uint64_t)(a16 + kh * (16 * kARow >> 4) + k * 2);
-              const uint64_t bd = MIR ? b_hi | (uint64_t)(w16 + (2 - kh) * (kWTile >> 4) + k * 128)   // mirrored row tap, 16 f rows on
-                                      : b_hi | (uint64_t)(w16 + (ck * 3 + kh) * (kWTile >> 4) + k * 2);
-              ptx::mma_f16(d, ad, bd, idesc, (ck | kh | k) != 0);
-            }
-          ptx::mma_commit(&empty[s]);
+              for (int k = 0; k < KC / 16; ++k) {
+                const uint64_t ad = a_hi | (uint64_t)(a16 + kh * (16 * kARow >> 4) + k * 2);
+                const uint64_t bd = MIR ? b_hi | (uint64_t)(w16 + (2 - kh) * (kWTile >> 4) + k * 128)   // mirrored row tap, 16 f rows on
+                                        : b_hi | (uint64_t)(w16 + (ck * 3 + kh) * (kWTile >> 4) + k * 2);
+                ptx::mma_f16(d, ad, bd, idesc, (ck | kh | k) != 0);
+              }
+          }
+          ptx::mma_commit(&empty[rg.s]);
         }
-        __syncwarp();
+        if (ok) ptx::mma_commit(&tfull[acc]);
       }
-      if (ok && lane == 0) ptx::mma_commit(&tfull[acc]);
-      __syncwarp();
     }
+    __syncwarp();
   } else if (XF && warp >= kFoldThreads / 32) {
     // normalisation warps: a thread owns one 16-byte channel chunk (8 channels) of one box column and walks the 10 rows.
     // The tile's own 14 x 8 pixels of a leave through a TMA store: the threads copy them from registers into a dense staging
@@ -690,19 +731,20 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     const int j = xt & 7, col = xt >> 3;                   // logical chunk, box column (0..15)
     const uint32_t off0 = (uint32_t)col * 128 + (uint32_t)((j ^ (col & 7)) * 16);  // 128-byte swizzle: the row's low bits are col's
     uint32_t it = 0;
+    Ring rg;
     float sc[8], sh[8];
     int coef_ck = -1;  // channel chunk whose coefficients the registers hold
     bool go = true;
     for (int t = blockIdx.x; go && t < p.total_tiles; t += gridDim.x) {
-      const int m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * 14, h0 = ((m / p.tiles_w) % p.tiles_h) * 8, n = m / (p.tiles_w * p.tiles_h);
+      const TileAt at = tile_at(t, p.tg);
+      const int w0 = at.w * 14, h0 = at.h * 8, n = at.n;
       const int w = w0 - 1 + col;
       const bool w_in = w >= 0 && w < p.W, w_own = col >= 1 && col <= 14;
-      for (int ck = 0; ck < p.kchunks; ++ck, ++it) {
+      for (int ck = 0; ck < p.kchunks; ++ck, ++it, rg.next(p.stages)) {
         if ((int)(it % kXfGroups) != xgrp) continue;
         const uint32_t jt = it / kXfGroups;  // this group's iteration count
-        const int s = it % p.stages;
-        const uint32_t ph = (it / p.stages) & 1;
+        const int s = rg.s;
+        const uint32_t ph = rg.ph;
         if (ck != coef_ck) {
           coef_ck = ck;
 #pragma unroll
@@ -788,11 +830,9 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       }
     }
     uint32_t tl = grp;
-    // 32-bit tile arithmetic (the host keeps total_tiles below 2^30): 64-bit divisions here cost about a quarter of the tile time
     for (int t = blockIdx.x + grp * gridDim.x; t < p.total_tiles; t += 2 * gridDim.x, tl += 2) {
-      const int nt = t % p.n_tiles;
-      const int m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * kTW, h0 = ((m / p.tiles_w) % p.tiles_h) * kTH, n = m / (p.tiles_w * p.tiles_h);
+      const TileAt at = tile_at(t, p.tg);
+      const int nt = at.nt, w0 = at.w * kTW, h0 = at.h * kTH, n = at.n;
       const uint32_t acc = tl % kAccs, aph = (tl / kAccs) & 1;
       ptx::mbar_wait(&tfull[acc], aph, abort_flag);
       ptx::tc_fence_after();
@@ -1083,51 +1123,46 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 
   if (warp == 0) {
     // ---------------- producer: the CTA's weights once, then per tile one dh box and (stats >= 2) the y2 tile
-    if (lane == 0 && blockIdx.x < p.total_tiles) {
-      ptx::mbar_expect_tx(wfull, (uint32_t)(3 * kWTile));
+    if (ptx::elect_one()) {
+      if (blockIdx.x < p.total_tiles) {
+        ptx::mbar_expect_tx(wfull, (uint32_t)(3 * kWTile));
 #pragma unroll
-      for (int kh = 0; kh < 3; ++kh) ptx::tma_load_4d(wres + kh * kWTile, &tm_w, wfull, (int)(blockIdx.x % p.n_tiles) * 64, 0, 0, kh);
+        for (int kh = 0; kh < 3; ++kh) ptx::tma_load_4d(wres + kh * kWTile, &tm_w, wfull, (int)(blockIdx.x % p.n_tiles) * 64, 0, 0, kh);
+      }
+      Ring rg, yr;
+      for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, rg.next(p.stages)) {
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * 8, h0 = at.h * 32, n = at.n;
+        if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) break;
+        ptx::mbar_expect_tx(&full[rg.s], (uint32_t)kBox);
+        ptx::tma_load_4d(smem + (size_t)rg.s * kStage, &tm_x, &full[rg.s], 0, w0 - 1, h0 - 1, n);
+        if (p.stats >= 2) {
+          if (!ptx::mbar_wait(&yempty[yr.s], yr.ph ^ 1, abort_flag)) break;
+          ptx::mbar_expect_tx(&yfull[yr.s], (uint32_t)kTile);
+          ptx::tma_load_4d(ybuf + yr.s * kTile, &tm_y2, &yfull[yr.s], (int)at.nt * 64, w0, h0, n);
+          yr.next(kWideYSlots);
+        }
+      }
     }
     __syncwarp();
-    uint32_t tl = 0;
-    for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
-      const int m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * 8, h0 = ((m / p.tiles_w) % p.tiles_h) * 32, n = m / (p.tiles_w * p.tiles_h);
-      const int s = tl % p.stages;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&empty[s], ((tl / p.stages) & 1) ^ 1, abort_flag))) break;
-      if (lane == 0) {
-        ptx::mbar_expect_tx(&full[s], (uint32_t)kBox);
-        ptx::tma_load_4d(smem + (size_t)s * kStage, &tm_x, &full[s], 0, w0 - 1, h0 - 1, n);
-      }
-      __syncwarp();
-      if (p.stats >= 2) {
-        const uint32_t slot = tl % kWideYSlots;
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&yempty[slot], ((tl / kWideYSlots) & 1) ^ 1, abort_flag))) break;
-        if (lane == 0) {
-          ptx::mbar_expect_tx(&yfull[slot], (uint32_t)kTile);
-          ptx::tma_load_4d(ybuf + slot * kTile, &tm_y2, &yfull[slot], (t % p.n_tiles) * 64, w0, h0, n);
-        }
-        __syncwarp();
-      }
-    }
   } else if (warp == 1) {
     // ---------------- issuer: nine instructions per tile, D[channel][pixel] += Wa_mirrored(tap)[channel][f] * dh[pixel + tap][f]
     constexpr uint32_t idesc = ptx::idesc_bf16(64, 256, 1, 0);
     const uint64_t a_hi = ptx::sdesc(0, KC * 128, 1024, 2);          // weight tile of a tap: [f][64 c], MN-major
     const uint64_t b_hi = ptx::sdesc(0, 16, 10 * kARow, kALayout);   // pixels: next 8-pixel group = next box row
     const uint32_t w16 = ptx::smem_u32(wres) >> 4;
-    uint32_t tl = 0;
-    bool ok = blockIdx.x >= p.total_tiles || __all_sync(0xffffffffu, ptx::mbar_wait(wfull, 0, abort_flag));
-    for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
-      const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag))) break;
-      ptx::tc_fence_after();
-      const int s = tl % p.stages;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&full[s], (tl / p.stages) & 1, abort_flag))) break;
-      ptx::tc_fence_after();
-      if (lane == 0) {
+    if (ptx::elect_one()) {
+      Ring rg;
+      uint32_t tl = 0;
+      const bool ok = blockIdx.x >= p.total_tiles || ptx::mbar_wait(wfull, 0, abort_flag);
+      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl, rg.next(p.stages)) {
+        const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
+        if (!ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag)) break;
+        ptx::tc_fence_after();
+        if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) break;
+        ptx::tc_fence_after();
         const uint32_t d = tmem_base + acc * 256;
-        const uint32_t x16 = ptx::smem_u32(smem + (size_t)s * kStage) >> 4;
+        const uint32_t x16 = (ptx::smem_u32(smem) + rg.s * kStage) >> 4;
 #pragma unroll
         for (int kh = 0; kh < 3; ++kh)
 #pragma unroll
@@ -1138,11 +1173,11 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
               const uint64_t bd = b_hi | (uint64_t)(x16 + ((kh * 10 + kw) * kARow >> 4) + k * 2);
               ptx::mma_f16(d, ad, bd, idesc, (kh | kw | k) != 0);
             }
-        ptx::mma_commit(&empty[s]);
+        ptx::mma_commit(&empty[rg.s]);
         ptx::mma_commit(&tfull[acc]);
       }
-      __syncwarp();
     }
+    __syncwarp();
   } else {
     // ---------------- two epilogue groups of 128 threads; group g takes the tiles tl = g, g + 2, ... (accumulator g)
     const int grp = (threadIdx.x - 64) >> 7;
@@ -1169,9 +1204,8 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     }
     uint32_t tl = grp;
     for (int t = blockIdx.x + grp * gridDim.x; t < p.total_tiles; t += 2 * gridDim.x, tl += 2) {
-      const int nt = t % p.n_tiles;
-      const int m = t / p.n_tiles;
-      const int w0 = (m % p.tiles_w) * 8, h0 = ((m / p.tiles_w) % p.tiles_h) * 32, n = m / (p.tiles_w * p.tiles_h);
+      const TileAt at = tile_at(t, p.tg);
+      const int nt = at.nt, w0 = at.w * 8, h0 = at.h * 32, n = at.n;
       const uint32_t acc = grp, aph = (tl >> 1) & 1;
       ptx::mbar_wait(&tfull[acc], aph, abort_flag);
       ptx::tc_fence_after();
@@ -1294,6 +1328,7 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 struct WgParams {
   int N, H, W, Cin, Cout;
   int BW, BH, tiles_w, tiles_h, pix_tiles, ci_chunks, co_chunks, splits, stages, stride, BI;
+  TileGrid tg;
   float* part;      // [splits][9][Cout][Cin]
   int32_t* status;
 };
@@ -1358,54 +1393,50 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    uint32_t it = 0;
-    for (int t = t0; t < t1; ++t, ++it) {
-      const int s = it % kStages;
-      const uint32_t ph = (it / kStages) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag))) break;
-      if (lane == 0) {
-        const int w0 = (t % p.tiles_w) * p.BW, h0 = ((t / p.tiles_w) % p.tiles_h) * p.BH, n = (t / (p.tiles_w * p.tiles_h)) * p.BI;
-        uint8_t* st = smem + (size_t)s * stage_bytes;
-        ptx::mbar_expect_tx(&full[s], (uint32_t)(3 * copy_bytes + kAtoms * kBTile));
+    if (ptx::elect_one()) {  // producer and issuer: one thread runs the whole loop, as in the forward kernels
+      Ring rg;
+      for (int t = t0; t < t1; ++t, rg.next(kStages)) {
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
+        if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) break;
+        uint64_t* fb = &full[rg.s];
+        uint8_t* st = smem + (size_t)rg.s * stage_bytes;
+        ptx::mbar_expect_tx(fb, (uint32_t)(3 * copy_bytes + kAtoms * kBTile));
 #pragma unroll
         for (int kw = 0; kw < 3; ++kw)
-          ptx::tma_load_4d(st + kw * copy_bytes, &tm_x, &full[s], cic * 64, p.stride * w0 + kw - 1, p.stride * h0 + khg - 1, n);
+          ptx::tma_load_4d(st + kw * copy_bytes, &tm_x, fb, cic * 64, p.stride * w0 + kw - 1, p.stride * h0 + khg - 1, n);
 #pragma unroll
-        for (int a = 0; a < kAtoms; ++a)
-          ptx::tma_load_4d(st + 3 * copy_bytes + a * 16384, &tm_dy, &full[s], coc * NB + a * 64, w0, h0, n);
+        for (int a = 0; a < kAtoms; ++a) ptx::tma_load_4d(st + 3 * copy_bytes + a * 16384, &tm_dy, fb, coc * NB + a * 64, w0, h0, n);
       }
-      __syncwarp();
     }
+    __syncwarp();
   } else if (warp == 1) {
     constexpr uint32_t idesc = ptx::idesc_bf16(128, NB, 1, 1);
-    uint32_t it = 0;
-    bool ok = true;
-    for (int t = t0; t < t1; ++t, ++it) {
-      const int s = it % kStages;
-      const uint32_t ph = (it / kStages) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph, abort_flag))) { ok = false; break; }
-      ptx::tc_fence_after();
-      if (lane == 0) {
-        const uint32_t xb = ptx::smem_u32(smem + (size_t)s * stage_bytes);
+    // descriptors differ only in the address field; the second stacked chunk sits one tap tile further
+    const uint64_t a_copy_hi = ptx::sdesc(0, copy_bytes, 1024, 2);
+    const uint64_t b_hi = ptx::sdesc(0, 16384, 8 * kBRow, kBLayout);  // next 64-channel atom: 16 KB further
+    constexpr uint32_t copy16 = (uint32_t)copy_bytes >> 4;
+    if (ptx::elect_one()) {
+      Ring rg;
+      bool ok = true;
+      for (int t = t0; t < t1; ++t, rg.next(kStages)) {
+        if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
+        ptx::tc_fence_after();
+        const uint32_t xb = ptx::smem_u32(smem) + rg.s * stage_bytes;
         const uint32_t x16 = xb >> 4, g16 = (xb + 3 * copy_bytes) >> 4;
-        const uint32_t copy16 = (uint32_t)copy_bytes >> 4;
-        // descriptors differ only in the address field; the second stacked chunk sits one tap tile further
-        const uint64_t a_copy_hi = ptx::sdesc(0, copy_bytes, 1024, 2);
-        const uint64_t b_hi = ptx::sdesc(0, 16384, 8 * kBRow, kBLayout);  // next 64-channel atom: 16 KB further
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const uint32_t k16 = k * 128;  // 16 pixels x 128 bytes, in 16-byte units
           const uint64_t bd = b_hi | (uint64_t)(g16 + k * kBRow);
-          const uint32_t acc = (it | k) != 0;
+          const uint32_t acc = t > t0 || k != 0;
           // taps (kh,0) and (kh,1): second chunk one tile further; tap (kh,2): rows 64..127 unused
           ptx::mma_f16(tmem_base, a_copy_hi | (uint64_t)(x16 + k16), bd, idesc, acc);
           ptx::mma_f16(tmem_base + NB, a_copy_hi | (uint64_t)(x16 + 2 * copy16 + k16), bd, idesc, acc);
         }
-        ptx::mma_commit(&empty[s]);
+        ptx::mma_commit(&empty[rg.s]);
       }
-      __syncwarp();
+      if (ok) ptx::mma_commit(done);
     }
-    if (ok && lane == 0) ptx::mma_commit(done);
     __syncwarp();
   } else {
     // epilogue: after the last MMA, lane m of tensor memory = row m of the stacked (tap, ci) chunks
@@ -1506,49 +1537,46 @@ conv_wgrad_kw_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    uint32_t it = 0;
-    for (int t = t0; t < t1; ++t, ++it) {
-      const int s = it % stages;
-      const uint32_t ph = (it / stages) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag))) break;
-      if (lane == 0) {
-        const int w0 = (t % p.tiles_w) * p.BW, h0 = ((t / p.tiles_w) % p.tiles_h) * p.BH, n = t / (p.tiles_w * p.tiles_h);
-        uint8_t* st = smem + (size_t)s * stage_bytes;
-        ptx::mbar_expect_tx(&full[s], (uint32_t)(box_bytes + 3 * kBTile));
-        ptx::tma_load_4d(st, &tm_x, &full[s], cic * 64, w0, h0 - 1, n);
+    if (ptx::elect_one()) {
+      Ring rg;
+      for (int t = t0; t < t1; ++t, rg.next(stages)) {
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n;
+        if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) break;
+        uint64_t* fb = &full[rg.s];
+        uint8_t* st = smem + (size_t)rg.s * stage_bytes;
+        ptx::mbar_expect_tx(fb, (uint32_t)(box_bytes + 3 * kBTile));
+        ptx::tma_load_4d(st, &tm_x, fb, cic * 64, w0, h0 - 1, n);
 #pragma unroll
         for (int kw = 0; kw < 3; ++kw)  // gradient column j = j' - kw + 1
-          ptx::tma_load_4d(st + box_bytes + kw * kBTile, &tm_dy, &full[s], coc * NB, w0 - kw + 1, h0, n);
+          ptx::tma_load_4d(st + box_bytes + kw * kBTile, &tm_dy, fb, coc * NB, w0 - kw + 1, h0, n);
       }
-      __syncwarp();
     }
+    __syncwarp();
   } else if (warp == 1) {
     constexpr uint32_t idesc = ptx::idesc_bf16(128, 3 * NB, 1, 1);
     const uint64_t a_hi = ptx::sdesc(0, p.BW * 128, 1024, 2);      // second 64 rows: one image row further
     const uint64_t b_hi = ptx::sdesc(0, kBTile, 8 * kBRow, kBLayout);  // next N atom: next shifted tile
     const uint32_t row16 = (uint32_t)(p.BW * 128) >> 4;
-    uint32_t it = 0;
-    bool ok = true;
-    for (int t = t0; t < t1; ++t, ++it) {
-      const int s = it % stages;
-      const uint32_t ph = (it / stages) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph, abort_flag))) { ok = false; break; }
-      ptx::tc_fence_after();
-      if (lane == 0) {
-        const uint32_t xb = ptx::smem_u32(smem + (size_t)s * stage_bytes);
+    if (ptx::elect_one()) {
+      Ring rg;
+      bool ok = true;
+      for (int t = t0; t < t1; ++t, rg.next(stages)) {
+        if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
+        ptx::tc_fence_after();
+        const uint32_t xb = ptx::smem_u32(smem) + rg.s * stage_bytes;
         const uint32_t x16 = xb >> 4, g16 = (xb + box_bytes) >> 4;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const uint64_t bd = b_hi | (uint64_t)(g16 + k * kBRow);   // 16 pixels x kBRow bytes = k * kBRow sixteen-byte units
-          const uint32_t acc = (it | k) != 0;
+          const uint32_t acc = t > t0 || k != 0;
           ptx::mma_f16(tmem_base, a_hi | (uint64_t)(x16 + k * 128), bd, idesc, acc);                      // kh = 0 | 1
           ptx::mma_f16(tmem_base + kAcc, a_hi | (uint64_t)(x16 + 2 * row16 + k * 128), bd, idesc, acc);  // kh = 2 | unused
         }
-        ptx::mma_commit(&empty[s]);
+        ptx::mma_commit(&empty[rg.s]);
       }
-      __syncwarp();
+      if (ok) ptx::mma_commit(done);
     }
-    if (ok && lane == 0) ptx::mma_commit(done);
     __syncwarp();
   } else {
     const int lg = warp & 3, m = lg * 32 + lane;
@@ -1643,44 +1671,41 @@ conv_wgrad_gx_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    uint32_t it = 0;
-    for (int t = t0; t < t1; ++t, ++it) {
-      const int s = it % stages;
-      const uint32_t ph = (it / stages) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag))) break;
-      if (lane == 0) {
-        const int w0 = (t % p.tiles_w) * p.BW, h0 = ((t / p.tiles_w) % p.tiles_h) * p.BH, n = t / (p.tiles_w * p.tiles_h);
-        uint8_t* st = smem + (size_t)s * stage_bytes;
-        ptx::mbar_expect_tx(&full[s], (uint32_t)(box_bytes + 3 * kGTile));
-        ptx::tma_load_4d(st, &tm_x, &full[s], cic * 64, w0, h0 - 1, n);
+    if (ptx::elect_one()) {
+      Ring rg;
+      for (int t = t0; t < t1; ++t, rg.next(stages)) {
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n;
+        if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) break;
+        uint64_t* fb = &full[rg.s];
+        uint8_t* st = smem + (size_t)rg.s * stage_bytes;
+        ptx::mbar_expect_tx(fb, (uint32_t)(box_bytes + 3 * kGTile));
+        ptx::tma_load_4d(st, &tm_x, fb, cic * 64, w0, h0 - 1, n);
 #pragma unroll
         for (int kw = 0; kw < 3; ++kw)  // gradient column j = j' - kw + 1
-          ptx::tma_load_4d(st + box_bytes + kw * kGTile, &tm_dy, &full[s], 0, w0 - kw + 1, h0, n);
+          ptx::tma_load_4d(st + box_bytes + kw * kGTile, &tm_dy, fb, 0, w0 - kw + 1, h0, n);
       }
-      __syncwarp();
     }
+    __syncwarp();
   } else if (warp == 1) {
     constexpr uint32_t idesc = ptx::idesc_bf16(4 * NB, 192, 1, 1);
     const uint64_t a_hi = ptx::sdesc(0, kGTile, 8 * kBRow, kGLayout);  // next M atom: next shifted tile
     const uint64_t b_hi = ptx::sdesc(0, p.BW * 128, 1024, 2);          // next N atom: one image row further (next kh)
-    uint32_t it = 0;
-    bool ok = true;
-    for (int t = t0; t < t1; ++t, ++it) {
-      const int s = it % stages;
-      const uint32_t ph = (it / stages) & 1;
-      if (!__all_sync(0xffffffffu, ptx::mbar_wait(&full[s], ph, abort_flag))) { ok = false; break; }
-      ptx::tc_fence_after();
-      if (lane == 0) {
-        const uint32_t xb = ptx::smem_u32(smem + (size_t)s * stage_bytes);
+    if (ptx::elect_one()) {
+      Ring rg;
+      bool ok = true;
+      for (int t = t0; t < t1; ++t, rg.next(stages)) {
+        if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
+        ptx::tc_fence_after();
+        const uint32_t xb = ptx::smem_u32(smem) + rg.s * stage_bytes;
         const uint32_t x16 = xb >> 4, g16 = (xb + box_bytes) >> 4;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          ptx::mma_f16(tmem_base, a_hi | (uint64_t)(g16 + k * kBRow), b_hi | (uint64_t)(x16 + k * 128), idesc, (it | k) != 0);
-        ptx::mma_commit(&empty[s]);
+          ptx::mma_f16(tmem_base, a_hi | (uint64_t)(g16 + k * kBRow), b_hi | (uint64_t)(x16 + k * 128), idesc, t > t0 || k != 0);
+        ptx::mma_commit(&empty[rg.s]);
       }
-      __syncwarp();
+      if (ok) ptx::mma_commit(done);
     }
-    if (ok && lane == 0) ptx::mma_commit(done);
     __syncwarp();
   } else {
     const int lg = warp & 3;  // = column tap kw of this warp's rows
@@ -1969,6 +1994,7 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
   p.tiles_w = (W + TW - 1) / TW; p.tiles_h = (H + TH - 1) / TH; p.total_tiles = N * p.tiles_w * p.tiles_h * p.n_tiles;
   if ((long long)N * p.tiles_w * p.tiles_h * p.n_tiles > (1ll << 30)) return NF_EUNSUPPORTED;
   p.stats = stats; p.red = red; p.status = status; p.bias = bias; p.out = (bf16*)y;
+  p.tg = tile_grid(p.n_tiles, p.tiles_w, p.tiles_h);
   const size_t a_bytes = wide ? ((size_t)34 * 10 * KC * 2 + 1023) / 1024 * 1024
                          : uf2 ? ((size_t)18 * 10 * KC * 2 + 1023) / 1024 * 1024 : (size_t)(uf ? 3 : 1) * 10 * 16 * KC * 2;
   const size_t wbytes = epi == 2 ? (size_t)9 * KC * 128 : (size_t)9 * p.kchunks * G * 128;
@@ -2052,6 +2078,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   p.bias = bias; p.out = (bf16*)y;
   p.total_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w * p.n_tiles;
   p.stride = stride; p.BI = pl.BI;
+  p.tg = tile_grid(p.n_tiles, p.tiles_w, p.tiles_h);
   p.kchunks = epi == 2 ? 1 : Cin / 64; p.stages = pl.stages; p.stats = stats; p.red = red; p.status = status;
   p.tm_y2 = my;
   if (stats == 2) {
@@ -2201,6 +2228,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
   p.N = N; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout; p.BW = pl.BW; p.BH = pl.BH;
   p.tiles_w = W / pl.BW; p.tiles_h = H / pl.BH; p.pix_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w;
   p.stride = stride; p.BI = pl.BI;
+  p.tg = tile_grid(1, p.tiles_w, p.tiles_h);
   p.ci_chunks = Cin / 64; p.co_chunks = aux ? 1 : Cout / pl.NB; p.splits = pl.splits; p.part = part; p.status = status;
   p.stages = pl.stages;
   if (pl.GX)
