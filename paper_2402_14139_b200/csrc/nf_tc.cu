@@ -108,8 +108,8 @@ struct TcPlan {
 // BMN : 0 = weights [tap][co][ci] read K-major (forward); 1 = weights [tap][f][c] read MN-major with the
 //       taps mirrored, which makes the same kernel the input-gradient convolution da = dh (*) Wa^T.
 // PT  : 1 = one TMA box per tap: stride-2 convolutions (the box is gathered with element stride 2, so the
-//       three row taps cannot share a box) and feature maps smaller than a tile, where a tile spans BI whole
-//       images (8x8x2, 4x4x8, 2x2x32); p.H, p.W are the OUTPUT sizes.
+//       three row taps cannot share a box), feature maps smaller than a tile, where a tile spans BI whole
+//       images (8x8x2, 4x4x8, 2x2x32), and maps that no tile divides; p.H, p.W are the OUTPUT sizes.
 // RW  : 1 = all nine weight tiles of the CTA's channel tile stay resident in shared memory for the whole
 //       kernel (single 64-channel K chunk, 9*BN*128 bytes); the pipeline then carries activations only.
 template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0>
@@ -284,6 +284,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     const int r = lg * 32 + lane;     // row of the tile = pixel (r % BW, r / BW)
     constexpr int kRowsPer = BN >= 128 ? 128 : 64;  // rows each thread sums for its channel
     const int sc = et % BN, shalf = et / BN;        // stats: channel and row half of this thread
+    const int rw = r % p.BW, rh = (r / p.BW) % p.BH;  // place of the thread's pixel in its tile
     float ssum = 0.f, ssq = 0.f;
     float ssum2 = 0.f, ssq2 = 0.f;                  // BN = 256: the thread's second channel, sc + 128
     uint32_t tl = 0;
@@ -310,6 +311,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
       ptx::named_barrier(1, 128);
       if (!*epi_go) break;
+      const bool inside = w0 + rw < p.W && h0 + rh < p.H;  // a pixel over the edge is staged as zero: it adds nothing to the sums
 #pragma unroll
       for (int j = 0; j < BN / 32; ++j) {
         uint32_t v[32];
@@ -331,7 +333,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             const __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
             w[e] = *reinterpret_cast<const uint32_t*>(&b2);
           }
-          *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (r & 7)) * 16)) = make_uint4(w[0], w[1], w[2], w[3]);
+          *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (r & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
         }
       }
       ptx::tc_fence_before();
@@ -405,6 +407,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const int et = threadIdx.x - 64;
       const int lg = warp & 3;
       const int r = lg * 32 + lane;
+      const int rw = r % p.BW, rh = (r / p.BW) % p.BH, img = r / (p.BW * p.BH);  // place of the thread's pixel in its tile
       uint32_t tl = 0;
       for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
         const TileAt at = tile_at(t, p.tg);
@@ -415,9 +418,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         if (et == 0) *epi_go = *abort_flag ? 0 : 1;
         ptx::named_barrier(1, 128);
         if (!*epi_go) break;
-        const int img = r / (p.BW * p.BH);  // image of this pixel inside a multi-image tile
-        const bool img_ok = n + img < p.N;
-        bf16* dst = p.out + (((size_t)(n + img) * p.H + h0 + (r / p.BW) % p.BH) * p.W + w0 + r % p.BW) * p.Cout;
+        const bool img_ok = n + img < p.N && w0 + rw < p.W && h0 + rh < p.H;
+        bf16* dst = p.out + (((size_t)(n + img) * p.H + h0 + rh) * p.W + w0 + rw) * p.Cout;
 #pragma unroll
         for (int j = 0; j < BN / 16; ++j) {
           uint32_t v[16];
@@ -1828,20 +1830,43 @@ int sm_count() {
 // mode 0: main forward (y + statistics), 1: aux forward (bias + ReLU, Cout = F), 2: aux input gradient
 // (Cin = F <= 64 and a multiple of 8, Cout a multiple of 64, mirrored MN-major weights).
 // H, W: OUTPUT size (equal to the input size for stride 1).
-// Pixel tile of 128 output pixels: a BW x BH patch of one image, or (per-tap mode only) BI whole images
-// of a small feature map.  Returns false when the size does not tile.
-bool pick_tile(int H, int W, bool allow_multi, int* BW, int* BH, int* BI) {
+// Pixel tile of 128 output pixels: a BW x BH patch of one image, or (per-tap mode only) of BI images at once.
+// Sizes that no patch divides (14, 7, 28, odd ones) take the per-tap mode with the powers of two BW * BH * BI = 128 that cover
+// the N x H x W pixels with the fewest tiles (7x7 maps: one pixel of 128 images; 14x14: 2x2 pixels of 32): loads beyond an
+// edge read zeros, stores are clipped, the epilogue zeroes what hangs over.  Where several cover equally well the one with
+// the largest patch is taken: neighbouring taps then find most of their pixels in L2.
+void pick_tile(int N, int H, int W, int* BW, int* BH, int* BI) {
   const int cand[3][2] = {{16, 8}, {32, 4}, {8, 16}};
   for (auto& c : cand)
     if (W % c[0] == 0 && H % c[1] == 0) {
       *BW = c[0]; *BH = c[1]; *BI = 1;
-      return true;
+      return;
     }
-  if (allow_multi && W * H <= 64 && 128 % (W * H) == 0 && (W & (W - 1)) == 0) {  // 8x8, 4x4, 2x2, 8x4, 1x1 ...
+  if (W * H <= 64 && 128 % (W * H) == 0 && (W & (W - 1)) == 0) {  // 8x8, 4x4, 2x2, 8x4, 1x1 ...
     *BW = W; *BH = H; *BI = 128 / (W * H);
-    return true;
+    return;
   }
-  return false;
+  long best = -1;
+  for (int bi = 1; bi <= 128; bi *= 2)
+    for (int bw = 1; bw * bi <= 128; bw *= 2) {
+      const int bh = 128 / (bi * bw);
+      const long tiles = (long)((N + bi - 1) / bi) * ((H + bh - 1) / bh) * ((W + bw - 1) / bw);
+      if (best < 0 || tiles < best) {
+        best = tiles;
+        *BW = bw; *BH = bh; *BI = bi;
+      }
+    }
+}
+bool tiles_exactly(int H, int W, int BW, int BH) { return W % BW == 0 && H % BH == 0; }
+// Whether a problem goes to the tensor cores at all.  Maps that tile exactly always do; the others from 8192 output pixels on
+// (64 tiles).  Below that a layer is a few launch-sized kernels either way, its gradients hang on a few thousand ReLU
+// decisions, and the CUDA-core kernels' fp32 sums (0.01 % of the bf16 outputs off the nearest value, against 0.04 - 0.13 %
+// here, 256 channels at 14x14) are worth more than the time: 0.9 % -> 6 % of a gradient's norm moves between the two on 648
+// pixels, 1 % on 12 000.
+bool tc_size_ok(int N, int H, int W) {
+  int BW, BH, BI;
+  pick_tile(N, H, W, &BW, &BH, &BI);
+  return tiles_exactly(H, W, BW, BH) && (BI == 1 || W * H * BI == 128) ? true : (long)N * H * W >= 8192;
 }
 
 // ybuf = 1 reserves the y2 tile of the fused BatchNorm-backward sums (as large as the output staging)
@@ -1850,8 +1875,8 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   if (stride == 2 && (epi != 0 || Cin % 64)) return pl;
   if (epi == 2 ? (Cin > 64 || Cin % 8 || Cout % 64) : (Cin % 64 != 0)) return pl;
   if (epi == 0 ? (Cout % 64 != 0) : epi == 1 ? (Cout > 64) : false) return pl;
-  if (!pick_tile(H, W, true, &pl.BW, &pl.BH, &pl.BI)) return pl;
-  pl.PT = (stride == 2 || pl.BI > 1) ? 1 : 0;
+  pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
+  pl.PT = (stride == 2 || pl.BI > 1 || pl.BW < 8 || pl.BW > 32 || !tiles_exactly(H, W, pl.BW, pl.BH)) ? 1 : 0;
   if (epi == 0 && Cout % 256 == 0) pl.PT = 1;  // 256-wide instructions need the per-tap form (one tap of weights per stage)
   pl.BN = epi != 1 ? (Cout % 128 == 0 ? 128 : 64) : (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64);
   if (epi == 0 && pl.PT && Cout % 256 == 0) pl.BN = 256;  // per-tap form: weights of one tap and 256 channels are 32 KB a stage
@@ -1869,7 +1894,8 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   pl.smem = (size_t)st * stage + fixed;
   pl.parts = pl.BN >= 128 ? 1 : 128 / pl.BN;
   const int n_tiles = epi != 1 ? Cout / pl.BN : 1;
-  const long total = (long)((N + pl.BI - 1) / pl.BI) * (H / pl.BH) * (W / pl.BW) * n_tiles;
+  const long total = (long)((N + pl.BI - 1) / pl.BI) * ((H + pl.BH - 1) / pl.BH) * ((W + pl.BW - 1) / pl.BW) * n_tiles;
+  if (total >= (1l << 30)) return pl;
   long g = sm_count();
   g -= g % n_tiles;  // every CTA keeps one channel tile for its whole life
   if (g < n_tiles) g = n_tiles;
@@ -2074,7 +2100,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   }
   FwdParams p{};
   p.N = N; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout;
-  p.BW = pl.BW; p.BH = pl.BH; p.tiles_w = W / pl.BW; p.tiles_h = H / pl.BH; p.n_tiles = epi != 1 ? Cout / pl.BN : 1;
+  p.BW = pl.BW; p.BH = pl.BH; p.tiles_w = (W + pl.BW - 1) / pl.BW; p.tiles_h = (H + pl.BH - 1) / pl.BH; p.n_tiles = epi != 1 ? Cout / pl.BN : 1;
   p.bias = bias; p.out = (bf16*)y;
   p.total_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w * p.n_tiles;
   p.stride = stride; p.BI = pl.BI;
@@ -2131,8 +2157,8 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
   WgPlan pl{};
   if (Cin % 64 || (stride == 2 && aux)) return pl;
   if (aux ? (Cout > 64 || Cout % 8) : (Cout % 64 != 0)) return pl;
-  if (!pick_tile(H, W, true, &pl.BW, &pl.BH, &pl.BI)) return pl;
-  pl.PT = (stride == 2 || pl.BI > 1) ? 1 : 0;
+  pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
+  pl.PT = (stride == 2 || pl.BI > 1 || pl.BW < 8 || pl.BW > 32 || !tiles_exactly(H, W, pl.BW, pl.BH)) ? 1 : 0;
   pl.NB = aux ? (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64) : 64;
   if (!aux && pl.PT) pl.NB = Cout % 256 == 0 ? 256 : Cout % 128 == 0 ? 128 : 64;  // per-tap form: as wide an instruction as Cout allows
   pl.GX = (aux && !pl.PT && pl.NB <= 32) ? 1 : 0;  // few filters: one instruction per 16 pixels with the gradient on the M side
@@ -2145,7 +2171,8 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
   pl.smem = (size_t)pl.stages * stage + 1024 + 1024;
   if (pl.smem > 232448) return pl;
   const int blocks = (Cin / 64) * (aux ? 1 : Cout / pl.NB);
-  const long pix_tiles = (long)((N + pl.BI - 1) / pl.BI) * (H / pl.BH) * (W / pl.BW);
+  const long pix_tiles = (long)((N + pl.BI - 1) / pl.BI) * ((H + pl.BH - 1) / pl.BH) * ((W + pl.BW - 1) / pl.BW);
+  if (pix_tiles >= (1l << 30)) return pl;
   const int groups = pl.PT ? 3 : 1;  // kernel rows handled by separate CTAs
   // pixel splits per (chunk pair, kernel-row group): the count whose CTAs fill whole waves of SMs best (smallest on ties),
   // e.g. 512 -> 512 channels with three row groups: 192 units -> 3 splits = 576 CTAs = 3.9 waves instead of 1.3
@@ -2226,7 +2253,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
   if ((rc = make_map4(&mg, dy, dg, bg)) != NF_OK) return rc;
   WgParams p{};
   p.N = N; p.H = H; p.W = W; p.Cin = Cin; p.Cout = Cout; p.BW = pl.BW; p.BH = pl.BH;
-  p.tiles_w = W / pl.BW; p.tiles_h = H / pl.BH; p.pix_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w;
+  p.tiles_w = (W + pl.BW - 1) / pl.BW; p.tiles_h = (H + pl.BH - 1) / pl.BH; p.pix_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w;
   p.stride = stride; p.BI = pl.BI;
   p.tg = tile_grid(1, p.tiles_w, p.tiles_h);
   p.ci_chunks = Cin / 64; p.co_chunks = aux ? 1 : Cout / pl.NB; p.splits = pl.splits; p.part = part; p.status = status;
@@ -2262,12 +2289,14 @@ void nf_tc_select(nf_layer* L) {
   // batch is copied once per step into a 64-channel zero-padded tensor (as large as the layer's output) and the main conv
   // then runs on the ordinary 64-channel kernels.  21 times the arithmetic, a third of the time (VGG first layer at 64 x 64,
   // 1260 images: forward + weight gradient 2.6 ms -> 0.9 ms including the copy).
-  if (L->Cin <= 8 && plan_fwd(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok &&
+  const bool main_ok = tc_size_ok(L->o.N, L->Ho, L->Wo), aux_ok = tc_size_ok(L->o.N, L->Ha, L->Wa);
+  if (L->Cin <= 8 && main_ok && plan_fwd(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok &&
       plan_wgrad(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok)
     L->cin_pad = 64;
   const int Cin = L->cin_pad ? L->cin_pad : L->Cin;
-  if (plan_fwd(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[0] = 1;
-  if (plan_wgrad(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[1] = 1;
+  if (main_ok && plan_fwd(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[0] = 1;
+  if (main_ok && plan_wgrad(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[1] = 1;
+  if (!aux_ok) return;
   if (wide_aux(L)) {  // more than 64 filters: the aux conv runs on the kernels of the main conv
     if (plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok) L->fam[2] = 1;
     if (plan_wgrad(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok && plan_fwd(L->Ha, L->Wa, L->F, L->Cout, L->o.N, 0).ok) L->fam[3] = 1;
@@ -2440,6 +2469,7 @@ int nf_tc_aux_wgrad(nf_layer* L, const void* a) {
 }
 
 size_t nf_tc_conv3x3_wgrad_scratch_floats(int N, int H, int W, int Cin, int Cout, int stride) {
+  if (!tc_size_ok(N, (H - 1) / stride + 1, (W - 1) / stride + 1)) return 0;
   const WgPlan pl = plan_wgrad((H - 1) / stride + 1, (W - 1) / stride + 1, Cin, Cout, N, 0, stride);
   return pl.ok ? pl.part_floats : 0;
 }
@@ -2455,6 +2485,7 @@ int nf_tc_op_status_ptr(int32_t** out) {
 }
 
 int nf_tc_conv3x3_forward(const void* x, const void* w, int N, int H, int W, int Cin, int Cout, int stride, void* y) {
+  if (!tc_size_ok(N, (H - 1) / stride + 1, (W - 1) / stride + 1)) return NF_EUNSUPPORTED;
   int32_t* st = nullptr;
   if (nf_tc_op_status_ptr(&st) != NF_OK) return NF_ECUDA;
   int nb = 0;
@@ -2463,6 +2494,7 @@ int nf_tc_conv3x3_forward(const void* x, const void* w, int N, int H, int W, int
 
 int nf_tc_conv3x3_wgrad(const void* x, const void* g, int N, int H, int W, int Cin, int Cout, int stride, float* part,
                         size_t part_floats, float* dw) {
+  if (!tc_size_ok(N, (H - 1) / stride + 1, (W - 1) / stride + 1)) return NF_EUNSUPPORTED;
   int32_t* st = nullptr;
   if (nf_tc_op_status_ptr(&st) != NF_OK) return NF_ECUDA;
   return run_wgrad(N, H, W, Cin, Cout, x, g, part, part_floats, dw, st, 0, stride);
