@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(256) conv_direct_kernel(const T* __restrict__ 
                                                           const T* __restrict__ w, long ws_tap, long ws_co,
                                                           long ws_ci, int flip, const float* __restrict__ bias,
                                                           int relu, int s, int Co, int Ho, int Wo, T* __restrict__ y) {
+  nf_pdl_begin();
   __shared__ float xs[3][CT_P * 2 + 2][CT_CI];
   __shared__ float wsm[9][CT_CO][CT_CI + 1];
   const int wt = (Wo + CT_P - 1) / CT_P, ct = (Co + CT_CO - 1) / CT_CO;
@@ -73,6 +74,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) wgrad_direct_kernel(const T* __restrict__ x, int N, int H, int W, int Ci,
                                                            const T* __restrict__ g, int Co, int s, int Ho, int Wo,
                                                            int splits, float* __restrict__ part) {
+  nf_pdl_begin();
   __shared__ float gs[WG_J][16];
   __shared__ float xs[3][WG_J * 2 + 2][16];
   const int cit = (Ci + 15) / 16, cot = (Co + 15) / 16;
@@ -123,6 +125,7 @@ __global__ void __launch_bounds__(256) wgrad_direct_kernel(const T* __restrict__
 // out[i] = sum over the splits of part[k][i]: 32 consecutive elements x 8 lanes over the splits per block; a lane adds its
 // splits in index order with four loads in flight, the lane sums are added in lane order (fixed order, no atomics)
 __global__ void __launch_bounds__(256) sum_splits_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
+  nf_pdl_begin();
   __shared__ float sm[8][33];
   const size_t i = (size_t)blockIdx.x * 32 + threadIdx.x;
   float s = 0.f;
@@ -173,6 +176,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) conv_smallc_kernel(const T* __restrict__ x, int N, int H, int W, int Ci,
                                                           const T* __restrict__ w, int s, int Co, int Ho, int Wo,
                                                           T* __restrict__ y) {
+  nf_pdl_begin();
   extern __shared__ float wsm[];  // [tap][ci][co]
   for (int e = threadIdx.y * 32 + threadIdx.x; e < 9 * Ci * Co; e += blockDim.x * blockDim.y) {
     const int co = e % Co, ci = (e / Co) % Ci, t = e / (Co * Ci);
@@ -221,6 +225,7 @@ template <typename T>
 __global__ void __launch_bounds__(512) wgrad_smallc_kernel(const T* __restrict__ x, int N, int H, int W, int Ci,
                                                            const T* __restrict__ g, int Co, int s, int Ho, int Wo,
                                                            int splits, float* __restrict__ part) {
+  nf_pdl_begin();
   extern __shared__ float sm[];           // xrow[(R-1)*s + 3][W + 2][4]  then  red[4][Co][36]
   constexpr int R = 4;                    // output rows staged per synchronisation
   const int xr = (R - 1) * s + 3;
@@ -287,10 +292,10 @@ int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void*
     if (nblk_ > 148 * 16) nblk_ = 148 * 16;
     const unsigned grid = (unsigned)nblk_;
     if (dtype == NF_F32)
-      conv_smallc_kernel<float><<<grid, blk, sm, g_nf_stream>>>((const float*)x, N, H, W, Ci, (const float*)w,
+      nf_launch(conv_smallc_kernel<float>, grid, blk, sm, (const float*)x, N, H, W, Ci, (const float*)w,
                                                                                    stride, Co, Ho, Wo, (float*)y);
     else
-      conv_smallc_kernel<bf16><<<grid, blk, sm, g_nf_stream>>>((const bf16*)x, N, H, W, Ci, (const bf16*)w,
+      nf_launch(conv_smallc_kernel<bf16>, grid, blk, sm, (const bf16*)x, N, H, W, Ci, (const bf16*)w,
                                                                                   stride, Co, Ho, Wo, (bf16*)y);
     NF_LAUNCHED();
     return NF_OK;
@@ -298,10 +303,10 @@ int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void*
   const long blocks = (long)N * Ho * ((Wo + CT_P - 1) / CT_P) * ((Co + CT_CO - 1) / CT_CO);
   if (blocks <= 0 || blocks > 0x7fffffffL) return NF_EUNSUPPORTED;
   if (dtype == NF_F32)
-    conv_direct_kernel<float><<<(unsigned)blocks, 256, 0, g_nf_stream>>>(
+    nf_launch(conv_direct_kernel<float>, (unsigned)blocks, 256, 0, 
         (const float*)x, N, H, W, Ci, (const float*)w, ws_tap, ws_co, ws_ci, flip, bias, relu, stride, Co, Ho, Wo, (float*)y);
   else
-    conv_direct_kernel<bf16><<<(unsigned)blocks, 256, 0, g_nf_stream>>>(
+    nf_launch(conv_direct_kernel<bf16>, (unsigned)blocks, 256, 0, 
         (const bf16*)x, N, H, W, Ci, (const bf16*)w, ws_tap, ws_co, ws_ci, flip, bias, relu, stride, Co, Ho, Wo, (bf16*)y);
   NF_LAUNCHED();
   return NF_OK;
@@ -335,25 +340,25 @@ int nf_k_wgrad(int dtype, const void* x, int N, int H, int W, int Ci, const void
       attr_done = true;
     }
     if (dtype == NF_F32)
-      wgrad_smallc_kernel<float><<<splits, blk, sm, g_nf_stream>>>((const float*)x, N, H, W, Ci, (const float*)g, Co, stride, Ho, Wo,
+      nf_launch(wgrad_smallc_kernel<float>, splits, blk, sm, (const float*)x, N, H, W, Ci, (const float*)g, Co, stride, Ho, Wo,
                                                                  splits, part);
     else
-      wgrad_smallc_kernel<bf16><<<splits, blk, sm, g_nf_stream>>>((const bf16*)x, N, H, W, Ci, (const bf16*)g, Co, stride, Ho, Wo,
+      nf_launch(wgrad_smallc_kernel<bf16>, splits, blk, sm, (const bf16*)x, N, H, W, Ci, (const bf16*)g, Co, stride, Ho, Wo,
                                                                 splits, part);
     NF_LAUNCHED();
-    sum_splits_kernel<<<(unsigned)((n + 31) / 32), dim3(32, 8), 0, g_nf_stream>>>(part, splits, n, dw);
+    nf_launch(sum_splits_kernel, (unsigned)((n + 31) / 32), dim3(32, 8), 0, part, splits, n, dw);
     NF_LAUNCHED();
     return NF_OK;
   }
   const unsigned blocks = (unsigned)(((Ci + 15) / 16) * ((Co + 15) / 16) * splits);
   if (dtype == NF_F32)
-    wgrad_direct_kernel<float><<<blocks, 256, 0, g_nf_stream>>>((const float*)x, N, H, W, Ci, (const float*)g, Co,
+    nf_launch(wgrad_direct_kernel<float>, blocks, 256, 0, (const float*)x, N, H, W, Ci, (const float*)g, Co,
                                                                 stride, Ho, Wo, splits, part);
   else
-    wgrad_direct_kernel<bf16><<<blocks, 256, 0, g_nf_stream>>>((const bf16*)x, N, H, W, Ci, (const bf16*)g, Co,
+    nf_launch(wgrad_direct_kernel<bf16>, blocks, 256, 0, (const bf16*)x, N, H, W, Ci, (const bf16*)g, Co,
                                                                stride, Ho, Wo, splits, part);
   NF_LAUNCHED();
-  sum_splits_kernel<<<(unsigned)((n + 31) / 32), dim3(32, 8), 0, g_nf_stream>>>(part, splits, n, dw);
+  nf_launch(sum_splits_kernel, (unsigned)((n + 31) / 32), dim3(32, 8), 0, part, splits, n, dw);
   NF_LAUNCHED();
   return NF_OK;
 }

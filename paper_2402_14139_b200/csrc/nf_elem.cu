@@ -61,6 +61,7 @@ struct BnBwdFn {  // (dz, dz*xhat)
 template <typename T, typename Fn>
 __global__ void __launch_bounds__(256) channel_reduce_kernel(const T* __restrict__ s0, const T* __restrict__ s1, size_t P,
                                                              int C, Fn fn, float* __restrict__ red) {
+  nf_pdl_begin();
   __shared__ float sm[2][256];
   const int lanes = pow2ceil_cap256(C), planes = 256 / lanes;
   const int lc = threadIdx.x % lanes, pl = threadIdx.x / lanes;
@@ -133,6 +134,7 @@ __device__ __forceinline__ void reduce_partials32(const float* __restrict__ red,
 __global__ void bn_finalize_kernel(const float* __restrict__ red, int nb, int C, double M, const float* __restrict__ gamma,
                                    const float* __restrict__ beta, float eps, float bnm, float* scale, float* shift,
                                    float* mu, float* invstd, float* rmean, float* rvar) {
+  nf_pdl_begin();
   double S, Q;
   reduce_partials32(red, nb, C, S, Q);
   const int c = blockIdx.x * 32 + threadIdx.x;
@@ -156,6 +158,7 @@ __global__ void bn_finalize_kernel(const float* __restrict__ red, int nb, int C,
 // Data-parallel BatchNorm: a rank turns its per-block partials into per-channel totals (fp64, [2][C]) that the
 // ranks add up; the statistics and the backward sums are then finished from the totals of the whole batch.
 __global__ void partial_totals_kernel(const float* __restrict__ red, int nb, int C, double* __restrict__ tot) {
+  nf_pdl_begin();
   double S, Q;
   reduce_partials32(red, nb, C, S, Q);
   const int c = blockIdx.x * 32 + threadIdx.x;
@@ -167,6 +170,7 @@ __global__ void partial_totals_kernel(const float* __restrict__ red, int nb, int
 __global__ void bn_finalize_tot_kernel(const double* __restrict__ tot, int C, double M, const float* __restrict__ gamma,
                                        const float* __restrict__ beta, float eps, float bnm, float* scale, float* shift, float* mu,
                                        float* invstd, float* rmean, float* rvar) {
+  nf_pdl_begin();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   const double m = tot[c] / M;
@@ -185,6 +189,7 @@ __global__ void bn_finalize_tot_kernel(const double* __restrict__ tot, int C, do
 // the gradients of gamma and beta are divided by the number of ranks: the sum over ranks that follows restores them
 __global__ void bn_bwd_finalize_tot_kernel(const double* __restrict__ tot, int C, double inv_world, float* sdz, float* sdzx, float* gg,
                                            float* gb) {
+  nf_pdl_begin();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   sdz[c] = (float)tot[c];
@@ -195,6 +200,7 @@ __global__ void bn_bwd_finalize_tot_kernel(const double* __restrict__ tot, int C
 
 __global__ void bn_eval_coeffs_kernel(int C, const float* gamma, const float* beta, float eps, const float* rmean,
                                       const float* rvar, float* scale, float* shift) {
+  nf_pdl_begin();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= C) return;
   const double is = 1.0 / sqrt((double)rvar[c] + (double)eps);
@@ -206,6 +212,7 @@ __global__ void bn_eval_coeffs_kernel(int C, const float* gamma, const float* be
 template <typename T>
 __global__ void bn_apply_kernel(const T* __restrict__ y, int Ho, int Wo, int C, int pool, const float* __restrict__ scale,
                                 const float* __restrict__ shift, size_t total, T* __restrict__ out, const T* __restrict__ skip) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int c = (int)(e % C);
@@ -236,6 +243,7 @@ __device__ __forceinline__ void bin_range(int u, int H, int& lo, int& hi) {
 // the same for bins of at most 16 pixels: one thread per output p[n][f*4 + bin] (consecutive threads = consecutive channels)
 template <typename T>
 __global__ void avgpool_small_kernel(const T* __restrict__ h, int Ha, int Wa, int F, size_t total, float* __restrict__ p) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int f = (int)(e % F), bin = (int)((e / F) % 4);
@@ -251,6 +259,7 @@ __global__ void avgpool_small_kernel(const T* __restrict__ h, int Ha, int Wa, in
 
 template <typename T>
 __global__ void __launch_bounds__(256) avgpool_kernel(const T* __restrict__ h, int Ha, int Wa, int F, float* __restrict__ p) {
+  nf_pdl_begin();
   __shared__ float sm[256];
   const int n = blockIdx.x / 4, bin = blockIdx.x % 4, u = bin / 2, v = bin % 2;
   int i0, i1, j0, j1;
@@ -284,6 +293,7 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const T* __restrict__ h, i
 template <typename T>
 __global__ void __launch_bounds__(256) auxmax_kernel(const T* __restrict__ h, int Ha, int Wa, int F, float* __restrict__ p,
                                                      int32_t* __restrict__ parg) {
+  nf_pdl_begin();
   __shared__ float sv[256];
   __shared__ int si[256];
   const int n = blockIdx.x / 4, bin = blockIdx.x % 4, u = bin / 2, v = bin % 2;
@@ -325,6 +335,7 @@ __global__ void __launch_bounds__(256) auxmax_kernel(const T* __restrict__ h, in
 template <typename T>
 __global__ void dh_max_kernel(const T* __restrict__ h, const float* __restrict__ dp, const int32_t* __restrict__ parg, int Ha, int Wa,
                               int F, size_t total, T* __restrict__ dh) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int f = (int)(e % F);
@@ -360,6 +371,7 @@ __global__ void __launch_bounds__(256) fc_ce_kernel(const float* __restrict__ p,
                                                     float* __restrict__ logits, float* __restrict__ dlogits,
                                                     float* __restrict__ dp, float* __restrict__ lossn, int32_t* status,
                                                     int loss_kind, int n_scale) {
+  nf_pdl_begin();
   extern __shared__ float dyn[];
   float* ps = dyn;          // [D]
   float* ls = dyn + D;      // [K]
@@ -448,6 +460,7 @@ __global__ void __launch_bounds__(256) fc_ce_kernel(const float* __restrict__ p,
 __global__ void __launch_bounds__(256) fc_predict_kernel(const float* __restrict__ p, int D, int K, const float* __restrict__ Wf,
                                                          const float* __restrict__ bf, float* __restrict__ logits,
                                                          int32_t* __restrict__ pred) {
+  nf_pdl_begin();
   extern __shared__ float dyn[];
   float* ps = dyn;
   __shared__ float bv[256];
@@ -482,6 +495,7 @@ __global__ void __launch_bounds__(256) fc_wgrad_kernel(const float* __restrict__
                                                        const float* __restrict__ lossn, int N, int D, int K,
                                                        float* __restrict__ gWf, float* __restrict__ gbf,
                                                        float* __restrict__ loss_out, int32_t* status, int n_scale) {
+  nf_pdl_begin();
   // Sums over the batch run as four interleaved chains (samples n % 4) that are combined in a fixed order, and the
   // two scalar sums are spread over a warp: the serial chains of one load per sample were pure latency.
   const int k = blockIdx.x, t = threadIdx.x;
@@ -522,6 +536,7 @@ __global__ void __launch_bounds__(256) fc_wgrad_kernel(const float* __restrict__
 template <typename T>
 __global__ void dh_kernel(const T* __restrict__ h, const float* __restrict__ dp, int Ha, int Wa, int F, size_t total,
                           T* __restrict__ dh) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int f = (int)(e % F);
@@ -548,6 +563,7 @@ __global__ void dh_kernel(const T* __restrict__ h, const float* __restrict__ dp,
 }
 
 __global__ void sum_partials_kernel(const float* __restrict__ red, int nb, int C, int which, float* __restrict__ out) {
+  nf_pdl_begin();
   double S, Q;
   reduce_partials32(red, nb, C, S, Q);
   const int c = blockIdx.x * 32 + threadIdx.x;
@@ -557,6 +573,7 @@ __global__ void sum_partials_kernel(const float* __restrict__ red, int nb, int C
 
 __global__ void bn_bwd_finalize_kernel(const float* __restrict__ red, int nb, int C, float* sdz, float* sdzx, float* gg,
                                        float* gb) {
+  nf_pdl_begin();
   double a, b;
   reduce_partials32(red, nb, C, a, b);
   const int c = blockIdx.x * 32 + threadIdx.x;
@@ -574,6 +591,7 @@ __global__ void bn_bwd_apply_kernel(const T* __restrict__ y, const T* __restrict
                                     const float* __restrict__ mu, const float* __restrict__ invstd,
                                     const float* __restrict__ sdz, const float* __restrict__ sdzx, float invM,
                                     size_t total, T* __restrict__ dy, const T* __restrict__ skip) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int c = (int)(e % C);
@@ -589,6 +607,7 @@ template <typename T>
 __global__ void write_dz_kernel(const T* __restrict__ y, const T* __restrict__ da, int Ho, int Wo, int C, int pool,
                                 const float* __restrict__ scale, const float* __restrict__ shift, const T* __restrict__ skip,
                                 size_t total, T* __restrict__ dz) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int c = (int)(e % C);
@@ -597,6 +616,7 @@ __global__ void write_dz_kernel(const T* __restrict__ y, const T* __restrict__ d
 
 // xpad[p][0..Cp) = (x[p][0..C), 0, ...): one thread per 8-channel chunk (16 bytes) of the padded pixel, C <= 8
 __global__ void pad_channels_kernel(const bf16* __restrict__ x, size_t P, int C, int Cp8, uint4* __restrict__ xpad) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= P * Cp8) return;
   const size_t p = e / Cp8;
@@ -609,12 +629,14 @@ __global__ void pad_channels_kernel(const bf16* __restrict__ x, size_t P, int C,
   xpad[e] = v;
 }
 __global__ void pad_weights_kernel(const bf16* __restrict__ w, size_t rows, int C, int Cp, bf16* __restrict__ wpad) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= rows * Cp) return;
   const int c = (int)(e % Cp);
   wpad[e] = c < C ? w[(e / Cp) * C + c] : __float2bfloat16(0.f);
 }
 __global__ void unpad_grad_kernel(const float* __restrict__ gwpad, size_t rows, int C, int Cp, float* __restrict__ gw) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= rows * C) return;
   gw[e] = gwpad[(e / C) * Cp + e % C];
@@ -625,6 +647,7 @@ __global__ void unpad_grad_kernel(const float* __restrict__ gwpad, size_t rows, 
 // gradient, 16-byte stores of value and momentum, one 8-byte store of the four bf16 copies.  Blocks are dealt to arenas
 // through the table of first-block indices.
 __global__ void __launch_bounds__(256) sgd_multi_kernel(const SgdTable tb, float lr, float mu) {
+  nf_pdl_begin();
   int a = 0;
   while (a + 1 < tb.count && (int)blockIdx.x >= tb.first_block[a + 1]) ++a;
   const size_t i4 = (size_t)(blockIdx.x - tb.first_block[a]) * blockDim.x + threadIdx.x;
@@ -642,6 +665,7 @@ __global__ void __launch_bounds__(256) sgd_multi_kernel(const SgdTable tb, float
 }
 
 __global__ void shadow_kernel(const float* __restrict__ val, bf16* __restrict__ shadow, size_t n) {
+  nf_pdl_begin();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) shadow[i] = __float2bfloat16_rn(val[i]);
 }
@@ -651,6 +675,7 @@ __global__ void shadow_kernel(const float* __restrict__ val, bf16* __restrict__ 
 __global__ void gather_kernel(const uint4* __restrict__ cache, const int32_t* __restrict__ cache_labels, int cache_rows,
                               const int32_t* __restrict__ idx, int count, size_t row16, uint4* __restrict__ out,
                               int32_t* __restrict__ out_labels, int32_t* __restrict__ status) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (size_t)count * row16) return;
   const size_t r = e / row16, k = e % row16;
@@ -688,6 +713,7 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
 __global__ void __launch_bounds__(256) bn_apply_vec_kernel(const uint4* __restrict__ y, int C8, const float* __restrict__ scale,
                                                            const float* __restrict__ shift, size_t total8,
                                                            uint4* __restrict__ out) {
+  nf_pdl_begin();
   extern __shared__ float cs[];  // scale[C], shift[C]
   const int C = C8 * 8;
   for (int i = threadIdx.x; i < C; i += 256) {
@@ -709,6 +735,7 @@ __global__ void __launch_bounds__(256) bn_apply_vec_kernel(const uint4* __restri
 // per-thread constants variant (256 % C8 == 0)
 __global__ void __launch_bounds__(256) bn_apply_vec2_kernel(const uint4* __restrict__ y, int C8, const float* __restrict__ scale,
                                                             const float* __restrict__ shift, size_t total8, uint4* __restrict__ out) {
+  nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8];
 #pragma unroll
@@ -741,6 +768,7 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __r
                                                                 size_t P, int C8, const float* __restrict__ scale,
                                                                 const float* __restrict__ shift, const float* __restrict__ mu,
                                                                 const float* __restrict__ invstd, float* __restrict__ red) {
+  nf_pdl_begin();
   __shared__ float sm[16][256];
   const int C = C8 * 8;
   const int planes = 256 / C8, g = threadIdx.x % C8, pl = threadIdx.x / C8;
@@ -808,6 +836,7 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec_kernel(const uint4* __re
                                                                const float* __restrict__ mu, const float* __restrict__ invstd,
                                                                const float* __restrict__ sdz, const float* __restrict__ sdzx,
                                                                float invM, size_t total8, uint4* __restrict__ dy) {
+  nf_pdl_begin();
   extern __shared__ float cs[];  // per channel: scale, shift, mu, invstd, sdz/M, sdzx/M
   const int C = C8 * 8;
   for (int i = threadIdx.x; i < C; i += 256) {
@@ -858,6 +887,7 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const uint4* __r
                                                                 const float* __restrict__ mu, const float* __restrict__ invstd,
                                                                 const float* __restrict__ sdz, const float* __restrict__ sdzx,
                                                                 float invM, size_t total8, uint4* __restrict__ dy) {
+  nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8], K1[8], K0[8];
 #pragma unroll
@@ -903,6 +933,7 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const uint4* __r
 // partial sums of (v, v^2) of a bf16 tensor; same layout of partials as channel_reduce_kernel
 __global__ void __launch_bounds__(256) channel_sums_vec_kernel(const uint4* __restrict__ src, size_t P, int C8,
                                                                float* __restrict__ red) {
+  nf_pdl_begin();
   __shared__ float sm[16][256];
   const int C = C8 * 8;
   const int planes = 256 / C8, g = threadIdx.x % C8, pl = threadIdx.x / C8;
@@ -939,6 +970,7 @@ __global__ void __launch_bounds__(256) channel_sums_vec_kernel(const uint4* __re
 // thread, fused with the per-filter sum of dh (the aux bias gradient): red[(block*2+0)*F + f].
 __global__ void __launch_bounds__(256) dh_vec_kernel(const uint4* __restrict__ h, const float* __restrict__ dp, int Ha, int Wa,
                                                      int F8, size_t P, uint4* __restrict__ dh, float* __restrict__ red) {
+  nf_pdl_begin();
   __shared__ float sm[8][256];
   const int F = F8 * 8;
   const int planes = 256 / F8, g = threadIdx.x % F8, pl = threadIdx.x / F8;
@@ -999,6 +1031,7 @@ __global__ void __launch_bounds__(256) dh_vec_kernel(const uint4* __restrict__ h
 // average pool, stage 1: partial bin sums over a slice of rows; part[(n*4+bin)*S + s][F]
 __global__ void __launch_bounds__(256) avgpool_part_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, int S,
                                                                float* __restrict__ part) {
+  nf_pdl_begin();
   __shared__ float sm[8][256];
   const int F = F8 * 8;
   const int planes = 256 / F8, g = threadIdx.x % F8, pl = threadIdx.x / F8;
@@ -1048,6 +1081,7 @@ __global__ void __launch_bounds__(256) avgpool_part_vec_kernel(const uint4* __re
 // sums are added in lane order.
 __global__ void __launch_bounds__(256) pool_finish_kernel(const float* __restrict__ part, int th, int tw, int F, float inv_cnt,
                                                           float* __restrict__ p) {
+  nf_pdl_begin();
   __shared__ float sm[256];
   const int n = blockIdx.x >> 2, bin = blockIdx.x & 3, u = bin >> 1, v = bin & 1;
   const int lanes = 256 / F, f = threadIdx.x % F, ln = threadIdx.x / F;
@@ -1081,6 +1115,7 @@ __global__ void __launch_bounds__(256) pool_finish_kernel(const float* __restric
 // stored in bf16; per-block partial sums of the stored values for the bias gradient, laid out as dh_vec_kernel does.
 __global__ void __launch_bounds__(256) dh_mask_vec_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ dp, int Ha, int Wa,
                                                           int F8, size_t P, uint4* __restrict__ dh, float* __restrict__ red) {
+  nf_pdl_begin();
   __shared__ float sm[8][256];
   __shared__ __align__(16) float tab[4][4][64];  // dp / |bin| of up to four images, [image][bin][channel]: 16-byte reads per thread
   const int F = F8 * 8;
@@ -1148,6 +1183,7 @@ __global__ void __launch_bounds__(256) dh_mask_vec_kernel(const uint8_t* __restr
 }
 
 __global__ void avgpool_finish_kernel(const float* __restrict__ part, int N, int F, int S, float inv_cnt, float* __restrict__ p) {
+  nf_pdl_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N * 4 * F) return;
   const int f = e % F, bin = (e / F) % 4, n = e / (4 * F);
@@ -1177,6 +1213,7 @@ __device__ __forceinline__ size_t win_base(size_t q, int Ho, int Wo, int C8) {  
 __global__ void __launch_bounds__(256) bn_apply_pool_vec_kernel(const uint4* __restrict__ y, int Ho, int Wo, int C8,
                                                                 const float* __restrict__ scale, const float* __restrict__ shift,
                                                                 size_t total8, uint4* __restrict__ out) {
+  nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8];
 #pragma unroll
@@ -1221,6 +1258,7 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_pool_vec_kernel(const uint4
                                                                      const float* __restrict__ scale, const float* __restrict__ shift,
                                                                      const float* __restrict__ mu, const float* __restrict__ invstd,
                                                                      float* __restrict__ red) {
+  nf_pdl_begin();
   __shared__ float sm[16][256];
   const int C = C8 * 8;
   const int planes = 256 / C8, g = threadIdx.x % C8, pl = threadIdx.x / C8;
@@ -1269,6 +1307,7 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_pool_vec_kernel(const uint4*
                                                                     const float* __restrict__ invstd, const float* __restrict__ sdz,
                                                                     const float* __restrict__ sdzx, float invM, size_t total8,
                                                                     uint4* __restrict__ dy) {
+  nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8], K1[8], K0[8];
 #pragma unroll
@@ -1326,14 +1365,14 @@ int nf_k_channel_sums(int dtype, const void* src, size_t P, int C, float* red, s
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
   if (vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    channel_sums_vec_kernel<<<nb, 256, 0, g_nf_stream>>>((const uint4*)src, P, C / 8, red);
+    nf_launch(channel_sums_vec_kernel, nb, 256, 0, (const uint4*)src, P, C / 8, red);
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;
   }
   DISPATCH(dtype,
-           (channel_reduce_kernel<float, StatsFn><<<nb, 256, 0, g_nf_stream>>>((const float*)src, nullptr, P, C, StatsFn(), red)),
-           (channel_reduce_kernel<bf16, StatsFn><<<nb, 256, 0, g_nf_stream>>>((const bf16*)src, nullptr, P, C, StatsFn(), red)));
+           (nf_launch(channel_reduce_kernel<float, StatsFn>, nb, 256, 0, (const float*)src, nullptr, P, C, StatsFn(), red)),
+           (nf_launch(channel_reduce_kernel<bf16, StatsFn>, nb, 256, 0, (const bf16*)src, nullptr, P, C, StatsFn(), red)));
   NF_LAUNCHED();
   *nblocks = nb;
   return NF_OK;
@@ -1342,35 +1381,35 @@ int nf_k_channel_sums(int dtype, const void* src, size_t P, int C, float* red, s
 int nf_k_bn_finalize(const float* red, int nblocks, int C, double M, const float* gamma, const float* beta,
                        float eps, float bn_momentum, float* scale, float* shift, float* mu, float* invstd,
                        float* rmean, float* rvar) {
-  bn_finalize_kernel<<<nblk(C, 32), dim3(32, 32), 0, g_nf_stream>>>(red, nblocks, C, M, gamma, beta, eps, bn_momentum, scale,
+  nf_launch(bn_finalize_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, M, gamma, beta, eps, bn_momentum, scale,
                                                             shift, mu, invstd, rmean, rvar);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_partial_totals(const float* red, int nblocks, int C, double* tot) {
-  partial_totals_kernel<<<nblk(C, 32), dim3(32, 32), 0, g_nf_stream>>>(red, nblocks, C, tot);
+  nf_launch(partial_totals_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, tot);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_bn_finalize_tot(const double* tot, int C, double M, const float* gamma, const float* beta, float eps, float bn_momentum,
                            float* scale, float* shift, float* mu, float* invstd, float* rmean, float* rvar) {
-  bn_finalize_tot_kernel<<<nblk(C, 128), 128, 0, g_nf_stream>>>(tot, C, M, gamma, beta, eps, bn_momentum, scale, shift, mu, invstd,
+  nf_launch(bn_finalize_tot_kernel, nblk(C, 128), 128, 0, tot, C, M, gamma, beta, eps, bn_momentum, scale, shift, mu, invstd,
                                                                 rmean, rvar);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_bn_bwd_finalize_tot(const double* tot, int C, int world, float* sdz, float* sdzx, float* ggamma, float* gbeta) {
-  bn_bwd_finalize_tot_kernel<<<nblk(C, 128), 128, 0, g_nf_stream>>>(tot, C, 1.0 / (double)world, sdz, sdzx, ggamma, gbeta);
+  nf_launch(bn_bwd_finalize_tot_kernel, nblk(C, 128), 128, 0, tot, C, 1.0 / (double)world, sdz, sdzx, ggamma, gbeta);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_bn_eval_coeffs(int C, const float* gamma, const float* beta, float eps, const float* rmean,
                           const float* rvar, float* scale, float* shift) {
-  bn_eval_coeffs_kernel<<<nblk(C, 128), 128, 0, g_nf_stream>>>(C, gamma, beta, eps, rmean, rvar, scale, shift);
+  nf_launch(bn_eval_coeffs_kernel, nblk(C, 128), 128, 0, C, gamma, beta, eps, rmean, rvar, scale, shift);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1380,31 +1419,31 @@ int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int po
   const size_t total = (size_t)N * (pool ? Ho / 2 : Ho) * (pool ? Wo / 2 : Wo) * C;
   if (skip) {  // residual layers take the generic kernels
     DISPATCH(dtype,
-             (bn_apply_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)y, Ho, Wo, C, pool, scale, shift, total, (float*)out, (const float*)skip)),
-             (bn_apply_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)y, Ho, Wo, C, pool, scale, shift, total, (bf16*)out, (const bf16*)skip)));
+             (nf_launch(bn_apply_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, Ho, Wo, C, pool, scale, shift, total, (float*)out, (const float*)skip)),
+             (nf_launch(bn_apply_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)y, Ho, Wo, C, pool, scale, shift, total, (bf16*)out, (const bf16*)skip)));
     NF_LAUNCHED();
     return NF_OK;
   }
   if (pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    bn_apply_pool_vec_kernel<<<vec_blocks(total / 8), 256, 0, g_nf_stream>>>((const uint4*)y, Ho, Wo, C / 8, scale, shift, total / 8,
+    nf_launch(bn_apply_pool_vec_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, Ho, Wo, C / 8, scale, shift, total / 8,
                                                                             (uint4*)out);
     NF_LAUNCHED();
     return NF_OK;
   }
   if (vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    bn_apply_vec2_kernel<<<vec_blocks(total / 8), 256, 0, g_nf_stream>>>((const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out);
+    nf_launch(bn_apply_vec2_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out);
     NF_LAUNCHED();
     return NF_OK;
   }
   if (vec_ok(dtype, C, pool)) {
-    bn_apply_vec_kernel<<<vec_blocks(total / 8), 256, 2 * C * sizeof(float), g_nf_stream>>>((const uint4*)y, C / 8, scale, shift,
+    nf_launch(bn_apply_vec_kernel, vec_blocks(total / 8), 256, 2 * C * sizeof(float), (const uint4*)y, C / 8, scale, shift,
                                                                                          total / 8, (uint4*)out);
     NF_LAUNCHED();
     return NF_OK;
   }
   DISPATCH(dtype,
-           (bn_apply_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)y, Ho, Wo, C, pool, scale, shift, total, (float*)out, nullptr)),
-           (bn_apply_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)y, Ho, Wo, C, pool, scale, shift, total, (bf16*)out, nullptr)));
+           (nf_launch(bn_apply_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, Ho, Wo, C, pool, scale, shift, total, (float*)out, nullptr)),
+           (nf_launch(bn_apply_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)y, Ho, Wo, C, pool, scale, shift, total, (bf16*)out, nullptr)));
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1422,9 +1461,9 @@ int nf_k_avgpool_fast(const void* h, int N, int Ha, int Wa, int F, float* part, 
   if ((long)(Ha / 2) * (Wa / 2) <= 16) return NF_EUNSUPPORTED;  // tiny maps: the caller's generic path has a kernel for them
   const int S = nf_k_avgpool_slices(N, Ha, Wa);
   if ((size_t)N * 4 * S * F > part_floats) return NF_EUNSUPPORTED;
-  avgpool_part_vec_kernel<<<N * 4 * S, 256, 0, g_nf_stream>>>((const uint4*)h, Ha, Wa, F / 8, S, part);
+  nf_launch(avgpool_part_vec_kernel, N * 4 * S, 256, 0, (const uint4*)h, Ha, Wa, F / 8, S, part);
   NF_LAUNCHED();
-  avgpool_finish_kernel<<<nblk((size_t)N * 4 * F, 256), 256, 0, g_nf_stream>>>(part, N, F, S, 1.f / (float)((Ha / 2) * (Wa / 2)), p);
+  nf_launch(avgpool_finish_kernel, nblk((size_t)N * 4 * F, 256), 256, 0, part, N, F, S, 1.f / (float)((Ha / 2) * (Wa / 2)), p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1432,7 +1471,7 @@ int nf_k_avgpool_fast(const void* h, int N, int Ha, int Wa, int F, float* part, 
 // dh with the fused aux-bias gradient partials (bf16, F % 8 == 0, even sizes); nblocks partials in red
 int nf_k_pool_finish(const float* part, int N, int th, int tw, int F, float inv_cnt, float* p) {
   if (F < 1 || F > 256) return NF_EUNSUPPORTED;
-  pool_finish_kernel<<<N * 4, 256, 0, g_nf_stream>>>(part, th, tw, F, inv_cnt, p);
+  nf_launch(pool_finish_kernel, N * 4, 256, 0, part, th, tw, F, inv_cnt, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1444,7 +1483,7 @@ int nf_k_dh_mask(const uint8_t* mask, const float* dp, int N, int Ha, int Wa, in
   if (P >= ((size_t)1 << 31)) return NF_EUNSUPPORTED;
   const int nb = nf_k_channel_blocks(P, F);
   if ((size_t)nb * 2 * F > red_floats) return NF_ENOWS;
-  dh_mask_vec_kernel<<<nb, 256, 0, g_nf_stream>>>(mask, dp, Ha, Wa, F / 8, P, (uint4*)dh, red);
+  nf_launch(dh_mask_vec_kernel, nb, 256, 0, mask, dp, Ha, Wa, F / 8, P, (uint4*)dh, red);
   NF_LAUNCHED();
   *nblocks = nb;
   return NF_OK;
@@ -1456,7 +1495,7 @@ int nf_k_dh_fast(const void* h, const float* dp, int N, int Ha, int Wa, int F, v
   const size_t P = (size_t)N * Ha * Wa;
   const int nb = nf_k_channel_blocks(P, F);
   if ((size_t)nb * 2 * F > red_floats) return NF_EUNSUPPORTED;
-  dh_vec_kernel<<<nb, 256, 0, g_nf_stream>>>((const uint4*)h, dp, Ha, Wa, F / 8, P, (uint4*)dh, red);
+  nf_launch(dh_vec_kernel, nb, 256, 0, (const uint4*)h, dp, Ha, Wa, F / 8, P, (uint4*)dh, red);
   NF_LAUNCHED();
   *nblocks = nb;
   return NF_OK;
@@ -1465,13 +1504,13 @@ int nf_k_dh_fast(const void* h, const float* dp, int N, int Ha, int Wa, int F, v
 int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* p) {
   if ((long)((Ha + 1) / 2) * ((Wa + 1) / 2) <= 16) {  // tiny maps (late blocks train at thousands of samples): a thread per output
     const size_t total = (size_t)N * 4 * F;
-    DISPATCH(dtype, (avgpool_small_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)h, Ha, Wa, F, total, p)),
-             (avgpool_small_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)h, Ha, Wa, F, total, p)));
+    DISPATCH(dtype, (nf_launch(avgpool_small_kernel<float>, nblk(total, 256), 256, 0, (const float*)h, Ha, Wa, F, total, p)),
+             (nf_launch(avgpool_small_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)h, Ha, Wa, F, total, p)));
     NF_LAUNCHED();
     return NF_OK;
   }
-  DISPATCH(dtype, (avgpool_kernel<float><<<N * 4, 256, 0, g_nf_stream>>>((const float*)h, Ha, Wa, F, p)),
-           (avgpool_kernel<bf16><<<N * 4, 256, 0, g_nf_stream>>>((const bf16*)h, Ha, Wa, F, p)));
+  DISPATCH(dtype, (nf_launch(avgpool_kernel<float>, N * 4, 256, 0, (const float*)h, Ha, Wa, F, p)),
+           (nf_launch(avgpool_kernel<bf16>, N * 4, 256, 0, (const bf16*)h, Ha, Wa, F, p)));
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1480,13 +1519,14 @@ int nf_k_fc_ce(const float* p, const int32_t* labels, int N, int D, int K, const
                  float* logits, float* dlogits, float* dp, float* lossn, int32_t* status, int loss_kind, int n_scale) {
   const size_t smem = (size_t)(D + K) * sizeof(float);
   if (smem > 40000) return NF_EUNSUPPORTED;
-  fc_ce_kernel<<<N, 256, smem, g_nf_stream>>>(p, labels, N, D, K, Wf, bf, logits, dlogits, dp, lossn, status, loss_kind, n_scale);
+  nf_launch(fc_ce_kernel, N, 256, smem, p, labels, N, D, K, Wf, bf, logits, dlogits, dp, lossn, status, loss_kind, n_scale);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 __global__ void __launch_bounds__(256) count_equal_kernel(const int32_t* __restrict__ a, const int32_t* __restrict__ b, long long n,
                                                           unsigned long long* __restrict__ count) {
+  nf_pdl_begin();
   unsigned c = 0;
   for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += 256LL * gridDim.x) c += a[i] == b[i];
   c = __reduce_add_sync(0xffffffffu, c);
@@ -1495,7 +1535,7 @@ __global__ void __launch_bounds__(256) count_equal_kernel(const int32_t* __restr
 
 int nf_k_count_equal(const int32_t* a, const int32_t* b, long long n, unsigned long long* count) {
   const int blocks = (int)std::min<long long>((n + 255) / 256, 1184);
-  count_equal_kernel<<<blocks, 256, 0, g_nf_stream>>>(a, b, n, count);
+  nf_launch(count_equal_kernel, blocks, 256, 0, a, b, n, count);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1503,20 +1543,21 @@ int nf_k_count_equal(const int32_t* a, const int32_t* b, long long n, unsigned l
 int nf_k_fc_predict(const float* p, int N, int D, int K, const float* Wf, const float* bf, float* logits, int32_t* pred) {
   const size_t smem = (size_t)D * sizeof(float);
   if (smem > 40000) return NF_EUNSUPPORTED;
-  fc_predict_kernel<<<N, 256, smem, g_nf_stream>>>(p, D, K, Wf, bf, logits, pred);
+  nf_launch(fc_predict_kernel, N, 256, smem, p, D, K, Wf, bf, logits, pred);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_fc_wgrad(const float* p, const float* dlogits, const float* lossn, int N, int D, int K, float* gWf,
                     float* gbf, float* loss_out, int32_t* status, int n_scale) {
-  fc_wgrad_kernel<<<K, 256, 0, g_nf_stream>>>(p, dlogits, lossn, N, D, K, gWf, gbf, loss_out, status, n_scale);
+  nf_launch(fc_wgrad_kernel, K, 256, 0, p, dlogits, lossn, N, D, K, gWf, gbf, loss_out, status, n_scale);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 // out[8 - tap][c][f] = w[tap][f][c]: the weights of the input-gradient convolution written as a forward convolution
 __global__ void flip_weights_kernel(const bf16* __restrict__ w, int F, int C, bf16* __restrict__ out) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (size_t)9 * F * C) return;
   const int f = (int)(e % F), c = (int)((e / F) % C), tap = (int)(e / ((size_t)F * C));
@@ -1524,36 +1565,36 @@ __global__ void flip_weights_kernel(const bf16* __restrict__ w, int F, int C, bf
 }
 
 int nf_k_flip_weights(const bf16* w, int F, int C, bf16* out) {
-  flip_weights_kernel<<<nblk((size_t)9 * F * C, 256), 256, 0, g_nf_stream>>>(w, F, C, out);
+  nf_launch(flip_weights_kernel, nblk((size_t)9 * F * C, 256), 256, 0, w, F, C, out);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_auxmax(int dtype, const void* h, int N, int Ha, int Wa, int F, float* p, int32_t* parg) {
-  DISPATCH(dtype, (auxmax_kernel<float><<<N * 4, 256, 0, g_nf_stream>>>((const float*)h, Ha, Wa, F, p, parg)),
-           (auxmax_kernel<bf16><<<N * 4, 256, 0, g_nf_stream>>>((const bf16*)h, Ha, Wa, F, p, parg)));
+  DISPATCH(dtype, (nf_launch(auxmax_kernel<float>, N * 4, 256, 0, (const float*)h, Ha, Wa, F, p, parg)),
+           (nf_launch(auxmax_kernel<bf16>, N * 4, 256, 0, (const bf16*)h, Ha, Wa, F, p, parg)));
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_dh_max(int dtype, const void* h, const float* dp, const int32_t* parg, int N, int Ha, int Wa, int F, void* dh) {
   const size_t total = (size_t)N * Ha * Wa * F;
-  DISPATCH(dtype, (dh_max_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)h, dp, parg, Ha, Wa, F, total, (float*)dh)),
-           (dh_max_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)h, dp, parg, Ha, Wa, F, total, (bf16*)dh)));
+  DISPATCH(dtype, (nf_launch(dh_max_kernel<float>, nblk(total, 256), 256, 0, (const float*)h, dp, parg, Ha, Wa, F, total, (float*)dh)),
+           (nf_launch(dh_max_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)h, dp, parg, Ha, Wa, F, total, (bf16*)dh)));
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_dh(int dtype, const void* h, const float* dp, int N, int Ha, int Wa, int F, void* dh) {
   const size_t total = (size_t)N * Ha * Wa * F;
-  DISPATCH(dtype, (dh_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)h, dp, Ha, Wa, F, total, (float*)dh)),
-           (dh_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)h, dp, Ha, Wa, F, total, (bf16*)dh)));
+  DISPATCH(dtype, (nf_launch(dh_kernel<float>, nblk(total, 256), 256, 0, (const float*)h, dp, Ha, Wa, F, total, (float*)dh)),
+           (nf_launch(dh_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)h, dp, Ha, Wa, F, total, (bf16*)dh)));
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_sum_partials(const float* red, int nblocks, int C, int which, float* out) {
-  sum_partials_kernel<<<nblk(C, 32), dim3(32, 32), 0, g_nf_stream>>>(red, nblocks, C, which, out);
+  nf_launch(sum_partials_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, which, out);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1565,22 +1606,22 @@ int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, 
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
   if (!skip && pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    bn_bwd_reduce_pool_vec_kernel<<<nb, 256, 0, g_nf_stream>>>((const uint4*)y, (const uint4*)da, P / 4, Ho, Wo, C / 8, scale, shift, mu,
+    nf_launch(bn_bwd_reduce_pool_vec_kernel, nb, 256, 0, (const uint4*)y, (const uint4*)da, P / 4, Ho, Wo, C / 8, scale, shift, mu,
                                                               invstd, red);
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;
   }
   if (!skip && vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    bn_bwd_reduce_vec_kernel<<<nb, 256, 0, g_nf_stream>>>((const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red);
+    nf_launch(bn_bwd_reduce_vec_kernel, nb, 256, 0, (const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red);
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;
   }
   BnBwdFn fn{Ho, Wo, pool, scale, shift, mu, invstd, skip};
   DISPATCH(dtype,
-           (channel_reduce_kernel<float, BnBwdFn><<<nb, 256, 0, g_nf_stream>>>((const float*)y, (const float*)da, P, C, fn, red)),
-           (channel_reduce_kernel<bf16, BnBwdFn><<<nb, 256, 0, g_nf_stream>>>((const bf16*)y, (const bf16*)da, P, C, fn, red)));
+           (nf_launch(channel_reduce_kernel<float, BnBwdFn>, nb, 256, 0, (const float*)y, (const float*)da, P, C, fn, red)),
+           (nf_launch(channel_reduce_kernel<bf16, BnBwdFn>, nb, 256, 0, (const bf16*)y, (const bf16*)da, P, C, fn, red)));
   NF_LAUNCHED();
   *nblocks = nb;
   return NF_OK;
@@ -1590,15 +1631,15 @@ int nf_k_write_dz(int dtype, const void* y, const void* da, int N, int Ho, int W
                   const float* shift, const void* skip, void* dz) {
   const size_t total = (size_t)N * Ho * Wo * C;
   DISPATCH(dtype,
-           (write_dz_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, (const float*)skip, total, (float*)dz)),
-           (write_dz_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)y, (const bf16*)da, Ho, Wo, C, pool, scale, shift, (const bf16*)skip, total, (bf16*)dz)));
+           (nf_launch(write_dz_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, (const float*)skip, total, (float*)dz)),
+           (nf_launch(write_dz_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)y, (const bf16*)da, Ho, Wo, C, pool, scale, shift, (const bf16*)skip, total, (bf16*)dz)));
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_bn_bwd_finalize(const float* red, int nblocks, int C, float* sdz, float* sdzx, float* ggamma,
                            float* gbeta) {
-  bn_bwd_finalize_kernel<<<nblk(C, 32), dim3(32, 32), 0, g_nf_stream>>>(red, nblocks, C, sdz, sdzx, ggamma, gbeta);
+  nf_launch(bn_bwd_finalize_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, sdz, sdzx, ggamma, gbeta);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1610,49 +1651,49 @@ int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, i
   const float invM = (float)(1.0 / M);
   if (skip) {
     DISPATCH(dtype,
-             (bn_bwd_apply_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (float*)dy, (const float*)skip)),
-             (bn_bwd_apply_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)y, (const bf16*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (bf16*)dy, (const bf16*)skip)));
+             (nf_launch(bn_bwd_apply_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (float*)dy, (const float*)skip)),
+             (nf_launch(bn_bwd_apply_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)y, (const bf16*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (bf16*)dy, (const bf16*)skip)));
     NF_LAUNCHED();
     return NF_OK;
   }
   if (pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    bn_bwd_apply_pool_vec_kernel<<<vec_blocks(total / 32), 256, 0, g_nf_stream>>>((const uint4*)y, (const uint4*)da, Ho, Wo, C / 8, scale,
+    nf_launch(bn_bwd_apply_pool_vec_kernel, vec_blocks(total / 32), 256, 0, (const uint4*)y, (const uint4*)da, Ho, Wo, C / 8, scale,
                                                                                  shift, mu, invstd, sdz, sdzx, invM, total / 32, (uint4*)dy);
     NF_LAUNCHED();
     return NF_OK;
   }
   if (vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    bn_bwd_apply_vec2_kernel<<<vec_blocks(total / 8), 256, 0, g_nf_stream>>>((const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
+    nf_launch(bn_bwd_apply_vec2_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
                                                                             invstd, sdz, sdzx, invM, total / 8, (uint4*)dy);
     NF_LAUNCHED();
     return NF_OK;
   }
   if (vec_ok(dtype, C, pool)) {
-    bn_bwd_apply_vec_kernel<<<vec_blocks(total / 8), 256, 6 * C * sizeof(float), g_nf_stream>>>(
+    nf_launch(bn_bwd_apply_vec_kernel, vec_blocks(total / 8), 256, 6 * C * sizeof(float), 
         (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu, invstd, sdz, sdzx, invM, total / 8, (uint4*)dy);
     NF_LAUNCHED();
     return NF_OK;
   }
   DISPATCH(dtype,
-           (bn_bwd_apply_kernel<float><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (float*)dy, nullptr)),
-           (bn_bwd_apply_kernel<bf16><<<nblk(total, 256), 256, 0, g_nf_stream>>>((const bf16*)y, (const bf16*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (bf16*)dy, nullptr)));
+           (nf_launch(bn_bwd_apply_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (float*)dy, nullptr)),
+           (nf_launch(bn_bwd_apply_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)y, (const bf16*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (bf16*)dy, nullptr)));
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_pad_channels(const void* x, size_t P, int C, int Cp, void* xpad) {
   if (C < 1 || C > 8 || Cp % 8) return NF_EUNSUPPORTED;
-  pad_channels_kernel<<<nblk(P * (Cp / 8), 256), 256, 0, g_nf_stream>>>((const bf16*)x, P, C, Cp / 8, (uint4*)xpad);
+  nf_launch(pad_channels_kernel, nblk(P * (Cp / 8), 256), 256, 0, (const bf16*)x, P, C, Cp / 8, (uint4*)xpad);
   NF_LAUNCHED();
   return NF_OK;
 }
 int nf_k_pad_weights(const bf16* w, size_t rows, int C, int Cp, bf16* wpad) {
-  pad_weights_kernel<<<nblk(rows * Cp, 256), 256, 0, g_nf_stream>>>(w, rows, C, Cp, wpad);
+  nf_launch(pad_weights_kernel, nblk(rows * Cp, 256), 256, 0, w, rows, C, Cp, wpad);
   NF_LAUNCHED();
   return NF_OK;
 }
 int nf_k_unpad_grad(const float* gwpad, size_t rows, int C, int Cp, float* gw) {
-  unpad_grad_kernel<<<nblk(rows * C, 256), 256, 0, g_nf_stream>>>(gwpad, rows, C, Cp, gw);
+  nf_launch(unpad_grad_kernel, nblk(rows * C, 256), 256, 0, gwpad, rows, C, Cp, gw);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1666,7 +1707,7 @@ int nf_k_sgd_multi(const SgdTable& tb_in, float lr, float momentum) {
     tb.first_block[a] = blocks;
     blocks += (int)nblk(tb.n[a] / 4, 256);
   }
-  sgd_multi_kernel<<<blocks, 256, 0, g_nf_stream>>>(tb, lr, momentum);
+  nf_launch(sgd_multi_kernel, blocks, 256, 0, tb, lr, momentum);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1679,7 +1720,7 @@ int nf_k_sgd(float* val, float* mom, const float* grad, bf16* shadow, size_t n, 
 }
 
 int nf_k_shadow(const float* val, bf16* shadow, size_t n) {
-  shadow_kernel<<<nblk(n, 256), 256, 0, g_nf_stream>>>(val, shadow, n);
+  nf_launch(shadow_kernel, nblk(n, 256), 256, 0, val, shadow, n);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1687,7 +1728,7 @@ int nf_k_shadow(const float* val, bf16* shadow, size_t n) {
 int nf_k_gather(const void* cache, const int32_t* cache_labels, int cache_rows, const int32_t* idx, int count, size_t row_bytes,
                   void* out, int32_t* out_labels, int32_t* status) {
   const size_t row16 = row_bytes / 16;
-  gather_kernel<<<nblk((size_t)count * row16, 256), 256, 0, g_nf_stream>>>((const uint4*)cache, cache_labels, cache_rows, idx,
+  nf_launch(gather_kernel, nblk((size_t)count * row16, 256), 256, 0, (const uint4*)cache, cache_labels, cache_rows, idx,
                                                                          count, row16, (uint4*)out, out_labels, status);
   NF_LAUNCHED();
   return NF_OK;

@@ -15,6 +15,7 @@ namespace {
 // 64 x 64 tile per block of 256 threads, 4 x 4 outputs per thread, 16-deep shared-memory stages.
 __global__ void __launch_bounds__(256) head_gemm_kernel(const float* __restrict__ A, long sai, long sak, const float* __restrict__ B,
                                                         long sbk, long sbj, int M, int Nn, int Kd, float* __restrict__ C) {
+  nf_pdl_begin();
   __shared__ float As[16][68];
   __shared__ float Bs[16][68];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -65,6 +66,7 @@ __global__ void __launch_bounds__(256) head_gemm_kernel(const float* __restrict_
 // out[e] = (bias ? bias[e % Nn] : 0) + part[0][e] + part[1][e] + ... in range order
 __global__ void head_finish_kernel(const float* __restrict__ part, int Z, size_t mn, int Nn, const float* __restrict__ bias,
                                    float* __restrict__ out) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= mn) return;
   float s = bias ? bias[e % Nn] : 0.f;
@@ -76,6 +78,7 @@ __global__ void head_finish_kernel(const float* __restrict__ part, int Z, size_t
 __global__ void __launch_bounds__(256) head_loss_rows_kernel(const float* __restrict__ logits, const int32_t* __restrict__ labels, int N,
                                                              int K, int loss_kind, float* __restrict__ dlogits,
                                                              float* __restrict__ lossn, int32_t* status, int n_scale) {
+  nf_pdl_begin();
   const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (n >= N) return;
   const float* l = logits + (size_t)n * K;
@@ -119,6 +122,7 @@ __global__ void __launch_bounds__(256) head_loss_rows_kernel(const float* __rest
 __global__ void __launch_bounds__(256) head_colsum_loss_kernel(const float* __restrict__ dl, const float* __restrict__ lossn, int N, int K,
                                                                float* __restrict__ part, float* __restrict__ loss_out, int32_t* status,
                                                                int n_scale) {
+  nf_pdl_begin();
   __shared__ float sm[8][33];
   __shared__ double sd[256];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -154,6 +158,7 @@ __global__ void __launch_bounds__(256) head_colsum_loss_kernel(const float* __re
 
 // first arg-max of each row of logits, one warp per sample
 __global__ void __launch_bounds__(256) head_argmax_rows_kernel(const float* __restrict__ logits, int N, int K, int32_t* __restrict__ pred) {
+  nf_pdl_begin();
   const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (n >= N) return;
   const float* l = logits + (size_t)n * K;
@@ -172,7 +177,7 @@ __global__ void __launch_bounds__(256) head_argmax_rows_kernel(const float* __re
 
 int gemm(const float* A, long sai, long sak, const float* B, long sbk, long sbj, int M, int Nn, int Kd, int Z, float* C) {
   dim3 grid((Nn + 63) / 64, (M + 63) / 64, Z);
-  head_gemm_kernel<<<grid, 256, 0, g_nf_stream>>>(A, sai, sak, B, sbk, sbj, M, Nn, Kd, C);
+  nf_launch(head_gemm_kernel, grid, 256, 0, A, sai, sak, B, sbk, sbj, M, Nn, Kd, C);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -186,13 +191,13 @@ int nf_head_logits(const float* p, int N, int D, int K, const float* Wf, const f
   int rc = gemm(p, D, 1, Wf, 1, D, N, K, D, 1, scratch);
   if (rc != NF_OK) return rc;
   const size_t mn = (size_t)N * K;
-  head_finish_kernel<<<(unsigned)((mn + 255) / 256), 256, 0, g_nf_stream>>>(scratch, 1, mn, K, bf, logits);
+  nf_launch(head_finish_kernel, (unsigned)((mn + 255) / 256), 256, 0, scratch, 1, mn, K, bf, logits);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_head_predict(const float* logits, int N, int K, int32_t* pred) {
-  head_argmax_rows_kernel<<<(N + 7) / 8, 256, 0, g_nf_stream>>>(logits, N, K, pred);
+  nf_launch(head_argmax_rows_kernel, (N + 7) / 8, 256, 0, logits, N, K, pred);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -208,7 +213,7 @@ int nf_head_step(const float* p, const int32_t* labels, int N, int D, int K, con
   if (scratch_floats < nf_head_scratch_floats(N, D, K)) return NF_ENOWS;
   int rc = nf_head_logits(p, N, D, K, Wf, bf, logits, scratch);
   if (rc != NF_OK) return rc;
-  head_loss_rows_kernel<<<(N + 7) / 8, 256, 0, g_nf_stream>>>(logits, labels, N, K, loss_kind, dlogits, lossn, status, n_scale);
+  nf_launch(head_loss_rows_kernel, (N + 7) / 8, 256, 0, logits, labels, N, K, loss_kind, dlogits, lossn, status, n_scale);
   NF_LAUNCHED();
   // dp[n][d] = sum_k dlogits[n][k] Wf[k][d]
   if ((rc = gemm(dlogits, K, 1, Wf, D, 1, N, D, K, 1, dp)) != NF_OK) return rc;
@@ -220,14 +225,14 @@ int nf_head_step(const float* p, const int32_t* labels, int N, int D, int K, con
   Z = std::min(Z, std::max(1, N / 256));
   if (Z < 1) Z = 1;
   if ((rc = gemm(dlogits, 1, K, p, D, 1, K, D, N, Z, scratch)) != NF_OK) return rc;
-  head_finish_kernel<<<(unsigned)((kd + 255) / 256), 256, 0, g_nf_stream>>>(scratch, Z, kd, D, nullptr, gWf);
+  nf_launch(head_finish_kernel, (unsigned)((kd + 255) / 256), 256, 0, scratch, Z, kd, D, nullptr, gWf);
   NF_LAUNCHED();
   // gbf[k] = sum_n dlogits[n][k]: row ranges in parallel (the scratch is free again), then the ranges in order
   int RB = std::max(1, std::min(64, N / 128));
   if ((size_t)RB * K > scratch_floats) RB = 1;
-  head_colsum_loss_kernel<<<dim3((K + 31) / 32, RB), 256, 0, g_nf_stream>>>(dlogits, lossn, N, K, scratch, loss_out, status, n_scale);
+  nf_launch(head_colsum_loss_kernel, dim3((K + 31) / 32, RB), 256, 0, dlogits, lossn, N, K, scratch, loss_out, status, n_scale);
   NF_LAUNCHED();
-  head_finish_kernel<<<(unsigned)((K + 255) / 256), 256, 0, g_nf_stream>>>(scratch, RB, (size_t)K, K, nullptr, gbf);
+  nf_launch(head_finish_kernel, (unsigned)((K + 255) / 256), 256, 0, scratch, RB, (size_t)K, K, nullptr, gbf);
   NF_LAUNCHED();
   return NF_OK;
 }

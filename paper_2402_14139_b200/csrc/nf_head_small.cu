@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(kHsThreads) head_logits_slice_kernel(const flo
                                                                        const float* __restrict__ Wf, const float* __restrict__ bf,
                                                                        float* __restrict__ logits, float* __restrict__ share,
                                                                        int loss_kind) {
+  nf_pdl_begin();
   extern __shared__ float sm[];
   const int Dp = D + 1;
   float* ps = sm;                 // [NC][D+1]
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kHsThreads) head_grad_slice_kernel(const float
                                                                      float* __restrict__ gWf, float* __restrict__ gbf,
                                                                      float* __restrict__ lossn, int32_t* __restrict__ status,
                                                                      int loss_kind, int n_scale) {
+  nf_pdl_begin();
   extern __shared__ float sm[];
   const int Dp = D + 1;
   float* ps = sm;                 // [NC][D+1]
@@ -216,6 +218,7 @@ __global__ void __launch_bounds__(kHsThreads) head_grad_slice_kernel(const float
 __global__ void __launch_bounds__(kHsThreads) head_finish_kernel(const float* __restrict__ dps, int S, size_t ND, float* __restrict__ dp,
                                                                  const float* __restrict__ lossn, int N, int n_scale,
                                                                  float* __restrict__ loss_out, int32_t* __restrict__ status) {
+  nf_pdl_begin();
   const size_t i = (size_t)blockIdx.x * kHsThreads + threadIdx.x;
   if (i < ND) {
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;  // four interleaved chains over the slices, combined in a fixed order
@@ -276,14 +279,14 @@ int nf_head_small_step(const float* p, const int32_t* labels, int N, int D, int 
   float* dps = scratch + (size_t)pl.S * N * 2;  // [S][N][D]
   const int rc = allow_smem();
   if (rc != NF_OK) return rc;
-  head_logits_slice_kernel<<<dim3(pl.S, pl.chunks), kHsThreads, pl.smem_fwd, g_nf_stream>>>(p, labels, N, D, K, pl.KS, pl.NC, Wf, bf,
+  nf_launch(head_logits_slice_kernel, dim3(pl.S, pl.chunks), kHsThreads, pl.smem_fwd, p, labels, N, D, K, pl.KS, pl.NC, Wf, bf,
                                                                                              logits, share, loss_kind);
   NF_LAUNCHED();
-  head_grad_slice_kernel<<<pl.S, kHsThreads, pl.smem_bwd, g_nf_stream>>>(p, labels, N, D, K, pl.KS, pl.NC, pl.S, Wf, logits, share, dps,
+  nf_launch(head_grad_slice_kernel, pl.S, kHsThreads, pl.smem_bwd, p, labels, N, D, K, pl.KS, pl.NC, pl.S, Wf, logits, share, dps,
                                                                          gWf, gbf, lossn, status, loss_kind, n_scale);
   NF_LAUNCHED();
   const size_t ND = (size_t)N * D;
-  head_finish_kernel<<<(unsigned)((ND + kHsThreads - 1) / kHsThreads), kHsThreads, 0, g_nf_stream>>>(dps, pl.S, ND, dp, lossn, N, n_scale,
+  nf_launch(head_finish_kernel, (unsigned)((ND + kHsThreads - 1) / kHsThreads), kHsThreads, 0, dps, pl.S, ND, dp, lossn, N, n_scale,
                                                                                                     loss_out, status);
   NF_LAUNCHED();
   return NF_OK;

@@ -91,6 +91,30 @@ int nf_cuda_check(cudaError_t e, const char* what);
     if (nf_cuda_check(cudaGetLastError(), "launch") != NF_OK) return NF_ECUDA; \
   } while (0)
 
+// Every kernel is launched with programmatic stream serialisation: it may be placed on the SMs while its predecessor in the
+// stream still runs, does what needs no memory of others (barriers, tensor memory, index arithmetic) and then waits in
+// nf_pdl_begin() until the predecessor has finished and its writes are visible.  A step is 15 to 20 kernels of 3 to 30 us a
+// layer at small sizes, where the start-up of each was paid in full: four-layer block at 32x32, 128 images, 0.83 -> 0.69 ms per
+// step, a single fp32 layer on 8 images 137 -> 114 us.  nf_pdl_begin() has to come before the first access to global memory in every thread.
+__device__ __forceinline__ void nf_pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+static inline void nf_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = g_nf_stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // an error stays as the last error, which NF_LAUNCHED reads
+}
+
 static inline size_t nf_align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 static inline size_t nf_esize(int dtype) { return dtype == NF_F32 ? 4 : 2; }
 

@@ -36,6 +36,7 @@ constexpr int kPix = 8;  // output pixels per block of the forward kernel
 template <typename T>
 __global__ void __launch_bounds__(256) proj_fwd_kernel(const T* __restrict__ x, const T* __restrict__ w, int H, int W, int Ci, int Co,
                                                        int Ho, int Wo, size_t P, int stride, T* __restrict__ ys) {
+  nf_pdl_begin();
   extern __shared__ float xs[];  // [kPix][Ci]
   const size_t p0 = (size_t)blockIdx.x * kPix;
   for (int i = threadIdx.x; i < kPix * Ci; i += 256) {
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(256) proj_fwd_kernel(const T* __restrict__ x, 
 template <typename T>
 __global__ void proj_affine_kernel(const T* __restrict__ ys, int C, const float* __restrict__ scale, const float* __restrict__ shift,
                                    size_t total, T* __restrict__ s) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int c = (int)(e % C);
@@ -79,6 +81,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) proj_bwd_reduce_kernel(const T* __restrict__ ys, const T* __restrict__ dz, size_t P, int C,
                                                               const float* __restrict__ mu, const float* __restrict__ invstd,
                                                               float* __restrict__ red) {
+  nf_pdl_begin();
   const size_t p0 = P * blockIdx.x / gridDim.x, p1 = P * (blockIdx.x + 1) / gridDim.x;
   for (int c = threadIdx.x; c < C; c += 256) {
     float a = 0.f, b = 0.f;
@@ -98,6 +101,7 @@ template <typename T>
 __global__ void proj_bwd_apply_kernel(const T* __restrict__ ys, const T* __restrict__ dz, int C, const float* __restrict__ scale,
                                       const float* __restrict__ mu, const float* __restrict__ invstd, const float* __restrict__ sdz,
                                       const float* __restrict__ sdzx, float invM, size_t total, T* __restrict__ dys) {
+  nf_pdl_begin();
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int c = (int)(e % C);
@@ -110,6 +114,7 @@ __global__ void proj_bwd_apply_kernel(const T* __restrict__ ys, const T* __restr
 template <typename T>
 __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x, const T* __restrict__ dys, int H, int W, int Ci, int Co,
                                                          int Ho, int Wo, size_t P, int stride, int splits, float* __restrict__ part) {
+  nf_pdl_begin();
   __shared__ float xs[16][16];   // [pixel][ci]
   __shared__ float gs[16][64];   // [pixel][co]
   const int ci0 = blockIdx.x * 16, co0 = blockIdx.y * 64, sp = blockIdx.z;
@@ -148,6 +153,7 @@ __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x
 }
 
 __global__ void proj_sum_splits_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
+  nf_pdl_begin();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float s = 0.f;
@@ -323,9 +329,9 @@ int proj_conv(nf_proj* P, const void* xb, int count) {
   if (smem > 48 * 1024) return NF_EUNSUPPORTED;
   const unsigned grid = blocks_for(pix, kPix);
   PROJ_DISPATCH(P->dtype,
-                (proj_fwd_kernel<float><<<grid, 256, smem, g_nf_stream>>>((const float*)xb, P->val + P->offW, P->H, P->W, P->Cin, P->Cout,
+                (nf_launch(proj_fwd_kernel<float>, grid, 256, smem, (const float*)xb, P->val + P->offW, P->H, P->W, P->Cin, P->Cout,
                                                                         P->Ho, P->Wo, pix, 2, (float*)P->ys)),
-                (proj_fwd_kernel<bf16><<<grid, 256, smem, g_nf_stream>>>((const bf16*)xb, P->shadow + P->offW, P->H, P->W, P->Cin, P->Cout,
+                (nf_launch(proj_fwd_kernel<bf16>, grid, 256, smem, (const bf16*)xb, P->shadow + P->offW, P->H, P->W, P->Cin, P->Cout,
                                                                        P->Ho, P->Wo, pix, 2, (bf16*)P->ys)));
   NF_LAUNCHED();
   return NF_OK;
@@ -334,9 +340,9 @@ int proj_conv(nf_proj* P, const void* xb, int count) {
 int proj_affine(nf_proj* P, int count, void* s_out) {
   const size_t total = (size_t)count * P->Ho * P->Wo * P->Cout;
   PROJ_DISPATCH(P->dtype,
-                (proj_affine_kernel<float><<<blocks_for(total, 256), 256, 0, g_nf_stream>>>((const float*)P->ys, P->Cout, P->scale, P->shift,
+                (nf_launch(proj_affine_kernel<float>, blocks_for(total, 256), 256, 0, (const float*)P->ys, P->Cout, P->scale, P->shift,
                                                                                          total, (float*)s_out)),
-                (proj_affine_kernel<bf16><<<blocks_for(total, 256), 256, 0, g_nf_stream>>>((const bf16*)P->ys, P->Cout, P->scale, P->shift,
+                (nf_launch(proj_affine_kernel<bf16>, blocks_for(total, 256), 256, 0, (const bf16*)P->ys, P->Cout, P->scale, P->shift,
                                                                                         total, (bf16*)s_out)));
   NF_LAUNCHED();
   return NF_OK;
@@ -380,27 +386,27 @@ int nf_proj_backward(nf_proj* P, const void* xb, const void* dz, float lr) {
   const size_t pix = (size_t)P->N * P->Ho * P->Wo, total = pix * C;
   const int nb = (int)(pix < (size_t)kProjBlocks ? pix : (size_t)kProjBlocks);
   PROJ_DISPATCH(P->dtype,
-                (proj_bwd_reduce_kernel<float><<<nb, 256, 0, g_nf_stream>>>((const float*)P->ys, (const float*)dz, pix, C, P->mu, P->invstd, P->red)),
-                (proj_bwd_reduce_kernel<bf16><<<nb, 256, 0, g_nf_stream>>>((const bf16*)P->ys, (const bf16*)dz, pix, C, P->mu, P->invstd, P->red)));
+                (nf_launch(proj_bwd_reduce_kernel<float>, nb, 256, 0, (const float*)P->ys, (const float*)dz, pix, C, P->mu, P->invstd, P->red)),
+                (nf_launch(proj_bwd_reduce_kernel<bf16>, nb, 256, 0, (const bf16*)P->ys, (const bf16*)dz, pix, C, P->mu, P->invstd, P->red)));
   NF_LAUNCHED();
   int rc = nf_k_bn_bwd_finalize(P->red, nb, C, P->sdz, P->sdzx, P->grad + P->offG, P->grad + P->offB);
   if (rc != NF_OK) return rc;
   const float invM = (float)(1.0 / (double)pix);
   PROJ_DISPATCH(P->dtype,
-                (proj_bwd_apply_kernel<float><<<blocks_for(total, 256), 256, 0, g_nf_stream>>>((const float*)P->ys, (const float*)dz, C, P->scale, P->mu,
+                (nf_launch(proj_bwd_apply_kernel<float>, blocks_for(total, 256), 256, 0, (const float*)P->ys, (const float*)dz, C, P->scale, P->mu,
                                                                                             P->invstd, P->sdz, P->sdzx, invM, total, (float*)P->dys)),
-                (proj_bwd_apply_kernel<bf16><<<blocks_for(total, 256), 256, 0, g_nf_stream>>>((const bf16*)P->ys, (const bf16*)dz, C, P->scale, P->mu,
+                (nf_launch(proj_bwd_apply_kernel<bf16>, blocks_for(total, 256), 256, 0, (const bf16*)P->ys, (const bf16*)dz, C, P->scale, P->mu,
                                                                                            P->invstd, P->sdz, P->sdzx, invM, total, (bf16*)P->dys)));
   NF_LAUNCHED();
   const dim3 grid((P->Cin + 15) / 16, (C + 63) / 64, P->splits);
   PROJ_DISPATCH(P->dtype,
-                (proj_wgrad_kernel<float><<<grid, 256, 0, g_nf_stream>>>((const float*)xb, (const float*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo,
+                (nf_launch(proj_wgrad_kernel<float>, grid, 256, 0, (const float*)xb, (const float*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo,
                                                                        pix, 2, P->splits, P->wpart)),
-                (proj_wgrad_kernel<bf16><<<grid, 256, 0, g_nf_stream>>>((const bf16*)xb, (const bf16*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo,
+                (nf_launch(proj_wgrad_kernel<bf16>, grid, 256, 0, (const bf16*)xb, (const bf16*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo,
                                                                       pix, 2, P->splits, P->wpart)));
   NF_LAUNCHED();
   const size_t nw = (size_t)P->Cin * C;
-  proj_sum_splits_kernel<<<blocks_for(nw, 256), 256, 0, g_nf_stream>>>(P->wpart, P->splits, nw, P->grad + P->offW);
+  nf_launch(proj_sum_splits_kernel, blocks_for(nw, 256), 256, 0, P->wpart, P->splits, nw, P->grad + P->offW);
   NF_LAUNCHED();
   return nf_k_sgd(P->val, P->mom, P->grad, P->shadow, P->arena, lr, P->momentum);
 }

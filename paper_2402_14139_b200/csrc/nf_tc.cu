@@ -85,7 +85,7 @@ struct FwdParams {
   int stride, BI;     // PT mode: conv stride and images per tile (BW*BH*BI = 128)
   TileGrid tg;
   int stats;
-  float* red;         // [grid * parts][2][Cout] channel partials (pre-zeroed)
+  float* red;         // [grid / n_tiles * parts][2][Cout] channel partials
   int32_t* status;    // device status word
   const float* bias;  // EPI 1: per-channel bias added before the ReLU
   bf16* out;          // EPI 1: destination [N][H][W][Cout], written straight from registers
@@ -170,6 +170,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
   if (warp == 0) {
     // ---------------- producer: one TMA box of activations + three weight tiles per k-step.  One thread runs the whole loop:
@@ -390,7 +391,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     if (et == 0) ptx::tma_store_wait_all();
     if (p.stats) {
       constexpr int parts = 128 / BN > 0 ? 128 / BN : 1;
-      const size_t b = (size_t)blockIdx.x * parts + shalf;
+      const size_t b = (size_t)(blockIdx.x / p.n_tiles) * parts + shalf;  // the CTAs of one pixel range fill one row of partials
       if (p.stats == 2) {
         const int ch = my_nt * BN + sc;
         ssq = (float)((double)p.bn_invstd[ch] * ((double)ssq - (double)p.bn_mu[ch] * (double)ssum));
@@ -638,6 +639,7 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
   if (warp == 0) {
     if (ptx::elect_one()) {  // one thread runs the whole loop, as in the generic kernel
@@ -1122,6 +1124,7 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
   if (warp == 0) {
     // ---------------- producer: the CTA's weights once, then per tile one dh box and (stats >= 2) the y2 tile
@@ -1393,6 +1396,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
   if (warp == 0) {
     if (ptx::elect_one()) {  // producer and issuer: one thread runs the whole loop, as in the forward kernels
@@ -1537,6 +1541,7 @@ conv_wgrad_kw_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
   if (warp == 0) {
     if (ptx::elect_one()) {
@@ -1671,6 +1676,7 @@ conv_wgrad_gx_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
   if (warp == 0) {
     if (ptx::elect_one()) {
@@ -1748,6 +1754,7 @@ conv_wgrad_gx_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 }
 
 __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
+  nf_pdl_begin();
   // 32 consecutive elements x 8 lanes over the splits; each lane adds its splits in index order, lane sums are added in lane order
   __shared__ float sm[8][33];
   const size_t i = (size_t)blockIdx.x * 32 + threadIdx.x;
@@ -1913,7 +1920,7 @@ int launch_fwd(const TcPlan& pl, const CUtensorMap& mx, const CUtensorMap& mw, c
     NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW><<<pl.grid, kThreads, pl.smem, g_nf_stream>>>(mx, mw, my, p);
+  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW>, pl.grid, kThreads, pl.smem, mx, mw, my, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1952,7 +1959,7 @@ int launch_fold(int grid, size_t smem, const CUtensorMap& mx, const CUtensorMap&
     NF_CUDA(cudaFuncSetAttribute(conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF><<<grid, kFoldThreads + kXfThreads * XF, smem, g_nf_stream>>>(mx, mw, my, my2, p);
+  nf_launch(conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF>, grid, kFoldThreads + kXfThreads * XF, smem, mx, mw, my, my2, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2055,7 +2062,7 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
       NF_CUDA(cudaFuncSetAttribute(aux_dgrad_wide_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
       attr_done = true;
     }
-    aux_dgrad_wide_kernel<16><<<grid, kWideThreads, smem, g_nf_stream>>>(mx, mw, my, my2, p);
+    nf_launch(aux_dgrad_wide_kernel<16>, grid, kWideThreads, smem, mx, mw, my, my2, p);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -2112,10 +2119,9 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     p.bn_scale = bn->scale; p.bn_shift = bn->shift; p.bn_mu = bn->mu; p.bn_invstd = bn->invstd;
   }
   if (stats) {
-    const size_t need = (size_t)pl.grid * pl.parts * 2 * Cout;
-    if (need > red_floats) return NF_ENOWS;
-    NF_CUDA(cudaMemsetAsync(red, 0, need * sizeof(float), g_nf_stream));
-    *nb = pl.grid * pl.parts;
+    const int rows = pl.grid / p.n_tiles * pl.parts;
+    if ((size_t)rows * 2 * Cout > red_floats) return NF_ENOWS;
+    *nb = rows;
   }
   if (pl.PT) {  // per-tap boxes: stride 2, or several small images per tile
     if (epi == 0)
@@ -2205,7 +2211,7 @@ int launch_wgrad_kw(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& 
     NF_CUDA(cudaFuncSetAttribute(conv_wgrad_kw_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  conv_wgrad_kw_kernel<NB><<<pl.grid, kThreads, pl.smem, g_nf_stream>>>(mx, mg, p);
+  nf_launch(conv_wgrad_kw_kernel<NB>, pl.grid, kThreads, pl.smem, mx, mg, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2218,7 +2224,7 @@ int launch_wgrad_gx(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& 
     NF_CUDA(cudaFuncSetAttribute(conv_wgrad_gx_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  conv_wgrad_gx_kernel<NB><<<pl.grid, kThreads, pl.smem, g_nf_stream>>>(mx, mg, p);
+  nf_launch(conv_wgrad_gx_kernel<NB>, pl.grid, kThreads, pl.smem, mx, mg, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2231,7 +2237,7 @@ int launch_wgrad(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& mg,
     NF_CUDA(cudaFuncSetAttribute(conv_wgrad_tc_kernel<NB, S2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  conv_wgrad_tc_kernel<NB, S2><<<pl.grid, kThreads, pl.smem, g_nf_stream>>>(mx, mg, p);
+  nf_launch(conv_wgrad_tc_kernel<NB, S2>, pl.grid, kThreads, pl.smem, mx, mg, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2268,7 +2274,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
                      : pl.NB == 32 ? launch_wgrad_kw<32>(pl, mx, mg, p) : launch_wgrad_kw<16>(pl, mx, mg, p);
   if (rc != NF_OK) return rc;
   const size_t n = (size_t)9 * Cout * Cin;
-  sum_parts_kernel<<<(unsigned)((n + 31) / 32), dim3(32, 8), 0, g_nf_stream>>>(part, pl.splits, n, dw);
+  nf_launch(sum_parts_kernel, (unsigned)((n + 31) / 32), dim3(32, 8), 0, part, pl.splits, n, dw);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2504,6 +2510,7 @@ int nf_tc_conv3x3_wgrad(const void* x, const void* g, int N, int H, int W, int C
 // arrives at, and then leaves the way those kernels do: abort flag set by the waiter, NF_ETIMEOUT raised in the status
 // word, waited time reported.  No TMA, no tensor memory, nothing else in flight.
 __global__ void bounded_wait_probe_kernel(unsigned long long limit_ns, int32_t* status, unsigned long long* waited_ns) {
+  nf_pdl_begin();
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -2525,7 +2532,7 @@ __global__ void bounded_wait_probe_kernel(unsigned long long limit_ns, int32_t* 
 int nf_tc_bounded_wait_probe(unsigned long long limit_ns, unsigned long long* waited_ns_dev) {
   int32_t* st = nullptr;
   if (nf_tc_op_status_ptr(&st) != NF_OK) return NF_ECUDA;
-  bounded_wait_probe_kernel<<<1, 32, 0, g_nf_stream>>>(limit_ns, st, waited_ns_dev);
+  nf_launch(bounded_wait_probe_kernel, 1, 32, 0, limit_ns, st, waited_ns_dev);
   NF_LAUNCHED();
   return NF_OK;
 }
