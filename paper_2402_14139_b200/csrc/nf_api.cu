@@ -395,7 +395,15 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   trace_begin(3);
   // h_masked: the aux forward left pooling partials (L->wpart) and a sign mask (in L->h) instead of h
   const bool h_masked = fused_bn_aux && nf_tc_aux_pool_fused(L);
-  if (h_masked) {
+  // heads of ordinary size: one block per sample does all of it, and writes dh where the sample's h fits its shared memory
+  int sample_mode = L->o.aux_pool == NF_POOL_AVG && !nf_head_is_large(N, D, K) ? nf_head_sample_mode(dt, Ha, Wa, F, K) : 0;
+  if (sample_mode == 2 && (h_masked || (size_t)N * F > L->red_floats)) sample_mode = 1;
+  if (sample_mode) {
+    const NfHeadIo io{h_masked ? nullptr : L->h, L->wpart, labels, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->p, L->logits,
+                      L->dlogits, L->dp, L->lossn, L->status, sample_mode == 2 ? L->dh : nullptr, L->red, g + L->off[NF_P_WF],
+                      g + L->off[NF_P_BF], g + L->off[NF_P_BA], loss_out};
+    NF_TRY(nf_head_sample_step(io, dt, N, Ha, Wa, F, K, L->o.loss, n_scale));
+  } else if (h_masked) {
     NF_TRY(nf_k_pool_finish(L->wpart, N, Ha / 8, Wa / 14, F, 1.f / (float)((Ha / 2) * (Wa / 2)), L->p));
   } else if (L->o.aux_pool == NF_POOL_MAX) {
     NF_TRY(nf_k_auxmax(dt, L->h, N, Ha, Wa, F, L->p, L->parg));
@@ -404,7 +412,8 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     if (rc == NF_EUNSUPPORTED) rc = nf_k_avgpool(dt, L->h, N, Ha, Wa, F, L->p);
     if (rc != NF_OK) return rc;
   }
-  if (nf_head_is_large(N, D, K)) {  // late blocks: tens of thousands of samples, up to 1024 head inputs
+  if (sample_mode) {
+  } else if (nf_head_is_large(N, D, K)) {  // late blocks: tens of thousands of samples, up to 1024 head inputs
     NF_TRY(nf_head_step(L->p, labels, N, D, K, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->logits, L->dlogits, L->dp,
                         L->lossn, L->status, L->o.loss, g + L->off[NF_P_WF], g + L->off[NF_P_BF], loss_out, L->wpart,
                         L->wpart_floats, n_scale));
@@ -423,7 +432,8 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   trace_end();
   trace_begin(4);
   int dh_nb = 0;
-  if (h_masked) {
+  if (sample_mode == 2) {
+  } else if (h_masked) {
     NF_TRY(nf_k_dh_mask((const uint8_t*)L->h, L->dp, N, Ha, Wa, F, L->dh, L->red, L->red_floats, &dh_nb));
   } else if (L->o.aux_pool == NF_POOL_MAX) {
     NF_TRY(nf_k_dh_max(dt, L->h, L->dp, L->parg, N, Ha, Wa, F, L->dh));
@@ -441,7 +451,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   } else {
     NF_TRY(nf_k_wgrad(dt, act_out, N, Ha, Wa, Co, L->dh, F, 1, L->wpart, L->wpart_floats, g + L->off[NF_P_WA]));
   }
-  if (!dh_nb) {
+  if (!dh_nb && sample_mode != 2) {
     NF_TRY(nf_k_channel_sums(dt, L->dh, (size_t)N * Ha * Wa, F, L->red, L->red_floats, &nb));
     NF_TRY(nf_k_sum_partials(L->red, nb, F, 0, g + L->off[NF_P_BA]));
   }

@@ -156,6 +156,20 @@ int nf_head_predict(const float* logits, int N, int K, int32_t* pred);
 int nf_head_step(const float* p, const int32_t* labels, int N, int D, int K, const float* Wf, const float* bf, float* logits,
                  float* dlogits, float* dp, float* lossn, int32_t* status, int loss_kind, float* gWf, float* gbf, float* loss_out,
                  float* scratch, size_t scratch_floats, int n_scale);
+// head with one block per sample (nf_head_sample.cu): pool, linear layer, loss, dp and (mode 2) dh with the aux bias gradient
+struct NfHeadIo {
+  const void* h;      // aux output, or NULL with
+  const float* part;  // the pooling partials of the fused aux forward
+  const int32_t* labels;
+  const float *Wf, *bf;
+  float *p, *logits, *dlogits, *dp, *lossn;
+  int32_t* status;
+  void* dh;           // mode 2, else NULL
+  float* bred;        // [N][F] scratch (with dh)
+  float *gWf, *gbf, *gba, *loss_out;
+};
+int nf_head_sample_mode(int dtype, int Ha, int Wa, int F, int K);
+int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, int F, int K, int loss_kind, int n_scale);
 // small-batch head (nf_head_small.cu): class-sliced forward + backward of the linear layer and the loss; 0 floats = not covered
 size_t nf_head_small_scratch_floats(int N, int D, int K);
 int nf_head_small_step(const float* p, const int32_t* labels, int N, int D, int K, const float* Wf, const float* bf, float* logits,
