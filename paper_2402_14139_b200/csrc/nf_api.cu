@@ -445,7 +445,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     }
     if (rc != NF_OK) return rc;
   }
-  if (dh_nb) NF_TRY(nf_k_sum_partials(L->red, dh_nb, F, 0, g + L->off[NF_P_BA]));
+  if (dh_nb) NF_TRY(nf_k_sum_partials(L->red, dh_nb, F, g + L->off[NF_P_BA]));
   if (L->fam[3]) {
     NF_TRY(nf_tc_aux_wgrad(L, act_out));
   } else {
@@ -453,7 +453,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   }
   if (!dh_nb && sample_mode != 2) {
     NF_TRY(nf_k_channel_sums(dt, L->dh, (size_t)N * Ha * Wa, F, L->red, L->red_floats, &nb));
-    NF_TRY(nf_k_sum_partials(L->red, nb, F, 0, g + L->off[NF_P_BA]));
+    NF_TRY(nf_k_sum_partials(L->red, nb, F, g + L->off[NF_P_BA]));
   }
   trace_end();
   // gradient at the aux input

@@ -93,42 +93,52 @@ __global__ void __launch_bounds__(256) channel_reduce_kernel(const T* __restrict
 }
 
 
-// Sums the per-block partials of 32 consecutive channels: block (32 channels x 32 lanes over the partials),
-// fp64, fixed order.  Returns the two totals to the threads with threadIdx.y == 0.
-__device__ __forceinline__ void reduce_partials32(const float* __restrict__ red, int nb, int C, double& S, double& Q) {
-  __shared__ double sm[2][32][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
+// Sums the per-block partials of 8 consecutive channels in fp64, in a fixed order: block of 1024 threads = 8 channels x 128 lanes
+// over the partials.  Returns the two totals to one thread per channel (t = 32 * channel of the block).
+// These kernels are one dependent chain: the start-up, a trip to L2, a reduction, and the fetch of their own cold instructions.
+// So the code is kept short (an 8-fold unrolled form with predicated loads ran 3 us slower than it is now) and the lanes many.
+constexpr int kRedCh = 8, kRedThreads = 1024;
+__device__ __forceinline__ void reduce_partials8(const float* __restrict__ red, int nb, int C, double& S, double& Q) {
+  __shared__ double sm[2][32][kRedCh + 1];
+  const int t = threadIdx.x, ch = t & 7;
+  const int c = blockIdx.x * kRedCh + ch;
   double a = 0.0, b = 0.0;
   if (c < C) {
-    int k = threadIdx.y;
-    for (; k + 7 * 32 < nb; k += 8 * 32) {  // eight independent pairs of loads in flight, added in index order
-      float u[8], v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        u[j] = red[((size_t)(k + 32 * j) * 2 + 0) * C + c];
-        v[j] = red[((size_t)(k + 32 * j) * 2 + 1) * C + c];
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        a += (double)u[j];
-        b += (double)v[j];
-      }
-    }
-    for (; k < nb; k += 32) {
-      a += (double)red[((size_t)k * 2 + 0) * C + c];
-      b += (double)red[((size_t)k * 2 + 1) * C + c];
+    const float* r = red + (size_t)(t >> 3) * 2 * C + c;
+#pragma unroll 1
+    for (int k = t >> 3; k < nb; k += 2 * 128, r += (size_t)2 * 128 * 2 * C) {
+      const bool two = k + 128 < nb;
+      const float u0 = r[0], v0 = r[C], u1 = two ? r[(size_t)128 * 2 * C] : 0.f, v1 = two ? r[(size_t)128 * 2 * C + C] : 0.f;
+      a += (double)u0 + (double)u1;
+      b += (double)v0 + (double)v1;
     }
   }
-  sm[0][threadIdx.y][threadIdx.x] = a;
-  sm[1][threadIdx.y][threadIdx.x] = b;
+#pragma unroll 1
+  for (int o = 8; o < 32; o <<= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if ((t & 31) < 8) {
+    sm[0][t >> 5][ch] = a;
+    sm[1][t >> 5][ch] = b;
+  }
   __syncthreads();
   S = 0.0;
   Q = 0.0;
-  if (threadIdx.y == 0)
-    for (int k = 0; k < 32; ++k) {
-      S += sm[0][k][threadIdx.x];
-      Q += sm[1][k][threadIdx.x];
+  if (t < 32 * kRedCh) {
+    S = sm[0][t & 31][t >> 5];
+    Q = sm[1][t & 31][t >> 5];
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+      S += __shfl_xor_sync(0xffffffffu, S, o);
+      Q += __shfl_xor_sync(0xffffffffu, Q, o);
     }
+  }
+}
+// channel whose totals thread t holds, or C
+__device__ __forceinline__ int reduced_channel(int C) {
+  const int c = blockIdx.x * kRedCh + (int)(threadIdx.x >> 5);
+  return (threadIdx.x & 31) == 0 && threadIdx.x < 32 * kRedCh && c < C ? c : C;
 }
 
 __global__ void bn_finalize_kernel(const float* __restrict__ red, int nb, int C, double M, const float* __restrict__ gamma,
@@ -136,9 +146,9 @@ __global__ void bn_finalize_kernel(const float* __restrict__ red, int nb, int C,
                                    float* mu, float* invstd, float* rmean, float* rvar) {
   nf_pdl_begin();
   double S, Q;
-  reduce_partials32(red, nb, C, S, Q);
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  if (c >= C || threadIdx.y != 0) return;
+  reduce_partials8(red, nb, C, S, Q);
+  const int c = reduced_channel(C);
+  if (c >= C) return;
   const double m = S / M;
   double v = Q / M - m * m;
   if (v < 0.0) v = 0.0;
@@ -160,9 +170,9 @@ __global__ void bn_finalize_kernel(const float* __restrict__ red, int nb, int C,
 __global__ void partial_totals_kernel(const float* __restrict__ red, int nb, int C, double* __restrict__ tot) {
   nf_pdl_begin();
   double S, Q;
-  reduce_partials32(red, nb, C, S, Q);
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  if (c >= C || threadIdx.y != 0) return;
+  reduce_partials8(red, nb, C, S, Q);
+  const int c = reduced_channel(C);
+  if (c >= C) return;
   tot[c] = S;
   tot[C + c] = Q;
 }
@@ -562,22 +572,22 @@ __global__ void dh_kernel(const T* __restrict__ h, const float* __restrict__ dp,
   stf(dh, e, g);
 }
 
-__global__ void sum_partials_kernel(const float* __restrict__ red, int nb, int C, int which, float* __restrict__ out) {
+__global__ void sum_partials_kernel(const float* __restrict__ red, int nb, int C, float* __restrict__ out) {
   nf_pdl_begin();
   double S, Q;
-  reduce_partials32(red, nb, C, S, Q);
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  if (c >= C || threadIdx.y != 0) return;
-  out[c] = (float)(which ? Q : S);
+  reduce_partials8(red, nb, C, S, Q);
+  const int c = reduced_channel(C);
+  if (c >= C) return;
+  out[c] = (float)S;
 }
 
 __global__ void bn_bwd_finalize_kernel(const float* __restrict__ red, int nb, int C, float* sdz, float* sdzx, float* gg,
                                        float* gb) {
   nf_pdl_begin();
   double a, b;
-  reduce_partials32(red, nb, C, a, b);
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  if (c >= C || threadIdx.y != 0) return;
+  reduce_partials8(red, nb, C, a, b);
+  const int c = reduced_channel(C);
+  if (c >= C) return;
   sdz[c] = (float)a;
   sdzx[c] = (float)b;
   gb[c] = (float)a;
@@ -640,6 +650,51 @@ __global__ void unpad_grad_kernel(const float* __restrict__ gwpad, size_t rows, 
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= rows * C) return;
   gw[e] = gwpad[(e / C) * Cp + e % C];
+}
+
+// out[i] = sum over the splits of part[k][i], in a fixed order.  V consecutive elements per thread (4: 16-byte loads) and LN lanes
+// over the splits per block of 256; a lane adds its splits in index order with four in flight, then the lanes are added in
+// order.  Many splits of few elements (148 of 36 864) want lanes, few splits of many elements a thread each.
+template <int V, int LN>
+__global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
+  nf_pdl_begin();
+  constexpr int kCols = 256 / LN;
+  __shared__ float sm[LN][kCols * V];
+  const int tx = threadIdx.x % kCols, ty = threadIdx.x / kCols;
+  const size_t i = ((size_t)blockIdx.x * kCols + tx) * V;
+  float s[V];
+#pragma unroll
+  for (int e = 0; e < V; ++e) s[e] = 0.f;
+  if (i < n) {
+    const float* src = part + (size_t)ty * n + i;
+#pragma unroll 4
+    for (int k = ty; k < splits; k += LN, src += (size_t)LN * n) {
+      if constexpr (V == 4) {
+        const float4 w = *reinterpret_cast<const float4*>(src);
+        s[0] += w.x; s[1] += w.y; s[2] += w.z; s[3] += w.w;
+      } else {
+        s[0] += *src;
+      }
+    }
+  }
+  if constexpr (LN > 1) {
+#pragma unroll
+    for (int e = 0; e < V; ++e) sm[ty][tx * V + e] = s[e];
+    __syncthreads();
+    if (threadIdx.x < kCols * V) {  // one thread per element
+      float v = sm[0][threadIdx.x];
+#pragma unroll
+      for (int l = 1; l < LN; ++l) v += sm[l][threadIdx.x];
+      const size_t o = (size_t)blockIdx.x * kCols * V + threadIdx.x;
+      if (o < n) out[o] = v;
+    }
+  } else if (i < n) {
+    if constexpr (V == 4) {
+      *reinterpret_cast<float4*>(out + i) = make_float4(s[0], s[1], s[2], s[3]);
+    } else {
+      out[i] = s[0];
+    }
+  }
 }
 
 // Momentum SGD over up to kSgdMaxArenas parameter arenas in one launch (all layers of a block).  An arena is a multiple
@@ -1381,14 +1436,14 @@ int nf_k_channel_sums(int dtype, const void* src, size_t P, int C, float* red, s
 int nf_k_bn_finalize(const float* red, int nblocks, int C, double M, const float* gamma, const float* beta,
                        float eps, float bn_momentum, float* scale, float* shift, float* mu, float* invstd,
                        float* rmean, float* rvar) {
-  nf_launch(bn_finalize_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, M, gamma, beta, eps, bn_momentum, scale,
+  nf_launch(bn_finalize_kernel, nblk(C, kRedCh), kRedThreads, 0, red, nblocks, C, M, gamma, beta, eps, bn_momentum, scale,
                                                             shift, mu, invstd, rmean, rvar);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 int nf_k_partial_totals(const float* red, int nblocks, int C, double* tot) {
-  nf_launch(partial_totals_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, tot);
+  nf_launch(partial_totals_kernel, nblk(C, kRedCh), kRedThreads, 0, red, nblocks, C, tot);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1593,8 +1648,8 @@ int nf_k_dh(int dtype, const void* h, const float* dp, int N, int Ha, int Wa, in
   return NF_OK;
 }
 
-int nf_k_sum_partials(const float* red, int nblocks, int C, int which, float* out) {
-  nf_launch(sum_partials_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, which, out);
+int nf_k_sum_partials(const float* red, int nblocks, int C, float* out) {
+  nf_launch(sum_partials_kernel, nblk(C, kRedCh), kRedThreads, 0, red, nblocks, C, out);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1639,7 +1694,7 @@ int nf_k_write_dz(int dtype, const void* y, const void* da, int N, int Ho, int W
 
 int nf_k_bn_bwd_finalize(const float* red, int nblocks, int C, float* sdz, float* sdzx, float* ggamma,
                            float* gbeta) {
-  nf_launch(bn_bwd_finalize_kernel, nblk(C, 32), dim3(32, 32), 0, red, nblocks, C, sdz, sdzx, ggamma, gbeta);
+  nf_launch(bn_bwd_finalize_kernel, nblk(C, kRedCh), kRedThreads, 0, red, nblocks, C, sdz, sdzx, ggamma, gbeta);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -1694,6 +1749,22 @@ int nf_k_pad_weights(const bf16* w, size_t rows, int C, int Cp, bf16* wpad) {
 }
 int nf_k_unpad_grad(const float* gwpad, size_t rows, int C, int Cp, float* gw) {
   nf_launch(unpad_grad_kernel, nblk(rows * C, 256), 256, 0, gwpad, rows, C, Cp, gw);
+  NF_LAUNCHED();
+  return NF_OK;
+}
+
+int nf_k_sum_parts(const float* part, int splits, size_t n, float* out) {
+  const bool vec = n % 4 == 0 && (((uintptr_t)part | (uintptr_t)out) & 15) == 0;
+  if (splits >= 16 && n <= 16384) {
+    if (vec) nf_launch(sum_parts_kernel<4, 32>, nblk(n, 32), 256, 0, part, splits, n, out);
+    else nf_launch(sum_parts_kernel<1, 8>, nblk(n, 32), 256, 0, part, splits, n, out);
+  } else if (splits >= 16) {
+    if (vec) nf_launch(sum_parts_kernel<4, 8>, nblk(n, 128), 256, 0, part, splits, n, out);
+    else nf_launch(sum_parts_kernel<1, 8>, nblk(n, 32), 256, 0, part, splits, n, out);
+  } else {
+    if (vec) nf_launch(sum_parts_kernel<4, 1>, nblk(n, 1024), 256, 0, part, splits, n, out);
+    else nf_launch(sum_parts_kernel<1, 1>, nblk(n, 256), 256, 0, part, splits, n, out);
+  }
   NF_LAUNCHED();
   return NF_OK;
 }

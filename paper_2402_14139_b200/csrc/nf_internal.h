@@ -124,6 +124,8 @@ int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void*
 int nf_k_wgrad_splits(int N, int Ho, int Ci, int Co);
 int nf_k_wgrad(int dtype, const void* x, int N, int H, int W, int Ci, const void* g, int Co, int stride,
                  float* part, size_t part_floats, float* dw);
+// out[i] = sum over k of part[k][i], i < n: the split partials of a weight gradient
+int nf_k_sum_parts(const float* part, int splits, size_t n, float* out);
 int nf_k_channel_blocks(size_t P, int C);
 int nf_k_channel_sums(int dtype, const void* src, size_t P, int C, float* red, size_t red_floats, int* nblocks);
 int nf_k_bn_finalize(const float* red, int nblocks, int C, double M, const float* gamma, const float* beta,
@@ -183,7 +185,7 @@ int nf_k_fc_predict(const float* p, int N, int D, int K, const float* Wf, const 
 int nf_k_fc_wgrad(const float* p, const float* dlogits, const float* lossn, int N, int D, int K, float* gWf,
                     float* gbf, float* loss_out, int32_t* status, int n_scale);
 int nf_k_dh(int dtype, const void* h, const float* dp, int N, int Ha, int Wa, int F, void* dh);
-int nf_k_sum_partials(const float* red, int nblocks, int C, int which, float* out);
+int nf_k_sum_partials(const float* red, int nblocks, int C, float* out);
 int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
                          const float* scale, const float* shift, const float* mu, const float* invstd, float* red,
                          size_t red_floats, int* nblocks, const void* skip = nullptr);
