@@ -464,16 +464,15 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   } else {
     NF_TRY(nf_k_conv(dt, L->dh, N, Ha, Wa, F, Wx, (long)F * Co, 1, Co, 1, nullptr, 0, 1, Co, L->da));
   }
-  // a trainable shortcut joined at the BatchNorm output gets the gradient at that sum
-  if (L->skip_grad) NF_TRY(nf_k_write_dz(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->skip, L->skip_grad));
   trace_end();
-  // back through pool / ReLU / BatchNorm
+  // back through pool / ReLU / BatchNorm; a trainable shortcut joined at the BatchNorm output gets the gradient dz at that sum
   trace_begin(5);
   if (bn_nb) {
     nb = bn_nb;
+    if (L->skip_grad) NF_TRY(nf_k_write_dz(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->skip, L->skip_grad));
   } else {
     NF_TRY(nf_k_bn_bwd_reduce(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->mu, L->invstd, L->red,
-                                L->red_floats, &nb, L->skip));
+                                L->red_floats, &nb, L->skip, L->skip_grad));
   }
   if (!all) return nf_k_partial_totals(L->red, nb, Co, L->dptot + 2 * Co);
   }

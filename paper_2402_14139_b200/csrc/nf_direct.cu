@@ -6,64 +6,208 @@
 
 namespace {
 
-// ------------------------------------------------------------------ direct 3x3 convolution, pad 1
-// y[n,i,j,co] = act(bias[co] + sum_{kh,kw,ci} w(tap,co,ci) * x[n, i*s+kh-1, j*s+kw-1, ci]).
+// ------------------------------------------------------------------ direct convolution, 3x3 with pad 1 or 1x1
+// y[n,i,j,co] = act(bias[co] + sum_{kh,kw,ci} w(tap,co,ci) * x[n, i*s+kh-pad, j*s+kw-pad, ci]).
 // Weight element (tap,co,ci) sits at w[t*ws_tap + co*ws_co + ci*ws_ci] with t = tap, or 8-tap when
 // flip is set (flip + swapped strides turn the same kernel into the input-gradient convolution).
-constexpr int CT_P = 16, CT_CO = 16, CT_CI = 32;
+//
+// A block owns PX output pixels (of any images) x CO channels, a thread TP x TC of them; per step (chunk of CK input channels, tap)
+// the operands go to shared memory transposed, the next step's loads fly meanwhile, one barrier per step.  Every output is ONE
+// fp32 chain over chunk, tap, channel, whatever the tile, so the tile is chosen by size alone: 64 x 64 where that fills the
+// chip, 32 x 32 below, 64 x 16 for few output channels.  (The earlier kernel gave each block 16 pixels of one row and 16 channels
+// and each thread one output: 2 loads per multiply-add, 7 TFLOP/s; 16 -> 8 channels on 8 images of 32x32 20 us.)
+struct ConvArgs {
+  const void* x;
+  const void* w;
+  void* y;
+  const float* bias;
+  long ws_tap, ws_co, ws_ci;
+  int H, W, Ci, Co, Ho, Wo, stride, taps, flip, relu;
+  uint32_t P;  // output pixels
+};
+
+// WCO: 1 = eight consecutive output channels of the weights are contiguous, 0 = eight input channels.  VEC: rows of eight are
+// whole and aligned; otherwise elements are fetched one by one.
+template <typename T, int PX, int CO, int CK, int TP, int TC, int WCO, int VEC>
+__global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(const ConvArgs a) {
+  nf_pdl_begin();
+  constexpr int kThr = (PX / TP) * (CO / TC), kXU = PX * CK / 8, kWU = CO * CK / 8;  // units of eight values per step
+  constexpr int kXN = (kXU + kThr - 1) / kThr, kWN = (kWU + kThr - 1) / kThr;
+  // column q of row c is kept at q ^ (8 * (c / 8)) (mod the row): the transposing stores then hit different banks
+  constexpr int kXM = PX >= 32 ? 24 : 8, kWM = CO >= 32 ? 24 : 8;
+  __shared__ __align__(16) float xs[2][CK][PX];
+  __shared__ __align__(16) float ws[2][CK][CO];
+  const T* __restrict__ x = reinterpret_cast<const T*>(a.x);
+  const T* __restrict__ w = reinterpret_cast<const T*>(a.w);
+  const int t = threadIdx.x, tc = t % (CO / TC), tp = t / (CO / TC);
+  const uint32_t p0 = blockIdx.x * PX;
+  const int co0 = blockIdx.y * CO, pad = a.taps == 9 ? 1 : 0;
+
+  int xi[kXN], xj[kXN];   // input row and column of the unit's pixel at tap (0, 0)
+  size_t xb[kXN];         // its image's first element; pixels past the end: marked by a row far outside
+#pragma unroll
+  for (int u = 0; u < kXN; ++u) {
+    const int e = t + u * kThr;
+    const uint32_t p = p0 + e / (CK / 8);
+    const uint32_t r = p / a.Wo, n = r / a.Ho;
+    xj[u] = (int)(p - r * a.Wo) * a.stride - pad;
+    xi[u] = p < a.P && e < kXU ? (int)(r - n * a.Ho) * a.stride - pad : -1000000;
+    xb[u] = (size_t)n * a.H * a.W * a.Ci;
+  }
+  float xr[kXN][8], wr[kWN][8];
+  auto fetch = [&](int c0, int tap) {
+    const int kh = tap / 3, kw = tap - kh * 3;
+#pragma unroll
+    for (int u = 0; u < kXN; ++u) {
+      const int e = t + u * kThr, ci = c0 + (e % (CK / 8)) * 8;
+      const int ii = xi[u] + kh, jj = xj[u] + kw;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) xr[u][q] = 0.f;
+      if (ii >= 0 && ii < a.H && jj >= 0 && jj < a.W && ci < a.Ci) {
+        const T* src = x + xb[u] + ((size_t)ii * a.W + jj) * a.Ci + ci;
+        if constexpr (VEC) {
+          ld8(src, xr[u]);
+        } else {
+          for (int q = 0; q < 8 && ci + q < a.Ci; ++q) xr[u][q] = ldf(src, q);
+        }
+      }
+    }
+    const size_t tb = (size_t)(a.flip ? 8 - tap : tap) * a.ws_tap;
+#pragma unroll
+    for (int u = 0; u < kWN; ++u) {
+      const int e = t + u * kThr;
+      const int ci = c0 + (WCO ? e / (CO / 8) : (e % (CK / 8)) * 8), co = co0 + (WCO ? (e % (CO / 8)) * 8 : e / (CK / 8));
+#pragma unroll
+      for (int q = 0; q < 8; ++q) wr[u][q] = 0.f;
+      if (e < kWU && ci < a.Ci && co < a.Co) {
+        const T* src = w + tb + (size_t)co * a.ws_co + (size_t)ci * a.ws_ci;
+        if constexpr (VEC) {
+          ld8(src, wr[u]);
+        } else {
+          for (int q = 0; q < 8 && (WCO ? co + q < a.Co : ci + q < a.Ci); ++q) wr[u][q] = ldf(src, (size_t)q * (WCO ? a.ws_co : a.ws_ci));
+        }
+      }
+    }
+  };
+  auto put = [&](int b) {
+#pragma unroll
+    for (int u = 0; u < kXN; ++u) {
+      const int e = t + u * kThr;
+      if (e < kXU) {
+        const int cc = e % (CK / 8), px = e / (CK / 8);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) xs[b][cc * 8 + q][px ^ ((cc * 8) & kXM)] = xr[u][q];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kWN; ++u) {
+      const int e = t + u * kThr;
+      if (e < kWU) {
+        if constexpr (WCO) {
+          const int c = e / (CO / 8), q0 = (e % (CO / 8)) * 8;
+          float* dst = &ws[b][c][q0 ^ (c & ~7 & kWM)];
+          *reinterpret_cast<float4*>(dst) = make_float4(wr[u][0], wr[u][1], wr[u][2], wr[u][3]);
+          *reinterpret_cast<float4*>(dst + 4) = make_float4(wr[u][4], wr[u][5], wr[u][6], wr[u][7]);
+        } else {
+          const int cc = e % (CK / 8), co = e / (CK / 8);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) ws[b][cc * 8 + q][co ^ ((cc * 8) & kWM)] = wr[u][q];
+        }
+      }
+    }
+  };
+
+  float acc[TP][TC];
+#pragma unroll
+  for (int i = 0; i < TP; ++i)
+#pragma unroll
+    for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
+  fetch(0, 0);
+  put(0);
+  __syncthreads();
+  int c0 = 0, tap = 0, b = 0;
+  while (true) {
+    int nc = c0, nt = tap + 1;
+    if (nt == a.taps) {
+      nt = 0;
+      nc += CK;
+    }
+    const bool more = nc < a.Ci;
+    if (more) fetch(nc, nt);
+#pragma unroll 8
+    for (int c = 0; c < CK; ++c) {
+      float xv[TP], wv[TC];
+      const float* xp = &xs[b][c][(tp * TP) ^ (c & ~7 & kXM)];
+      const float* wp = &ws[b][c][(tc * TC) ^ (c & ~7 & kWM)];
+      if constexpr (TP == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(xp);
+        xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
+      } else {
+        const float2 v = *reinterpret_cast<const float2*>(xp);
+        xv[0] = v.x; xv[1] = v.y;
+      }
+      if constexpr (TC == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(wp);
+        wv[0] = v.x; wv[1] = v.y; wv[2] = v.z; wv[3] = v.w;
+      } else {
+        const float2 v = *reinterpret_cast<const float2*>(wp);
+        wv[0] = v.x; wv[1] = v.y;
+      }
+#pragma unroll
+      for (int i = 0; i < TP; ++i)
+#pragma unroll
+        for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
+    }
+    if (!more) break;
+    put(b ^ 1);
+    __syncthreads();
+    b ^= 1;
+    c0 = nc;
+    tap = nt;
+  }
+  T* y = reinterpret_cast<T*>(a.y);
+#pragma unroll
+  for (int i = 0; i < TP; ++i) {
+    const uint32_t p = p0 + tp * TP + i;
+    if (p >= a.P) break;
+#pragma unroll
+    for (int j = 0; j < TC; ++j) {
+      const int co = co0 + tc * TC + j;
+      if (co < a.Co) {
+        float v = acc[i][j];
+        if (a.bias) v += a.bias[co];
+        if (a.relu) v = fmaxf(v, 0.f);
+        stf(y, (size_t)p * a.Co + co, v);
+      }
+    }
+  }
+}
+
+template <typename T, int PX, int CO, int CK, int TP, int TC>
+int launch_direct(const ConvArgs& a) {
+  const dim3 grid((unsigned)((a.P + PX - 1) / PX), (unsigned)((a.Co + CO - 1) / CO));
+  const int thr = (PX / TP) * (CO / TC);
+  const bool wco = a.ws_co == 1 && a.ws_ci != 1;
+  const bool vec = a.Ci % 8 == 0 && (((uintptr_t)a.x | (uintptr_t)a.w) & 15) == 0 && (wco ? a.Co % 8 == 0 && a.ws_ci % 8 == 0 : a.ws_ci == 1 && a.ws_co % 8 == 0) &&
+                   a.ws_tap % 8 == 0;
+  if (wco)
+    vec ? nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 1, 1>, grid, thr, 0, a)
+        : nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 1, 0>, grid, thr, 0, a);
+  else
+    vec ? nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 0, 1>, grid, thr, 0, a)
+        : nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 0, 0>, grid, thr, 0, a);
+  NF_LAUNCHED();
+  return NF_OK;
+}
 
 template <typename T>
-__global__ void __launch_bounds__(256) conv_direct_kernel(const T* __restrict__ x, int N, int H, int W, int Ci,
-                                                          const T* __restrict__ w, long ws_tap, long ws_co,
-                                                          long ws_ci, int flip, const float* __restrict__ bias,
-                                                          int relu, int s, int Co, int Ho, int Wo, T* __restrict__ y) {
-  nf_pdl_begin();
-  __shared__ float xs[3][CT_P * 2 + 2][CT_CI];
-  __shared__ float wsm[9][CT_CO][CT_CI + 1];
-  const int wt = (Wo + CT_P - 1) / CT_P, ct = (Co + CT_CO - 1) / CT_CO;
-  long b = blockIdx.x;
-  const int jt = b % wt; b /= wt;
-  const int cot = b % ct; b /= ct;
-  const int i = b % Ho;
-  const int n = b / Ho;
-  const int tid = threadIdx.x, co_l = tid % CT_CO, p_l = tid / CT_CO;
-  const int j0 = jt * CT_P, co0 = cot * CT_CO;
-  const int cols = (CT_P - 1) * s + 3;
-  float acc = 0.f;
-  for (int c0 = 0; c0 < Ci; c0 += CT_CI) {
-    const int cn = min(CT_CI, Ci - c0);
-    for (int e = tid; e < 3 * cols * CT_CI; e += 256) {
-      const int c = e % CT_CI, col = (e / CT_CI) % cols, r = e / (CT_CI * cols);
-      const int ii = i * s + r - 1, jj = j0 * s + col - 1;
-      float v = 0.f;
-      if (c < cn && ii >= 0 && ii < H && jj >= 0 && jj < W) v = ldf(x, (((size_t)n * H + ii) * W + jj) * Ci + c0 + c);
-      xs[r][col][c] = v;
-    }
-    for (int e = tid; e < 9 * CT_CO * CT_CI; e += 256) {
-      const int c = e % CT_CI, co = (e / CT_CI) % CT_CO, t = e / (CT_CI * CT_CO);
-      float v = 0.f;
-      if (c < cn && co0 + co < Co)
-        v = ldf(w, (size_t)((flip ? 8 - t : t) * ws_tap + (co0 + co) * ws_co + (c0 + c) * ws_ci));
-      wsm[t][co][c] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kh = 0; kh < 3; ++kh)
-#pragma unroll
-      for (int kw = 0; kw < 3; ++kw) {
-        const float* xr = xs[kh][p_l * s + kw];
-        const float* wr = wsm[kh * 3 + kw][co_l];
-#pragma unroll 8
-        for (int c = 0; c < CT_CI; ++c) acc = fmaf(xr[c], wr[c], acc);
-      }
-    __syncthreads();
-  }
-  const int j = j0 + p_l, co = co0 + co_l;
-  if (j < Wo && co < Co) {
-    if (bias) acc += bias[co];
-    if (relu) acc = fmaxf(acc, 0.f);
-    stf(y, (((size_t)n * Ho + i) * Wo + j) * Co + co, acc);
-  }
+int run_direct(const ConvArgs& a) {
+  // chunks of 16 where there are no more than 16 input channels: the same chain, half the shared memory work
+  if (a.Co <= 16) return a.Ci <= 16 ? launch_direct<T, 64, 16, 16, 2, 2>(a) : launch_direct<T, 64, 16, 32, 2, 2>(a);
+  // 64 x 64 tiles from one block per SM on (148): below that, four times as many blocks of 32 x 32 finish sooner
+  const long big = (long)((a.P + 63) / 64) * ((a.Co + 63) / 64);
+  if (big >= 148) return launch_direct<T, 64, 64, 32, 4, 4>(a);
+  return launch_direct<T, 32, 32, 32, 2, 2>(a);
 }
 
 // ------------------------------------------------------------------ direct weight gradient
@@ -270,16 +414,16 @@ int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void*
     NF_LAUNCHED();
     return NF_OK;
   }
-  const long blocks = (long)N * Ho * ((Wo + CT_P - 1) / CT_P) * ((Co + CT_CO - 1) / CT_CO);
-  if (blocks <= 0 || blocks > 0x7fffffffL) return NF_EUNSUPPORTED;
-  if (dtype == NF_F32)
-    nf_launch(conv_direct_kernel<float>, (unsigned)blocks, 256, 0, 
-        (const float*)x, N, H, W, Ci, (const float*)w, ws_tap, ws_co, ws_ci, flip, bias, relu, stride, Co, Ho, Wo, (float*)y);
-  else
-    nf_launch(conv_direct_kernel<bf16>, (unsigned)blocks, 256, 0, 
-        (const bf16*)x, N, H, W, Ci, (const bf16*)w, ws_tap, ws_co, ws_ci, flip, bias, relu, stride, Co, Ho, Wo, (bf16*)y);
-  NF_LAUNCHED();
-  return NF_OK;
+  return nf_k_conv_taps(dtype, x, N, H, W, Ci, w, 9, ws_tap, ws_co, ws_ci, flip, bias, relu, stride, Co, y);
+}
+
+int nf_k_conv_taps(int dtype, const void* x, int N, int H, int W, int Ci, const void* w, int taps, long ws_tap, long ws_co, long ws_ci,
+                   int flip, const float* bias, int relu, int stride, int Co, void* y) {
+  const int Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
+  const long P = (long)N * Ho * Wo;
+  if (P <= 0 || P > 0x7fffff00L || (Co + 15) / 16 > 65535) return NF_EUNSUPPORTED;
+  const ConvArgs a{x, w, y, bias, ws_tap, ws_co, ws_ci, H, W, Ci, Co, Ho, Wo, stride, taps, flip, relu, (uint32_t)P};
+  return dtype == NF_F32 ? run_direct<float>(a) : run_direct<bf16>(a);
 }
 
 int nf_k_wgrad_splits(int N, int Ho, int Ci, int Co) {

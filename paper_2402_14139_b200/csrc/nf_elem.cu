@@ -788,8 +788,12 @@ __global__ void __launch_bounds__(256) bn_apply_vec_kernel(const uint4* __restri
 
 
 // per-thread constants variant (256 % C8 == 0)
+// MODE of this and the two backward kernels below: 0 = ReLU, 1 = a shortcut tensor of y's shape is added before the ReLU, 2 = no
+// activation (a projection shortcut).  One element per thread took 18 us where 16-byte accesses take 5 (33 MB).
+template <int MODE>
 __global__ void __launch_bounds__(256) bn_apply_vec2_kernel(const uint4* __restrict__ y, int C8, const float* __restrict__ scale,
-                                                            const float* __restrict__ shift, size_t total8, uint4* __restrict__ out) {
+                                                            const float* __restrict__ shift, size_t total8, uint4* __restrict__ out,
+                                                            const uint4* __restrict__ skip) {
   nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8];
@@ -804,25 +808,35 @@ __global__ void __launch_bounds__(256) bn_apply_vec2_kernel(const uint4* __restr
     const bool two = e1 < total8;
     const uint4 ya = __ldg(y + e0);
     const uint4 yb = two ? __ldg(y + e1) : ya;
-    float v[8];
+    float v[8], k[8];
+    uint4 sa, sb;
+    if constexpr (MODE == 1) {
+      sa = __ldg(skip + e0);
+      sb = two ? __ldg(skip + e1) : sa;
+      unpack8(sa, k);
+    }
     unpack8(ya, v);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = fmaxf(fmaf(v[i], A[i], B[i]), 0.f);
+    for (int i = 0; i < 8; ++i) v[i] = MODE == 2 ? fmaf(v[i], A[i], B[i]) : fmaxf(fmaf(v[i], A[i], B[i]) + (MODE == 1 ? k[i] : 0.f), 0.f);
     out[e0] = pack8(v);
     if (two) {
       unpack8(yb, v);
+      if constexpr (MODE == 1) unpack8(sb, k);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = fmaxf(fmaf(v[i], A[i], B[i]), 0.f);
+      for (int i = 0; i < 8; ++i) v[i] = MODE == 2 ? fmaf(v[i], A[i], B[i]) : fmaxf(fmaf(v[i], A[i], B[i]) + (MODE == 1 ? k[i] : 0.f), 0.f);
       out[e1] = pack8(v);
     }
   }
 }
 
-// partial sums of (dz, dz*xhat) with dz = da * 1[y*scale+shift > 0]; red[(block*2+k)*C + c]
+// partial sums of (dz, dz*xhat) with dz = da * 1[y*scale+shift (+ skip) > 0]; red[(block*2+k)*C + c].  MODE 1 also
+// writes dz where a trainable shortcut wants it (dz_out not NULL).
+template <int MODE>
 __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da,
                                                                 size_t P, int C8, const float* __restrict__ scale,
                                                                 const float* __restrict__ shift, const float* __restrict__ mu,
-                                                                const float* __restrict__ invstd, float* __restrict__ red) {
+                                                                const float* __restrict__ invstd, float* __restrict__ red,
+                                                                const uint4* __restrict__ skip, uint4* __restrict__ dz_out) {
   nf_pdl_begin();
   __shared__ float sm[16][256];
   const int C = C8 * 8;
@@ -835,38 +849,34 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __r
     a[i] = 0.f; b[i] = 0.f;
   }
   const size_t p0 = P * blockIdx.x / gridDim.x, p1 = P * (blockIdx.x + 1) / gridDim.x;
-  if (pl < planes) {
-    size_t p = p0 + pl;
-    for (; p + planes < p1; p += 2 * (size_t)planes) {  // two pixels per iteration: four 16-byte loads in flight
-      const uint4 y0 = __ldg(y + p * C8 + g), d0 = __ldg(da + p * C8 + g);
-      const uint4 y1 = __ldg(y + (p + planes) * C8 + g), d1 = __ldg(da + (p + planes) * C8 + g);
-      float yv[8], dv[8];
-      unpack8(y0, yv);
-      unpack8(d0, dv);
+  constexpr int kU = 4;  // pixels per trip: eight (with a shortcut twelve) 16-byte loads in flight
+  for (size_t p = p0 + pl; p < p1; p += (size_t)kU * planes) {
+    uint4 yq[kU], dq[kU], sq[kU];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float dz = fmaf(yv[i], sc[i], sh[i]) > 0.f ? dv[i] : 0.f;
-        a[i] += dz;
-        b[i] = fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
-      }
-      unpack8(y1, yv);
-      unpack8(d1, dv);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float dz = fmaf(yv[i], sc[i], sh[i]) > 0.f ? dv[i] : 0.f;
-        a[i] += dz;
-        b[i] = fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
+    for (int u = 0; u < kU; ++u) {
+      const size_t q = p + (size_t)u * planes;
+      if (q < p1) {
+        yq[u] = __ldg(y + q * C8 + g);
+        dq[u] = __ldg(da + q * C8 + g);
+        if constexpr (MODE == 1) sq[u] = __ldg(skip + q * C8 + g);
       }
     }
-    for (; p < p1; p += planes) {
-      float yv[8], dv[8];
-      unpack8(__ldg(y + p * C8 + g), yv);
-      unpack8(__ldg(da + p * C8 + g), dv);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float dz = fmaf(yv[i], sc[i], sh[i]) > 0.f ? dv[i] : 0.f;
-        a[i] += dz;
-        b[i] = fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
+    for (int u = 0; u < kU; ++u) {
+      const size_t q = p + (size_t)u * planes;
+      if (q < p1) {
+        float yv[8], dv[8], kv[8];
+        unpack8(yq[u], yv);
+        unpack8(dq[u], dv);
+        if constexpr (MODE == 1) unpack8(sq[u], kv);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float dz = MODE == 2 || fmaf(yv[i], sc[i], sh[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
+          a[i] += dz;
+          b[i] = fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
+          dv[i] = dz;
+        }
+        if (MODE == 1 && dz_out) dz_out[q * C8 + g] = pack8(dv);
       }
     }
   }
@@ -937,11 +947,13 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec_kernel(const uint4* __re
 // Same result with per-thread constants: when 256 % C8 == 0 a thread keeps its 8 channels over the whole
 // grid-stride loop, and dy = s*dz + k1*y + k0 with k1 = -s*m2*invstd, k0 = s*(m2*invstd*mu - m1),
 // m1 = sum(dz)/M, m2 = sum(dz*xhat)/M: five instructions per element.
+template <int MODE>
 __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da, int C8,
                                                                 const float* __restrict__ scale, const float* __restrict__ shift,
                                                                 const float* __restrict__ mu, const float* __restrict__ invstd,
                                                                 const float* __restrict__ sdz, const float* __restrict__ sdzx,
-                                                                float invM, size_t total8, uint4* __restrict__ dy) {
+                                                                float invM, size_t total8, uint4* __restrict__ dy,
+                                                                const uint4* __restrict__ skip) {
   nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8], K1[8], K0[8];
@@ -963,21 +975,28 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const uint4* __r
       yb = __ldg(y + e1);
       db = __ldg(da + e1);
     }
-    float yv[8], dv[8], o[8];
+    float yv[8], dv[8], kv[8], o[8];
+    uint4 sa, sb;
+    if constexpr (MODE == 1) {
+      sa = __ldg(skip + e0);
+      sb = two ? __ldg(skip + e1) : sa;
+      unpack8(sa, kv);
+    }
     unpack8(ya, yv);
     unpack8(da0, dv);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float dz = fmaf(yv[i], A[i], B[i]) > 0.f ? dv[i] : 0.f;
+      const float dz = MODE == 2 || fmaf(yv[i], A[i], B[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
       o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i], K0[i]));
     }
     dy[e0] = pack8(o);
     if (two) {
       unpack8(yb, yv);
       unpack8(db, dv);
+      if constexpr (MODE == 1) unpack8(sb, kv);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const float dz = fmaf(yv[i], A[i], B[i]) > 0.f ? dv[i] : 0.f;
+        const float dz = MODE == 2 || fmaf(yv[i], A[i], B[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
         o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i], K0[i]));
       }
       dy[e1] = pack8(o);
@@ -1472,7 +1491,13 @@ int nf_k_bn_eval_coeffs(int C, const float* gamma, const float* beta, float eps,
 int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int pool, const float* scale,
                     const float* shift, void* out, const void* skip) {
   const size_t total = (size_t)N * (pool ? Ho / 2 : Ho) * (pool ? Wo / 2 : Wo) * C;
-  if (skip) {  // residual layers take the generic kernels
+  if (skip && vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
+    nf_launch(bn_apply_vec2_kernel<1>, vec_blocks(total / 8), 256, 0, (const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out,
+              (const uint4*)skip);
+    NF_LAUNCHED();
+    return NF_OK;
+  }
+  if (skip) {  // residual layers with a pool or odd channel counts take the generic kernels
     DISPATCH(dtype,
              (nf_launch(bn_apply_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, Ho, Wo, C, pool, scale, shift, total, (float*)out, (const float*)skip)),
              (nf_launch(bn_apply_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)y, Ho, Wo, C, pool, scale, shift, total, (bf16*)out, (const bf16*)skip)));
@@ -1486,7 +1511,8 @@ int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int po
     return NF_OK;
   }
   if (vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_apply_vec2_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out);
+    nf_launch(bn_apply_vec2_kernel<0>, vec_blocks(total / 8), 256, 0, (const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out,
+              nullptr);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1656,10 +1682,15 @@ int nf_k_sum_partials(const float* red, int nblocks, int C, float* out) {
 
 int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
                          const float* scale, const float* shift, const float* mu, const float* invstd, float* red,
-                         size_t red_floats, int* nblocks, const void* skip) {
+                         size_t red_floats, int* nblocks, const void* skip, void* dz_out) {
   const size_t P = (size_t)N * Ho * Wo;
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
+  const bool vec = vec_ok(dtype, C, pool) && 256 % (C / 8) == 0;
+  if (dz_out && !(skip && vec)) {  // else the reduction below writes it
+    const int rc = nf_k_write_dz(dtype, y, da, N, Ho, Wo, C, pool, scale, shift, skip, dz_out);
+    if (rc != NF_OK) return rc;
+  }
   if (!skip && pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
     nf_launch(bn_bwd_reduce_pool_vec_kernel, nb, 256, 0, (const uint4*)y, (const uint4*)da, P / 4, Ho, Wo, C / 8, scale, shift, mu,
                                                               invstd, red);
@@ -1667,8 +1698,13 @@ int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, 
     *nblocks = nb;
     return NF_OK;
   }
-  if (!skip && vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_bwd_reduce_vec_kernel, nb, 256, 0, (const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red);
+  if (vec) {
+    if (skip)
+      nf_launch(bn_bwd_reduce_vec_kernel<1>, nb, 256, 0, (const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red,
+                (const uint4*)skip, (uint4*)dz_out);
+    else
+      nf_launch(bn_bwd_reduce_vec_kernel<0>, nb, 256, 0, (const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red,
+                nullptr, nullptr);
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;
@@ -1704,6 +1740,12 @@ int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, i
                         const float* sdz, const float* sdzx, double M, void* dy, const void* skip) {
   const size_t total = (size_t)N * Ho * Wo * C;
   const float invM = (float)(1.0 / M);
+  if (skip && vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
+    nf_launch(bn_bwd_apply_vec2_kernel<1>, vec_blocks(total / 8), 256, 0, (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
+              invstd, sdz, sdzx, invM, total / 8, (uint4*)dy, (const uint4*)skip);
+    NF_LAUNCHED();
+    return NF_OK;
+  }
   if (skip) {
     DISPATCH(dtype,
              (nf_launch(bn_bwd_apply_kernel<float>, nblk(total, 256), 256, 0, (const float*)y, (const float*)da, Ho, Wo, C, pool, scale, shift, mu, invstd, sdz, sdzx, invM, total, (float*)dy, (const float*)skip)),
@@ -1718,8 +1760,8 @@ int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, i
     return NF_OK;
   }
   if (vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_bwd_apply_vec2_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
-                                                                            invstd, sdz, sdzx, invM, total / 8, (uint4*)dy);
+    nf_launch(bn_bwd_apply_vec2_kernel<0>, vec_blocks(total / 8), 256, 0, (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
+              invstd, sdz, sdzx, invM, total / 8, (uint4*)dy, nullptr);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1801,6 +1843,35 @@ int nf_k_gather(const void* cache, const int32_t* cache_labels, int cache_rows, 
   const size_t row16 = row_bytes / 16;
   nf_launch(gather_kernel, nblk((size_t)count * row16, 256), 256, 0, (const uint4*)cache, cache_labels, cache_rows, idx,
                                                                          count, row16, (uint4*)out, out_labels, status);
+  NF_LAUNCHED();
+  return NF_OK;
+}
+
+// ---- BatchNorm without an activation (projection shortcut), bf16 with 8 | C and C / 8 a divisor of 256; NF_EUNSUPPORTED otherwise
+static bool plain_ok(int dtype, int C) { return vec_ok(dtype, C, 0) && 256 % (C / 8) == 0; }
+int nf_k_bn_plain_apply(int dtype, const void* y, size_t P, int C, const float* scale, const float* shift, void* out) {
+  if (!plain_ok(dtype, C)) return NF_EUNSUPPORTED;
+  const size_t total8 = P * C / 8;
+  nf_launch(bn_apply_vec2_kernel<2>, vec_blocks(total8), 256, 0, (const uint4*)y, C / 8, scale, shift, total8, (uint4*)out, nullptr);
+  NF_LAUNCHED();
+  return NF_OK;
+}
+int nf_k_bn_plain_bwd_reduce(int dtype, const void* y, const void* dz, size_t P, int C, const float* mu, const float* invstd, float* red,
+                             size_t red_floats, int* nblocks) {
+  if (!plain_ok(dtype, C)) return NF_EUNSUPPORTED;
+  const int nb = nf_k_channel_blocks(P, C);
+  if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
+  nf_launch(bn_bwd_reduce_vec_kernel<2>, nb, 256, 0, (const uint4*)y, (const uint4*)dz, P, C / 8, mu, mu, mu, invstd, red, nullptr, nullptr);
+  NF_LAUNCHED();
+  *nblocks = nb;
+  return NF_OK;
+}
+int nf_k_bn_plain_bwd_apply(int dtype, const void* y, const void* dz, size_t P, int C, const float* scale, const float* mu,
+                            const float* invstd, const float* sdz, const float* sdzx, double M, void* dy) {
+  if (!plain_ok(dtype, C)) return NF_EUNSUPPORTED;
+  const size_t total8 = P * C / 8;
+  nf_launch(bn_bwd_apply_vec2_kernel<2>, vec_blocks(total8), 256, 0, (const uint4*)y, (const uint4*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx,
+            (float)(1.0 / M), total8, (uint4*)dy, nullptr);
   NF_LAUNCHED();
   return NF_OK;
 }

@@ -30,19 +30,6 @@ struct HeadArgs {
   int loss_kind, n_scale;
 };
 
-__device__ __forceinline__ void load8(const bf16* p, float (&v)[8]) {
-  const uint4 u = *reinterpret_cast<const uint4*>(p);
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    v[2 * i] = __uint_as_float(w[i] << 16);
-    v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-  }
-}
-__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
-  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
 __device__ __forceinline__ void store8(bf16* p, float (&v)[8]) {  // v becomes the values as stored
   uint32_t w[4];
 #pragma unroll
@@ -103,7 +90,7 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
       float v[4][8];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (q0 + u * kStep < px) load8(hn + (size_t)(q0 + u * kStep) * F + g * 8, v[u]);
+        if (q0 + u * kStep < px) ld8(hn + (size_t)(q0 + u * kStep) * F + g * 8, v[u]);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int q = q0 + u * kStep;
@@ -287,8 +274,8 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
     const int i = q / a.Wa, j = q - i * a.Wa;
     const int rc = i < r0 ? 0 : i >= r1 ? 1 : 2, cc = j < c0 ? 0 : j >= c1 ? 1 : 2;
     float v[8], o[8];
-    load8(hs + (size_t)q * F + g * 8, v);
-    load8(tab + (rc * 3 + cc) * F + g * 8, o);
+    ld8(hs + (size_t)q * F + g * 8, v);
+    ld8(tab + (rc * 3 + cc) * F + g * 8, o);
 #pragma unroll
     for (int e = 0; e < 8; ++e) o[e] = v[e] > 0.f ? o[e] : 0.f;
     store8(dhn + (size_t)q * F + g * 8, o);

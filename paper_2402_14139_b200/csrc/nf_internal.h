@@ -121,6 +121,9 @@ static inline size_t nf_esize(int dtype) { return dtype == NF_F32 ? 4 : 2; }
 // ---- generic CUDA-core kernels (nf_k_kernels.cu): any shape, fp32 or bf16 storage, fp32 accumulate
 int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void* w, long ws_tap, long ws_co,
                 long ws_ci, int flip, const float* bias, int relu, int stride, int Co, void* y);
+// the general form: taps = 9 (3x3, pad 1) or 1 (1x1, no pad)
+int nf_k_conv_taps(int dtype, const void* x, int N, int H, int W, int Ci, const void* w, int taps, long ws_tap, long ws_co, long ws_ci,
+                   int flip, const float* bias, int relu, int stride, int Co, void* y);
 int nf_k_wgrad_splits(int N, int Ho, int Ci, int Co);
 int nf_k_wgrad(int dtype, const void* x, int N, int H, int W, int Ci, const void* g, int Co, int stride,
                  float* part, size_t part_floats, float* dw);
@@ -188,12 +191,17 @@ int nf_k_dh(int dtype, const void* h, const float* dp, int N, int Ha, int Wa, in
 int nf_k_sum_partials(const float* red, int nblocks, int C, float* out);
 int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
                          const float* scale, const float* shift, const float* mu, const float* invstd, float* red,
-                         size_t red_floats, int* nblocks, const void* skip = nullptr);
+                         size_t red_floats, int* nblocks, const void* skip = nullptr, void* dz_out = nullptr);  // dz_out: dz is written too
 int nf_k_bn_bwd_finalize(const float* red, int nblocks, int C, float* sdz, float* sdzx, float* ggamma,
                            float* gbeta);
 int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
                         const float* scale, const float* shift, const float* mu, const float* invstd,
                         const float* sdz, const float* sdzx, double M, void* dy, const void* skip = nullptr);
+int nf_k_bn_plain_apply(int dtype, const void* y, size_t P, int C, const float* scale, const float* shift, void* out);
+int nf_k_bn_plain_bwd_reduce(int dtype, const void* y, const void* dz, size_t P, int C, const float* mu, const float* invstd, float* red,
+                             size_t red_floats, int* nblocks);
+int nf_k_bn_plain_bwd_apply(int dtype, const void* y, const void* dz, size_t P, int C, const float* scale, const float* mu,
+                            const float* invstd, const float* sdz, const float* sdzx, double M, void* dy);
 int nf_k_write_dz(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool, const float* scale,
                   const float* shift, const void* skip, void* dz);
 // channel padding of a first layer's input and weights, and the gradient of the real channels out of the padded result

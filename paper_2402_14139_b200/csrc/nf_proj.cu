@@ -30,41 +30,6 @@ struct nf_proj {
 
 namespace {
 
-constexpr int kPix = 8;  // output pixels per block of the forward kernel
-
-// ys[pix][co] = sum_ci w[ci][co] * x[n][s*i][s*j][ci]; block: kPix pixels, thread <-> output channel (strided over Cout)
-template <typename T>
-__global__ void __launch_bounds__(256) proj_fwd_kernel(const T* __restrict__ x, const T* __restrict__ w, int H, int W, int Ci, int Co,
-                                                       int Ho, int Wo, size_t P, int stride, T* __restrict__ ys) {
-  nf_pdl_begin();
-  extern __shared__ float xs[];  // [kPix][Ci]
-  const size_t p0 = (size_t)blockIdx.x * kPix;
-  for (int i = threadIdx.x; i < kPix * Ci; i += 256) {
-    const size_t p = p0 + i / Ci;
-    float v = 0.f;
-    if (p < P) {
-      const int j = (int)(p % Wo), r = (int)((p / Wo) % Ho);
-      const size_t n = p / ((size_t)Wo * Ho);
-      v = ldf(x, ((n * H + (size_t)r * stride) * W + (size_t)j * stride) * Ci + i % Ci);
-    }
-    xs[i] = v;
-  }
-  __syncthreads();
-  for (int co = threadIdx.x; co < Co; co += 256) {
-    float acc[kPix];
-#pragma unroll
-    for (int q = 0; q < kPix; ++q) acc[q] = 0.f;
-    for (int ci = 0; ci < Ci; ++ci) {
-      const float wv = ldf(w, (size_t)ci * Co + co);
-#pragma unroll
-      for (int q = 0; q < kPix; ++q) acc[q] = fmaf(wv, xs[q * Ci + ci], acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < kPix; ++q)
-      if (p0 + q < P) stf(ys, (p0 + q) * Co + co, acc[q]);
-  }
-}
-
 // s = ys * scale + shift (no activation: the sum with the layer's BatchNorm output passes through the layer's ReLU)
 template <typename T>
 __global__ void proj_affine_kernel(const T* __restrict__ ys, int C, const float* __restrict__ scale, const float* __restrict__ shift,
@@ -109,56 +74,79 @@ __global__ void proj_bwd_apply_kernel(const T* __restrict__ ys, const T* __restr
   stf(dys, e, scale[c] * (ldf(dz, e) - sdz[c] * invM - sh * sdzx[c] * invM));
 }
 
-// part[split][ci][co] = sum over the split's pixel range (ascending) of dys[pix][co] * x[n][s*i][s*j][ci];
-// block: 16 input channels x 64 output channels, thread <-> (4 input channels, one output channel)
-template <typename T>
+// part[split][ci][co] = sum over the split's pixel range (ascending) of dys[pix][co] * x[n][s*i][s*j][ci].  Block: 64 x 64 channels,
+// a thread 4 x 4 of them, 32 pixels per step with the next step's loads in flight; both operands lie in shared memory as they
+// do in memory, a pixel's channels in a row.  (16 x 64 channels with 16-pixel steps and one output row per thread took 132 us on
+// 64 -> 128 channels and 32 768 pixels.)
+template <typename T, int VEC>
 __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x, const T* __restrict__ dys, int H, int W, int Ci, int Co,
-                                                         int Ho, int Wo, size_t P, int stride, int splits, float* __restrict__ part) {
+                                                         int Ho, int Wo, uint32_t P, int stride, int splits, float* __restrict__ part) {
   nf_pdl_begin();
-  __shared__ float xs[16][16];   // [pixel][ci]
-  __shared__ float gs[16][64];   // [pixel][co]
-  const int ci0 = blockIdx.x * 16, co0 = blockIdx.y * 64, sp = blockIdx.z;
-  const size_t p0 = P * sp / splits, p1 = P * (sp + 1) / splits;
-  const int tco = threadIdx.x & 63, tci = (threadIdx.x >> 6) * 4;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (size_t pb = p0; pb < p1; pb += 16) {
-    {
-      const int q = threadIdx.x >> 4, c = threadIdx.x & 15;
-      const size_t p = pb + q;
-      float v = 0.f;
-      if (p < p1 && ci0 + c < Ci) {
-        const int j = (int)(p % Wo), r = (int)((p / Wo) % Ho);
-        const size_t n = p / ((size_t)Wo * Ho);
-        v = ldf(x, ((n * H + (size_t)r * stride) * W + (size_t)j * stride) * Ci + ci0 + c);
-      }
-      xs[q][c] = v;
-    }
-    for (int i = threadIdx.x; i < 16 * 64; i += 256) {
-      const int q = i >> 6, c = i & 63;
-      const size_t p = pb + q;
-      gs[q][c] = (p < p1 && co0 + c < Co) ? ldf(dys, p * Co + co0 + c) : 0.f;
-    }
-    __syncthreads();
+  __shared__ __align__(16) float xs[2][32][64];
+  __shared__ __align__(16) float gs[2][32][64];
+  const int ci0 = blockIdx.x * 64, co0 = blockIdx.y * 64, sp = blockIdx.z, t = threadIdx.x;
+  const uint32_t p0 = (uint32_t)((size_t)P * sp / splits), p1 = (uint32_t)((size_t)P * (sp + 1) / splits);
+  const int q = t >> 3, c = (t & 7) * 8;  // the thread's pixel and channels of a step
+  const int ti = (t >> 4) * 4, to = (t & 15) * 4;
+  float xr[8], gr[8];
+  auto row = [&](const T* src, int c0, int C, float(&v)[8]) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const float g = gs[q][tco];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] = fmaf(g, xs[q][tci + u], acc[u]);
+    for (int e = 0; e < 8; ++e) v[e] = 0.f;
+    if (c0 >= C) return;
+    if constexpr (VEC) {
+      ld8(src + c0, v);
+    } else {
+      for (int e = 0; e < 8 && c0 + e < C; ++e) v[e] = ldf(src, c0 + e);
     }
+  };
+  auto fetch = [&](uint32_t pb) {
+    const uint32_t p = pb + q;
+    if (p < p1) {
+      const uint32_t r = p / Wo, n = r / Ho;
+      row(x + (((size_t)n * H + (size_t)(r - n * Ho) * stride) * W + (size_t)(p - r * Wo) * stride) * Ci, ci0 + c, Ci, xr);
+      row(dys + (size_t)p * Co, co0 + c, Co, gr);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) xr[e] = gr[e] = 0.f;
+    }
+  };
+  auto put = [&](int b) {
+#pragma unroll
+    for (int e = 0; e < 8; e += 4) {
+      *reinterpret_cast<float4*>(&xs[b][q][c + e]) = make_float4(xr[e], xr[e + 1], xr[e + 2], xr[e + 3]);
+      *reinterpret_cast<float4*>(&gs[b][q][c + e]) = make_float4(gr[e], gr[e + 1], gr[e + 2], gr[e + 3]);
+    }
+  };
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  fetch(p0);
+  put(0);
+  __syncthreads();
+  int b = 0;
+  for (uint32_t pb = p0; pb < p1; pb += 32) {
+    const bool more = pb + 32 < p1;
+    if (more) fetch(pb + 32);
+#pragma unroll 8
+    for (int k = 0; k < 32; ++k) {
+      const float4 xv = *reinterpret_cast<const float4*>(&xs[b][k][ti]), gv = *reinterpret_cast<const float4*>(&gs[b][k][to]);
+      const float xa[4] = {xv.x, xv.y, xv.z, xv.w}, ga[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ga[j], xa[i], acc[i][j]);
+    }
+    if (more) put(b ^ 1);
     __syncthreads();
+    b ^= 1;
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
-    if (ci0 + tci + u < Ci && co0 + tco < Co) part[((size_t)sp * Ci + ci0 + tci + u) * Co + co0 + tco] = acc[u];
-}
-
-__global__ void proj_sum_splits_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
-  nf_pdl_begin();
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float s = 0.f;
-  for (int k = 0; k < splits; ++k) s += part[(size_t)k * n + i];
-  out[i] = s;
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (ci0 + ti + i < Ci && co0 + to + j < Co) part[((size_t)sp * Ci + ci0 + ti + i) * Co + co0 + to + j] = acc[i][j];
 }
 
 inline unsigned blocks_for(size_t n, int per) { return (unsigned)((n + per - 1) / per); }
@@ -191,10 +179,10 @@ size_t proj_plan(nf_proj* P, char* base) {
   P->red_floats = r1 > r2 ? r1 : r2;
   P->red = (float*)take(P->red_floats * 4);
   const size_t pix = (size_t)P->N * P->Ho * P->Wo;
-  const int tiles = ((P->Cin + 15) / 16) * ((P->Cout + 63) / 64);
-  long sp = 592 / tiles;  // about four waves of blocks
+  const int tiles = ((P->Cin + 63) / 64) * ((P->Cout + 63) / 64);
+  long sp = 296 / tiles;  // two blocks per SM
   if (sp < 1) sp = 1;
-  if ((size_t)sp > (pix + 15) / 16) sp = (long)((pix + 15) / 16);
+  if ((size_t)sp > (pix + 31) / 32) sp = (long)((pix + 31) / 32);
   P->splits = (int)sp;
   P->wpart = (float*)take((size_t)sp * P->Cin * P->Cout * 4);
   (void)state_end;
@@ -324,21 +312,15 @@ namespace {
   } while (0)
 
 int proj_conv(nf_proj* P, const void* xb, int count) {
-  const size_t pix = (size_t)count * P->Ho * P->Wo;
-  const size_t smem = (size_t)kPix * P->Cin * sizeof(float);
-  if (smem > 48 * 1024) return NF_EUNSUPPORTED;
-  const unsigned grid = blocks_for(pix, kPix);
-  PROJ_DISPATCH(P->dtype,
-                (nf_launch(proj_fwd_kernel<float>, grid, 256, smem, (const float*)xb, P->val + P->offW, P->H, P->W, P->Cin, P->Cout,
-                                                                        P->Ho, P->Wo, pix, 2, (float*)P->ys)),
-                (nf_launch(proj_fwd_kernel<bf16>, grid, 256, smem, (const bf16*)xb, P->shadow + P->offW, P->H, P->W, P->Cin, P->Cout,
-                                                                       P->Ho, P->Wo, pix, 2, (bf16*)P->ys)));
-  NF_LAUNCHED();
-  return NF_OK;
+  if (P->Cin > 1536) return NF_EUNSUPPORTED;
+  const void* w = P->dtype == NF_F32 ? (const void*)(P->val + P->offW) : (const void*)(P->shadow + P->offW);
+  return nf_k_conv_taps(P->dtype, xb, count, P->H, P->W, P->Cin, w, 1, 0, 1, P->Cout, 0, nullptr, 0, 2, P->Cout, P->ys);
 }
 
 int proj_affine(nf_proj* P, int count, void* s_out) {
-  const size_t total = (size_t)count * P->Ho * P->Wo * P->Cout;
+  const size_t pix = (size_t)count * P->Ho * P->Wo, total = pix * P->Cout;
+  const int rc = nf_k_bn_plain_apply(P->dtype, P->ys, pix, P->Cout, P->scale, P->shift, s_out);
+  if (rc != NF_EUNSUPPORTED) return rc;
   PROJ_DISPATCH(P->dtype,
                 (nf_launch(proj_affine_kernel<float>, blocks_for(total, 256), 256, 0, (const float*)P->ys, P->Cout, P->scale, P->shift,
                                                                                          total, (float*)s_out)),
@@ -384,30 +366,41 @@ int nf_proj_backward(nf_proj* P, const void* xb, const void* dz, float lr) {
   if (((uintptr_t)xb | (uintptr_t)dz) & 15) return NF_EALIGN;
   const int C = P->Cout;
   const size_t pix = (size_t)P->N * P->Ho * P->Wo, total = pix * C;
-  const int nb = (int)(pix < (size_t)kProjBlocks ? pix : (size_t)kProjBlocks);
-  PROJ_DISPATCH(P->dtype,
-                (nf_launch(proj_bwd_reduce_kernel<float>, nb, 256, 0, (const float*)P->ys, (const float*)dz, pix, C, P->mu, P->invstd, P->red)),
-                (nf_launch(proj_bwd_reduce_kernel<bf16>, nb, 256, 0, (const bf16*)P->ys, (const bf16*)dz, pix, C, P->mu, P->invstd, P->red)));
-  NF_LAUNCHED();
-  int rc = nf_k_bn_bwd_finalize(P->red, nb, C, P->sdz, P->sdzx, P->grad + P->offG, P->grad + P->offB);
+  int nb = 0;
+  int rc = nf_k_bn_plain_bwd_reduce(P->dtype, P->ys, dz, pix, C, P->mu, P->invstd, P->red, P->red_floats, &nb);
+  if (rc == NF_EUNSUPPORTED) {
+    nb = (int)(pix < (size_t)kProjBlocks ? pix : (size_t)kProjBlocks);
+    PROJ_DISPATCH(P->dtype,
+                  (nf_launch(proj_bwd_reduce_kernel<float>, nb, 256, 0, (const float*)P->ys, (const float*)dz, pix, C, P->mu, P->invstd, P->red)),
+                  (nf_launch(proj_bwd_reduce_kernel<bf16>, nb, 256, 0, (const bf16*)P->ys, (const bf16*)dz, pix, C, P->mu, P->invstd, P->red)));
+    NF_LAUNCHED();
+  } else if (rc != NF_OK) {
+    return rc;
+  }
+  rc = nf_k_bn_bwd_finalize(P->red, nb, C, P->sdz, P->sdzx, P->grad + P->offG, P->grad + P->offB);
   if (rc != NF_OK) return rc;
-  const float invM = (float)(1.0 / (double)pix);
-  PROJ_DISPATCH(P->dtype,
-                (nf_launch(proj_bwd_apply_kernel<float>, blocks_for(total, 256), 256, 0, (const float*)P->ys, (const float*)dz, C, P->scale, P->mu,
-                                                                                            P->invstd, P->sdz, P->sdzx, invM, total, (float*)P->dys)),
-                (nf_launch(proj_bwd_apply_kernel<bf16>, blocks_for(total, 256), 256, 0, (const bf16*)P->ys, (const bf16*)dz, C, P->scale, P->mu,
-                                                                                           P->invstd, P->sdz, P->sdzx, invM, total, (bf16*)P->dys)));
+  rc = nf_k_bn_plain_bwd_apply(P->dtype, P->ys, dz, pix, C, P->scale, P->mu, P->invstd, P->sdz, P->sdzx, (double)pix, P->dys);
+  if (rc == NF_EUNSUPPORTED) {
+    const float invM = (float)(1.0 / (double)pix);
+    PROJ_DISPATCH(P->dtype,
+                  (nf_launch(proj_bwd_apply_kernel<float>, blocks_for(total, 256), 256, 0, (const float*)P->ys, (const float*)dz, C, P->scale,
+                             P->mu, P->invstd, P->sdz, P->sdzx, invM, total, (float*)P->dys)),
+                  (nf_launch(proj_bwd_apply_kernel<bf16>, blocks_for(total, 256), 256, 0, (const bf16*)P->ys, (const bf16*)dz, C, P->scale, P->mu,
+                             P->invstd, P->sdz, P->sdzx, invM, total, (bf16*)P->dys)));
+    NF_LAUNCHED();
+  } else if (rc != NF_OK) {
+    return rc;
+  }
+  if (pix > 0x7fffffffu) return NF_EUNSUPPORTED;
+  const dim3 grid((P->Cin + 63) / 64, (C + 63) / 64, P->splits);
+  const bool vec = P->Cin % 8 == 0 && C % 8 == 0;
+#define PROJ_WGRAD(T, V)                                                                                                              \
+  nf_launch(proj_wgrad_kernel<T, V>, grid, 256, 0, (const T*)xb, (const T*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo, (uint32_t)pix, 2, \
+            P->splits, P->wpart)
+  PROJ_DISPATCH(P->dtype, (vec ? PROJ_WGRAD(float, 1) : PROJ_WGRAD(float, 0)), (vec ? PROJ_WGRAD(bf16, 1) : PROJ_WGRAD(bf16, 0)));
+#undef PROJ_WGRAD
   NF_LAUNCHED();
-  const dim3 grid((P->Cin + 15) / 16, (C + 63) / 64, P->splits);
-  PROJ_DISPATCH(P->dtype,
-                (nf_launch(proj_wgrad_kernel<float>, grid, 256, 0, (const float*)xb, (const float*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo,
-                                                                       pix, 2, P->splits, P->wpart)),
-                (nf_launch(proj_wgrad_kernel<bf16>, grid, 256, 0, (const bf16*)xb, (const bf16*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo,
-                                                                      pix, 2, P->splits, P->wpart)));
-  NF_LAUNCHED();
-  const size_t nw = (size_t)P->Cin * C;
-  nf_launch(proj_sum_splits_kernel, blocks_for(nw, 256), 256, 0, P->wpart, P->splits, nw, P->grad + P->offW);
-  NF_LAUNCHED();
+  if ((rc = nf_k_sum_parts(P->wpart, P->splits, (size_t)P->Cin * C, P->grad + P->offW)) != NF_OK) return rc;
   return nf_k_sgd(P->val, P->mom, P->grad, P->shadow, P->arena, lr, P->momentum);
 }
 

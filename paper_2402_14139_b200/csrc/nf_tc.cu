@@ -12,6 +12,8 @@
 //   sum and sum of squares of the stored (rounded) values are accumulated per CTA for BatchNorm.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "nf_ptx.cuh"
 #include "nf_tc.h"
 
@@ -1837,11 +1839,11 @@ void pick_tile(int N, int H, int W, int* BW, int* BH, int* BI) {
     }
 }
 bool tiles_exactly(int H, int W, int BW, int BH) { return W % BW == 0 && H % BH == 0; }
-// Whether a problem goes to the tensor cores at all.  Maps that tile exactly always do; the others from 8192 output pixels on
-// (64 tiles).  Below that a layer is a few launch-sized kernels either way, its gradients hang on a few thousand ReLU
-// decisions, and the CUDA-core kernels' fp32 sums (0.01 % of the bf16 outputs off the nearest value, against 0.04 - 0.13 %
-// here, 256 channels at 14x14) are worth more than the time: 0.9 % -> 6 % of a gradient's norm moves between the two on 648
-// pixels, 1 % on 12 000.
+// Whether a FORWARD convolution goes to the tensor cores.  Maps that tile exactly always do; the others from 8192 output pixels
+// on (64 tiles).  Below that a layer's gradients hang on a few thousand ReLU decisions, and the CUDA-core kernels' fp32 sums (0.01 %
+// of the bf16 outputs off the nearest value, against 0.04 - 0.13 % here, 256 channels at 14x14) are worth more than the time: up
+// to 6 % of a gradient's norm moves between the two on 648 pixels, 1 % on 12 000.  The gradients themselves decide nothing and
+// always run here.
 bool tc_size_ok(int N, int H, int W) {
   int BW, BH, BI;
   pick_tile(N, H, W, &BW, &BH, &BI);
@@ -2271,14 +2273,13 @@ void nf_tc_select(nf_layer* L) {
     L->cin_pad = 64;
   const int Cin = L->cin_pad ? L->cin_pad : L->Cin;
   if (main_ok && plan_fwd(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[0] = 1;
-  if (main_ok && plan_wgrad(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[1] = 1;
-  if (!aux_ok) return;
+  if (plan_wgrad(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[1] = 1;
   if (wide_aux(L)) {  // more than 64 filters: the aux conv runs on the kernels of the main conv
-    if (plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok) L->fam[2] = 1;
+    if (aux_ok && plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok) L->fam[2] = 1;
     if (plan_wgrad(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok && plan_fwd(L->Ha, L->Wa, L->F, L->Cout, L->o.N, 0).ok) L->fam[3] = 1;
     return;
   }
-  if (plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 1).ok) L->fam[2] = 1;
+  if (aux_ok && plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 1).ok) L->fam[2] = 1;
   if (plan_wgrad(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 1).ok && plan_fwd(L->Ha, L->Wa, L->F, L->Cout, L->o.N, 2).ok) L->fam[3] = 1;
 }
 
@@ -2444,10 +2445,17 @@ int nf_tc_aux_wgrad(nf_layer* L, const void* a) {
                    L->status, wide_aux(L) ? 0 : 1);
 }
 
+// The stand-alone weight gradient takes maps that no tile divides only where its split partials need no more scratch than the
+// CUDA-core kernel would, or fit the library's own array: what a caller's scratch was enough for stays accepted.
+static bool standalone_wgrad_ok(int N, int Ho, int Wo, int Cin, int Cout, const WgPlan& pl) {
+  const size_t limit = std::max((size_t)nf_k_wgrad_splits(N, Ho, Cin, Cout) * 9 * Cout * Cin, (size_t)NF_STATIC_SCRATCH_BYTES / sizeof(float));
+  return pl.ok && (tiles_exactly(Ho, Wo, pl.BW, pl.BH) || pl.part_floats <= limit);
+}
+
 size_t nf_tc_conv3x3_wgrad_scratch_floats(int N, int H, int W, int Cin, int Cout, int stride) {
-  if (!tc_size_ok(N, (H - 1) / stride + 1, (W - 1) / stride + 1)) return 0;
-  const WgPlan pl = plan_wgrad((H - 1) / stride + 1, (W - 1) / stride + 1, Cin, Cout, N, 0, stride);
-  return pl.ok ? pl.part_floats : 0;
+  const int Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
+  const WgPlan pl = plan_wgrad(Ho, Wo, Cin, Cout, N, 0, stride);
+  return standalone_wgrad_ok(N, Ho, Wo, Cin, Cout, pl) ? pl.part_floats : 0;
 }
 
 static __device__ int32_t g_op_status;  // status word of the stand-alone operations (one per device that loads the library)
@@ -2470,7 +2478,8 @@ int nf_tc_conv3x3_forward(const void* x, const void* w, int N, int H, int W, int
 
 int nf_tc_conv3x3_wgrad(const void* x, const void* g, int N, int H, int W, int Cin, int Cout, int stride, float* part,
                         size_t part_floats, float* dw) {
-  if (!tc_size_ok(N, (H - 1) / stride + 1, (W - 1) / stride + 1)) return NF_EUNSUPPORTED;
+  const int Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
+  if (!standalone_wgrad_ok(N, Ho, Wo, Cin, Cout, plan_wgrad(Ho, Wo, Cin, Cout, N, 0, stride))) return NF_EUNSUPPORTED;
   int32_t* st = nullptr;
   if (nf_tc_op_status_ptr(&st) != NF_OK) return NF_ECUDA;
   return run_wgrad(N, H, W, Cin, Cout, x, g, part, part_floats, dw, st, 0, stride);
