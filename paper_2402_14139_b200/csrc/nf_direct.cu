@@ -28,15 +28,15 @@ struct ConvArgs {
 
 // WCO: 1 = eight consecutive output channels of the weights are contiguous, 0 = eight input channels.  VEC: rows of eight are
 // whole and aligned; otherwise elements are fetched one by one.
-template <typename T, int PX, int CO, int CK, int TP, int TC, int WCO, int VEC>
+template <typename T, int PX, int CO, int CK, int TP, int TC, int SPB, int WCO, int VEC>
 __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(const ConvArgs a) {
   nf_pdl_begin();
   constexpr int kThr = (PX / TP) * (CO / TC), kXU = PX * CK / 8, kWU = CO * CK / 8;  // units of eight values per step
   constexpr int kXN = (kXU + kThr - 1) / kThr, kWN = (kWU + kThr - 1) / kThr;
   // column q of row c is kept at q ^ (8 * (c / 8)) (mod the row): the transposing stores then hit different banks
   constexpr int kXM = PX >= 32 ? 24 : 8, kWM = CO >= 32 ? 24 : 8;
-  __shared__ __align__(16) float xs[2][CK][PX];
-  __shared__ __align__(16) float ws[2][CK][CO];
+  __shared__ __align__(16) float xs[2][SPB][CK][PX];
+  __shared__ __align__(16) float ws[2][SPB][CK][CO];
   const T* __restrict__ x = reinterpret_cast<const T*>(a.x);
   const T* __restrict__ w = reinterpret_cast<const T*>(a.w);
   const int t = threadIdx.x, tc = t % (CO / TC), tp = t / (CO / TC);
@@ -54,8 +54,8 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
     xi[u] = p < a.P && e < kXU ? (int)(r - n * a.Ho) * a.stride - pad : -1000000;
     xb[u] = (size_t)n * a.H * a.W * a.Ci;
   }
-  float xr[kXN][8], wr[kWN][8];
-  auto fetch = [&](int c0, int tap) {
+  float xr_[SPB][kXN][8], wr_[SPB][kWN][8];
+  auto fetch = [&](int c0, int tap, float(&xr)[kXN][8], float(&wr)[kWN][8]) {
     const int kh = tap / 3, kw = tap - kh * 3;
 #pragma unroll
     for (int u = 0; u < kXN; ++u) {
@@ -89,14 +89,14 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
       }
     }
   };
-  auto put = [&](int b) {
+  auto put = [&](float(&xs)[CK][PX], float(&ws)[CK][CO], const float(&xr)[kXN][8], const float(&wr)[kWN][8]) {
 #pragma unroll
     for (int u = 0; u < kXN; ++u) {
       const int e = t + u * kThr;
       if (e < kXU) {
         const int cc = e % (CK / 8), px = e / (CK / 8);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) xs[b][cc * 8 + q][px ^ ((cc * 8) & kXM)] = xr[u][q];
+        for (int q = 0; q < 8; ++q) xs[cc * 8 + q][px ^ ((cc * 8) & kXM)] = xr[u][q];
       }
     }
 #pragma unroll
@@ -105,13 +105,13 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
       if (e < kWU) {
         if constexpr (WCO) {
           const int c = e / (CO / 8), q0 = (e % (CO / 8)) * 8;
-          float* dst = &ws[b][c][q0 ^ (c & ~7 & kWM)];
+          float* dst = &ws[c][q0 ^ (c & ~7 & kWM)];
           *reinterpret_cast<float4*>(dst) = make_float4(wr[u][0], wr[u][1], wr[u][2], wr[u][3]);
           *reinterpret_cast<float4*>(dst + 4) = make_float4(wr[u][4], wr[u][5], wr[u][6], wr[u][7]);
         } else {
           const int cc = e % (CK / 8), co = e / (CK / 8);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) ws[b][cc * 8 + q][co ^ ((cc * 8) & kWM)] = wr[u][q];
+          for (int q = 0; q < 8; ++q) ws[cc * 8 + q][co ^ ((cc * 8) & kWM)] = wr[u][q];
         }
       }
     }
@@ -122,44 +122,52 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
   for (int i = 0; i < TP; ++i)
 #pragma unroll
     for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
-  fetch(0, 0);
-  put(0);
+  // steps (chunk, tap) go SPB at a time; `taps` is a multiple of SPB wherever SPB > 1
+#pragma unroll
+  for (int i = 0; i < SPB; ++i) fetch(0, i, xr_[i], wr_[i]);
+#pragma unroll
+  for (int i = 0; i < SPB; ++i) put(xs[0][i], ws[0][i], xr_[i], wr_[i]);
   __syncthreads();
   int c0 = 0, tap = 0, b = 0;
   while (true) {
-    int nc = c0, nt = tap + 1;
+    int nc = c0, nt = tap + SPB;
     if (nt == a.taps) {
       nt = 0;
       nc += CK;
     }
     const bool more = nc < a.Ci;
-    if (more) fetch(nc, nt);
+    if (more)
+#pragma unroll
+      for (int i = 0; i < SPB; ++i) fetch(nc, nt + i, xr_[i], wr_[i]);
+#pragma unroll 1
+    for (int st = 0; st < SPB; ++st)
 #pragma unroll 8
-    for (int c = 0; c < CK; ++c) {
-      float xv[TP], wv[TC];
-      const float* xp = &xs[b][c][(tp * TP) ^ (c & ~7 & kXM)];
-      const float* wp = &ws[b][c][(tc * TC) ^ (c & ~7 & kWM)];
-      if constexpr (TP == 4) {
-        const float4 v = *reinterpret_cast<const float4*>(xp);
-        xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
-      } else {
-        const float2 v = *reinterpret_cast<const float2*>(xp);
-        xv[0] = v.x; xv[1] = v.y;
-      }
-      if constexpr (TC == 4) {
-        const float4 v = *reinterpret_cast<const float4*>(wp);
-        wv[0] = v.x; wv[1] = v.y; wv[2] = v.z; wv[3] = v.w;
-      } else {
-        const float2 v = *reinterpret_cast<const float2*>(wp);
-        wv[0] = v.x; wv[1] = v.y;
-      }
+      for (int c = 0; c < CK; ++c) {
+        float xv[TP], wv[TC];
+        const float* xp = &xs[b][st][c][(tp * TP) ^ (c & ~7 & kXM)];
+        const float* wp = &ws[b][st][c][(tc * TC) ^ (c & ~7 & kWM)];
+        if constexpr (TP == 4) {
+          const float4 v = *reinterpret_cast<const float4*>(xp);
+          xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
+        } else {
+          const float2 v = *reinterpret_cast<const float2*>(xp);
+          xv[0] = v.x; xv[1] = v.y;
+        }
+        if constexpr (TC == 4) {
+          const float4 v = *reinterpret_cast<const float4*>(wp);
+          wv[0] = v.x; wv[1] = v.y; wv[2] = v.z; wv[3] = v.w;
+        } else {
+          const float2 v = *reinterpret_cast<const float2*>(wp);
+          wv[0] = v.x; wv[1] = v.y;
+        }
 #pragma unroll
-      for (int i = 0; i < TP; ++i)
+        for (int i = 0; i < TP; ++i)
 #pragma unroll
-        for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
-    }
+          for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
+      }
     if (!more) break;
-    put(b ^ 1);
+#pragma unroll
+    for (int i = 0; i < SPB; ++i) put(xs[b ^ 1][i], ws[b ^ 1][i], xr_[i], wr_[i]);
     __syncthreads();
     b ^= 1;
     c0 = nc;
@@ -183,7 +191,7 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
   }
 }
 
-template <typename T, int PX, int CO, int CK, int TP, int TC>
+template <typename T, int PX, int CO, int CK, int TP, int TC, int SPB>
 int launch_direct(const ConvArgs& a) {
   const dim3 grid((unsigned)((a.P + PX - 1) / PX), (unsigned)((a.Co + CO - 1) / CO));
   const int thr = (PX / TP) * (CO / TC);
@@ -191,23 +199,27 @@ int launch_direct(const ConvArgs& a) {
   const bool vec = a.Ci % 8 == 0 && (((uintptr_t)a.x | (uintptr_t)a.w) & 15) == 0 && (wco ? a.Co % 8 == 0 && a.ws_ci % 8 == 0 : a.ws_ci == 1 && a.ws_co % 8 == 0) &&
                    a.ws_tap % 8 == 0;
   if (wco)
-    vec ? nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 1, 1>, grid, thr, 0, a)
-        : nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 1, 0>, grid, thr, 0, a);
+    vec ? nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, SPB, 1, 1>, grid, thr, 0, a)
+        : nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, SPB, 1, 0>, grid, thr, 0, a);
   else
-    vec ? nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 0, 1>, grid, thr, 0, a)
-        : nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, 0, 0>, grid, thr, 0, a);
+    vec ? nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, SPB, 0, 1>, grid, thr, 0, a)
+        : nf_launch(conv_direct_kernel<T, PX, CO, CK, TP, TC, SPB, 0, 0>, grid, thr, 0, a);
   NF_LAUNCHED();
   return NF_OK;
 }
 
 template <typename T>
 int run_direct(const ConvArgs& a) {
-  // chunks of 16 where there are no more than 16 input channels: the same chain, half the shared memory work
-  if (a.Co <= 16) return a.Ci <= 16 ? launch_direct<T, 64, 16, 16, 2, 2>(a) : launch_direct<T, 64, 16, 32, 2, 2>(a);
+  // Few output channels: 64 x 16 tiles; with at most 16 input channels (chunks of 16: the same chain, half the shared memory work)
+  // a step is so short that the trip to L2 shows, so three taps share one (16 -> 8 channels on 8 images of 32x32: 10.7 -> 6 us)
+  if (a.Co <= 16) {
+    if (a.Ci > 16) return launch_direct<T, 64, 16, 32, 2, 2, 1>(a);
+    return a.taps == 9 ? launch_direct<T, 64, 16, 16, 2, 2, 3>(a) : launch_direct<T, 64, 16, 16, 2, 2, 1>(a);
+  }
   // 64 x 64 tiles from one block per SM on (148): below that, four times as many blocks of 32 x 32 finish sooner
   const long big = (long)((a.P + 63) / 64) * ((a.Co + 63) / 64);
-  if (big >= 148) return launch_direct<T, 64, 64, 32, 4, 4>(a);
-  return launch_direct<T, 32, 32, 32, 2, 2>(a);
+  if (big >= 148) return launch_direct<T, 64, 64, 32, 4, 4, 1>(a);
+  return launch_direct<T, 32, 32, 32, 2, 2, 1>(a);
 }
 
 // ------------------------------------------------------------------ direct weight gradient

@@ -652,9 +652,9 @@ __global__ void unpad_grad_kernel(const float* __restrict__ gwpad, size_t rows, 
   gw[e] = gwpad[(e / C) * Cp + e % C];
 }
 
-// out[i] = sum over the splits of part[k][i], in a fixed order.  V consecutive elements per thread (4: 16-byte loads) and LN lanes
-// over the splits per block of 256; a lane adds its splits in index order with four in flight, then the lanes are added in
-// order.  Many splits of few elements (148 of 36 864) want lanes, few splits of many elements a thread each.
+// out[i] = sum over the splits of part[k][i]: eight chains (split k in chain k % 8) in index order, the chains added in order.  V
+// consecutive elements per thread (4: 16-byte loads); LN = 8: a thread per chain, for many splits of few elements (148 of
+// 36 864); LN = 1: one thread runs all chains, for fewer than 16 splits (at most two terms each) of many elements.
 template <int V, int LN>
 __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
   nf_pdl_begin();
@@ -665,19 +665,25 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
   float s[V];
 #pragma unroll
   for (int e = 0; e < V; ++e) s[e] = 0.f;
-  if (i < n) {
-    const float* src = part + (size_t)ty * n + i;
-#pragma unroll 4
-    for (int k = ty; k < splits; k += LN, src += (size_t)LN * n) {
-      if constexpr (V == 4) {
-        const float4 w = *reinterpret_cast<const float4*>(src);
-        s[0] += w.x; s[1] += w.y; s[2] += w.z; s[3] += w.w;
-      } else {
-        s[0] += *src;
+  auto term = [&](int k, float(&v)[V]) {
+    const float* src = part + (size_t)k * n + i;
+    if constexpr (V == 4) {
+      const float4 w = *reinterpret_cast<const float4*>(src);
+      v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+    } else {
+      v[0] = *src;
+    }
+  };
+  if constexpr (LN > 1) {
+    if (i < n) {
+#pragma unroll 8
+      for (int k = ty; k < splits; k += LN) {
+        float v[V];
+        term(k, v);
+#pragma unroll
+        for (int e = 0; e < V; ++e) s[e] += v[e];
       }
     }
-  }
-  if constexpr (LN > 1) {
 #pragma unroll
     for (int e = 0; e < V; ++e) sm[ty][tx * V + e] = s[e];
     __syncthreads();
@@ -689,6 +695,17 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
       if (o < n) out[o] = v;
     }
   } else if (i < n) {
+    const int heads = splits < 8 ? splits : 8;
+#pragma unroll 4
+    for (int k = 0; k < heads; ++k) {
+      float v[V], w[V];
+      term(k, v);
+#pragma unroll
+      for (int e = 0; e < V; ++e) w[e] = 0.f;
+      if (k + 8 < splits) term(k + 8, w);
+#pragma unroll
+      for (int e = 0; e < V; ++e) s[e] += v[e] + w[e];
+    }
     if constexpr (V == 4) {
       *reinterpret_cast<float4*>(out + i) = make_float4(s[0], s[1], s[2], s[3]);
     } else {
@@ -764,6 +781,24 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
   return u;
 }
 
+// Eight consecutive values of either storage type, loaded but not yet unpacked
+template <typename T> struct Vec8;
+template <> struct Vec8<bf16> {
+  uint4 u;
+  __device__ __forceinline__ void load(const bf16* p, size_t e) { u = __ldg(reinterpret_cast<const uint4*>(p) + e); }
+  __device__ __forceinline__ void get(float (&f)[8]) const { unpack8(u, f); }
+};
+template <> struct Vec8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p, size_t e) {
+    a = __ldg(reinterpret_cast<const float4*>(p) + 2 * e);
+    b = __ldg(reinterpret_cast<const float4*>(p) + 2 * e + 1);
+  }
+  __device__ __forceinline__ void get(float (&f)[8]) const {
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w; f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+  }
+};
+
 // out = ReLU(y*scale+shift); grid-stride over (pixel, channel group)
 __global__ void __launch_bounds__(256) bn_apply_vec_kernel(const uint4* __restrict__ y, int C8, const float* __restrict__ scale,
                                                            const float* __restrict__ shift, size_t total8,
@@ -790,10 +825,10 @@ __global__ void __launch_bounds__(256) bn_apply_vec_kernel(const uint4* __restri
 // per-thread constants variant (256 % C8 == 0)
 // MODE of this and the two backward kernels below: 0 = ReLU, 1 = a shortcut tensor of y's shape is added before the ReLU, 2 = no
 // activation (a projection shortcut).  One element per thread took 18 us where 16-byte accesses take 5 (33 MB).
-template <int MODE>
-__global__ void __launch_bounds__(256) bn_apply_vec2_kernel(const uint4* __restrict__ y, int C8, const float* __restrict__ scale,
-                                                            const float* __restrict__ shift, size_t total8, uint4* __restrict__ out,
-                                                            const uint4* __restrict__ skip) {
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256) bn_apply_vec2_kernel(const T* __restrict__ y, int C8, const float* __restrict__ scale,
+                                                            const float* __restrict__ shift, size_t total8, T* __restrict__ out,
+                                                            const T* __restrict__ skip) {
   nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
   float A[8], B[8];
@@ -804,43 +839,42 @@ __global__ void __launch_bounds__(256) bn_apply_vec2_kernel(const uint4* __restr
   }
   const size_t stride = (size_t)gridDim.x * 256;
   for (size_t e0 = (size_t)blockIdx.x * 256 + threadIdx.x; e0 < total8; e0 += 2 * stride) {
-    const size_t e1 = e0 + stride;
-    const bool two = e1 < total8;
-    const uint4 ya = __ldg(y + e0);
-    const uint4 yb = two ? __ldg(y + e1) : ya;
-    float v[8], k[8];
-    uint4 sa, sb;
-    if constexpr (MODE == 1) {
-      sa = __ldg(skip + e0);
-      sb = two ? __ldg(skip + e1) : sa;
-      unpack8(sa, k);
-    }
-    unpack8(ya, v);
+    Vec8<T> yq[2], sq[2];
+    const int m = e0 + stride < total8 ? 2 : 1;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = MODE == 2 ? fmaf(v[i], A[i], B[i]) : fmaxf(fmaf(v[i], A[i], B[i]) + (MODE == 1 ? k[i] : 0.f), 0.f);
-    out[e0] = pack8(v);
-    if (two) {
-      unpack8(yb, v);
-      if constexpr (MODE == 1) unpack8(sb, k);
+    for (int u = 0; u < 2; ++u)
+      if (u < m) {
+        yq[u].load(y, e0 + u * stride);
+        if constexpr (MODE == 1) sq[u].load(skip, e0 + u * stride);
+      }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = MODE == 2 ? fmaf(v[i], A[i], B[i]) : fmaxf(fmaf(v[i], A[i], B[i]) + (MODE == 1 ? k[i] : 0.f), 0.f);
-      out[e1] = pack8(v);
-    }
+    for (int u = 0; u < 2; ++u)
+      if (u < m) {
+        float v[8], k[8];
+        yq[u].get(v);
+        if constexpr (MODE == 1) sq[u].get(k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = MODE == 2 ? fmaf(v[i], A[i], B[i]) : fmaxf(fmaf(v[i], A[i], B[i]) + (MODE == 1 ? k[i] : 0.f), 0.f);
+        st8(out + (e0 + u * stride) * 8, v);
+      }
   }
 }
 
-// partial sums of (dz, dz*xhat) with dz = da * 1[y*scale+shift (+ skip) > 0]; red[(block*2+k)*C + c].  MODE 1 also
-// writes dz where a trainable shortcut wants it (dz_out not NULL).
-template <int MODE>
-__global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da,
-                                                                size_t P, int C8, const float* __restrict__ scale,
+// partial sums of (dz, dz*xhat) with dz = da * 1[y*scale+shift (+ skip) > 0]; red[(range*2+k)*C + c] over `ranges` pixel ranges.
+// MODE 1 also writes dz where a trainable shortcut wants it (dz_out not NULL).  A range has `planes` interleaved chains per
+// channel, added in order; a thread runs 8 channels of a chain, so a range takes C / 8 * planes threads and a block several
+// ranges where that is less than 256.  Four pixels per trip: eight (with a shortcut twelve) 16-byte loads in flight.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const T* __restrict__ y, const T* __restrict__ da,
+                                                                size_t P, int C8, int planes, int ranges, const float* __restrict__ scale,
                                                                 const float* __restrict__ shift, const float* __restrict__ mu,
                                                                 const float* __restrict__ invstd, float* __restrict__ red,
-                                                                const uint4* __restrict__ skip, uint4* __restrict__ dz_out) {
+                                                                const T* __restrict__ skip, T* __restrict__ dz_out) {
   nf_pdl_begin();
   __shared__ float sm[16][256];
-  const int C = C8 * 8;
-  const int planes = 256 / C8, g = threadIdx.x % C8, pl = threadIdx.x / C8;
+  const int C = C8 * 8, thr = C8 * planes;  // threads per range: a divisor of 256
+  const int lt = threadIdx.x % thr, g = lt % C8, pl = lt / C8;
+  const int rng = blockIdx.x * (256 / thr) + threadIdx.x / thr;
   const int c0 = g * 8;
   float sc[8], sh[8], m[8], is[8], a[8], b[8];
 #pragma unroll
@@ -848,17 +882,17 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __r
     sc[i] = scale[c0 + i]; sh[i] = shift[c0 + i]; m[i] = mu[c0 + i]; is[i] = invstd[c0 + i];
     a[i] = 0.f; b[i] = 0.f;
   }
-  const size_t p0 = P * blockIdx.x / gridDim.x, p1 = P * (blockIdx.x + 1) / gridDim.x;
-  constexpr int kU = 4;  // pixels per trip: eight (with a shortcut twelve) 16-byte loads in flight
+  const size_t p0 = rng < ranges ? P * rng / ranges : P, p1 = rng < ranges ? P * (rng + 1) / ranges : P;
+  constexpr int kU = 4;
   for (size_t p = p0 + pl; p < p1; p += (size_t)kU * planes) {
-    uint4 yq[kU], dq[kU], sq[kU];
+    Vec8<T> yq[kU], dq[kU], sq[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const size_t q = p + (size_t)u * planes;
       if (q < p1) {
-        yq[u] = __ldg(y + q * C8 + g);
-        dq[u] = __ldg(da + q * C8 + g);
-        if constexpr (MODE == 1) sq[u] = __ldg(skip + q * C8 + g);
+        yq[u].load(y, q * C8 + g);
+        dq[u].load(da, q * C8 + g);
+        if constexpr (MODE == 1) sq[u].load(skip, q * C8 + g);
       }
     }
 #pragma unroll
@@ -866,17 +900,17 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __r
       const size_t q = p + (size_t)u * planes;
       if (q < p1) {
         float yv[8], dv[8], kv[8];
-        unpack8(yq[u], yv);
-        unpack8(dq[u], dv);
-        if constexpr (MODE == 1) unpack8(sq[u], kv);
+        yq[u].get(yv);
+        dq[u].get(dv);
+        if constexpr (MODE == 1) sq[u].get(kv);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const float dz = MODE == 2 || fmaf(yv[i], sc[i], sh[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
           a[i] += dz;
-          b[i] = fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
+          b[i] = MODE == 1 ? fmaf(dz * (yv[i] - m[i]), is[i], b[i]) : fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
           dv[i] = dz;
         }
-        if (MODE == 1 && dz_out) dz_out[q * C8 + g] = pack8(dv);
+        if (MODE == 1 && dz_out) st8(dz_out + (q * C8 + g) * 8, dv);
       }
     }
   }
@@ -886,13 +920,15 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const uint4* __r
     sm[8 + i][threadIdx.x] = b[i];
   }
   __syncthreads();
-  // thread t < 2*C finishes value k = t / C of channel c = t % C
-  for (int t = threadIdx.x; t < 2 * C; t += 256) {
-    const int k = t / C, c = t % C, gg = c / 8, i = c % 8;
-    float s = 0.f;
-    for (int q = 0; q < planes; ++q) s += sm[k * 8 + i][q * C8 + gg];
-    red[((size_t)blockIdx.x * 2 + k) * C + c] = s;
-  }
+  // value k = t / C of channel c = t % C, one thread each, for every range of the block
+  const int base = threadIdx.x / thr * thr;
+  if (rng < ranges)
+    for (int t = lt; t < 2 * C; t += thr) {
+      const int k = t / C, c = t % C, gg = c / 8, i = c % 8;
+      float s = 0.f;
+      for (int q = 0; q < planes; ++q) s += sm[k * 8 + i][base + q * C8 + gg];
+      red[((size_t)rng * 2 + k) * C + c] = s;
+    }
 }
 
 // dy = scale * (dz - sum(dz)/M - xhat * sum(dz*xhat)/M)
@@ -947,65 +983,63 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec_kernel(const uint4* __re
 // Same result with per-thread constants: when 256 % C8 == 0 a thread keeps its 8 channels over the whole
 // grid-stride loop, and dy = s*dz + k1*y + k0 with k1 = -s*m2*invstd, k0 = s*(m2*invstd*mu - m1),
 // m1 = sum(dz)/M, m2 = sum(dz*xhat)/M: five instructions per element.
-template <int MODE>
-__global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da, int C8,
+template <typename T, int MODE>
+__global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const T* __restrict__ y, const T* __restrict__ da, int C8,
                                                                 const float* __restrict__ scale, const float* __restrict__ shift,
                                                                 const float* __restrict__ mu, const float* __restrict__ invstd,
                                                                 const float* __restrict__ sdz, const float* __restrict__ sdzx,
-                                                                float invM, size_t total8, uint4* __restrict__ dy,
-                                                                const uint4* __restrict__ skip) {
+                                                                float invM, size_t total8, T* __restrict__ dy, const T* __restrict__ skip) {
   nf_pdl_begin();
   const int c0 = (threadIdx.x % C8) * 8;
-  float A[8], B[8], K1[8], K0[8];
+  float A[8], B[8], K1[8], K0[8], M1[8], IS[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const float s = scale[c0 + i], m1 = sdz[c0 + i] * invM, m2 = sdzx[c0 + i] * invM, is = invstd[c0 + i];
     A[i] = s;
     B[i] = shift[c0 + i];
-    K1[i] = -s * m2 * is;
-    K0[i] = s * (m2 * is * mu[c0 + i] - m1);
+    if constexpr (MODE == 1) {  // the generic kernel's form, term by term
+      M1[i] = mu[c0 + i]; IS[i] = is; K1[i] = sdzx[c0 + i]; K0[i] = sdz[c0 + i];
+    } else {
+      K1[i] = -s * m2 * is;
+      K0[i] = s * (m2 * is * mu[c0 + i] - m1);
+    }
   }
   const size_t stride = (size_t)gridDim.x * 256;
   for (size_t e0 = (size_t)blockIdx.x * 256 + threadIdx.x; e0 < total8; e0 += 2 * stride) {
-    const size_t e1 = e0 + stride;
-    const bool two = e1 < total8;
-    const uint4 ya = __ldg(y + e0), da0 = __ldg(da + e0);
-    uint4 yb = ya, db = da0;
-    if (two) {
-      yb = __ldg(y + e1);
-      db = __ldg(da + e1);
-    }
-    float yv[8], dv[8], kv[8], o[8];
-    uint4 sa, sb;
-    if constexpr (MODE == 1) {
-      sa = __ldg(skip + e0);
-      sb = two ? __ldg(skip + e1) : sa;
-      unpack8(sa, kv);
-    }
-    unpack8(ya, yv);
-    unpack8(da0, dv);
+    Vec8<T> yq[2], dq[2], sq[2];
+    const int m = e0 + stride < total8 ? 2 : 1;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float dz = MODE == 2 || fmaf(yv[i], A[i], B[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
-      o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i], K0[i]));
-    }
-    dy[e0] = pack8(o);
-    if (two) {
-      unpack8(yb, yv);
-      unpack8(db, dv);
-      if constexpr (MODE == 1) unpack8(sb, kv);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float dz = MODE == 2 || fmaf(yv[i], A[i], B[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
-        o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i], K0[i]));
+    for (int u = 0; u < 2; ++u)
+      if (u < m) {
+        yq[u].load(y, e0 + u * stride);
+        dq[u].load(da, e0 + u * stride);
+        if constexpr (MODE == 1) sq[u].load(skip, e0 + u * stride);
       }
-      dy[e1] = pack8(o);
-    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (u < m) {
+        float yv[8], dv[8], kv[8], o[8];
+        yq[u].get(yv);
+        dq[u].get(dv);
+        if constexpr (MODE == 1) sq[u].get(kv);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float dz = MODE == 2 || fmaf(yv[i], A[i], B[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
+          if constexpr (MODE == 1) {
+            const float xh = (yv[i] - M1[i]) * IS[i];
+            o[i] = A[i] * (dz - K0[i] * invM - xh * K1[i] * invM);
+          } else {
+            o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i], K0[i]));
+          }
+        }
+        st8(dy + (e0 + u * stride) * 8, o);
+      }
   }
 }
 
-// partial sums of (v, v^2) of a bf16 tensor; same layout of partials as channel_reduce_kernel
-__global__ void __launch_bounds__(256) channel_sums_vec_kernel(const uint4* __restrict__ src, size_t P, int C8,
+// partial sums of (v, v^2); same layout of partials as channel_reduce_kernel
+template <typename T>
+__global__ void __launch_bounds__(256) channel_sums_vec_kernel(const T* __restrict__ src, size_t P, int C8,
                                                                float* __restrict__ red) {
   nf_pdl_begin();
   __shared__ float sm[16][256];
@@ -1016,14 +1050,22 @@ __global__ void __launch_bounds__(256) channel_sums_vec_kernel(const uint4* __re
   for (int i = 0; i < 8; ++i) a[i] = b[i] = 0.f;
   const size_t p0 = P * blockIdx.x / gridDim.x, p1 = P * (blockIdx.x + 1) / gridDim.x;
   if (pl < planes)
-    for (size_t p = p0 + pl; p < p1; p += planes) {
-      float v[8];
-      unpack8(__ldg(src + p * C8 + g), v);
+    for (size_t p = p0 + pl; p < p1; p += 4 * (size_t)planes) {  // four loads in flight, added in index order
+      Vec8<T> q[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        a[i] += v[i];
-        b[i] = fmaf(v[i], v[i], b[i]);
-      }
+      for (int u = 0; u < 4; ++u)
+        if (p + (size_t)u * planes < p1) q[u].load(src, (p + (size_t)u * planes) * C8 + g);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (p + (size_t)u * planes < p1) {
+          float v[8];
+          q[u].get(v);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            a[i] += v[i];
+            b[i] = fmaf(v[i], v[i], b[i]);
+          }
+        }
     }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -1411,6 +1453,8 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_pool_vec_kernel(const uint4*
 }
 
 inline bool vec_ok(int dtype, int C, int pool) { return dtype == NF_BF16 && C % 8 == 0 && C <= 1024 && !pool; }
+// either storage type: a thread keeps its eight channels over its whole loop
+inline bool vec2_ok(int C, int pool) { return C % 8 == 0 && C <= 2048 && 256 % (C / 8) == 0 && !pool; }
 inline int vec_blocks(size_t work_items) {
   size_t b = (work_items + 256 * 8 - 1) / (256 * 8);
   if (b < 1) b = 1;
@@ -1438,8 +1482,9 @@ int nf_k_channel_blocks(size_t P, int C) {
 int nf_k_channel_sums(int dtype, const void* src, size_t P, int C, float* red, size_t red_floats, int* nblocks) {
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
-  if (vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    nf_launch(channel_sums_vec_kernel, nb, 256, 0, (const uint4*)src, P, C / 8, red);
+  if (vec2_ok(C, 0)) {
+    DISPATCH(dtype, (nf_launch(channel_sums_vec_kernel<float>, nb, 256, 0, (const float*)src, P, C / 8, red)),
+             (nf_launch(channel_sums_vec_kernel<bf16>, nb, 256, 0, (const bf16*)src, P, C / 8, red)));
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;
@@ -1491,9 +1536,11 @@ int nf_k_bn_eval_coeffs(int C, const float* gamma, const float* beta, float eps,
 int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int pool, const float* scale,
                     const float* shift, void* out, const void* skip) {
   const size_t total = (size_t)N * (pool ? Ho / 2 : Ho) * (pool ? Wo / 2 : Wo) * C;
-  if (skip && vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_apply_vec2_kernel<1>, vec_blocks(total / 8), 256, 0, (const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out,
-              (const uint4*)skip);
+  if (vec2_ok(C, pool)) {
+#define NF_APPLY(T, M) \
+  nf_launch(bn_apply_vec2_kernel<T, M>, vec_blocks(total / 8), 256, 0, (const T*)y, C / 8, scale, shift, total / 8, (T*)out, (const T*)skip)
+    DISPATCH(dtype, (skip ? NF_APPLY(float, 1) : NF_APPLY(float, 0)), (skip ? NF_APPLY(bf16, 1) : NF_APPLY(bf16, 0)));
+#undef NF_APPLY
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1507,12 +1554,6 @@ int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int po
   if (pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
     nf_launch(bn_apply_pool_vec_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, Ho, Wo, C / 8, scale, shift, total / 8,
                                                                             (uint4*)out);
-    NF_LAUNCHED();
-    return NF_OK;
-  }
-  if (vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_apply_vec2_kernel<0>, vec_blocks(total / 8), 256, 0, (const uint4*)y, C / 8, scale, shift, total / 8, (uint4*)out,
-              nullptr);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1686,7 +1727,7 @@ int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, 
   const size_t P = (size_t)N * Ho * Wo;
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
-  const bool vec = vec_ok(dtype, C, pool) && 256 % (C / 8) == 0;
+  const bool vec = vec2_ok(C, pool);
   if (dz_out && !(skip && vec)) {  // else the reduction below writes it
     const int rc = nf_k_write_dz(dtype, y, da, N, Ho, Wo, C, pool, scale, shift, skip, dz_out);
     if (rc != NF_OK) return rc;
@@ -1699,12 +1740,13 @@ int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, 
     return NF_OK;
   }
   if (vec) {
-    if (skip)
-      nf_launch(bn_bwd_reduce_vec_kernel<1>, nb, 256, 0, (const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red,
-                (const uint4*)skip, (uint4*)dz_out);
-    else
-      nf_launch(bn_bwd_reduce_vec_kernel<0>, nb, 256, 0, (const uint4*)y, (const uint4*)da, P, C / 8, scale, shift, mu, invstd, red,
-                nullptr, nullptr);
+    // without a shortcut a range is a block's 256 / (C / 8) chains; with one, the generic kernel's (256 channels and chains)
+    const int planes = skip ? 256 / pow2ceil_cap256(C) : 256 / (C / 8), per = 256 / (C / 8 * planes);
+#define NF_REDUCE(T, M)                                                                                                                  \
+  nf_launch(bn_bwd_reduce_vec_kernel<T, M>, nblk(nb, per), 256, 0, (const T*)y, (const T*)da, P, C / 8, planes, nb, scale, shift, mu, invstd, red, \
+            (const T*)skip, (T*)dz_out)
+    DISPATCH(dtype, (skip ? NF_REDUCE(float, 1) : NF_REDUCE(float, 0)), (skip ? NF_REDUCE(bf16, 1) : NF_REDUCE(bf16, 0)));
+#undef NF_REDUCE
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;
@@ -1740,9 +1782,12 @@ int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, i
                         const float* sdz, const float* sdzx, double M, void* dy, const void* skip) {
   const size_t total = (size_t)N * Ho * Wo * C;
   const float invM = (float)(1.0 / M);
-  if (skip && vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_bwd_apply_vec2_kernel<1>, vec_blocks(total / 8), 256, 0, (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
-              invstd, sdz, sdzx, invM, total / 8, (uint4*)dy, (const uint4*)skip);
+  if (vec2_ok(C, pool)) {
+#define NF_APPLY(T, M)                                                                                                                       \
+  nf_launch(bn_bwd_apply_vec2_kernel<T, M>, vec_blocks(total / 8), 256, 0, (const T*)y, (const T*)da, C / 8, scale, shift, mu, invstd, sdz, sdzx, \
+            invM, total / 8, (T*)dy, (const T*)skip)
+    DISPATCH(dtype, (skip ? NF_APPLY(float, 1) : NF_APPLY(float, 0)), (skip ? NF_APPLY(bf16, 1) : NF_APPLY(bf16, 0)));
+#undef NF_APPLY
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1756,12 +1801,6 @@ int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, i
   if (pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
     nf_launch(bn_bwd_apply_pool_vec_kernel, vec_blocks(total / 32), 256, 0, (const uint4*)y, (const uint4*)da, Ho, Wo, C / 8, scale,
                                                                                  shift, mu, invstd, sdz, sdzx, invM, total / 32, (uint4*)dy);
-    NF_LAUNCHED();
-    return NF_OK;
-  }
-  if (vec_ok(dtype, C, pool) && 256 % (C / 8) == 0) {
-    nf_launch(bn_bwd_apply_vec2_kernel<0>, vec_blocks(total / 8), 256, 0, (const uint4*)y, (const uint4*)da, C / 8, scale, shift, mu,
-              invstd, sdz, sdzx, invM, total / 8, (uint4*)dy, nullptr);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1797,10 +1836,7 @@ int nf_k_unpad_grad(const float* gwpad, size_t rows, int C, int Cp, float* gw) {
 
 int nf_k_sum_parts(const float* part, int splits, size_t n, float* out) {
   const bool vec = n % 4 == 0 && (((uintptr_t)part | (uintptr_t)out) & 15) == 0;
-  if (splits >= 16 && n <= 16384) {
-    if (vec) nf_launch(sum_parts_kernel<4, 32>, nblk(n, 32), 256, 0, part, splits, n, out);
-    else nf_launch(sum_parts_kernel<1, 8>, nblk(n, 32), 256, 0, part, splits, n, out);
-  } else if (splits >= 16) {
+  if (splits >= 16) {
     if (vec) nf_launch(sum_parts_kernel<4, 8>, nblk(n, 128), 256, 0, part, splits, n, out);
     else nf_launch(sum_parts_kernel<1, 8>, nblk(n, 32), 256, 0, part, splits, n, out);
   } else {
@@ -1847,31 +1883,34 @@ int nf_k_gather(const void* cache, const int32_t* cache_labels, int cache_rows, 
   return NF_OK;
 }
 
-// ---- BatchNorm without an activation (projection shortcut), bf16 with 8 | C and C / 8 a divisor of 256; NF_EUNSUPPORTED otherwise
-static bool plain_ok(int dtype, int C) { return vec_ok(dtype, C, 0) && 256 % (C / 8) == 0; }
+// ---- BatchNorm without an activation (projection shortcut); NF_EUNSUPPORTED for channel counts the kernels above do not take
 int nf_k_bn_plain_apply(int dtype, const void* y, size_t P, int C, const float* scale, const float* shift, void* out) {
-  if (!plain_ok(dtype, C)) return NF_EUNSUPPORTED;
-  const size_t total8 = P * C / 8;
-  nf_launch(bn_apply_vec2_kernel<2>, vec_blocks(total8), 256, 0, (const uint4*)y, C / 8, scale, shift, total8, (uint4*)out, nullptr);
+  if (!vec2_ok(C, 0)) return NF_EUNSUPPORTED;
+  const size_t n8 = P * C / 8;
+  DISPATCH(dtype, (nf_launch(bn_apply_vec2_kernel<float, 2>, vec_blocks(n8), 256, 0, (const float*)y, C / 8, scale, shift, n8, (float*)out, nullptr)),
+           (nf_launch(bn_apply_vec2_kernel<bf16, 2>, vec_blocks(n8), 256, 0, (const bf16*)y, C / 8, scale, shift, n8, (bf16*)out, nullptr)));
   NF_LAUNCHED();
   return NF_OK;
 }
 int nf_k_bn_plain_bwd_reduce(int dtype, const void* y, const void* dz, size_t P, int C, const float* mu, const float* invstd, float* red,
                              size_t red_floats, int* nblocks) {
-  if (!plain_ok(dtype, C)) return NF_EUNSUPPORTED;
-  const int nb = nf_k_channel_blocks(P, C);
+  if (!vec2_ok(C, 0)) return NF_EUNSUPPORTED;
+  const int nb = std::min(nf_k_channel_blocks(P, C), 296);  // two blocks per SM: each pays for its channel constants and its reduction
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
-  nf_launch(bn_bwd_reduce_vec_kernel<2>, nb, 256, 0, (const uint4*)y, (const uint4*)dz, P, C / 8, mu, mu, mu, invstd, red, nullptr, nullptr);
+  const int planes = 256 / (C / 8);
+  DISPATCH(dtype, (nf_launch(bn_bwd_reduce_vec_kernel<float, 2>, nb, 256, 0, (const float*)y, (const float*)dz, P, C / 8, planes, nb, mu, mu, mu, invstd, red, nullptr, nullptr)),
+           (nf_launch(bn_bwd_reduce_vec_kernel<bf16, 2>, nb, 256, 0, (const bf16*)y, (const bf16*)dz, P, C / 8, planes, nb, mu, mu, mu, invstd, red, nullptr, nullptr)));
   NF_LAUNCHED();
   *nblocks = nb;
   return NF_OK;
 }
 int nf_k_bn_plain_bwd_apply(int dtype, const void* y, const void* dz, size_t P, int C, const float* scale, const float* mu,
                             const float* invstd, const float* sdz, const float* sdzx, double M, void* dy) {
-  if (!plain_ok(dtype, C)) return NF_EUNSUPPORTED;
-  const size_t total8 = P * C / 8;
-  nf_launch(bn_bwd_apply_vec2_kernel<2>, vec_blocks(total8), 256, 0, (const uint4*)y, (const uint4*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx,
-            (float)(1.0 / M), total8, (uint4*)dy, nullptr);
+  if (!vec2_ok(C, 0)) return NF_EUNSUPPORTED;
+  const size_t n8 = P * C / 8;
+  const float invM = (float)(1.0 / M);
+  DISPATCH(dtype, (nf_launch(bn_bwd_apply_vec2_kernel<float, 2>, vec_blocks(n8), 256, 0, (const float*)y, (const float*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx, invM, n8, (float*)dy, nullptr)),
+           (nf_launch(bn_bwd_apply_vec2_kernel<bf16, 2>, vec_blocks(n8), 256, 0, (const bf16*)y, (const bf16*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx, invM, n8, (bf16*)dy, nullptr)));
   NF_LAUNCHED();
   return NF_OK;
 }

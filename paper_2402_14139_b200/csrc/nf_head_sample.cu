@@ -30,22 +30,6 @@ struct HeadArgs {
   int loss_kind, n_scale;
 };
 
-__device__ __forceinline__ void store8(bf16* p, float (&v)[8]) {  // v becomes the values as stored
-  uint32_t w[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-    w[i] = *reinterpret_cast<const uint32_t*>(&b);
-    v[2 * i] = __uint_as_float(w[i] << 16);
-    v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-  }
-  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-__device__ __forceinline__ void store8(float* p, float (&v)[8]) {
-  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-  *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
-}
-
 // reduction over the block; every thread gets the result
 __device__ __forceinline__ float block_all(float v, float* sm, bool is_max) {
 #pragma unroll
@@ -95,7 +79,7 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
       for (int u = 0; u < 4; ++u) {
         const int q = q0 + u * kStep;
         if (q < px) {
-          if (a.dh) store8(hs + (size_t)q * F + g * 8, v[u]);
+          if (a.dh) st8(hs + (size_t)q * F + g * 8, v[u]);
           const int i = q / a.Wa, j = q - i * a.Wa;
 #pragma unroll
           for (int b = 0; b < 4; ++b) {
@@ -278,7 +262,7 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
     ld8(tab + (rc * 3 + cc) * F + g * 8, o);
 #pragma unroll
     for (int e = 0; e < 8; ++e) o[e] = v[e] > 0.f ? o[e] : 0.f;
-    store8(dhn + (size_t)q * F + g * 8, o);
+    st8(dhn + (size_t)q * F + g * 8, o);
 #pragma unroll
     for (int e = 0; e < 8; ++e) bs[e] += o[e];  // the bias gradient sums the values as stored
   }
