@@ -396,13 +396,9 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   // h_masked: the aux forward left pooling partials (L->wpart) and a sign mask (in L->h) instead of h
   const bool h_masked = fused_bn_aux && nf_tc_aux_pool_fused(L);
   // heads of ordinary size: one block per sample does all of it, and writes dh where the sample's h fits its shared memory
-  int sample_mode = L->o.aux_pool == NF_POOL_AVG && !nf_head_is_large(N, D, K) ? nf_head_sample_mode(dt, Ha, Wa, F, K) : 0;
+  int sample_mode = L->o.aux_pool == NF_POOL_AVG && !nf_head_is_large(N, D, K) ? nf_head_sample_mode(dt, N, Ha, Wa, F, K) : 0;
   if (sample_mode == 2 && (h_masked || (size_t)N * F > L->red_floats)) sample_mode = 1;
-  if (sample_mode) {
-    const NfHeadIo io{h_masked ? nullptr : L->h, L->wpart, labels, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->p, L->logits,
-                      L->dlogits, L->dp, L->lossn, L->status, sample_mode == 2 ? L->dh : nullptr, L->red, g + L->off[NF_P_WF],
-                      g + L->off[NF_P_BF], g + L->off[NF_P_BA], loss_out};
-    NF_TRY(nf_head_sample_step(io, dt, N, Ha, Wa, F, K, L->o.loss, n_scale));
+  if (sample_mode == 2 || (h_masked && sample_mode)) {  // pooled by the head itself
   } else if (h_masked) {
     NF_TRY(nf_k_pool_finish(L->wpart, N, Ha / 8, Wa / 14, F, 1.f / (float)((Ha / 2) * (Wa / 2)), L->p));
   } else if (L->o.aux_pool == NF_POOL_MAX) {
@@ -413,6 +409,10 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     if (rc != NF_OK) return rc;
   }
   if (sample_mode) {
+    const NfHeadIo io{sample_mode == 2 ? L->h : nullptr, h_masked ? L->wpart : nullptr, labels, L->val + L->off[NF_P_WF],
+                      L->val + L->off[NF_P_BF], L->p, L->logits, L->dlogits, L->dp, L->lossn, L->status,
+                      sample_mode == 2 ? L->dh : nullptr, L->red, g + L->off[NF_P_WF], g + L->off[NF_P_BF], g + L->off[NF_P_BA], loss_out};
+    NF_TRY(nf_head_sample_step(io, dt, N, Ha, Wa, F, K, L->o.loss, n_scale));
   } else if (nf_head_is_large(N, D, K)) {  // late blocks: tens of thousands of samples, up to 1024 head inputs
     NF_TRY(nf_head_step(L->p, labels, N, D, K, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->logits, L->dlogits, L->dp,
                         L->lossn, L->status, L->o.loss, g + L->off[NF_P_WF], g + L->off[NF_P_BF], loss_out, L->wpart,

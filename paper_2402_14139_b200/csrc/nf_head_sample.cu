@@ -3,10 +3,15 @@
 //
 // These heads are pure latency (64 to 512 samples, at most a few million multiply-adds): as separate pool, pool-finish, loss,
 // weight-gradient, dh and bias kernels they took 55 of 215 us of a 32 x 32-pixel layer at 128 samples, each kernel a launch and a
-// few dependent trips to L2 (the weight gradient with one block per class and one load at a time alone 20 us).  Here a sample's
-// h is read once, kept in shared memory until dh is written, and every loop has several independent loads in flight.
-// fp32 throughout, every sum in a fixed order.
+// few dependent trips to L2 (the weight gradient with one block per class and one load at a time alone 20 us); now 12 + 3 us.
+// A sample's h is read once; its sign bits stay in shared memory until dh is written, the linear weights take h's place there.
+// Loads come in batches whose indexes are clamped instead of guarded, so that no branch separates them, and loops stay rolled:
+// at this size the fetch of unrolled code costs more than it saves.
+// fp32 throughout, every sum in a fixed order: the order of the kernels for large maps and batches (nf_elem.cu), so that a layer
+// computes the same bits whichever of them its size selects.
 #include <math.h>
+
+#include <algorithm>
 
 #include "nf_internal.h"
 #include "nf_ldst.cuh"
@@ -17,97 +22,190 @@ constexpr int kHT = 512;  // threads of the per-sample kernel: with at most one 
 constexpr int kWarps = kHT / 32;
 
 struct HeadArgs {
-  const void* h;        // [N][Ha][Wa][F], or NULL when the pooled inputs come from `part`
+  const void* h;        // [N][Ha][Wa][F], or NULL when the pooled inputs come from `part` or, where that is NULL too, are in p
   const float* part;    // pooling partials of the fused aux forward: [N][th][tw][4][F] (14 x 8-pixel tiles, four warps each)
+  int slices, planes;   // order of a bin's sum: `slices` ranges of its pixels, `planes` interleaved chains in each
+  int even, dh_even;    // the mean as a product with 1 / |bin| (else a quotient), in the pool and in dh
   int th, tw;
   int N, Ha, Wa, F, K;
   const int32_t* labels;
   const float *Wf, *bf;
   float *p, *logits, *dlogits, *dp, *lossn;
   int32_t* status;
-  void* dh;             // NULL: dh is written elsewhere
+  void* dh;             // with h; else dh is written elsewhere
   float* bred;          // [N][F] sums of the stored dh over the sample's pixels (with dh)
   int loss_kind, n_scale;
+  int groups;           // class ranges of the sums in dp
+  size_t off;           // where the offsets and the sign bits lie in shared memory
 };
 
-// reduction over the block; every thread gets the result
-__device__ __forceinline__ float block_all(float v, float* sm, bool is_max) {
+// eight values as they are in memory
+template <typename T> struct Raw8;
+template <> struct Raw8<bf16> {
+  uint4 u;
+  __device__ __forceinline__ void load(const bf16* p) { u = *reinterpret_cast<const uint4*>(p); }
+  __device__ __forceinline__ void store(bf16* p) const { *reinterpret_cast<uint4*>(p) = u; }
+  __device__ __forceinline__ uint32_t positive() const {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+    uint32_t b = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float u = __shfl_xor_sync(0xffffffffu, v, o);
-    v = is_max ? fmaxf(v, u) : v + u;
+    for (int i = 0; i < 4; ++i) {
+      b |= (__uint_as_float(w[i] << 16) > 0.f ? 1u : 0u) << (2 * i);
+      b |= (__uint_as_float(w[i] & 0xffff0000u) > 0.f ? 1u : 0u) << (2 * i + 1);
+    }
+    return b;
   }
-  __syncthreads();  // sm may still be read from the reduction before
+};
+template <> struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) {
+    a = *reinterpret_cast<const float4*>(p);
+    b = *reinterpret_cast<const float4*>(p + 4);
+  }
+  __device__ __forceinline__ void store(float* p) const {
+    *reinterpret_cast<float4*>(p) = a;
+    *reinterpret_cast<float4*>(p + 4) = b;
+  }
+  __device__ __forceinline__ uint32_t positive() const {
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t r = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r |= (v[i] > 0.f ? 1u : 0u) << i;
+    return r;
+  }
+};
+__device__ __forceinline__ float2 pair(const bf16* p) {
+  const uint32_t u = *reinterpret_cast<const uint32_t*>(p);
+  return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
+__device__ __forceinline__ float2 pair(const float* p) { return *reinterpret_cast<const float2*>(p); }
+
+// maximum over the block, for every thread
+__device__ __forceinline__ float block_max(float v, float* sm) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
   __syncthreads();
   v = sm[0];
 #pragma unroll
-  for (int w = 1; w < kWarps; ++w) v = is_max ? fmaxf(v, sm[w]) : v + sm[w];
+  for (int w = 1; w < kWarps; ++w) v = fmaxf(v, sm[w]);
+  __syncthreads();
+  return v;
+}
+// sum of the values of the first 256 threads as a binary tree (t with t + 128, + 64, ...), for every thread
+__device__ __forceinline__ float tree_sum256(float v, float* sm) {
+  const int t = threadIdx.x;
+  if (t < 256) sm[t] = v;
+  __syncthreads();
+  if (t < 32) {
+    float q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = sm[t + 32 * i] + sm[t + 32 * i + 128];
+    v = (q[0] + q[2]) + (q[1] + q[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (t == 0) sm[256] = v;
+  }
+  __syncthreads();
+  v = sm[256];
+  __syncthreads();
   return v;
 }
 
 // F8 = F / 8 in {1, 2, 4, 8}: a warp covers whole pixels, and its lanes with equal lane % F8 hold the same channels.
-template <typename T, int F8>
+// STAGE: the linear weights fit shared memory.
+template <typename T, int F8, bool STAGE>
 __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   nf_pdl_begin();
   constexpr int F = F8 * 8, D = 4 * F;
   extern __shared__ __align__(16) uint8_t dyn[];
   float* ps = reinterpret_cast<float*>(dyn);  // [D] pooled inputs, then their gradient
-  float* ls = ps + D;                         // [K] logits, then dlogits
+  float* ls = ps + D;                         // [K] bias, logits, dlogits
   float* rd = ls + ((a.K + 3) & ~3);          // [kWarps][D] reductions
   float* tab = rd + kWarps * D;               // [9][F] dh of a positive h, by row class and column class of its pixel
   T* hs = reinterpret_cast<T*>(tab + 9 * F);  // the sample's h
+  uint32_t* off = reinterpret_cast<uint32_t*>(dyn + a.off);  // byte offset in the image of a bin's k-th pixel
+  uint8_t* mask = reinterpret_cast<uint8_t*>(off + (((a.Ha + 1) / 2) * ((a.Wa + 1) / 2) + 3) / 4 * 4);  // bit e of [unit]: h > 0
   const int n = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int px = a.Ha * a.Wa, g = t % F8;
   // rows [0, r1) belong to the upper bins, [r0, Ha) to the lower ones: the middle row of an odd height to both; columns likewise
   const int r0 = a.Ha / 2, r1 = (a.Ha + 1) / 2, c0 = a.Wa / 2, c1 = (a.Wa + 1) / 2;
+  int lab = a.labels[n];
+  for (int k = t; k < a.K; k += kHT) ls[k] = a.bf[k];
 
   if (a.h) {
-    float s[4][8];
+    {
+      const T* src = reinterpret_cast<const T*>(a.h) + (size_t)n * px * F;
+      const int units = px * F8;  // of eight values
+#pragma unroll 1
+      for (int i0 = t; i0 < units; i0 += 8 * kHT) {
+        Raw8<T> q[8];
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+        for (int j = 0; j < 8; ++j) q[j].load(src + (size_t)min(i0 + j * kHT, units - 1) * 8);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) s[b][e] = 0.f;
-    const T* hn = reinterpret_cast<const T*>(a.h) + (size_t)n * px * F;
-    constexpr int kStep = kHT / F8;
-    for (int q0 = t / F8; q0 < px; q0 += 4 * kStep) {  // four loads in flight
-      float v[4][8];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (q0 + u * kStep < px) ld8(hn + (size_t)(q0 + u * kStep) * F + g * 8, v[u]);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int q = q0 + u * kStep;
-        if (q < px) {
-          if (a.dh) st8(hs + (size_t)q * F + g * 8, v[u]);
-          const int i = q / a.Wa, j = q - i * a.Wa;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const bool in = (b & 2 ? i >= r0 : i < r1) && (b & 1 ? j >= c0 : j < c1);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) s[b][e] += in ? v[u][e] : 0.f;
+        for (int j = 0; j < 8; ++j)
+          if (i0 + j * kHT < units) {
+            q[j].store(hs + (size_t)(i0 + j * kHT) * 8);
+            mask[i0 + j * kHT] = (uint8_t)q[j].positive();
           }
-        }
       }
     }
+    const int bw = c1, cnt = r1 * c1;  // all four bins have this size
+    for (int k = t; k < cnt; k += kHT) off[k] = (uint32_t)((k / bw) * a.Wa + k % bw) * F * sizeof(T);
+    __syncthreads();
+    // a thread per (bin, slice, channel pair): sixteen chains at a time, each in pixel order, added in chain order
+    for (int i = t; i < 2 * a.slices * F; i += kHT) {
+      const int f = (i % (F / 2)) * 2, sl = (i / (F / 2)) % a.slices, bin = i / (F / 2 * a.slices);
+      const uint8_t* hb = reinterpret_cast<const uint8_t*>(hs + ((size_t)(bin & 2 ? r0 : 0) * a.Wa + (bin & 1 ? c0 : 0)) * F + f);
+      const int k0 = cnt * sl / a.slices, k1 = cnt * (sl + 1) / a.slices;
+      float ta = 0.f, tb = 0.f;
+      const int planes = min(a.planes, k1 - k0);
+      const bool whole = planes % 16 == 0 && (k1 - k0) % a.planes == 0 && k0 % 4 == 0;
+#pragma unroll 1
+      for (int pl = 0; pl < planes; pl += 16) {
+        float ca[16], cb[16];
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+        for (int u = 0; u < 16; ++u) ca[u] = cb[u] = 0.f;
+#pragma unroll 1
+        for (int k = k0 + pl; k < k1; k += a.planes) {
+          uint32_t o[16];
+          if (whole) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
+            for (int u = 0; u < 16; u += 4) {
+              const uint4 x = *reinterpret_cast<const uint4*>(off + k + u);
+              o[u] = x.x; o[u + 1] = x.y; o[u + 2] = x.z; o[u + 3] = x.w;
+            }
+          } else {
 #pragma unroll
-        for (int o = 16; o >= F8; o >>= 1) s[b][e] += __shfl_xor_sync(0xffffffffu, s[b][e], o);
-        if (lane < F8) rd[warp * D + (lane * 8 + e) * 4 + b] = s[b][e];
+            for (int u = 0; u < 16; ++u) o[u] = off[min(k + u, cnt - 1)];
+          }
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            const float2 v = pair(reinterpret_cast<const T*>(hb + o[u]));
+            const bool in = whole || (k + u < k1 && pl + u < planes);
+            ca[u] += in ? v.x : 0.f;
+            cb[u] += in ? v.y : 0.f;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          ta += ca[u];
+          tb += cb[u];
+        }
       }
+      rd[sl * D + f * 4 + bin] = ta;
+      rd[sl * D + f * 4 + 4 + bin] = tb;
+    }
     __syncthreads();
     for (int d = t; d < D; d += kHT) {
       float v = 0.f;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) v += rd[w * D + d];
-      const int b = d & 3;
-      v /= (float)((b & 2 ? a.Ha - r0 : r1) * (b & 1 ? a.Wa - c0 : c1));
+      for (int sl = 0; sl < a.slices; ++sl) v += rd[sl * D + d];
+      v = a.even ? v * (1.f / (float)cnt) : v / (float)cnt;
       ps[d] = v;
       a.p[(size_t)n * D + d] = v;
     }
+  } else if (!a.part) {
+    for (int d = t; d < D; d += kHT) ps[d] = a.p[(size_t)n * D + d];
   } else {
     // a warp per bin and quarter of the bin's partials; lanes run over the channels
     const int qh = a.th / 2, qw = a.tw / 2, cnt = qh * qw * 4, b = warp & 3, sub = warp >> 2;
@@ -139,42 +237,71 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
   __syncthreads();
 
-  // logits: kLpc lanes per class, each with 4 (or 8) of the inputs in registers; four classes at a time per lane group
-  constexpr int kLpc = F < 32 ? F : 32, kVec = F / kLpc, kGroups = kHT / kLpc;
-  {
+  // The linear weights are read twice, by rows and by columns: through shared memory, in h's place, where they fit (rows padded
+  // against bank conflicts), else from L2.
+  constexpr int kRow = D + 4;
+  float* ws = reinterpret_cast<float*>(hs);
+  if constexpr (STAGE) {
+    const float4* src = reinterpret_cast<const float4*>(a.Wf);
+    const int units = a.K * (D / 4);
+#pragma unroll 1
+    for (int i0 = t; i0 < units; i0 += 8 * kHT) {
+      float4 q[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) q[j] = src[min(i0 + j * kHT, units - 1)];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (i0 + j * kHT < units) {
+          const int i = i0 + j * kHT;
+          *reinterpret_cast<float4*>(ws + (size_t)(i / (D / 4)) * kRow + (i % (D / 4)) * 4) = q[j];
+        }
+    }
+    __syncthreads();
+    // logits: a thread per class, inputs in order
+    for (int k = t; k < a.K; k += kHT) {
+      float v = ls[k];  // the bias
+      const float4* w = reinterpret_cast<const float4*>(ws + (size_t)k * kRow);
+      const float4* x = reinterpret_cast<const float4*>(ps);
+#pragma unroll 8
+      for (int d = 0; d < D / 4; ++d) {
+        const float4 wv = w[d], xv = x[d];
+        v = fmaf(wv.x, xv.x, v);
+        v = fmaf(wv.y, xv.y, v);
+        v = fmaf(wv.z, xv.z, v);
+        v = fmaf(wv.w, xv.w, v);
+      }
+      ls[k] = v;
+    }
+  } else {
+    // kLpc lanes per class, each with 4 (or 8) of the inputs in registers, kU classes at a time per lane group
+    constexpr int kLpc = F < 32 ? F : 32, kVec = F / kLpc, kGroups = kHT / kLpc, kU = kVec == 1 ? 8 : 4;
     const int l = t % kLpc, grp = t / kLpc;
     float4 x[kVec];
 #pragma unroll
     for (int v = 0; v < kVec; ++v) x[v] = *reinterpret_cast<const float4*>(ps + (l + v * kLpc) * 4);
-    for (int kb = 0; kb < a.K; kb += 4 * kGroups) {  // the same trips for every thread: whole warps in the shuffles
-      const int k0 = kb + grp;
-      float s[4];
+#pragma unroll 1
+    for (int kb = 0; kb < a.K; kb += kU * kGroups) {  // the same trips for every thread: whole warps in the shuffles
+      float4 w[kU][kVec];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int k = k0 + u * kGroups;
-        s[u] = 0.f;
-        if (k < a.K) {
+      for (int u = 0; u < kU; ++u)
 #pragma unroll
-          for (int v = 0; v < kVec; ++v) {
-            const float4 w = *reinterpret_cast<const float4*>(a.Wf + (size_t)k * D + (l + v * kLpc) * 4);
-            s[u] = fmaf(w.x, x[v].x, s[u]);
-            s[u] = fmaf(w.y, x[v].y, s[u]);
-            s[u] = fmaf(w.z, x[v].z, s[u]);
-            s[u] = fmaf(w.w, x[v].w, s[u]);
-          }
-        }
-      }
+        for (int v = 0; v < kVec; ++v)
+          w[u][v] = *reinterpret_cast<const float4*>(a.Wf + (size_t)min(kb + grp + u * kGroups, a.K - 1) * D + (l + v * kLpc) * 4);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < kU; ++u) {
+        float z = 0.f;
 #pragma unroll
-        for (int o = kLpc / 2; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-        const int k = k0 + u * kGroups;
-        if (l == 0 && k < a.K) ls[k] = s[u] + a.bf[k];
+        for (int v = 0; v < kVec; ++v) z = fmaf(w[u][v].x, x[v].x, fmaf(w[u][v].y, x[v].y, fmaf(w[u][v].z, x[v].z, fmaf(w[u][v].w, x[v].w, z))));
+#pragma unroll
+        for (int o = kLpc / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        const int k = kb + grp + u * kGroups;
+        if (l == 0 && k < a.K) ls[k] += z;
       }
     }
   }
+  const float* wrow = STAGE ? ws : a.Wf;
+  constexpr int pitch = STAGE ? kRow : D;
   __syncthreads();
-  int lab = a.labels[n];
   if (lab < 0 || lab >= a.K) {
     if (t == 0) atomicOr(a.status, NF_ELABEL);
     lab = lab < 0 ? 0 : a.K - 1;
@@ -184,22 +311,24 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   if (a.loss_kind == 1) {  // mean squared error against the one-hot target
     float se = 0.f;
     const float sc = 2.f / ((float)a.n_scale * (float)a.K);
-    for (int k = t; k < a.K; k += kHT) {
-      const float l = ls[k], e = l - (k == lab ? 1.f : 0.f);
-      se = fmaf(e, e, se);
-      lrow[k] = l;
-      grow[k] = e * sc;
-      ls[k] = e * sc;
-    }
-    se = block_all(se, rd, false);
+    if (t < 256)
+      for (int k = t; k < a.K; k += 256) {
+        const float l = ls[k], e = l - (k == lab ? 1.f : 0.f);
+        se = fmaf(e, e, se);
+        lrow[k] = l;
+        grow[k] = e * sc;
+        ls[k] = e * sc;
+      }
+    se = tree_sum256(se, rd);
     if (t == 0) a.lossn[n] = se / (float)a.K;
   } else {
     float mx = -INFINITY;
     for (int k = t; k < a.K; k += kHT) mx = fmaxf(mx, ls[k]);
-    mx = block_all(mx, rd, true);
+    mx = block_max(mx, rd);
     float se = 0.f;
-    for (int k = t; k < a.K; k += kHT) se += expf(ls[k] - mx);
-    se = block_all(se, rd, false);
+    if (t < 256)
+      for (int k = t; k < a.K; k += 256) se += expf(ls[k] - mx);
+    se = tree_sum256(se, rd);
     const float lse = mx + logf(se);
     if (t == 0) a.lossn[n] = lse - ls[lab];
     __syncthreads();
@@ -213,26 +342,25 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
   __syncthreads();
 
-  // dp[d] = sum_k dlogits[k] Wf[k][d]: the classes in kG contiguous ranges, the range sums added in order
-  constexpr int kG = kHT / D;
-  {
+  // dp[d] = sum_k dlogits[k] Wf[k][d]: the classes in contiguous ranges, each in order, the range sums added in order
+  const int kG = a.groups;
+  if (t < kG * D) {
     const int d = t % D, kg = t / D, per = (a.K + kG - 1) / kG, ka = kg * per, kb = min(a.K, ka + per);
     float s = 0.f;
-    int k = ka;
-    for (; k + 7 < kb; k += 8) {
-      float w[8];
+#pragma unroll 1
+    for (int k = ka; k < kb; k += 16) {
+      float w[16];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) w[u] = a.Wf[(size_t)(k + u) * D + d];
+      for (int u = 0; u < 16; ++u) w[u] = wrow[(size_t)min(k + u, kb - 1) * pitch + d];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) s = fmaf(ls[k + u], w[u], s);
+      for (int u = 0; u < 16; ++u)
+        if (k + u < kb) s = fmaf(ls[k + u], w[u], s);
     }
-    for (; k < kb; ++k) s = fmaf(ls[k], a.Wf[(size_t)k * D + d], s);
     rd[kg * D + d] = s;
   }
   __syncthreads();
   for (int d = t; d < D; d += kHT) {
     float v = 0.f;
-#pragma unroll
     for (int q = 0; q < kG; ++q) v += rd[q * D + d];
     a.dp[(size_t)n * D + d] = v;
     ps[d] = v;
@@ -245,7 +373,7 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int u = b >> 1, w = b & 1;
-      if ((rc == 2 || rc == u) && (cc == 2 || cc == w)) v += ps[f * 4 + b] / (float)((u ? a.Ha - r0 : r1) * (w ? a.Wa - c0 : c1));
+      if ((rc == 2 || rc == u) && (cc == 2 || cc == w)) v += a.dh_even ? ps[f * 4 + b] * (1.f / (float)(r1 * c1)) : ps[f * 4 + b] / (float)(r1 * c1);
     }
     tab[i] = v;
   }
@@ -254,15 +382,16 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
 #pragma unroll
   for (int e = 0; e < 8; ++e) bs[e] = 0.f;
   T* dhn = reinterpret_cast<T*>(a.dh) + (size_t)n * px * F;
-  for (int q = t / F8; q < px; q += kHT / F8) {
-    const int i = q / a.Wa, j = q - i * a.Wa;
-    const int rc = i < r0 ? 0 : i >= r1 ? 1 : 2, cc = j < c0 ? 0 : j >= c1 ? 1 : 2;
-    float v[8], o[8];
-    ld8(hs + (size_t)q * F + g * 8, v);
+#pragma unroll 2
+  for (int i = t; i < px * F8; i += kHT) {  // kHT is a multiple of F8: the thread's channels stay
+    const int q = i / F8, ii = q / a.Wa, jj = q - ii * a.Wa;
+    const int rc = ii < r0 ? 0 : ii >= r1 ? 1 : 2, cc = jj < c0 ? 0 : jj >= c1 ? 1 : 2;
+    const uint32_t bits = mask[i];
+    float o[8];
     ld8(tab + (rc * 3 + cc) * F + g * 8, o);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) o[e] = v[e] > 0.f ? o[e] : 0.f;
-    st8(dhn + (size_t)q * F + g * 8, o);
+    for (int e = 0; e < 8; ++e) o[e] = (bits >> e) & 1u ? o[e] : 0.f;
+    st8(dhn + (size_t)i * 8, o);
 #pragma unroll
     for (int e = 0; e < 8; ++e) bs[e] += o[e];  // the bias gradient sums the values as stored
   }
@@ -281,62 +410,75 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
 }
 
-// Sums over the batch.  Blocks [0, K * DT): class k = b / DT, inputs 32 (b % DT) ..: gWf, and gbf where b % DT == 0; 32 inputs x
-// 8 sample lanes, eight samples in flight per lane, lanes added in order.  Then FT blocks of 32 filters: gba from the per-sample
-// sums of dh (fp64, none when bred is NULL); the last block: the mean loss (fp64).
+// Sums over the batch.  Blocks [0, KT * DT): KC classes from KC (b / DT) on, inputs 64 (b % DT) ..: gWf, and gbf where b % DT == 0;
+// 64 inputs x 4 interleaved chains over the samples, combined as (0 + 1) + (2 + 3).  Then FT blocks of 32 filters: gba from the
+// per-sample sums of dh (fp64); the last block: the mean loss (fp64).
+template <int KC>
 __global__ void __launch_bounds__(256) head_batch_kernel(const float* __restrict__ p, const float* __restrict__ dl,
                                                          const float* __restrict__ lossn, const float* __restrict__ bred, int N, int D,
-                                                         int K, int DT, int FT, int F, float* __restrict__ gWf, float* __restrict__ gbf,
-                                                         float* __restrict__ gba, float* __restrict__ loss_out,
+                                                         int K, int KT, int DT, int FT, int F, float* __restrict__ gWf,
+                                                         float* __restrict__ gbf, float* __restrict__ gba, float* __restrict__ loss_out,
                                                          int32_t* __restrict__ status, int n_scale) {
   nf_pdl_begin();
   __shared__ double sd[8][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.x;
-  if (b < K * DT) {
-    float(*sf)[33] = reinterpret_cast<float(*)[33]>(sd);
-    const int k = b / DT, d = (b % DT) * 32 + tx;
-    float s = 0.f, sb = 0.f;
-    int n = ty;
-    for (; n + 56 < N; n += 64) {
-      float u[8], v[8];
+  if (b < KT * DT) {
+    __shared__ float sf[KC][4][64];
+    const int k0 = (b / DT) * KC, dx = threadIdx.x & 63, ch = threadIdx.x >> 6, d = (b % DT) * 64 + dx;
+    const int N4 = N & ~3;
+    float s[KC];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        u[e] = dl[(size_t)(n + 8 * e) * K + k];
-        v[e] = d < D ? p[(size_t)(n + 8 * e) * D + d] : 0.f;
-      }
+    for (int c = 0; c < KC; ++c) s[c] = 0.f;
+    if (d < D) {
+      // chain ch: samples ch, ch + 4, ... below N4; chain 0 goes on with the last one to three
+      const int cnt = N4 / 4, all = cnt + (ch == 0 ? N - N4 : 0);
+      constexpr int kU = KC == 1 ? 16 : 8;
+#pragma unroll 1
+      for (int j = 0; j < all; j += kU) {
+        float u[kU][KC], v[kU];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        s = fmaf(u[e], v[e], s);
-        sb += u[e];
+        for (int e = 0; e < kU; ++e) {
+          const int q = min(j + e, all - 1), n = q < cnt ? ch + 4 * q : N4 + q - cnt;
+          v[e] = p[(size_t)n * D + d];
+#pragma unroll
+          for (int c = 0; c < KC; ++c) u[e][c] = dl[(size_t)n * K + min(k0 + c, K - 1)];
+        }
+#pragma unroll
+        for (int e = 0; e < kU; ++e)
+#pragma unroll
+          for (int c = 0; c < KC; ++c) s[c] = j + e < all ? fmaf(u[e][c], v[e], s[c]) : s[c];
       }
     }
-    for (; n < N; n += 8) {
-      const float u = dl[(size_t)n * K + k];
-      s = fmaf(u, d < D ? p[(size_t)n * D + d] : 0.f, s);
-      sb += u;
-    }
-    sf[ty][tx] = s;
-    if (tx == 0) sf[ty][32] = sb;
+#pragma unroll
+    for (int c = 0; c < KC; ++c) sf[c][ch][dx] = s[c];
     __syncthreads();
-    if (ty == 0) {
-      float v = 0.f;
+    if (d < D)
+      for (int c = ch; c < KC; c += 4)
+        if (k0 + c < K) gWf[(size_t)(k0 + c) * D + d] = (sf[c][0][dx] + sf[c][1][dx]) + (sf[c][2][dx] + sf[c][3][dx]);
+    if (b % DT == 0 && ty < KC && k0 + ty < K) {
+      float c = 0.f;
+#pragma unroll 1
+      for (int n0 = tx; n0 < N; n0 += 128) {
+        float u[4];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v += sf[q][tx];
-      if (d < D) gWf[(size_t)k * D + d] = v;
-      if (tx == 0 && b % DT == 0) {
-        float c = 0.f;
+        for (int e = 0; e < 4; ++e) u[e] = dl[(size_t)min(n0 + 32 * e, N - 1) * K + k0 + ty];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) c += sf[q][32];
-        gbf[k] = c;
+        for (int e = 0; e < 4; ++e) c += n0 + 32 * e < N ? u[e] : 0.f;
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if (tx == 0) gbf[k0 + ty] = c;
     }
     return;
   }
-  const bool loss = b == K * DT + FT;
-  const int f = (b - K * DT) * 32 + tx;
+  const bool loss = b == KT * DT + FT;
+  const int f = (b - KT * DT) * 32 + tx;
   double s = 0.0;
   if (loss) {
-    for (int n = threadIdx.x; n < N; n += 256) s += (double)lossn[n];
+    if (ty == 0) {
+#pragma unroll 4
+      for (int n = tx; n < N; n += 32) s += (double)lossn[n];
+    }
   } else if (f < F) {
 #pragma unroll 8
     for (int n = ty; n < N; n += 8) s += (double)bred[(size_t)n * F + f];
@@ -344,9 +486,7 @@ __global__ void __launch_bounds__(256) head_batch_kernel(const float* __restrict
   sd[ty][tx] = s;
   __syncthreads();
   if (loss && ty == 0) {
-    double v = 0.0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v += sd[q][tx];
+    double v = s;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (tx == 0) {
@@ -364,29 +504,51 @@ __global__ void __launch_bounds__(256) head_batch_kernel(const float* __restrict
 
 constexpr size_t kSmemMax = 200 * 1024;
 
+// Summation order of the average pool, as the stand-alone pool kernels have it (nf_k_avgpool_fast, nf_k_avgpool)
+struct PoolOrder {
+  int slices, planes, even;
+};
+PoolOrder pool_order(int dtype, int N, int Ha, int Wa, int F) {
+  const bool even = Ha % 2 == 0 && Wa % 2 == 0;
+  if (dtype == NF_BF16 && even && (Ha / 2) * (Wa / 2) > 16) return {nf_k_avgpool_slices(N, Ha, Wa), 256 / (F / 8), 1};
+  const int cnt = ((Ha + 1) / 2) * ((Wa + 1) / 2);
+  if (dtype == NF_F32) return {std::max(1, std::min(kWarps, cnt / 16)), 16, 0};  // fp32 follows no other kernel's bits
+  return {1, cnt <= 16 ? 1 : 256 / F, 0};
+}
+size_t h_smem(int dtype, int Ha, int Wa, int F) { return (size_t)Ha * Wa * F * nf_esize(dtype); }
+size_t off_smem(int Ha, int Wa, int F) {  // offsets and sign bits
+  return (size_t)((((Ha + 1) / 2) * ((Wa + 1) / 2) + 3) / 4 * 4) * 4 + (size_t)Ha * Wa * (F / 8);
+}
 size_t fixed_smem(int F, int K) { return ((size_t)4 * F + ((K + 3) & ~3) + (size_t)kWarps * 4 * F + 9 * F) * 4; }
 
-template <typename T, int F8>
-int run_sample(const HeadArgs& a, size_t smem) {
+template <typename T, int F8, bool STAGE>
+int launch_sample(const HeadArgs& a, size_t smem) {
   static bool done[64];  // function attributes belong to a device's context: set once per device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
   if (!done[dev]) {
-    NF_CUDA(cudaFuncSetAttribute(head_sample_kernel<T, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    NF_CUDA(cudaFuncSetAttribute(head_sample_kernel<T, F8, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax + 1024));
     done[dev] = true;
   }
-  nf_launch(head_sample_kernel<T, F8>, a.N, kHT, smem, a);
+  nf_launch(head_sample_kernel<T, F8, STAGE>, a.N, kHT, smem, a);
   NF_LAUNCHED();
   return NF_OK;
+}
+template <typename T, int F8>
+int run_sample(const HeadArgs& a, size_t smem, bool stage) {
+  return stage ? launch_sample<T, F8, true>(a, smem) : launch_sample<T, F8, false>(a, smem);
 }
 
 }  // namespace
 
-// 0: not covered; 1: everything but dh; 2: dh as well.  Filters in 8, 16, 32, 64; dh where the sample's h fits beside the tables.
-int nf_head_sample_mode(int dtype, int Ha, int Wa, int F, int K) {
+// 0: not covered; 1: from pooled inputs (p, or the fused aux forward's partials); 2: from h, with dh, where the sample's h fits
+// beside the tables.  Filters in 8, 16, 32, 64.
+int nf_head_sample_mode(int dtype, int N, int Ha, int Wa, int F, int K) {
   if ((F != 8 && F != 16 && F != 32 && F != 64) || K > 16384 || Ha < 2 || Wa < 2) return 0;
   if (fixed_smem(F, K) > kSmemMax) return 0;
-  return fixed_smem(F, K) + (size_t)Ha * Wa * F * nf_esize(dtype) <= kSmemMax ? 2 : 1;
+  const PoolOrder o = pool_order(dtype, N, Ha, Wa, F);
+  const size_t need = fixed_smem(F, K) + h_smem(dtype, Ha, Wa, F) + off_smem(Ha, Wa, F);
+  return o.slices <= kWarps && need <= kSmemMax ? 2 : 1;
 }
 
 int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, int F, int K, int loss_kind, int n_scale) {
@@ -396,18 +558,34 @@ int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, in
   a.labels = io.labels; a.Wf = io.Wf; a.bf = io.bf;
   a.p = io.p; a.logits = io.logits; a.dlogits = io.dlogits; a.dp = io.dp; a.lossn = io.lossn; a.status = io.status;
   a.dh = io.dh; a.bred = io.bred; a.loss_kind = loss_kind; a.n_scale = n_scale;
-  const size_t smem = fixed_smem(F, K) + (io.dh ? (size_t)Ha * Wa * F * nf_esize(dtype) : 0);
+  const PoolOrder o = pool_order(dtype, N, Ha, Wa, F);
+  a.slices = o.slices; a.planes = o.planes; a.even = o.even;
+  a.dh_even = dtype == NF_BF16 && Ha % 2 == 0 && Wa % 2 == 0;
+  const int D = 4 * F;
+  // fixed tables, then h or the weights, then (with h) offsets and sign bits
+  const size_t tail = io.h ? off_smem(Ha, Wa, F) : 0;
+  size_t smem = fixed_smem(F, K) + (io.h ? h_smem(dtype, Ha, Wa, F) : 0);
+  const size_t with_w = fixed_smem(F, K) + (size_t)K * (D + 4) * 4;
+  const bool stage = with_w + tail <= kSmemMax;
+  if (stage && with_w > smem) smem = with_w;
+  smem = (smem + 15) & ~(size_t)15;
+  a.off = smem;
+  smem += tail;
+  // many classes per sample: as many ranges as there are threads; else the order of the kernel for heads that are not covered here
+  a.groups = (long)K >= 4L * N ? kHT / D : D <= 128 ? 256 / D : 1;
   int rc;
   if (dtype == NF_F32)
-    rc = F == 8 ? run_sample<float, 1>(a, smem) : F == 16 ? run_sample<float, 2>(a, smem)
-       : F == 32 ? run_sample<float, 4>(a, smem) : run_sample<float, 8>(a, smem);
+    rc = F == 8 ? run_sample<float, 1>(a, smem, stage) : F == 16 ? run_sample<float, 2>(a, smem, stage)
+       : F == 32 ? run_sample<float, 4>(a, smem, stage) : run_sample<float, 8>(a, smem, stage);
   else
-    rc = F == 8 ? run_sample<bf16, 1>(a, smem) : F == 16 ? run_sample<bf16, 2>(a, smem)
-       : F == 32 ? run_sample<bf16, 4>(a, smem) : run_sample<bf16, 8>(a, smem);
+    rc = F == 8 ? run_sample<bf16, 1>(a, smem, stage) : F == 16 ? run_sample<bf16, 2>(a, smem, stage)
+       : F == 32 ? run_sample<bf16, 4>(a, smem, stage) : run_sample<bf16, 8>(a, smem, stage);
   if (rc != NF_OK) return rc;
-  const int D = 4 * F, DT = (D + 31) / 32, FT = io.dh ? (F + 31) / 32 : 0;
-  nf_launch(head_batch_kernel, (unsigned)(K * DT + FT + 1), 256, 0, io.p, io.dlogits, io.lossn, io.bred, N, D, K, DT, FT, F, io.gWf, io.gbf, io.gba,
-            io.loss_out, io.status, n_scale);
+  const int DT = (D + 63) / 64, FT = io.dh ? (F + 31) / 32 : 0;
+  // four classes per block read the samples' inputs once between them; with few classes that would leave too few blocks
+  const int KC = K >= 512 ? 4 : 1, KT = (K + KC - 1) / KC;
+  nf_launch(KC == 4 ? head_batch_kernel<4> : head_batch_kernel<1>, (unsigned)(KT * DT + FT + 1), 256, 0, io.p, io.dlogits, io.lossn, io.bred, N, D, K,
+            KT, DT, FT, F, io.gWf, io.gbf, io.gba, io.loss_out, io.status, n_scale);
   NF_LAUNCHED();
   return NF_OK;
 }

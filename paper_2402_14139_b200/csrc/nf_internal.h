@@ -138,6 +138,7 @@ int nf_k_bn_eval_coeffs(int C, const float* gamma, const float* beta, float eps,
                           const float* rvar, float* scale, float* shift);
 int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int pool, const float* scale,
                     const float* shift, void* out, const void* skip = nullptr);
+int nf_k_avgpool_slices(int N, int Ha, int Wa);
 int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* p);
 // bf16 fast paths (F % 8 == 0, even Ha and Wa); NF_EUNSUPPORTED means "use the generic kernel"
 int nf_k_avgpool_fast(const void* h, int N, int Ha, int Wa, int F, float* part, size_t part_floats, float* p);
@@ -163,8 +164,8 @@ int nf_head_step(const float* p, const int32_t* labels, int N, int D, int K, con
                  float* scratch, size_t scratch_floats, int n_scale);
 // head with one block per sample (nf_head_sample.cu): pool, linear layer, loss, dp and (mode 2) dh with the aux bias gradient
 struct NfHeadIo {
-  const void* h;      // aux output, or NULL with
-  const float* part;  // the pooling partials of the fused aux forward
+  const void* h;      // mode 2: aux output; else NULL, with
+  const float* part;  // the pooling partials of the fused aux forward, or NULL: p holds the pooled inputs
   const int32_t* labels;
   const float *Wf, *bf;
   float *p, *logits, *dlogits, *dp, *lossn;
@@ -173,7 +174,7 @@ struct NfHeadIo {
   float* bred;        // [N][F] scratch (with dh)
   float *gWf, *gbf, *gba, *loss_out;
 };
-int nf_head_sample_mode(int dtype, int Ha, int Wa, int F, int K);
+int nf_head_sample_mode(int dtype, int N, int Ha, int Wa, int F, int K);
 int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, int F, int K, int loss_kind, int n_scale);
 // small-batch head (nf_head_small.cu): class-sliced forward + backward of the linear layer and the loss; 0 floats = not covered
 size_t nf_head_small_scratch_floats(int N, int D, int K);
