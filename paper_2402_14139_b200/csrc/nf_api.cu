@@ -459,7 +459,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   // gradient at the aux input
   trace_begin(8);
   int bn_nb = 0;  // > 0: the input-gradient kernel has already left the BatchNorm-backward partial sums in L->red
-  if (L->fam[3]) {
+  if (L->dgrad_tc) {
     NF_TRY(nf_tc_aux_dgrad(L, &bn_nb));
   } else {
     NF_TRY(nf_k_conv(dt, L->dh, N, Ha, Wa, F, Wx, (long)F * Co, 1, Co, 1, nullptr, 0, 1, Co, L->da));

@@ -64,6 +64,7 @@ struct nf_layer {
   float* stage_loss;
   // kernel families chosen at configure time: 0 = cuda-core, 1 = tcgen05
   int fam[4];
+  int dgrad_tc;                        // aux input gradient on tcgen05 (fam[3] says so of the aux weight gradient)
   // First layers (a few input channels, e.g. RGB): cin_pad = 64 makes the main conv run on the tensor-core kernels over a
   // copy of the input batch whose pixels are zero-padded to 64 channels; 0 = the input is used as it is.
   int cin_pad;

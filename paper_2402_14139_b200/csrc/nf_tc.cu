@@ -21,6 +21,7 @@ namespace {
 
 constexpr int kThreads = 192;  // warp 0: TMA producer, warp 1: MMA issuer + TMEM owner, warps 2-5: epilogue
 constexpr int kMaxStages = 8;
+constexpr int kSegSteps = 3;  // k-steps of 64 products per accumulator in the segmented forward
 // normalisation threads of the fused BatchNorm + aux forward: two groups of 128 that take the stages in turn.  A single group
 // was the slowest role of the kernel (busy 2350 of every 2450 cycles per tile while the issuer waited 520 on it: one warp per
 // scheduler cannot hide the latency of its load - arithmetic - store - fence chain).  Splitting the ten rows of ONE box over
@@ -98,9 +99,30 @@ struct FwdParams {
 };
 
 struct TcPlan {
-  int ok, BW, BH, BI, PT, BN, KC, RW, stages, grid, parts;
+  int ok, BW, BH, BI, PT, BN, KC, RW, SEG, stages, grid, parts;
   size_t smem;
 };
+
+// Sum of the next `n` segment accumulators (of four taken in turn; `taken` counts them) for one thread's row of BN columns.
+template <int BN>
+__device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& taken, uint64_t* tfull, uint64_t* tempty,
+                                             volatile int* abort_flag, float (&sum)[BN]) {
+  for (int i = 0; i < n; ++i, ++taken) {
+    const uint32_t acc = taken & 3;
+    ptx::mbar_wait(&tfull[acc], (taken >> 2) & 1, abort_flag);  // sets the abort flag itself when it gives up
+    ptx::tc_fence_after();
+#pragma unroll
+    for (int j = 0; j < BN / 16; ++j) {
+      uint32_t v[16];
+      ptx::tmem_ld16(tbase + acc * BN + j * 16, v);
+      ptx::tmem_ld_wait();
+#pragma unroll
+      for (int e = 0; e < 16; ++e) sum[j * 16 + e] = i ? sum[j * 16 + e] + __uint_as_float(v[e]) : __uint_as_float(v[e]);
+    }
+    ptx::tc_fence_before();
+    ptx::mbar_arrive(&tempty[acc]);
+  }
+}
 
 // EPI 0: y in bf16 through a TMA store plus BatchNorm partial sums (BN = 64 or 128).
 // EPI 1: bias + ReLU, channels [0, Cout) of a BN-wide tile written directly (aux conv; Cout <= BN <= 64,
@@ -114,7 +136,11 @@ struct TcPlan {
 //       images (8x8x2, 4x4x8, 2x2x32), and maps that no tile divides; p.H, p.W are the OUTPUT sizes.
 // RW  : 1 = all nine weight tiles of the CTA's channel tile stay resident in shared memory for the whole
 //       kernel (single 64-channel K chunk, 9*BN*128 bytes); the pipeline then carries activations only.
-template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0>
+// SEG : 1 (PT, forward only) = a new accumulator every kSegSteps k-steps, the segments added in fp32 by the epilogue.  The tensor
+//       core's running sum drops low bits on every instruction: over 2304 products 0.07 % of the bf16 outputs came out one unit
+//       off the nearest value, against 0.016 % of an fp32 chain.  Maps that no tile divides had such chains (they ran on the CUDA
+//       cores), and their layers are small enough for that to show; a segment's 192 products keep the error below theirs.
+template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0>
 __global__ void __launch_bounds__(kThreads, 1)
 conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                    const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ FwdParams p) {
@@ -135,8 +161,9 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   uint64_t* full = bars;
   uint64_t* empty = bars + kMaxStages;
   uint64_t* tfull = bars + 2 * kMaxStages;
-  uint64_t* tempty = tfull + 2;
-  uint64_t* wfull = tempty + 2;
+  constexpr uint32_t kAccs = SEG ? 4 : 2;
+  uint64_t* tempty = tfull + kAccs;
+  uint64_t* wfull = tempty + kAccs;
   uint64_t* yfull = wfull + 1;
   uint64_t* yempty = yfull + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(yempty + 1);
@@ -150,7 +177,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       ptx::mbar_init(&full[s], 1);
       ptx::mbar_init(&empty[s], 1);
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < (int)kAccs; ++a) {
       ptx::mbar_init(&tfull[a], 1);
       ptx::mbar_init(&tempty[a], 128);
     }
@@ -163,7 +190,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     ptx::prefetch_tmap(&tm_w);
     ptx::prefetch_tmap(&tm_y);
   }
-  constexpr uint32_t kTmemCols = 2 * BN < 32 ? 32 : 2 * BN;
+  static_assert(!SEG || (PT && !BMN && BN <= 128), "segmented accumulation: per-tap forward");
+  constexpr uint32_t kTmemCols = kAccs * BN < 32 ? 32 : kAccs * BN;
   if (warp == 1) {
     ptx::tmem_alloc(tmem_slot, kTmemCols);
     ptx::tmem_relinquish();
@@ -248,15 +276,21 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if constexpr (RW) {
         if (blockIdx.x < p.total_tiles) ok = ptx::mbar_wait(wfull, 0, abort_flag);
       }
-      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x, ++tl) {
-        const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
-        if (!ptx::mbar_wait(&tempty[acc], aph ^ 1, abort_flag)) break;
-        ptx::tc_fence_after();
-        const uint32_t d = tmem_base + acc * BN;
-        uint32_t accumulate = 0;
+      const int steps = (PT ? 9 : 3) * p.kchunks;
+      for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
+        uint32_t acc = 0, d = 0, accumulate = 0;
+        int step = 0;
         for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
           for (int tap = 0; tap < (PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+            if (step == 0 || (SEG && step % kSegSteps == 0)) {
+              acc = tl % kAccs;
+              if (!ptx::mbar_wait(&tempty[acc], ((tl / kAccs) & 1) ^ 1, abort_flag)) { ok = false; break; }
+              ++tl;
+              d = tmem_base + acc * BN;
+              accumulate = 0;
+            }
+            ++step;
             if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
             ptx::tc_fence_after();
             const uint32_t a_base = ptx::smem_u32(smem) + rg.s * stage_bytes;
@@ -273,9 +307,9 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                 accumulate = 1;
               }
             ptx::mma_commit(&empty[rg.s]);
+            if (step == steps || (SEG && step % kSegSteps == 0)) ptx::mma_commit(&tfull[acc]);
           }
         }
-        if (ok) ptx::mma_commit(&tfull[acc]);
       }
     }
     __syncwarp();
@@ -288,6 +322,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     constexpr int kRowsPer = BN >= 128 ? 128 : 64;  // rows each thread sums for its channel
     const int sc = et % BN, shalf = et / BN;        // stats: channel and row half of this thread
     const int rw = r % p.BW, rh = (r / p.BW) % p.BH;  // place of the thread's pixel in its tile
+    uint32_t sg = 0;                                  // SEG: segments taken so far
     float ssum = 0.f, ssq = 0.f;
     float ssum2 = 0.f, ssq2 = 0.f;                  // BN = 256: the thread's second channel, sc + 128
     uint32_t tl = 0;
@@ -306,8 +341,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const TileAt at = tile_at(t, p.tg);
       const int nt = at.nt, w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
       const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
-      ptx::mbar_wait(&tfull[acc], aph, abort_flag);  // sets the abort flag itself when it gives up
-      ptx::tc_fence_after();
+      float seg[SEG ? BN : 1];
+      if constexpr (SEG) {
+        add_segments<BN>(tmem_base + ((uint32_t)(lg * 32) << 16), (9 * p.kchunks + kSegSteps - 1) / kSegSteps, sg, tfull, tempty, abort_flag, seg);
+      } else {
+        ptx::mbar_wait(&tfull[acc], aph, abort_flag);  // sets the abort flag itself when it gives up
+        ptx::tc_fence_after();
+      }
       if (et == 0) {
         ptx::tma_store_wait_read();  // the previous tile's store has finished reading the staging tile
         *epi_go = *abort_flag ? 0 : 1;  // one thread decides for all 128, so nobody is left alone at a barrier
@@ -318,8 +358,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
       for (int j = 0; j < BN / 32; ++j) {
         uint32_t v[32];
-        ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 32, v);
-        ptx::tmem_ld_wait();
+        if constexpr (SEG) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(seg[j * 32 + e]);
+        } else {
+          ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 32, v);
+          ptx::tmem_ld_wait();
+        }
         uint8_t* sub = stg + ((j * 32) / 64) * 16384 + r * 128;
         const int u0 = ((j * 32) % 64) / 8;
 #pragma unroll
@@ -339,8 +384,10 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (r & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
         }
       }
-      ptx::tc_fence_before();
-      ptx::mbar_arrive(&tempty[acc]);
+      if constexpr (!SEG) {
+        ptx::tc_fence_before();
+        ptx::mbar_arrive(&tempty[acc]);
+      }
       ptx::fence_async_smem();
       ptx::named_barrier(1, 128);
       if (et == 0) {
@@ -411,13 +458,19 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const int lg = warp & 3;
       const int r = lg * 32 + lane;
       const int rw = r % p.BW, rh = (r / p.BW) % p.BH, img = r / (p.BW * p.BH);  // place of the thread's pixel in its tile
+      uint32_t sg = 0;
       uint32_t tl = 0;
       for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
         const TileAt at = tile_at(t, p.tg);
         const int w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
         const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
-        ptx::mbar_wait(&tfull[acc], aph, abort_flag);
-        ptx::tc_fence_after();
+        float seg[SEG ? BN : 1];
+        if constexpr (SEG) {
+          add_segments<BN>(tmem_base + ((uint32_t)(lg * 32) << 16), (9 * p.kchunks + kSegSteps - 1) / kSegSteps, sg, tfull, tempty, abort_flag, seg);
+        } else {
+          ptx::mbar_wait(&tfull[acc], aph, abort_flag);
+          ptx::tc_fence_after();
+        }
         if (et == 0) *epi_go = *abort_flag ? 0 : 1;
         ptx::named_barrier(1, 128);
         if (!*epi_go) break;
@@ -426,8 +479,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
         for (int j = 0; j < BN / 16; ++j) {
           uint32_t v[16];
-          ptx::tmem_ld16(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 16, v);
-          ptx::tmem_ld_wait();
+          if constexpr (SEG) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(seg[j * 16 + e]);
+          } else {
+            ptx::tmem_ld16(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 16, v);
+            ptx::tmem_ld_wait();
+          }
           if (j * 16 < p.Cout && img_ok) {
             uint32_t w[8];
 #pragma unroll
@@ -452,8 +510,10 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             }
           }
         }
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(&tempty[acc]);
+        if constexpr (!SEG) {
+          ptx::tc_fence_before();
+          ptx::mbar_arrive(&tempty[acc]);
+        }
       }
     }
   }
@@ -468,7 +528,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   }
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, 2 * BN);
+    ptx::tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -1816,16 +1876,17 @@ int sm_count() {
 // the N x H x W pixels with the fewest tiles (7x7 maps: one pixel of 128 images; 14x14: 2x2 pixels of 32): loads beyond an
 // edge read zeros, stores are clipped, the epilogue zeroes what hangs over.  Where several cover equally well the one with
 // the largest patch is taken: neighbouring taps then find most of their pixels in L2.
-void pick_tile(int N, int H, int W, int* BW, int* BH, int* BI) {
+// Returns whether the tiles divide the maps (a last tile may still lack images).
+bool pick_tile(int N, int H, int W, int* BW, int* BH, int* BI) {
   const int cand[3][2] = {{16, 8}, {32, 4}, {8, 16}};
   for (auto& c : cand)
     if (W % c[0] == 0 && H % c[1] == 0) {
       *BW = c[0]; *BH = c[1]; *BI = 1;
-      return;
+      return true;
     }
   if (W * H <= 64 && 128 % (W * H) == 0 && (W & (W - 1)) == 0) {  // 8x8, 4x4, 2x2, 8x4, 1x1 ...
     *BW = W; *BH = H; *BI = 128 / (W * H);
-    return;
+    return true;
   }
   long best = -1;
   for (int bi = 1; bi <= 128; bi *= 2)
@@ -1837,17 +1898,15 @@ void pick_tile(int N, int H, int W, int* BW, int* BH, int* BI) {
         *BW = bw; *BH = bh; *BI = bi;
       }
     }
+  return false;
 }
-bool tiles_exactly(int H, int W, int BW, int BH) { return W % BW == 0 && H % BH == 0; }
-// Whether a FORWARD convolution goes to the tensor cores.  Maps that tile exactly always do; the others from 8192 output pixels
-// on (64 tiles).  Below that a layer's gradients hang on a few thousand ReLU decisions, and the CUDA-core kernels' fp32 sums (0.01 %
-// of the bf16 outputs off the nearest value, against 0.04 - 0.13 % here, 256 channels at 14x14) are worth more than the time: up
-// to 6 % of a gradient's norm moves between the two on 648 pixels, 1 % on 12 000.  The gradients themselves decide nothing and
-// always run here.
+// Whether a convolution whose result is rounded for storage (forward, input gradient) goes to the tensor cores.  Maps that tile
+// exactly always do; the others from 8192 output pixels on (64 tiles).  Below that a layer's gradients hang on a few thousand ReLU
+// decisions, and an output one bfloat16 unit off moves them by up to several per cent in the next step; the CUDA-core kernels
+// give the same bits as they always have there.  The weight gradients stay in fp32 and always run here.
 bool tc_size_ok(int N, int H, int W) {
   int BW, BH, BI;
-  pick_tile(N, H, W, &BW, &BH, &BI);
-  return tiles_exactly(H, W, BW, BH) && (BI == 1 || W * H * BI == 128) ? true : (long)N * H * W >= 8192;
+  return pick_tile(N, H, W, &BW, &BH, &BI) || (long)N * H * W >= 8192;
 }
 
 // ybuf = 1 reserves the y2 tile of the fused BatchNorm-backward sums (as large as the output staging)
@@ -1856,11 +1915,12 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   if (stride == 2 && (epi != 0 || Cin % 64)) return pl;
   if (epi == 2 ? (Cin > 64 || Cin % 8 || Cout % 64) : (Cin % 64 != 0)) return pl;
   if (epi == 0 ? (Cout % 64 != 0) : epi == 1 ? (Cout > 64) : false) return pl;
-  pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
-  pl.PT = (stride == 2 || pl.BI > 1 || pl.BW < 8 || pl.BW > 32 || !tiles_exactly(H, W, pl.BW, pl.BH)) ? 1 : 0;
+  const bool exact = pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
+  pl.PT = (stride == 2 || pl.BI > 1 || !exact) ? 1 : 0;
+  pl.SEG = !exact && epi != 2;  // the input gradient is rounded but decides nothing
   if (epi == 0 && Cout % 256 == 0) pl.PT = 1;  // 256-wide instructions need the per-tap form (one tap of weights per stage)
   pl.BN = epi != 1 ? (Cout % 128 == 0 ? 128 : 64) : (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64);
-  if (epi == 0 && pl.PT && Cout % 256 == 0) pl.BN = 256;  // per-tap form: weights of one tap and 256 channels are 32 KB a stage
+  if (epi == 0 && pl.PT && !pl.SEG && Cout % 256 == 0) pl.BN = 256;  // per-tap form: weights of one tap and 256 channels are 32 KB a stage
   pl.KC = epi == 2 ? (Cin <= 16 ? 16 : Cin <= 32 ? 32 : 64) : 64;
   const size_t a_stride = pl.PT ? (size_t)128 * pl.KC * 2 : ((size_t)(pl.BH + 2) * pl.BW * pl.KC * 2 + 1023) & ~(size_t)1023;
   pl.RW = (!pl.PT && epi != 2 && Cin == 64 && pl.BN <= 64) ? 1 : 0;  // weights resident in shared memory
@@ -1886,15 +1946,15 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   return pl;
 }
 
-template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0>
+template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0>
 int launch_fwd(const TcPlan& pl, const CUtensorMap& mx, const CUtensorMap& mw, const CUtensorMap& my, const FwdParams& p) {
   static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
   bool& attr_done = attr_done_dev[current_device()];
   if (!attr_done) {
-    NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW>, pl.grid, kThreads, pl.smem, mx, mw, my, p);
+  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG>, pl.grid, kThreads, pl.smem, mx, mw, my, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2097,6 +2157,11 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     if ((size_t)rows * 2 * Cout > red_floats) return NF_ENOWS;
     *nb = rows;
   }
+  if (pl.SEG) {  // maps that no tile divides
+    if (epi == 0) return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
+    return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p)
+                       : pl.BN == 32 ? launch_fwd<32, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
+  }
   if (pl.PT) {  // per-tap boxes: stride 2, or several small images per tile
     if (epi == 0)
       return pl.BN == 256 ? launch_fwd<256, 0, 64, 0, 1>(pl, mx, mw, my, p)
@@ -2127,7 +2192,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
 }
 
 struct WgPlan {
-  int ok, BW, BH, BI, PT, NB, GX, splits, grid, stages;
+  int ok, exact, BW, BH, BI, PT, NB, GX, splits, grid, stages;
   size_t smem, part_floats;
 };
 
@@ -2137,8 +2202,8 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
   WgPlan pl{};
   if (Cin % 64 || (stride == 2 && aux)) return pl;
   if (aux ? (Cout > 64 || Cout % 8) : (Cout % 64 != 0)) return pl;
-  pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
-  pl.PT = (stride == 2 || pl.BI > 1 || pl.BW < 8 || pl.BW > 32 || !tiles_exactly(H, W, pl.BW, pl.BH)) ? 1 : 0;
+  pl.exact = pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
+  pl.PT = (stride == 2 || pl.BI > 1 || !pl.exact) ? 1 : 0;
   pl.NB = aux ? (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64) : 64;
   if (!aux && pl.PT) pl.NB = Cout % 256 == 0 ? 256 : Cout % 128 == 0 ? 128 : 64;  // per-tap form: as wide an instruction as Cout allows
   pl.GX = (aux && !pl.PT && pl.NB <= 32) ? 1 : 0;  // few filters: one instruction per 16 pixels with the gradient on the M side
@@ -2259,7 +2324,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
 static bool wide_aux(const nf_layer* L) { return L->F > 64 && L->F % 64 == 0; }
 
 void nf_tc_select(nf_layer* L) {
-  L->fam[0] = L->fam[1] = L->fam[2] = L->fam[3] = 0;
+  L->fam[0] = L->fam[1] = L->fam[2] = L->fam[3] = L->dgrad_tc = 0;
   L->cin_pad = 0;
   if (L->o.dtype != NF_BF16) return;
   // A first layer with a handful of input channels (RGB) is far too thin a contraction for useful tensor-core work (K = 27),
@@ -2277,10 +2342,12 @@ void nf_tc_select(nf_layer* L) {
   if (wide_aux(L)) {  // more than 64 filters: the aux conv runs on the kernels of the main conv
     if (aux_ok && plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok) L->fam[2] = 1;
     if (plan_wgrad(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 0).ok && plan_fwd(L->Ha, L->Wa, L->F, L->Cout, L->o.N, 0).ok) L->fam[3] = 1;
+    L->dgrad_tc = L->fam[3] && aux_ok;
     return;
   }
   if (aux_ok && plan_fwd(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 1).ok) L->fam[2] = 1;
   if (plan_wgrad(L->Ha, L->Wa, L->Cout, L->F, L->o.N, 1).ok && plan_fwd(L->Ha, L->Wa, L->F, L->Cout, L->o.N, 2).ok) L->fam[3] = 1;
+  L->dgrad_tc = L->fam[3] && aux_ok;
 }
 
 size_t nf_tc_scratch_floats(const nf_layer* L) {
@@ -2393,7 +2460,7 @@ int nf_tc_wgrad(nf_layer* L, const void* x) {
 // writes dy = BatchNorm-backward(da) directly, so da is never stored and the separate apply pass (read y and da, write dy)
 // disappears: 1.75 activation-sized tensors less memory traffic per layer step for one more read of the narrow dh.
 bool nf_tc_dgrad_two_pass(const nf_layer* L) {
-  return L->fam[3] && !wide_aux(L) && !L->o.maxpool && fold_ok(L->Ha, L->Wa, L->F, L->Cout, 2, 1, 3) &&
+  return L->dgrad_tc && !wide_aux(L) && !L->o.maxpool && fold_ok(L->Ha, L->Wa, L->F, L->Cout, 2, 1, 3) &&
          (size_t)(sm_count() / (L->Cout / 64)) * 8 * 2 * L->Cout <= L->red_floats;
 }
 
@@ -2449,7 +2516,7 @@ int nf_tc_aux_wgrad(nf_layer* L, const void* a) {
 // CUDA-core kernel would, or fit the library's own array: what a caller's scratch was enough for stays accepted.
 static bool standalone_wgrad_ok(int N, int Ho, int Wo, int Cin, int Cout, const WgPlan& pl) {
   const size_t limit = std::max((size_t)nf_k_wgrad_splits(N, Ho, Cin, Cout) * 9 * Cout * Cin, (size_t)NF_STATIC_SCRATCH_BYTES / sizeof(float));
-  return pl.ok && (tiles_exactly(Ho, Wo, pl.BW, pl.BH) || pl.part_floats <= limit);
+  return pl.ok && (pl.exact || pl.part_floats <= limit);
 }
 
 size_t nf_tc_conv3x3_wgrad_scratch_floats(int N, int H, int W, int Cin, int Cout, int stride) {
