@@ -7,8 +7,8 @@
 // A sample's h is read once; its sign bits stay in shared memory until dh is written, the linear weights take h's place there.
 // Loads come in batches whose indexes are clamped instead of guarded, so that no branch separates them, and loops stay rolled:
 // at this size the fetch of unrolled code costs more than it saves.
-// fp32 throughout, every sum in a fixed order: the order of the kernels for large maps and batches (nf_elem.cu), so that a layer
-// computes the same bits whichever of them its size selects.
+// fp32 throughout, every sum in a fixed order: the order of the kernels for other sizes (nf_elem.cu, nf_head_small.cu), so that a
+// layer computes the same bits whichever of them its size selects.
 #include <math.h>
 
 #include <algorithm>
@@ -36,6 +36,8 @@ struct HeadArgs {
   float* bred;          // [N][F] sums of the stored dh over the sample's pixels (with dh)
   int loss_kind, n_scale;
   int groups;           // class ranges of the sums in dp
+  int KS, S, parts;     // SL: classes per slice, slices, ranges their shares are folded in
+  int chunk;            // classes whose weights fit shared memory at a time
   size_t off;           // where the offsets and the sign bits lie in shared memory
 };
 
@@ -112,17 +114,19 @@ __device__ __forceinline__ float tree_sum256(float v, float* sm) {
   return v;
 }
 
+template <int F8> constexpr int kRd = kWarps * 32 * F8 < 1024 ? 1024 : kWarps * 32 * F8;
+
 // F8 = F / 8 in {1, 2, 4, 8}: a warp covers whole pixels, and its lanes with equal lane % F8 hold the same channels.
-// STAGE: the linear weights fit shared memory.
-template <typename T, int F8, bool STAGE>
+// STAGE: the linear weights fit shared memory.  SL: many classes per sample, sums by class slices as in nf_head_small.cu.
+template <typename T, int F8, bool STAGE, bool SL>
 __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   nf_pdl_begin();
   constexpr int F = F8 * 8, D = 4 * F;
   extern __shared__ __align__(16) uint8_t dyn[];
   float* ps = reinterpret_cast<float*>(dyn);  // [D] pooled inputs, then their gradient
   float* ls = ps + D;                         // [K] bias, logits, dlogits
-  float* rd = ls + ((a.K + 3) & ~3);          // [kWarps][D] reductions
-  float* tab = rd + kWarps * D;               // [9][F] dh of a positive h, by row class and column class of its pixel
+  float* rd = ls + ((a.K + 3) & ~3);          // reductions: [kWarps][D] or [4][256]
+  float* tab = rd + kRd<F8>;                  // [9][F] dh of a positive h, by row class and column class of its pixel
   T* hs = reinterpret_cast<T*>(tab + 9 * F);  // the sample's h
   uint32_t* off = reinterpret_cast<uint32_t*>(dyn + a.off);  // byte offset in the image of a bin's k-th pixel
   uint8_t* mask = reinterpret_cast<uint8_t*>(off + (((a.Ha + 1) / 2) * ((a.Wa + 1) / 2) + 3) / 4 * 4);  // bit e of [unit]: h > 0
@@ -207,29 +211,31 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   } else if (!a.part) {
     for (int d = t; d < D; d += kHT) ps[d] = a.p[(size_t)n * D + d];
   } else {
-    // a warp per bin and quarter of the bin's partials; lanes run over the channels
-    const int qh = a.th / 2, qw = a.tw / 2, cnt = qh * qw * 4, b = warp & 3, sub = warp >> 2;
-    constexpr int kSub = kWarps / 4;
-    for (int f = lane; f < F; f += 32) {
-      float v = 0.f;
-      int k = sub;
+    // per bin 256 / F chains over its partials, added in order; eight loads in flight
+    const int qh = a.th / 2, qw = a.tw / 2, cnt = qh * qw * 4;
+    constexpr int kLn = 256 / F;
+    for (int i = t; i < 1024; i += kHT) {
+      const int f = i % F, ln = (i % 256) / F, b = i / 256;
       const float* base = a.part + (((size_t)n * a.th + (b >> 1) * qh) * a.tw + (b & 1) * qw) * 4 * F + f;
-      auto at = [&](int kk) { return base[((size_t)((kk >> 2) / qw) * a.tw + (kk >> 2) % qw) * 4 * F + (size_t)(kk & 3) * F]; };
-      for (; k + 7 * kSub < cnt; k += 8 * kSub) {
+      float v = 0.f;
+#pragma unroll 1
+      for (int k = ln; k < cnt; k += 8 * kLn) {
         float u[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) u[e] = at(k + e * kSub);
+        for (int e = 0; e < 8; ++e) {
+          const int kk = min(k + e * kLn, cnt - 1), tq = kk >> 2;
+          u[e] = base[((size_t)(tq / qw) * a.tw + tq % qw) * 4 * F + (size_t)(kk & 3) * F];
+        }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v += u[e];
+        for (int e = 0; e < 8; ++e) v += k + e * kLn < cnt ? u[e] : 0.f;
       }
-      for (; k < cnt; k += kSub) v += at(k);
-      rd[sub * D + f * 4 + b] = v;
+      rd[i] = v;
     }
     __syncthreads();
     for (int d = t; d < D; d += kHT) {
       float v = 0.f;
-#pragma unroll
-      for (int w = 0; w < kSub; ++w) v += rd[w * D + d];
+#pragma unroll 4
+      for (int l = 0; l < kLn; ++l) v += rd[(d & 3) * 256 + l * F + (d >> 2)];
       v *= 1.f / (float)(r0 * c0);
       ps[d] = v;
       a.p[(size_t)n * D + d] = v;
@@ -237,13 +243,15 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
   __syncthreads();
 
-  // The linear weights are read twice, by rows and by columns: through shared memory, in h's place, where they fit (rows padded
-  // against bank conflicts), else from L2.
+  // The linear weights are read twice, by rows and by columns: by rows through shared memory, in h's place, `chunk` classes at a
+  // time (padded against bank conflicts); by columns from there where all of them fit, else from L2.
   constexpr int kRow = D + 4;
   float* ws = reinterpret_cast<float*>(hs);
-  if constexpr (STAGE) {
-    const float4* src = reinterpret_cast<const float4*>(a.Wf);
-    const int units = a.K * (D / 4);
+#pragma unroll 1
+  for (int kc = 0; kc < a.K; kc += a.chunk) {
+    const int kn = min(a.chunk, a.K - kc), units = kn * (D / 4);
+    const float4* src = reinterpret_cast<const float4*>(a.Wf + (size_t)kc * D);
+    if (kc) __syncthreads();
 #pragma unroll 1
     for (int i0 = t; i0 < units; i0 += 8 * kHT) {
       float4 q[8];
@@ -258,8 +266,8 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
     }
     __syncthreads();
     // logits: a thread per class, inputs in order
-    for (int k = t; k < a.K; k += kHT) {
-      float v = ls[k];  // the bias
+    for (int k = t; k < kn; k += kHT) {
+      float v = ls[kc + k];  // the bias
       const float4* w = reinterpret_cast<const float4*>(ws + (size_t)k * kRow);
       const float4* x = reinterpret_cast<const float4*>(ps);
 #pragma unroll 8
@@ -270,33 +278,7 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
         v = fmaf(wv.z, xv.z, v);
         v = fmaf(wv.w, xv.w, v);
       }
-      ls[k] = v;
-    }
-  } else {
-    // kLpc lanes per class, each with 4 (or 8) of the inputs in registers, kU classes at a time per lane group
-    constexpr int kLpc = F < 32 ? F : 32, kVec = F / kLpc, kGroups = kHT / kLpc, kU = kVec == 1 ? 8 : 4;
-    const int l = t % kLpc, grp = t / kLpc;
-    float4 x[kVec];
-#pragma unroll
-    for (int v = 0; v < kVec; ++v) x[v] = *reinterpret_cast<const float4*>(ps + (l + v * kLpc) * 4);
-#pragma unroll 1
-    for (int kb = 0; kb < a.K; kb += kU * kGroups) {  // the same trips for every thread: whole warps in the shuffles
-      float4 w[kU][kVec];
-#pragma unroll
-      for (int u = 0; u < kU; ++u)
-#pragma unroll
-        for (int v = 0; v < kVec; ++v)
-          w[u][v] = *reinterpret_cast<const float4*>(a.Wf + (size_t)min(kb + grp + u * kGroups, a.K - 1) * D + (l + v * kLpc) * 4);
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        float z = 0.f;
-#pragma unroll
-        for (int v = 0; v < kVec; ++v) z = fmaf(w[u][v].x, x[v].x, fmaf(w[u][v].y, x[v].y, fmaf(w[u][v].z, x[v].z, fmaf(w[u][v].w, x[v].w, z))));
-#pragma unroll
-        for (int o = kLpc / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        const int k = kb + grp + u * kGroups;
-        if (l == 0 && k < a.K) ls[k] += z;
-      }
+      ls[kc + k] = v;
     }
   }
   const float* wrow = STAGE ? ws : a.Wf;
@@ -308,7 +290,62 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
   float* lrow = a.logits + (size_t)n * a.K;
   float* grow = a.dlogits + (size_t)n * a.K;
-  if (a.loss_kind == 1) {  // mean squared error against the one-hot target
+  if constexpr (SL) {
+    // shares of the slices (maximum and sum of exponentials, or the squared error), folded in `parts` ranges, then those in order
+    float* sh = rd;  // [S][2]
+    for (int j = t; j < a.S; j += kHT) {
+      const int k0 = j * a.KS, k1 = min(a.K, k0 + a.KS);
+      float m = 0.f, q = 0.f;
+      if (a.loss_kind == 1) {
+        for (int k = k0; k < k1; ++k) {
+          const float e = ls[k] - (k == lab ? 1.f : 0.f);
+          q = fmaf(e, e, q);
+        }
+      } else {
+        m = -INFINITY;
+        for (int k = k0; k < k1; ++k) m = fmaxf(m, ls[k]);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) q += expf(ls[k] - m);
+      }
+      sh[2 * j] = m;
+      sh[2 * j + 1] = q;
+    }
+    __syncthreads();
+    auto fold = [&](float& m, float& q, float mj, float qj) {
+      if (a.loss_kind == 1) {
+        q += qj;
+      } else {
+        const float mm = fmaxf(m, mj);
+        q = q * expf(m - mm) + qj * expf(mj - mm);
+        m = mm;
+      }
+    };
+    float* fp = sh + 2 * a.S;  // [parts][2]
+    if (t < a.parts) {
+      float m = -INFINITY, q = 0.f;
+      for (int j = t; j < a.S; j += a.parts) fold(m, q, sh[2 * j], sh[2 * j + 1]);
+      fp[2 * t] = m;
+      fp[2 * t + 1] = q;
+    }
+    __syncthreads();
+    if (t == 0) {
+      float m = fp[0], q = fp[1];
+      for (int i = 1; i < a.parts; ++i)
+        if (a.loss_kind == 1 || fp[2 * i] > -INFINITY) fold(m, q, fp[2 * i], fp[2 * i + 1]);
+      const float lse = a.loss_kind == 1 ? q : m + logf(q);
+      fp[0] = lse;
+      a.lossn[n] = a.loss_kind == 1 ? q / (float)a.K : lse - ls[lab];
+    }
+    __syncthreads();
+    const float lse = fp[0], invN = 1.f / (float)a.n_scale, sc = 2.f / ((float)a.n_scale * (float)a.K);
+    for (int k = t; k < a.K; k += kHT) {
+      const float l = ls[k], hit = k == lab ? 1.f : 0.f;
+      const float gr = a.loss_kind == 1 ? (l - hit) * sc : (expf(l - lse) - hit) * invN;
+      lrow[k] = l;
+      grow[k] = gr;
+      ls[k] = gr;
+    }
+  } else if (a.loss_kind == 1) {  // mean squared error against the one-hot target
     float se = 0.f;
     const float sc = 2.f / ((float)a.n_scale * (float)a.K);
     if (t < 256)
@@ -342,10 +379,12 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
   __syncthreads();
 
-  // dp[d] = sum_k dlogits[k] Wf[k][d]: the classes in contiguous ranges, each in order, the range sums added in order
-  const int kG = a.groups;
-  if (t < kG * D) {
-    const int d = t % D, kg = t / D, per = (a.K + kG - 1) / kG, ka = kg * per, kb = min(a.K, ka + per);
+  // dp[d] = sum_k dlogits[k] Wf[k][d]: the classes in contiguous ranges, each in order.  The range sums are added in order, or (SL:
+  // the ranges are the slices) as four interleaved chains, (0 + 1) + (2 + 3).
+  const int kG = SL ? a.S : a.groups, per = SL ? a.KS : (a.K + kG - 1) / kG;
+  float* sums = SL ? ws : rd;  // [kG][D]
+  for (int i = t; i < kG * D; i += kHT) {
+    const int d = i % D, ka = i / D * per, kb = min(a.K, ka + per);
     float s = 0.f;
 #pragma unroll 1
     for (int k = ka; k < kb; k += 16) {
@@ -356,12 +395,21 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
       for (int u = 0; u < 16; ++u)
         if (k + u < kb) s = fmaf(ls[k + u], w[u], s);
     }
-    rd[kg * D + d] = s;
+    sums[i] = s;
   }
   __syncthreads();
   for (int d = t; d < D; d += kHT) {
     float v = 0.f;
-    for (int q = 0; q < kG; ++q) v += rd[q * D + d];
+    if constexpr (SL) {
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+      const int S4 = kG & ~3;
+#pragma unroll 4
+      for (int q = 0; q < S4; ++q) c[q & 3] += sums[q * D + d];
+      for (int q = S4; q < kG; ++q) c[0] += sums[q * D + d];
+      v = (c[0] + c[1]) + (c[2] + c[3]);
+    } else {
+      for (int q = 0; q < kG; ++q) v += sums[q * D + d];
+    }
     a.dp[(size_t)n * D + d] = v;
     ps[d] = v;
   }
@@ -410,10 +458,10 @@ __global__ void __launch_bounds__(kHT) head_sample_kernel(const HeadArgs a) {
   }
 }
 
-// Sums over the batch.  Blocks [0, KT * DT): KC classes from KC (b / DT) on, inputs 64 (b % DT) ..: gWf, and gbf where b % DT == 0;
-// 64 inputs x 4 interleaved chains over the samples, combined as (0 + 1) + (2 + 3).  Then FT blocks of 32 filters: gba from the
-// per-sample sums of dh (fp64); the last block: the mean loss (fp64).
-template <int KC>
+// Sums over the batch.  Blocks [0, KT * DT): gWf of 64 inputs from 64 (b % DT) on, and gbf where b % DT == 0.  SL 0: class b / DT, four
+// interleaved chains over the samples combined as (0 + 1) + (2 + 3); SL 1: four classes from 4 (b / DT) on, one chain each.  Then FT
+// blocks of 32 filters: gba from the per-sample sums of dh (fp64); the last block: the mean loss (fp64).
+template <bool SL>
 __global__ void __launch_bounds__(256) head_batch_kernel(const float* __restrict__ p, const float* __restrict__ dl,
                                                          const float* __restrict__ lossn, const float* __restrict__ bred, int N, int D,
                                                          int K, int KT, int DT, int FT, int F, float* __restrict__ gWf,
@@ -423,51 +471,51 @@ __global__ void __launch_bounds__(256) head_batch_kernel(const float* __restrict
   __shared__ double sd[8][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, b = blockIdx.x;
   if (b < KT * DT) {
-    __shared__ float sf[KC][4][64];
-    const int k0 = (b / DT) * KC, dx = threadIdx.x & 63, ch = threadIdx.x >> 6, d = (b % DT) * 64 + dx;
-    const int N4 = N & ~3;
-    float s[KC];
-#pragma unroll
-    for (int c = 0; c < KC; ++c) s[c] = 0.f;
-    if (d < D) {
-      // chain ch: samples ch, ch + 4, ... below N4; chain 0 goes on with the last one to three
-      const int cnt = N4 / 4, all = cnt + (ch == 0 ? N - N4 : 0);
-      constexpr int kU = KC == 1 ? 16 : 8;
+    float(*sf)[64] = reinterpret_cast<float(*)[64]>(sd);
+    const int dx = threadIdx.x & 63, ch = threadIdx.x >> 6, d = (b % DT) * 64 + dx;
+    const int k = SL ? (b / DT) * 4 + ch : b / DT;
+    float s = 0.f, sb = 0.f;
+    if (d < D && k < K) {
+      // samples ch, ch + 4, ... below N4; chain 0 goes on with the last one to three.  SL: all samples
+      const int N4 = SL ? 0 : N & ~3, cnt = N4 / 4, all = SL ? N : cnt + (ch == 0 ? N - N4 : 0);
 #pragma unroll 1
-      for (int j = 0; j < all; j += kU) {
-        float u[kU][KC], v[kU];
+      for (int j = 0; j < all; j += 16) {
+        float u[16], v[16];
 #pragma unroll
-        for (int e = 0; e < kU; ++e) {
+        for (int e = 0; e < 16; ++e) {
           const int q = min(j + e, all - 1), n = q < cnt ? ch + 4 * q : N4 + q - cnt;
           v[e] = p[(size_t)n * D + d];
-#pragma unroll
-          for (int c = 0; c < KC; ++c) u[e][c] = dl[(size_t)n * K + min(k0 + c, K - 1)];
+          u[e] = dl[(size_t)n * K + k];
         }
 #pragma unroll
-        for (int e = 0; e < kU; ++e)
-#pragma unroll
-          for (int c = 0; c < KC; ++c) s[c] = j + e < all ? fmaf(u[e][c], v[e], s[c]) : s[c];
+        for (int e = 0; e < 16; ++e)
+          if (j + e < all) {
+            s = fmaf(u[e], v[e], s);
+            sb += u[e];
+          }
       }
     }
-#pragma unroll
-    for (int c = 0; c < KC; ++c) sf[c][ch][dx] = s[c];
-    __syncthreads();
-    if (d < D)
-      for (int c = ch; c < KC; c += 4)
-        if (k0 + c < K) gWf[(size_t)(k0 + c) * D + d] = (sf[c][0][dx] + sf[c][1][dx]) + (sf[c][2][dx] + sf[c][3][dx]);
-    if (b % DT == 0 && ty < KC && k0 + ty < K) {
-      float c = 0.f;
+    if constexpr (SL) {
+      if (d < D && k < K) gWf[(size_t)k * D + d] = s;
+      if (b % DT == 0 && dx == 0 && k < K) gbf[k] = sb;
+    } else {
+      sf[ch][dx] = s;
+      __syncthreads();
+      if (ch == 0 && d < D) gWf[(size_t)k * D + d] = (sf[0][dx] + sf[1][dx]) + (sf[2][dx] + sf[3][dx]);
+      if (b % DT == 0 && ty == 7) {
+        float c = 0.f;
 #pragma unroll 1
-      for (int n0 = tx; n0 < N; n0 += 128) {
-        float u[4];
+        for (int n0 = tx; n0 < N; n0 += 128) {
+          float u[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) u[e] = dl[(size_t)min(n0 + 32 * e, N - 1) * K + k0 + ty];
+          for (int e = 0; e < 4; ++e) u[e] = dl[(size_t)min(n0 + 32 * e, N - 1) * K + k];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) c += n0 + 32 * e < N ? u[e] : 0.f;
+          for (int e = 0; e < 4; ++e) c += n0 + 32 * e < N ? u[e] : 0.f;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        if (tx == 0) gbf[k] = c;
       }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-      if (tx == 0) gbf[k0 + ty] = c;
     }
     return;
   }
@@ -519,24 +567,28 @@ size_t h_smem(int dtype, int Ha, int Wa, int F) { return (size_t)Ha * Wa * F * n
 size_t off_smem(int Ha, int Wa, int F) {  // offsets and sign bits
   return (size_t)((((Ha + 1) / 2) * ((Wa + 1) / 2) + 3) / 4 * 4) * 4 + (size_t)Ha * Wa * (F / 8);
 }
-size_t fixed_smem(int F, int K) { return ((size_t)4 * F + ((K + 3) & ~3) + (size_t)kWarps * 4 * F + 9 * F) * 4; }
+size_t fixed_smem(int F, int K) {
+  const int rd = std::max(kWarps * 4 * F, 1024);
+  return ((size_t)4 * F + ((K + 3) & ~3) + rd + 9 * F) * 4;
+}
 
-template <typename T, int F8, bool STAGE>
+template <typename T, int F8, bool STAGE, bool SL>
 int launch_sample(const HeadArgs& a, size_t smem) {
   static bool done[64];  // function attributes belong to a device's context: set once per device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
   if (!done[dev]) {
-    NF_CUDA(cudaFuncSetAttribute(head_sample_kernel<T, F8, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax + 1024));
+    NF_CUDA(cudaFuncSetAttribute(head_sample_kernel<T, F8, STAGE, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax + 1024));
     done[dev] = true;
   }
-  nf_launch(head_sample_kernel<T, F8, STAGE>, a.N, kHT, smem, a);
+  nf_launch(head_sample_kernel<T, F8, STAGE, SL>, a.N, kHT, smem, a);
   NF_LAUNCHED();
   return NF_OK;
 }
 template <typename T, int F8>
 int run_sample(const HeadArgs& a, size_t smem, bool stage) {
-  return stage ? launch_sample<T, F8, true>(a, smem) : launch_sample<T, F8, false>(a, smem);
+  if (a.S) return launch_sample<T, F8, false, true>(a, smem);
+  return stage ? launch_sample<T, F8, true, false>(a, smem) : launch_sample<T, F8, false, false>(a, smem);
 }
 
 }  // namespace
@@ -547,7 +599,12 @@ int nf_head_sample_mode(int dtype, int N, int Ha, int Wa, int F, int K) {
   if ((F != 8 && F != 16 && F != 32 && F != 64) || K > 16384 || Ha < 2 || Wa < 2) return 0;
   if (fixed_smem(F, K) > kSmemMax) return 0;
   const PoolOrder o = pool_order(dtype, N, Ha, Wa, F);
-  const size_t need = fixed_smem(F, K) + h_smem(dtype, Ha, Wa, F) + off_smem(Ha, Wa, F);
+  int KS, S, parts;
+  if (nf_head_slice_order(N, 4 * F, K, &KS, &S, &parts) &&
+      (2 * (S + parts) > std::max(kWarps * 4 * F, 1024) || fixed_smem(F, K) + (size_t)S * 16 * F + off_smem(Ha, Wa, F) > kSmemMax))
+    return 0;
+  if (fixed_smem(F, K) + 16 * (4 * F + 4) * 4 > kSmemMax) return 0;
+  const size_t need = fixed_smem(F, K) + std::max(h_smem(dtype, Ha, Wa, F), (size_t)16 * (4 * F + 4) * 4) + off_smem(Ha, Wa, F);
   return o.slices <= kWarps && need <= kSmemMax ? 2 : 1;
 }
 
@@ -564,15 +621,18 @@ int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, in
   const int D = 4 * F;
   // fixed tables, then h or the weights, then (with h) offsets and sign bits
   const size_t tail = io.h ? off_smem(Ha, Wa, F) : 0;
-  size_t smem = fixed_smem(F, K) + (io.h ? h_smem(dtype, Ha, Wa, F) : 0);
-  const size_t with_w = fixed_smem(F, K) + (size_t)K * (D + 4) * 4;
-  const bool stage = with_w + tail <= kSmemMax;
-  if (stage && with_w > smem) smem = with_w;
+  const size_t fixed = fixed_smem(F, K), row = (size_t)(D + 4) * 4;
+  size_t smem = fixed + (io.h ? h_smem(dtype, Ha, Wa, F) : 0);
+  const bool sliced = nf_head_slice_order(N, D, K, &a.KS, &a.S, &a.parts);
+  if (!sliced) a.S = 0;
+  a.chunk = (int)std::min<size_t>(K, (kSmemMax - fixed - tail) / row);
+  const bool stage = a.chunk == K && !sliced;
+  smem = std::max(smem, fixed + a.chunk * row);
+  if (sliced) smem = std::max(smem, fixed + (size_t)a.S * D * 4);
   smem = (smem + 15) & ~(size_t)15;
   a.off = smem;
   smem += tail;
-  // many classes per sample: as many ranges as there are threads; else the order of the kernel for heads that are not covered here
-  a.groups = (long)K >= 4L * N ? kHT / D : D <= 128 ? 256 / D : 1;
+  a.groups = D <= 128 ? 256 / D : 1;
   int rc;
   if (dtype == NF_F32)
     rc = F == 8 ? run_sample<float, 1>(a, smem, stage) : F == 16 ? run_sample<float, 2>(a, smem, stage)
@@ -582,10 +642,9 @@ int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, in
        : F == 32 ? run_sample<bf16, 4>(a, smem, stage) : run_sample<bf16, 8>(a, smem, stage);
   if (rc != NF_OK) return rc;
   const int DT = (D + 63) / 64, FT = io.dh ? (F + 31) / 32 : 0;
-  // four classes per block read the samples' inputs once between them; with few classes that would leave too few blocks
-  const int KC = K >= 512 ? 4 : 1, KT = (K + KC - 1) / KC;
-  nf_launch(KC == 4 ? head_batch_kernel<4> : head_batch_kernel<1>, (unsigned)(KT * DT + FT + 1), 256, 0, io.p, io.dlogits, io.lossn, io.bred, N, D, K,
-            KT, DT, FT, F, io.gWf, io.gbf, io.gba, io.loss_out, io.status, n_scale);
+  const int KT = sliced ? (K + 3) / 4 : K;
+  nf_launch(sliced ? head_batch_kernel<true> : head_batch_kernel<false>, (unsigned)(KT * DT + FT + 1), 256, 0, io.p, io.dlogits, io.lossn, io.bred, N, D,
+            K, KT, DT, FT, F, io.gWf, io.gbf, io.gba, io.loss_out, io.status, n_scale);
   NF_LAUNCHED();
   return NF_OK;
 }

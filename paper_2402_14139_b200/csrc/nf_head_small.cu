@@ -264,6 +264,15 @@ int allow_smem() {
 
 }  // namespace
 
+bool nf_head_slice_order(int N, int D, int K, int* KS, int* S, int* parts) {
+  const HsPlan pl = hs_plan(N, D, K);
+  if (!pl.ok) return false;
+  *KS = pl.KS;
+  *S = pl.S;
+  *parts = kHsThreads / pl.NC;
+  return true;
+}
+
 size_t nf_head_small_scratch_floats(int N, int D, int K) {
   const HsPlan pl = hs_plan(N, D, K);
   return pl.ok ? pl.scratch_floats : 0;

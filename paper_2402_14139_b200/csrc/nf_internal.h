@@ -179,6 +179,8 @@ int nf_head_sample_mode(int dtype, int N, int Ha, int Wa, int F, int K);
 int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, int F, int K, int loss_kind, int n_scale);
 // small-batch head (nf_head_small.cu): class-sliced forward + backward of the linear layer and the loss; 0 floats = not covered
 size_t nf_head_small_scratch_floats(int N, int D, int K);
+// whether that head takes the sizes, and its summation order: classes per slice, slices, ranges the slices' shares are folded in
+bool nf_head_slice_order(int N, int D, int K, int* KS, int* S, int* parts);
 int nf_head_small_step(const float* p, const int32_t* labels, int N, int D, int K, const float* Wf, const float* bf, float* logits,
                        float* dp, float* lossn, int32_t* status, int loss_kind, float* gWf, float* gbf, float* loss_out,
                        float* scratch, size_t scratch_floats, int n_scale);
