@@ -1084,6 +1084,9 @@ __global__ void __launch_bounds__(256) channel_sums_vec_kernel(const T* __restri
 
 // dh = 1[h>0] * dp[n][f*4+bin]/|bin| for even sizes (every pixel lies in exactly one bin), 8 filters per
 // thread, fused with the per-filter sum of dh (the aux bias gradient): red[(block*2+0)*F + f].
+// CACHE: the image's 8 x 4 gradients of a thread's channels stay in registers (from 128 filters on: few pixels per block and step,
+// where eight strided loads a pixel cost more than the 32 registers; 6366 maps of 8 x 8 x 256: 198 -> 130 us).
+template <bool CACHE>
 __global__ void __launch_bounds__(256) dh_vec_kernel(const uint4* __restrict__ h, const float* __restrict__ dp, int Ha, int Wa,
                                                      int F8, size_t P, uint4* __restrict__ dh, float* __restrict__ red) {
   nf_pdl_begin();
@@ -1095,6 +1098,8 @@ __global__ void __launch_bounds__(256) dh_vec_kernel(const uint4* __restrict__ h
 #pragma unroll
   for (int i = 0; i < 8; ++i) a[i] = 0.f;
   const size_t p0 = P * blockIdx.x / gridDim.x, p1 = P * (blockIdx.x + 1) / gridDim.x;
+  float4 dv[CACHE ? 8 : 1];
+  size_t cur = ~(size_t)0;
   auto one = [&](size_t p, const uint4 hq) {
     int i, j;
     size_t n;
@@ -1111,10 +1116,22 @@ __global__ void __launch_bounds__(256) dh_vec_kernel(const uint4* __restrict__ h
     const int bin = (i >= Ha / 2 ? 2 : 0) + (j >= Wa / 2 ? 1 : 0);
     float hv[8], o[8];
     unpack8(hq, hv);
-    const float* d = dp + n * 4 * F + (size_t)(g * 8) * 4 + bin;
+    if constexpr (CACHE) {
+      if (n != cur) {
+        cur = n;
+        const float4* d = reinterpret_cast<const float4*>(dp + n * 4 * F) + g * 8;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      o[e] = hv[e] > 0.f ? d[e * 4] * inv_bin : 0.f;
+        for (int e = 0; e < 8; ++e) dv[e] = __ldg(d + e);
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float top = bin & 1 ? dv[e].y : dv[e].x, bot = bin & 1 ? dv[e].w : dv[e].z;
+        o[e] = hv[e] > 0.f ? (bin & 2 ? bot : top) * inv_bin : 0.f;
+      }
+    } else {
+      const float* d = dp + n * 4 * F + (size_t)(g * 8) * 4 + bin;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[e] = hv[e] > 0.f ? d[e * 4] * inv_bin : 0.f;
     }
     const uint4 packed = pack8(o);
     dh[p * F8 + g] = packed;
@@ -1142,6 +1159,45 @@ __global__ void __launch_bounds__(256) dh_vec_kernel(const uint4* __restrict__ h
     red[((size_t)blockIdx.x * 2 + 0) * F + t] = s;
     red[((size_t)blockIdx.x * 2 + 1) * F + t] = 0.f;
   }
+}
+
+// avgpool_small for bf16, eight channels and all four bins per thread: 16-byte loads and stores, the same sums.  (One 2-byte load at
+// a time took 185 us on 6366 maps of 8 x 8 x 256, 208 MB.)
+__global__ void __launch_bounds__(256) avgpool_small_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, size_t total,
+                                                                float4* __restrict__ p) {
+  nf_pdl_begin();
+  const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (e >= total) return;
+  const size_t n = e / F8;
+  const uint4* hn = h + n * Ha * Wa * F8 + e % F8;
+  float o[4][8];
+#pragma unroll
+  for (int bin = 0; bin < 4; ++bin) {
+    int i0, i1, j0, j1;
+    bin_range(bin / 2, Ha, i0, i1);
+    bin_range(bin % 2, Wa, j0, j1);
+    float a[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) a[c] = 0.f;
+    for (int i = i0; i < i1; ++i) {
+      for (int j = j0; j < j1; j += 4) {
+        uint4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = __ldg(hn + (size_t)(i * Wa + min(j + u, j1 - 1)) * F8);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float v[8];
+          unpack8(q[u], v);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) a[c] = j + u < j1 ? a[c] + v[c] : a[c];
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) o[bin][c] = a[c] / (float)((i1 - i0) * (j1 - j0));
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) p[e * 8 + c] = make_float4(o[0][c], o[1][c], o[2][c], o[3][c]);
 }
 
 // average pool, stage 1: partial bin sums over a slice of rows; part[(n*4+bin)*S + s][F]
@@ -1351,25 +1407,28 @@ __global__ void __launch_bounds__(256) bn_apply_pool_vec_kernel(const uint4* __r
   }
 }
 
-// dz of the four window positions: the first maximum (scan order) of the bf16-rounded ReLU outputs takes da
-// if its pre-activation is positive.  arg[i] = winning position of channel i, or -1.
-__device__ __forceinline__ void pool_winner(const float (&yv)[4][8], const float (&A)[8], const float (&B)[8], int (&arg)[8]) {
+// Which of the four window positions of a channel pair (packed bf16 y in w[0..3]) receives the gradient: all-ones halves in keep[d]
+// where position d is the first maximum, in scan order, of the bf16-rounded ReLU outputs and that maximum is positive.  Two channels
+// per instruction from the conversion on: with one channel at a time the two kernels below were bound by these instructions.
+__device__ __forceinline__ void pool_winner2(const uint32_t (&w)[4], float A0, float A1, float B0, float B1, uint32_t (&keep)[4]) {
+  __nv_bfloat162 r[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float best = -1.f;
-    int a = 0;
-    float zbest = 0.f;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      const float z = fmaf(yv[d][i], A[i], B[i]);
-      const float r = __bfloat162float(__float2bfloat16_rn(fmaxf(z, 0.f)));
-      if (r > best) { best = r; a = d; zbest = z; }
-    }
-    arg[i] = zbest > 0.f ? a : -1;
+  for (int d = 0; d < 4; ++d) {
+    const float z0 = fmaf(__uint_as_float(w[d] << 16), A0, B0), z1 = fmaf(__uint_as_float(w[d] & 0xffff0000u), A1, B1);
+    uint32_t u;
+    asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(u) : "f"(z1), "f"(z0));
+    r[d] = *reinterpret_cast<const __nv_bfloat162*>(&u);
   }
+  const __nv_bfloat162 m = __hmax2(__hmax2(r[0], r[1]), __hmax2(r[2], r[3]));
+  const uint32_t pos = __hgt2_mask(m, __floats2bfloat162_rn(0.f, 0.f));
+  const uint32_t e0 = __heq2_mask(r[0], m), e1 = __heq2_mask(r[1], m), e2 = __heq2_mask(r[2], m);
+  keep[0] = pos & e0;
+  keep[1] = pos & e1 & ~e0;
+  keep[2] = pos & e2 & ~(e0 | e1);
+  keep[3] = pos & ~(e0 | e1 | e2);
 }
 
-__global__ void __launch_bounds__(256) bn_bwd_reduce_pool_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da,
+__global__ void __launch_bounds__(256, 2) bn_bwd_reduce_pool_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da,
                                                                      size_t Pq, int Ho, int Wo, int C8,
                                                                      const float* __restrict__ scale, const float* __restrict__ shift,
                                                                      const float* __restrict__ mu, const float* __restrict__ invstd,
@@ -1386,22 +1445,34 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_pool_vec_kernel(const uint4
     a[i] = 0.f; b[i] = 0.f;
   }
   const size_t q0 = Pq * blockIdx.x / gridDim.x, q1 = Pq * (blockIdx.x + 1) / gridDim.x;
-  for (size_t q = q0 + pl; q < q1; q += planes) {
+  // the next window's five loads fly while this one is worked on (one window at a time: 547 us for 1.25 GB)
+  uint4 nx[5];
+  auto fetch = [&](size_t q) {
     const size_t bb = win_base(q, Ho, Wo, C8) + g;
-    const uint4 v4[4] = {__ldg(y + bb), __ldg(y + bb + C8), __ldg(y + bb + (size_t)Wo * C8), __ldg(y + bb + (size_t)Wo * C8 + C8)};
-    float yv[4][8], dv[8];
+    nx[0] = __ldg(y + bb);
+    nx[1] = __ldg(y + bb + C8);
+    nx[2] = __ldg(y + bb + (size_t)Wo * C8);
+    nx[3] = __ldg(y + bb + (size_t)Wo * C8 + C8);
+    nx[4] = __ldg(da + q * C8 + g);
+  };
+  if (q0 + pl < q1) fetch(q0 + pl);
+  for (size_t q = q0 + pl; q < q1; q += planes) {
+    const uint4 v4[5] = {nx[0], nx[1], nx[2], nx[3], nx[4]};
+    if (q + planes < q1) fetch(q + planes);
+    const uint32_t* yw = reinterpret_cast<const uint32_t*>(v4);  // [window position][channel pair]
 #pragma unroll
-    for (int d = 0; d < 4; ++d) unpack8(v4[d], yv[d]);
-    unpack8(__ldg(da + q * C8 + g), dv);
-    int arg[8];
-    pool_winner(yv, A, B, arg);
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (arg[i] >= 0) {
-        const float yy = arg[i] == 0 ? yv[0][i] : arg[i] == 1 ? yv[1][i] : arg[i] == 2 ? yv[2][i] : yv[3][i];
-        a[i] += dv[i];
-        b[i] = fmaf(dv[i], (yy - m[i]) * is[i], b[i]);
-      }
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t w[4] = {yw[i], yw[4 + i], yw[8 + i], yw[12 + i]};
+      uint32_t k[4];
+      pool_winner2(w, A[2 * i], A[2 * i + 1], B[2 * i], B[2 * i + 1], k);
+      const uint32_t dd = yw[16 + i] & (k[0] | k[1] | k[2] | k[3]);
+      const uint32_t yy = (w[0] & k[0]) | (w[1] & k[1]) | (w[2] & k[2]) | (w[3] & k[3]);
+      const float d0 = __uint_as_float(dd << 16), d1 = __uint_as_float(dd & 0xffff0000u);
+      a[2 * i] += d0;
+      a[2 * i + 1] += d1;
+      b[2 * i] = fmaf(d0, (__uint_as_float(yy << 16) - m[2 * i]) * is[2 * i], b[2 * i]);
+      b[2 * i + 1] = fmaf(d1, (__uint_as_float(yy & 0xffff0000u) - m[2 * i + 1]) * is[2 * i + 1], b[2 * i + 1]);
+    }
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -1417,7 +1488,7 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_pool_vec_kernel(const uint4
   }
 }
 
-__global__ void __launch_bounds__(256) bn_bwd_apply_pool_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da, int Ho,
+__global__ void __launch_bounds__(256, 2) bn_bwd_apply_pool_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da, int Ho,
                                                                     int Wo, int C8, const float* __restrict__ scale,
                                                                     const float* __restrict__ shift, const float* __restrict__ mu,
                                                                     const float* __restrict__ invstd, const float* __restrict__ sdz,
@@ -1433,22 +1504,38 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_pool_vec_kernel(const uint4*
     K1[i] = -s * m2 * is;
     K0[i] = s * (m2 * is * mu[c0 + i] - m1);
   }
-  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < total8; e += (size_t)gridDim.x * 256) {  // e over pooled vectors
-    const size_t bb = win_base(div_small(e, C8), Ho, Wo, C8) + threadIdx.x % C8;
-    const size_t off[4] = {0, (size_t)C8, (size_t)Wo * C8, (size_t)Wo * C8 + C8};
-    float yv[4][8], dv[8];
+  const size_t off[4] = {0, (size_t)C8, (size_t)Wo * C8, (size_t)Wo * C8 + C8}, step = (size_t)gridDim.x * 256;
+  size_t e = (size_t)blockIdx.x * 256 + threadIdx.x, nb = 0;
+  uint4 nx[5];
+  auto fetch = [&](size_t i) {  // as in the reduction
+    nb = win_base(div_small(i, C8), Ho, Wo, C8) + threadIdx.x % C8;
 #pragma unroll
-    for (int d = 0; d < 4; ++d) unpack8(__ldg(y + bb + off[d]), yv[d]);
-    unpack8(__ldg(da + e), dv);
-    int arg[8];
-    pool_winner(yv, A, B, arg);
+    for (int d = 0; d < 4; ++d) nx[d] = __ldg(y + nb + off[d]);
+    nx[4] = __ldg(da + i);
+  };
+  if (e < total8) fetch(e);
+  for (; e < total8; e += step) {  // e over pooled vectors
+    const size_t bb = nb;
+    const uint4 v4[5] = {nx[0], nx[1], nx[2], nx[3], nx[4]};
+    if (e + step < total8) fetch(e + step);
+    const uint32_t* yw = reinterpret_cast<const uint32_t*>(v4);
+    uint32_t ow[4][4];
 #pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      float o[8];
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t w[4] = {yw[i], yw[4 + i], yw[8 + i], yw[12 + i]};
+      uint32_t k[4];
+      pool_winner2(w, A[2 * i], A[2 * i + 1], B[2 * i], B[2 * i + 1], k);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) o[i] = fmaf(A[i], arg[i] == d ? dv[i] : 0.f, fmaf(K1[i], yv[d][i], K0[i]));
-      dy[bb + off[d]] = pack8(o);
+      for (int d = 0; d < 4; ++d) {
+        const uint32_t dd = yw[16 + i] & k[d];
+        const float o0 = fmaf(A[2 * i], __uint_as_float(dd << 16), fmaf(K1[2 * i], __uint_as_float(w[d] << 16), K0[2 * i]));
+        const float o1 = fmaf(A[2 * i + 1], __uint_as_float(dd & 0xffff0000u), fmaf(K1[2 * i + 1], __uint_as_float(w[d] & 0xffff0000u), K0[2 * i + 1]));
+        const __nv_bfloat162 q = __floats2bfloat162_rn(o0, o1);
+        ow[d][i] = *reinterpret_cast<const uint32_t*>(&q);
+      }
     }
+#pragma unroll
+    for (int d = 0; d < 4; ++d) dy[bb + off[d]] = make_uint4(ow[d][0], ow[d][1], ow[d][2], ow[d][3]);
   }
 }
 
@@ -1617,7 +1704,7 @@ int nf_k_dh_fast(const void* h, const float* dp, int N, int Ha, int Wa, int F, v
   const size_t P = (size_t)N * Ha * Wa;
   const int nb = nf_k_channel_blocks(P, F);
   if ((size_t)nb * 2 * F > red_floats) return NF_EUNSUPPORTED;
-  nf_launch(dh_vec_kernel, nb, 256, 0, (const uint4*)h, dp, Ha, Wa, F / 8, P, (uint4*)dh, red);
+  nf_launch(F >= 128 ? dh_vec_kernel<true> : dh_vec_kernel<false>, nb, 256, 0, (const uint4*)h, dp, Ha, Wa, F / 8, P, (uint4*)dh, red);
   NF_LAUNCHED();
   *nblocks = nb;
   return NF_OK;
@@ -1625,6 +1712,12 @@ int nf_k_dh_fast(const void* h, const float* dp, int N, int Ha, int Wa, int F, v
 
 int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* p) {
   if ((long)((Ha + 1) / 2) * ((Wa + 1) / 2) <= 16) {  // tiny maps (late blocks train at thousands of samples): a thread per output
+    if (dtype == NF_BF16 && F % 8 == 0) {
+      const size_t groups = (size_t)N * (F / 8);
+      nf_launch(avgpool_small_vec_kernel, nblk(groups, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, groups, (float4*)p);
+      NF_LAUNCHED();
+      return NF_OK;
+    }
     const size_t total = (size_t)N * 4 * F;
     DISPATCH(dtype, (nf_launch(avgpool_small_kernel<float>, nblk(total, 256), 256, 0, (const float*)h, Ha, Wa, F, total, p)),
              (nf_launch(avgpool_small_kernel<bf16>, nblk(total, 256), 256, 0, (const bf16*)h, Ha, Wa, F, total, p)));
