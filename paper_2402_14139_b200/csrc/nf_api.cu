@@ -89,8 +89,10 @@ size_t plan(nf_layer* L, char* base, bool assign) {
   D->grad = (float*)c.take(L->arena * 4);
   D->shadow = (bf16*)c.take(L->arena * 2);
   D->wa_t = (bf16*)c.take(F > 64 ? (size_t)9 * Co * F * 2 : 0);
-  D->wpad = (bf16*)c.take(L->cin_pad ? (size_t)9 * Co * L->cin_pad * 2 : 0);
-  D->gwpad = (float*)c.take(L->cin_pad ? (size_t)9 * Co * L->cin_pad * 4 : 0);
+  // the padded copies are sized for 64 channels whichever padding is used: a layer's memory need, from which the blocks are
+  // planned, does not depend on it
+  D->wpad = (bf16*)c.take(L->cin_pad ? (size_t)9 * Co * 64 * 2 : 0);
+  D->gwpad = (float*)c.take(L->cin_pad ? (size_t)9 * Co * 64 * 4 : 0);
   D->rmean = (float*)c.take(Co * 4);
   D->rvar = (float*)c.take(Co * 4);
   D->scale = (float*)c.take(Co * 4);
@@ -106,7 +108,7 @@ size_t plan(nf_layer* L, char* base, bool assign) {
   D->dh = c.take(nh * es);
   D->da = c.take(na * es);
   D->act = c.take(na * es);
-  D->xpad = c.take(L->cin_pad ? N * L->H * L->W * L->cin_pad * es : 0);
+  D->xpad = c.take(L->cin_pad ? N * L->H * L->W * 64 * es : 0);
   D->p = (float*)c.take(N * 4 * F * 4);
   D->dp = (float*)c.take(N * 4 * F * 4);
   D->parg = (int32_t*)c.take(N * 4 * F * 4);
@@ -632,14 +634,16 @@ int nf_block_cache_n(nf_block* B, const void* x, void* out, int count) {
 static int layer_eval_forward(nf_layer* L, const void* in, int count, void* dst) {
   const int dt = L->o.dtype;
   const void* Wm = dt == NF_F32 ? (const void*)(L->val + L->off[NF_P_W]) : (const void*)(L->shadow + L->off[NF_P_W]);
+  NF_TRY(nf_k_bn_eval_coeffs(L->Cout, L->val + L->off[NF_P_GAMMA], L->val + L->off[NF_P_BETA], L->o.bn_eps, L->rmean, L->rvar,
+                               L->scale, L->shift));
   if (L->fam[0]) {
-    NF_TRY(nf_tc_conv_fwd_eval(L, in, count));
+    const bool fused = !L->o.maxpool && !L->skip;  // the convolution normalises in its epilogue: y is neither written nor read
+    NF_TRY(nf_tc_conv_fwd_eval(L, in, count, fused ? dst : nullptr));
+    if (fused) return NF_OK;
   } else {
     NF_TRY(nf_k_conv(dt, in, count, L->H, L->W, L->Cin, Wm, (long)L->Cout * L->Cin, L->Cin, 1, 0, nullptr, 0, L->o.stride,
                        L->Cout, L->y));
   }
-  NF_TRY(nf_k_bn_eval_coeffs(L->Cout, L->val + L->off[NF_P_GAMMA], L->val + L->off[NF_P_BETA], L->o.bn_eps, L->rmean, L->rvar,
-                               L->scale, L->shift));
   return nf_k_bn_apply(dt, L->y, count, L->Ho, L->Wo, L->Cout, L->o.maxpool, L->scale, L->shift, dst, L->skip);
 }
 

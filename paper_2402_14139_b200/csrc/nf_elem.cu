@@ -714,6 +714,14 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
   }
 }
 
+__global__ void unpad_grad_mirrored_kernel(const float* __restrict__ gwpad, int Co, int C, int Cp, float* __restrict__ gw) {
+  nf_pdl_begin();
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 9 * Co * C) return;
+  const int c = e % C, co = (e / C) % Co, tap = e / (C * Co);
+  gw[e] = gwpad[((size_t)(8 - tap) * Cp + c) * Co + co];
+}
+
 // Momentum SGD over up to kSgdMaxArenas parameter arenas in one launch (all layers of a block).  An arena is a multiple
 // of 64 floats and 256-byte aligned, so every thread owns four consecutive elements: 16-byte loads of value, momentum and
 // gradient, 16-byte stores of value and momentum, one 8-byte store of the four bf16 copies.  Blocks are dealt to arenas
@@ -1918,6 +1926,11 @@ int nf_k_pad_channels(const void* x, size_t P, int C, int Cp, void* xpad) {
 }
 int nf_k_pad_weights(const bf16* w, size_t rows, int C, int Cp, bf16* wpad) {
   nf_launch(pad_weights_kernel, nblk(rows * Cp, 256), 256, 0, w, rows, C, Cp, wpad);
+  NF_LAUNCHED();
+  return NF_OK;
+}
+int nf_k_unpad_grad_mirrored(const float* gwpad, int Co, int C, int Cp, float* gw) {
+  nf_launch(unpad_grad_mirrored_kernel, nblk((size_t)9 * Co * C, 256), 256, 0, gwpad, Co, C, Cp, gw);
   NF_LAUNCHED();
   return NF_OK;
 }

@@ -65,8 +65,8 @@ struct nf_layer {
   // kernel families chosen at configure time: 0 = cuda-core, 1 = tcgen05
   int fam[4];
   int dgrad_tc;                        // aux input gradient on tcgen05 (fam[3] says so of the aux weight gradient)
-  // First layers (a few input channels, e.g. RGB): cin_pad = 64 makes the main conv run on the tensor-core kernels over a
-  // copy of the input batch whose pixels are zero-padded to 64 channels; 0 = the input is used as it is.
+  // First layers (a few input channels, e.g. RGB): cin_pad = 16 or 64 makes the main conv run on the tensor-core kernels over a
+  // copy of the input batch whose pixels are zero-padded to that many channels; 0 = the input is used as it is.
   int cin_pad;
   void* xpad;                          // [N][H][W][cin_pad] (bf16)
   bf16* wpad;                          // [9][Cout][cin_pad] operand copy of W, zero beyond Cin
@@ -212,6 +212,8 @@ int nf_k_write_dz(int dtype, const void* y, const void* da, int N, int Ho, int W
 int nf_k_pad_channels(const void* x, size_t P, int C, int Cp, void* xpad);
 int nf_k_pad_weights(const bf16* w, size_t rows, int C, int Cp, bf16* wpad);
 int nf_k_unpad_grad(const float* gwpad, size_t rows, int C, int Cp, float* gw);
+// the same from [8 - tap][Cp][Co]
+int nf_k_unpad_grad_mirrored(const float* gwpad, int Co, int C, int Cp, float* gw);
 int nf_k_sgd(float* val, float* mom, const float* grad, bf16* shadow, size_t n, float lr, float momentum);
 // the same update over several arenas (the layers of a block) in one launch; first_block is filled by the callee
 enum { kSgdMaxArenas = 48 };

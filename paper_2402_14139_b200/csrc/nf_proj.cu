@@ -182,9 +182,8 @@ size_t proj_plan(nf_proj* P, char* base) {
   const int tiles = ((P->Cin + 63) / 64) * ((P->Cout + 63) / 64);
   long sp = 296 / tiles;  // two blocks per SM
   if (sp < 1) sp = 1;
-  if ((size_t)sp > (pix + 31) / 32) sp = (long)((pix + 31) / 32);
-  P->splits = (int)sp;
-  P->wpart = (float*)take((size_t)sp * P->Cin * P->Cout * 4);
+  P->wpart = (float*)take((size_t)sp * P->Cin * P->Cout * 4);  // for the full count: the need then grows by stored tensors alone
+  P->splits = (int)((size_t)sp > (pix + 31) / 32 ? (pix + 31) / 32 : (size_t)sp);
   (void)state_end;
   return nf_align_up(off, 256);
 }

@@ -103,6 +103,14 @@ struct TcPlan {
   size_t smem;
 };
 
+// With stats == 0 and bn_scale set, the forward writes ReLU(y * scale + shift) of the bf16-rounded y instead of y: BatchNorm with
+// running statistics, whose coefficients are known beforehand (cache fill, exits).  Two channels, packed:
+__device__ __forceinline__ uint32_t bn_relu2(uint32_t y, float2 sc, float2 sh) {
+  const __nv_bfloat162 b = __floats2bfloat162_rn(fmaxf(fmaf(__uint_as_float(y << 16), sc.x, sh.x), 0.f),
+                                                 fmaxf(fmaf(__uint_as_float(y & 0xffff0000u), sc.y, sh.y), 0.f));
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
+
 // Sum of the next `n` segment accumulators (of four taken in turn; `taken` counts them) for one thread's row of BN columns.
 template <int BN>
 __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& taken, uint64_t* tfull, uint64_t* tempty,
@@ -323,6 +331,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     const int sc = et % BN, shalf = et / BN;        // stats: channel and row half of this thread
     const int rw = r % p.BW, rh = (r / p.BW) % p.BH;  // place of the thread's pixel in its tile
     uint32_t sg = 0;                                  // SEG: segments taken so far
+    const bool post = !p.stats && p.bn_scale;
     float ssum = 0.f, ssq = 0.f;
     float ssum2 = 0.f, ssq2 = 0.f;                  // BN = 256: the thread's second channel, sc + 128
     uint32_t tl = 0;
@@ -380,6 +389,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             }
             const __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
             w[e] = *reinterpret_cast<const uint32_t*>(&b2);
+          }
+          if (post) {
+            const float* ps = p.bn_scale + nt * BN + j * 32 + q * 8;
+            const float* ph = p.bn_shift + nt * BN + j * 32 + q * 8;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              w[e] = bn_relu2(w[e], __ldg(reinterpret_cast<const float2*>(ps) + e), __ldg(reinterpret_cast<const float2*>(ph) + e));
           }
           *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (r & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
         }
@@ -643,7 +659,7 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   constexpr int kTW = UF == 2 ? 8 : UF ? 16 : 14;  // output columns of a tile
   constexpr int kTH = UF == 2 ? 16 : 8;            // output rows of a tile
   constexpr int kStatIters = UF ? 8 : 7;           // 16-row slices of the staged tile (128 or 112 pixels)
-  constexpr int kWTile = MIR ? 3 * KC * 128 : 3 * G * 128;  // one kernel row: [kw*G + co][64 ci], or mirrored [kw][f][64 c]
+  constexpr int kWTile = MIR ? 3 * KC * 128 : 3 * G * kARow;  // one kernel row: [kw*G + co][64 ci], or mirrored [kw][f][64 c]
   const int w_bytes = 3 * p.kchunks * kWTile; // [chunk][kh][kw*G + co][64 ci]
   uint8_t* wres = smem + (size_t)p.stages * kABytes;
   uint8_t* stg = wres + w_bytes;              // EPI 0: 112 (UF: 128) output pixels x 128 bytes
@@ -743,7 +759,7 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   } else if (warp == 1) {
     constexpr uint32_t idesc = ptx::idesc_bf16(128, UF ? G : 3 * G, 0, MIR);
     const uint64_t a_hi = ptx::sdesc(0, 16, (UF == 2 ? 10 : 8) * kARow, kALayout);  // UF 2: next 8-pixel group = next box row
-    const uint64_t b_hi = MIR ? ptx::sdesc(0, KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
+    const uint64_t b_hi = MIR ? ptx::sdesc(0, KC * 128, 1024, 2) : ptx::sdesc(0, 16, 8 * kARow, kALayout);
     const uint32_t w16 = ptx::smem_u32(wres) >> 4;
     if (ptx::elect_one()) {
       Ring rg;
@@ -951,6 +967,12 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         }
         }
         if constexpr (EPI == 0) {
+          if (!p.stats && p.bn_scale) {
+            const float2* ps = reinterpret_cast<const float2*>(p.bn_scale + nt * 64 + q * 16);
+            const float2* ph = reinterpret_cast<const float2*>(p.bn_shift + nt * 64 + q * 16);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) w[e] = bn_relu2(w[e], __ldg(ps + e), __ldg(ph + e));
+          }
           if (valid) {
             uint8_t* dst = stg_g + orow * 128;
             *reinterpret_cast<uint4*>(dst + (((2 * q) ^ (orow & 7)) * 16)) = vcol ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
@@ -1978,6 +2000,7 @@ bool fold_ok(int H, int W, int Cin, int Cout, int epi, int stride, int stats = 0
   // filters at 32 columns the folded form measured slower there (0.33 vs 0.25 ms), the fused form faster everywhere
   if (epi == 1 && W % 14 != 0 && extra_smem == 0) return false;
   if (epi == 2) return Cin <= 32 && Cin % 8 == 0 && Cout % 64 == 0;
+  if (Cin == 16 && epi == 0) return Cout == 64;  // first layers, padded to 16 channels
   if (Cin % 64) return false;
   if (epi == 0 ? (Cin != 64 || Cout != 64) : (Cout > 64 || Cout % 8)) return false;
   const size_t wbytes = (size_t)9 * (Cin / 64) * fold_group(Cout, epi) * 128;
@@ -2018,7 +2041,7 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
              size_t red_floats, int32_t* status, int* nb, int epi, const float* bias, const BnBwdIn* bn = nullptr,
              const XfIn* xf = nullptr) {
   const int G = fold_group(Cout, epi);
-  const int KC = epi == 2 ? (Cin <= 16 ? 16 : 32) : 64;
+  const int KC = epi == 2 ? (Cin <= 16 ? 16 : 32) : Cin < 64 ? 16 : 64;
   // input gradient on widths that also tile by 16: the unfolded form (three shifted boxes, no shift-add in the epilogue);
   // where the map tiles by 8 x 16 as well: its single-box form
   const bool uf = epi == 2 && W % 16 == 0;
@@ -2032,7 +2055,7 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
   // forward: weights [kh][kw][Cout][Cin], box = G rows of co x 64 ci for the three kw of one kh;
   // input gradient: weights [kh][kw][F][Cout], box = KC rows of f x 64 c for the three kw of one kh
   const uint64_t dw[4] = {(uint64_t)(epi == 2 ? Cout : Cin), (uint64_t)(epi == 2 ? Cin : Cout), 3, 3};
-  const uint32_t bw[4] = {64, (uint32_t)(epi == 2 ? KC : G), 3, 1};
+  const uint32_t bw[4] = {(uint32_t)(epi == 2 ? 64 : KC), (uint32_t)(epi == 2 ? KC : G), 3, 1};
   const uint64_t dy[4] = {(uint64_t)Cout, (uint64_t)W, (uint64_t)H, (uint64_t)N};
   const uint32_t by[4] = {64, (uint32_t)TW, (uint32_t)TH, 1};
   int rc;
@@ -2057,14 +2080,14 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
     p.bn_scale = bn->scale; p.bn_shift = bn->shift; p.bn_mu = bn->mu; p.bn_invstd = bn->invstd;
     p.bn_sdz = bn->sdz; p.bn_sdzx = bn->sdzx; p.inv_m = bn->inv_m;
   }
-  p.N = N; p.H = H; p.W = W; p.Cout = Cout; p.kchunks = epi == 2 ? 1 : Cin / 64; p.n_tiles = epi == 2 ? Cout / 64 : 1;
+  p.N = N; p.H = H; p.W = W; p.Cout = Cout; p.kchunks = epi == 2 || Cin < 64 ? 1 : Cin / 64; p.n_tiles = epi == 2 ? Cout / 64 : 1;
   p.tiles_w = (W + TW - 1) / TW; p.tiles_h = (H + TH - 1) / TH; p.total_tiles = N * p.tiles_w * p.tiles_h * p.n_tiles;
   if ((long long)N * p.tiles_w * p.tiles_h * p.n_tiles > (1ll << 30)) return NF_EUNSUPPORTED;
   p.stats = stats; p.red = red; p.status = status; p.bias = bias; p.out = (bf16*)y;
   p.tg = tile_grid(p.n_tiles, p.tiles_w, p.tiles_h);
   const size_t a_bytes = wide ? ((size_t)34 * 10 * KC * 2 + 1023) / 1024 * 1024
                          : uf2 ? ((size_t)18 * 10 * KC * 2 + 1023) / 1024 * 1024 : (size_t)(uf ? 3 : 1) * 10 * 16 * KC * 2;
-  const size_t wbytes = epi == 2 ? (size_t)9 * KC * 128 : (size_t)9 * p.kchunks * G * 128;
+  const size_t wbytes = epi == 2 ? (size_t)9 * KC * 128 : (size_t)9 * p.kchunks * G * KC * 2;
   const size_t fixed = wide ? wbytes + (size_t)(stats >= 2 ? 2 + kWideYSlots : 2) * 32768 + 1024 + 1024
                             : wbytes + (epi != 1 ? (stats >= 2 ? 2 + kYSlots : 2) * 16384 : xf ? 3 * kXfGroups * 112 * 128 : 0) + 1024 + 1024;
   int st = (int)((232448 - fixed) / a_bytes);
@@ -2088,6 +2111,7 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
                    : G == 32 ? launch_fold<32, 1, 64, 0, 0, 1>(grid, smem, mx, mw, my, my2, p)
                              : launch_fold<64, 1, 64, 0, 0, 1>(grid, smem, mx, mw, my, my2, p);
   }
+  if (epi == 0 && KC == 16) return launch_fold<64, 0, 16>(grid, smem, mx, mw, my, my2, p);
   if (epi == 0) return launch_fold<64, 0>(grid, smem, mx, mw, my, my2, p);
   if (wide) {
     static bool attr_done_dev[kMaxDevices];
@@ -2148,6 +2172,9 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   p.tg = tile_grid(p.n_tiles, p.tiles_w, p.tiles_h);
   p.kchunks = epi == 2 ? 1 : Cin / 64; p.stages = pl.stages; p.stats = stats; p.red = red; p.status = status;
   p.tm_y2 = my;
+  if (stats == 0 && bn) {
+    p.bn_scale = bn->scale; p.bn_shift = bn->shift;
+  }
   if (stats == 2) {
     if ((rc = make_map4(&p.tm_y2, bn->y2, dy, by)) != NF_OK) return rc;
     p.bn_scale = bn->scale; p.bn_shift = bn->shift; p.bn_mu = bn->mu; p.bn_invstd = bn->invstd;
@@ -2329,14 +2356,18 @@ void nf_tc_select(nf_layer* L) {
   if (L->o.dtype != NF_BF16) return;
   // A first layer with a handful of input channels (RGB) is far too thin a contraction for useful tensor-core work (K = 27),
   // but its CUDA-core kernels reach under a tenth of the memory bandwidth, and the tensor cores are idle anyway: the input
-  // batch is copied once per step into a 64-channel zero-padded tensor (as large as the layer's output) and the main conv
-  // then runs on the ordinary 64-channel kernels.  21 times the arithmetic, a third of the time (VGG first layer at 64 x 64,
-  // 1260 images: forward + weight gradient 2.6 ms -> 0.9 ms including the copy).
+  // batch is copied once per step into a zero-padded tensor whose pixels TMA can address, and the main conv runs on the ordinary
+  // kernels.  16 channels where the folded forward and the narrow weight gradient cover the shape (64 output channels; VGG first
+  // layer at 64 x 64, 1260 images: copy + forward 636 -> 300 us against 64 channels), else 64.
   const bool main_ok = tc_size_ok(L->o.N, L->Ho, L->Wo), aux_ok = tc_size_ok(L->o.N, L->Ha, L->Wa);
-  if (L->Cin <= 8 && main_ok && plan_fwd(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok &&
-      plan_wgrad(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok)
-    L->cin_pad = 64;
+  if (L->Cin <= 8 && main_ok) {
+    if (fold_ok(L->Ho, L->Wo, 16, L->Cout, 0, L->o.stride) && plan_wgrad(L->Ho, L->Wo, L->Cout, 16, L->o.N, 1).ok)
+      L->cin_pad = 16;
+    else if (plan_fwd(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok && plan_wgrad(L->Ho, L->Wo, 64, L->Cout, L->o.N, 0, L->o.stride).ok)
+      L->cin_pad = 64;
+  }
   const int Cin = L->cin_pad ? L->cin_pad : L->Cin;
+  if (L->cin_pad == 16) L->fam[0] = L->fam[1] = 1;
   if (main_ok && plan_fwd(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[0] = 1;
   if (plan_wgrad(L->Ho, L->Wo, Cin, L->Cout, L->o.N, 0, L->o.stride).ok) L->fam[1] = 1;
   if (wide_aux(L)) {  // more than 64 filters: the aux conv runs on the kernels of the main conv
@@ -2351,7 +2382,7 @@ void nf_tc_select(nf_layer* L) {
 }
 
 size_t nf_tc_scratch_floats(const nf_layer* L) {
-  const size_t a = L->fam[1] ? plan_wgrad(L->Ho, L->Wo, L->cin_pad ? L->cin_pad : L->Cin, L->Cout, L->o.N, 0, L->o.stride).part_floats : 0;
+  const size_t a = L->cin_pad == 16 ? plan_wgrad(L->Ho, L->Wo, L->Cout, 16, L->o.N, 1).part_floats : L->fam[1] ? plan_wgrad(L->Ho, L->Wo, L->cin_pad ? L->cin_pad : L->Cin, L->Cout, L->o.N, 0, L->o.stride).part_floats : 0;
   const size_t b = L->fam[3] ? plan_wgrad(L->Ha, L->Wa, L->Cout, L->F, L->o.N, wide_aux(L) ? 0 : 1).part_floats : 0;
   return a > b ? a : b;
 }
@@ -2392,17 +2423,14 @@ int nf_tc_conv_fwd(nf_layer* L, const void* x, int& nb) {
                  L->status, &nb, 0, nullptr, L->o.stride);
 }
 
-int nf_tc_conv_fwd_eval(nf_layer* L, const void* x, int count) {
-  int nb = 0;
-  if (L->cin_pad) {
-    const void *xin, *win;
-    int Cin;
-    const int rc = main_conv_operands(L, x, count, &xin, &win, &Cin);
-    if (rc != NF_OK) return rc;
-    return run_fwd(count, L->H, L->W, Cin, L->Cout, xin, win, L->y, 0, nullptr, 0, L->status, &nb, 0, nullptr, L->o.stride);
-  }
-  return run_fwd(count, L->H, L->W, L->Cin, L->Cout, x, L->shadow + L->off[NF_P_W], L->y, 0, nullptr, 0, L->status, &nb, 0,
-                 nullptr, L->o.stride);
+int nf_tc_conv_fwd_eval(nf_layer* L, const void* x, int count, void* act) {
+  int nb = 0, Cin;
+  const void *xin, *win;
+  const int rc = main_conv_operands(L, x, count, &xin, &win, &Cin);
+  if (rc != NF_OK) return rc;
+  const BnBwdIn bn{nullptr, L->scale, L->shift, nullptr, nullptr};
+  return run_fwd(count, L->H, L->W, Cin, L->Cout, xin, win, act ? act : L->y, 0, nullptr, 0, L->status, &nb, 0, nullptr, L->o.stride,
+                 act ? &bn : nullptr);
 }
 
 int nf_tc_aux_fwd(nf_layer* L, const void* a, int count) {
@@ -2446,10 +2474,16 @@ int nf_tc_bn_aux_fwd(nf_layer* L, void* act_out) {
 
 int nf_tc_wgrad(nf_layer* L, const void* x) {
   if (L->cin_pad) {  // the padded copy of this step's input is still in place (the forward made it); x itself is not read again
-    const int rc = run_wgrad(L->o.N, L->H, L->W, L->cin_pad, L->Cout, L->xpad, L->dy, L->wpart, L->wpart_floats, L->gwpad, L->status, 0,
-                             L->o.stride);
+    // 16 channels: the roles of input and gradient are exchanged, so that the narrow tensor takes the narrow side of the auxiliary
+    // weight gradient: with i' = i + kh - 1 the sum runs over the input's pixels and the gradient is shifted by 1 - kh, which gives
+    // [8 - tap][ci][co]
+    const bool narrow = L->cin_pad == 16;
+    const int rc = narrow ? run_wgrad(L->o.N, L->H, L->W, L->Cout, 16, L->dy, L->xpad, L->wpart, L->wpart_floats, L->gwpad, L->status, 1)
+                          : run_wgrad(L->o.N, L->H, L->W, L->cin_pad, L->Cout, L->xpad, L->dy, L->wpart, L->wpart_floats, L->gwpad, L->status, 0,
+                                      L->o.stride);
     if (rc != NF_OK) return rc;
-    return nf_k_unpad_grad(L->gwpad, (size_t)9 * L->Cout, L->Cin, L->cin_pad, L->grad + L->off[NF_P_W]);
+    return narrow ? nf_k_unpad_grad_mirrored(L->gwpad, L->Cout, L->Cin, 16, L->grad + L->off[NF_P_W])
+                  : nf_k_unpad_grad(L->gwpad, (size_t)9 * L->Cout, L->Cin, L->cin_pad, L->grad + L->off[NF_P_W]);
   }
   return run_wgrad(L->o.N, L->H, L->W, L->Cin, L->Cout, x, L->dy, L->wpart, L->wpart_floats, L->grad + L->off[NF_P_W],
                    L->status, 0, L->o.stride);

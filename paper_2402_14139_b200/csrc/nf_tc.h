@@ -8,8 +8,9 @@ void nf_tc_select(nf_layer* L);
 size_t nf_tc_scratch_floats(const nf_layer* L);
 // y = conv(x) in bf16 plus per-CTA channel partials (sum, sum of squares) in L->red; nb = partial count.
 int nf_tc_conv_fwd(nf_layer* L, const void* x, int& nb);
-// Same convolution for `count` samples without statistics (cache-filling forward).
-int nf_tc_conv_fwd_eval(nf_layer* L, const void* x, int count);
+// Same convolution for `count` samples without statistics (cache-filling forward): y, or, with act, straight to act = ReLU(y * scale +
+// shift) with the layer's current coefficients.
+int nf_tc_conv_fwd_eval(nf_layer* L, const void* x, int count, void* act);
 // grad(W) = wgrad(x, L->dy) into the gradient arena.
 int nf_tc_wgrad(nf_layer* L, const void* x);
 // Floats of channel-partial scratch (L->red) the tensor-core forward needs.
