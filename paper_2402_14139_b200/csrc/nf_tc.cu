@@ -103,7 +103,7 @@ struct TcPlan {
   size_t smem;
 };
 
-// With stats == 0 and bn_scale set, the forward writes ReLU(y * scale + shift) of the bf16-rounded y instead of y: BatchNorm with
+// POST = 1 (stats == 0): the forward writes ReLU(y * scale + shift) of the bf16-rounded y instead of y: BatchNorm with
 // running statistics, whose coefficients are known beforehand (cache fill, exits).  Two channels, packed:
 __device__ __forceinline__ uint32_t bn_relu2(uint32_t y, float2 sc, float2 sh) {
   const __nv_bfloat162 b = __floats2bfloat162_rn(fmaxf(fmaf(__uint_as_float(y << 16), sc.x, sh.x), 0.f),
@@ -148,7 +148,7 @@ __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& ta
 //       core's running sum drops low bits on every instruction: over 2304 products 0.07 % of the bf16 outputs came out one unit
 //       off the nearest value, against 0.016 % of an fp32 chain.  Maps that no tile divides had such chains (they ran on the CUDA
 //       cores), and their layers are small enough for that to show; a segment's 192 products keep the error below theirs.
-template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0>
+template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0>
 __global__ void __launch_bounds__(kThreads, 1)
 conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                    const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ FwdParams p) {
@@ -331,7 +331,6 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     const int sc = et % BN, shalf = et / BN;        // stats: channel and row half of this thread
     const int rw = r % p.BW, rh = (r / p.BW) % p.BH;  // place of the thread's pixel in its tile
     uint32_t sg = 0;                                  // SEG: segments taken so far
-    const bool post = !p.stats && p.bn_scale;
     float ssum = 0.f, ssq = 0.f;
     float ssum2 = 0.f, ssq2 = 0.f;                  // BN = 256: the thread's second channel, sc + 128
     uint32_t tl = 0;
@@ -390,7 +389,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             const __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
             w[e] = *reinterpret_cast<const uint32_t*>(&b2);
           }
-          if (post) {
+          if constexpr (POST) {
             const float* ps = p.bn_scale + nt * BN + j * 32 + q * 8;
             const float* ph = p.bn_shift + nt * BN + j * 32 + q * 8;
 #pragma unroll
@@ -639,7 +638,7 @@ struct FoldParams {
 // padding of a must be), write the tile's own 14 x 8 pixels of a to global memory (the layer's output activation) and
 // only then hand the stage to the issuer.  The separate normalisation pass (read y, write a) and this kernel's read of
 // a disappear; the halo pixels are normalised by both neighbours.
-template <int G, int EPI, int KC = 64, int MIR = 0, int UF = 0, int XF = 0>
+template <int G, int EPI, int KC = 64, int MIR = 0, int UF = 0, int XF = 0, int POST = 0>
 __global__ void __launch_bounds__(kFoldThreads + kXfThreads * XF, 1)
 conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                      const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_y2, const FoldParams p) {
@@ -967,7 +966,7 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         }
         }
         if constexpr (EPI == 0) {
-          if (!p.stats && p.bn_scale) {
+          if constexpr (POST) {
             const float2* ps = reinterpret_cast<const float2*>(p.bn_scale + nt * 64 + q * 16);
             const float2* ph = reinterpret_cast<const float2*>(p.bn_shift + nt * 64 + q * 16);
 #pragma unroll
@@ -1968,15 +1967,15 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   return pl;
 }
 
-template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0>
+template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0>
 int launch_fwd(const TcPlan& pl, const CUtensorMap& mx, const CUtensorMap& mw, const CUtensorMap& my, const FwdParams& p) {
   static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
   bool& attr_done = attr_done_dev[current_device()];
   if (!attr_done) {
-    NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG>, pl.grid, kThreads, pl.smem, mx, mw, my, p);
+  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, pl.grid, kThreads, pl.smem, mx, mw, my, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2007,16 +2006,16 @@ bool fold_ok(int H, int W, int Cin, int Cout, int epi, int stride, int stats = 0
   return wbytes + (epi == 0 ? 2 * 16384 : 0) + extra_smem + 2048 + 3 * 20480 <= 232448;
 }
 
-template <int G, int EPI, int KC = 64, int MIR = 0, int UF = 0, int XF = 0>
+template <int G, int EPI, int KC = 64, int MIR = 0, int UF = 0, int XF = 0, int POST = 0>
 int launch_fold(int grid, size_t smem, const CUtensorMap& mx, const CUtensorMap& mw, const CUtensorMap& my, const CUtensorMap& my2,
                 const FoldParams& p) {
   static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
   bool& attr_done = attr_done_dev[current_device()];
   if (!attr_done) {
-    NF_CUDA(cudaFuncSetAttribute(conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    NF_CUDA(cudaFuncSetAttribute(conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF>, grid, kFoldThreads + kXfThreads * XF, smem, mx, mw, my, my2, p);
+  nf_launch(conv_fwd_fold_kernel<G, EPI, KC, MIR, UF, XF, POST>, grid, kFoldThreads + kXfThreads * XF, smem, mx, mw, my, my2, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2111,6 +2110,8 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
                    : G == 32 ? launch_fold<32, 1, 64, 0, 0, 1>(grid, smem, mx, mw, my, my2, p)
                              : launch_fold<64, 1, 64, 0, 0, 1>(grid, smem, mx, mw, my, my2, p);
   }
+  if (epi == 0 && bn)  // evaluation: normalised in the epilogue
+    return KC == 16 ? launch_fold<64, 0, 16, 0, 0, 0, 1>(grid, smem, mx, mw, my, my2, p) : launch_fold<64, 0, 64, 0, 0, 0, 1>(grid, smem, mx, mw, my, my2, p);
   if (epi == 0 && KC == 16) return launch_fold<64, 0, 16>(grid, smem, mx, mw, my, my2, p);
   if (epi == 0) return launch_fold<64, 0>(grid, smem, mx, mw, my, my2, p);
   if (wide) {
@@ -2183,6 +2184,15 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     const int rows = pl.grid / p.n_tiles * pl.parts;
     if ((size_t)rows * 2 * Cout > red_floats) return NF_ENOWS;
     *nb = rows;
+  }
+  if (epi == 0 && stats == 0 && bn) {  // evaluation: normalised in the epilogue
+    if (pl.SEG)
+      return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 1, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 1, 1>(pl, mx, mw, my, p);
+    if (pl.PT)
+      return pl.BN == 256 ? launch_fwd<256, 0, 64, 0, 1, 0, 0, 1>(pl, mx, mw, my, p)
+           : pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 0, 1>(pl, mx, mw, my, p);
+    if (pl.RW) return launch_fwd<64, 0, 64, 0, 0, 1, 0, 1>(pl, mx, mw, my, p);
+    return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 0, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
   }
   if (pl.SEG) {  // maps that no tile divides
     if (epi == 0) return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
