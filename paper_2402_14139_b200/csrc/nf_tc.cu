@@ -1709,6 +1709,144 @@ conv_wgrad_kw_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   }
 }
 
+// ---------------------------------------------------------------- weight gradient, stride 1, 128 output channels on the M side
+// A CTA owns one column tap kw, 128 output channels and CC chunks of 64 input channels:
+//   A (M = 128) = the gradient tile of 128 output channels (two MN-major atoms),
+//   B (N = 192) = the three row taps of ONE activation box (rows h0 - 1 .. h0 + BH, columns shifted by kw - 1) as consecutive
+//                 64-channel atoms one image row apart,
+// so an instruction per 16 pixels and chunk yields three taps x 64 x 128 with no idle half: the forms with the activation on the M
+// side stack taps 0 | 1 and 2 | nothing and waste a quarter of the tensor pipe, and the per-tap one fetches each pixel three times
+// (112 KB of shared memory fill per 128 pixels and 3 x 64 x 256 products; here 72 KB for the same with CC = 2).  Tiles of BI images
+// (8x8x2, 4x4x8) have a box of BH + 2 rows per image; 16 consecutive pixels of the gradient tile must lie in one image:
+// BW * BH a multiple of 16.  The partial sums leave with 16-byte stores, a thread per output channel.
+template <int CC>
+__global__ void __launch_bounds__(kThreads, 1)
+conv_wgrad_row_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dy, const WgParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int box_bytes = p.BI * (p.BH + 2) * p.BW * 128;
+  const int stage_bytes = CC * box_bytes + 2 * 16384;
+  const int stages = p.stages;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)stages * stage_bytes);
+  uint64_t* full = bars;
+  uint64_t* empty = bars + kMaxStages;
+  uint64_t* done = bars + 2 * kMaxStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  constexpr uint32_t kCols = CC * 256;  // 192 used of each 256
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int blocks = p.ci_chunks * p.co_chunks;
+  const int blk = blockIdx.x % blocks, rest = blockIdx.x / blocks;
+  const int kw = rest % 3, sp = rest / 3;
+  const int cic = blk % p.ci_chunks, coc = blk / p.ci_chunks;
+  const int t0 = (int)((long)p.pix_tiles * sp / p.splits), t1 = (int)((long)p.pix_tiles * (sp + 1) / p.splits);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      ptx::mbar_init(&full[s], 1);
+      ptx::mbar_init(&empty[s], 1);
+    }
+    ptx::mbar_init(done, 1);
+    *abort_flag = 0;
+    ptx::fence_mbar_init();
+    ptx::prefetch_tmap(&tm_x);
+    ptx::prefetch_tmap(&tm_dy);
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc(tmem_slot, kCols);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
+
+  if (warp == 0) {
+    if (ptx::elect_one()) {
+      Ring rg;
+      for (int t = t0; t < t1; ++t, rg.next(stages)) {
+        const TileAt at = tile_at(t, p.tg);
+        const int w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
+        if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) break;
+        uint64_t* fb = &full[rg.s];
+        uint8_t* st = smem + (size_t)rg.s * stage_bytes;
+        ptx::mbar_expect_tx(fb, (uint32_t)stage_bytes);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) ptx::tma_load_4d(st + a * 16384, &tm_dy, fb, coc * 128 + a * 64, w0, h0, n);
+#pragma unroll
+        for (int c = 0; c < CC; ++c)
+          ptx::tma_load_4d(st + 32768 + c * box_bytes, &tm_x, fb, (cic * CC + c) * 64, w0 + kw - 1, h0 - 1, n);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    constexpr uint32_t idesc = ptx::idesc_bf16(128, 192, 1, 1);
+    const uint64_t a_hi = ptx::sdesc(0, 16384, 1024, 2);       // next 64 output channels: next atom
+    const uint64_t b_hi = ptx::sdesc(0, p.BW * 128, 1024, 2);  // next row tap: one image row further
+    const int per_img = p.BW * p.BH / 16;                      // 16-pixel steps per image of the tile
+    const uint32_t gap16 = (uint32_t)(2 * p.BW * 128) >> 4;    // the two halo rows between the images' boxes
+    if (ptx::elect_one()) {
+      Ring rg;
+      bool ok = true;
+      for (int t = t0; t < t1; ++t, rg.next(stages)) {
+        if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
+        ptx::tc_fence_after();
+        const uint32_t g16 = (ptx::smem_u32(smem) + rg.s * stage_bytes) >> 4;
+        uint32_t x16 = g16 + (32768 >> 4);
+        int left = per_img;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (left == 0) {
+            x16 += gap16;
+            left = per_img;
+          }
+          --left;
+#pragma unroll
+          for (int c = 0; c < CC; ++c)
+            ptx::mma_f16(tmem_base + c * 256, a_hi | (uint64_t)(g16 + k * 128), b_hi | (uint64_t)(x16 + ((c * box_bytes) >> 4) + k * 128), idesc,
+                         t > t0 || k != 0);
+        }
+        ptx::mma_commit(&empty[rg.s]);
+      }
+      if (ok) ptx::mma_commit(done);
+    }
+    __syncwarp();
+  } else {
+    const int lg = warp & 3, m = lg * 32 + lane;  // m: output channel of the CTA's 128
+    if (ptx::mbar_wait(done, 0, abort_flag) && t1 > t0) {
+      ptx::tc_fence_after();
+      const size_t plane = (size_t)p.Cout * p.Cin;
+      float* base = p.part + ((size_t)sp * 9 + kw) * plane + (size_t)(coc * 128 + m) * p.Cin + cic * CC * 64;
+#pragma unroll 1
+      for (int q = 0; q < CC * 12; ++q) {  // 16 input channels of one row tap at a time
+        const int c = q / 12, kh = (q / 4) % 3, b = q % 4;
+        uint32_t v[16];
+        ptx::tmem_ld16(tmem_base + ((uint32_t)(lg * 32) << 16) + c * 256 + kh * 64 + b * 16, v);
+        ptx::tmem_ld_wait();
+        float4* dst = reinterpret_cast<float4*>(base + (size_t)(kh * 3) * plane + c * 64 + b * 16);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          dst[e] = make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]), __uint_as_float(v[4 * e + 2]),
+                               __uint_as_float(v[4 * e + 3]));
+      }
+    }
+  }
+
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) {
+    if (threadIdx.x == 0) atomicOr(p.status, NF_ETIMEOUT);
+    const unsigned long long tt = ptx::globaltimer();
+    while (ptx::globaltimer() - tt < 2000000ull) __nanosleep(1000);
+  }
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem_base, kCols);
+  }
+}
+
 // ---------------------------------------------------------------- weight gradient, stride 1, few filters: gradient on the M side
 // An instruction holds the tensor pipe for about the same time whatever its shape, so for the auxiliary conv
 // (F <= 32 filters) the fewest instructions win.  Here the roles of conv_wgrad_kw_kernel are swapped:
@@ -2229,36 +2367,15 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
 }
 
 struct WgPlan {
-  int ok, exact, BW, BH, BI, PT, NB, GX, splits, grid, stages;
+  int ok, exact, BW, BH, BI, PT, NB, GX, ROW, splits, grid, stages;  // ROW: input-channel chunks per CTA of the row kernel, or 0
   size_t smem, part_floats;
 };
 
-// aux = 0: main conv (Cout a multiple of 64).  aux = 1: aux conv (Cout = F <= 64, a multiple of 8).
-// H, W: size of the gradient tensor (the conv OUTPUT; equals the input size for stride 1).
-WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int stride = 1) {
-  WgPlan pl{};
-  if (Cin % 64 || (stride == 2 && aux)) return pl;
-  if (aux ? (Cout > 64 || Cout % 8) : (Cout % 64 != 0)) return pl;
-  pl.exact = pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
-  pl.PT = (stride == 2 || pl.BI > 1 || !pl.exact) ? 1 : 0;
-  pl.NB = aux ? (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64) : 64;
-  if (!aux && pl.PT) pl.NB = Cout % 256 == 0 ? 256 : Cout % 128 == 0 ? 128 : 64;  // per-tap form: as wide an instruction as Cout allows
-  pl.GX = (aux && !pl.PT && pl.NB <= 32) ? 1 : 0;  // few filters: one instruction per 16 pixels with the gradient on the M side
-  size_t g_region = (size_t)(pl.GX ? 4 : 3) * 128 * pl.NB * 2;
-  if (g_region < 4096) g_region = 4096;
-  const size_t stage = pl.PT ? (size_t)49152 + (pl.NB > 64 ? pl.NB / 64 : 1) * 16384 : (size_t)(pl.BH + 2) * pl.BW * 128 + g_region;
-  pl.stages = pl.PT ? (pl.NB > 64 ? 2 : 3) : (int)((232448 - 2048) / stage);
-  if (pl.stages > kMaxStages) pl.stages = kMaxStages;
-  if (pl.stages < 2) return pl;
-  pl.smem = (size_t)pl.stages * stage + 1024 + 1024;
-  if (pl.smem > 232448) return pl;
-  const int blocks = (Cin / 64) * (aux ? 1 : Cout / pl.NB);
-  const long pix_tiles = (long)((N + pl.BI - 1) / pl.BI) * ((H + pl.BH - 1) / pl.BH) * ((W + pl.BW - 1) / pl.BW);
-  if (pix_tiles >= (1l << 30)) return pl;
-  const int groups = pl.PT ? 3 : 1;  // kernel rows handled by separate CTAs
-  // pixel splits per (chunk pair, kernel-row group): the count whose CTAs fill whole waves of SMs best (smallest on ties),
-  // e.g. 512 -> 512 channels with three row groups: 192 units -> 3 splits = 576 CTAs = 3.9 waves instead of 1.3
-  const int units = blocks * groups, sms = sm_count();
+// Pixel splits for `units` CTAs per split (channel chunk pairs x kernel rows or columns): the count whose CTAs fill whole waves of
+// SMs best (smallest on ties), e.g. 512 -> 512 channels with three row groups: 192 units -> 3 splits = 576 CTAs = 3.9 waves
+// instead of 1.3
+long wgrad_splits(int units, long pix_tiles) {
+  const int sms = sm_count();
   long base = sms / units;
   if (base < 1) base = 1;
   long sp = base;
@@ -2271,10 +2388,49 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
       sp = c;
     }
   }
-  if (sp > pix_tiles) sp = pix_tiles;
+  return sp > pix_tiles ? pix_tiles : sp;
+}
+
+// aux = 0: main conv (Cout a multiple of 64).  aux = 1: aux conv (Cout = F <= 64, a multiple of 8).
+// H, W: size of the gradient tensor (the conv OUTPUT; equals the input size for stride 1).
+WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int stride = 1) {
+  WgPlan pl{};
+  if (Cin % 64 || (stride == 2 && aux)) return pl;
+  if (aux ? (Cout > 64 || Cout % 8) : (Cout % 64 != 0)) return pl;
+  pl.exact = pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
+  pl.PT = (stride == 2 || pl.BI > 1 || !pl.exact) ? 1 : 0;
+  pl.NB = aux ? (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64) : 64;
+  if (!aux && pl.PT) pl.NB = Cout % 256 == 0 ? 256 : Cout % 128 == 0 ? 128 : 64;  // per-tap form: as wide an instruction as Cout allows
+  pl.GX = (aux && !pl.PT && pl.NB <= 32) ? 1 : 0;  // few filters: one instruction per 16 pixels with the gradient on the M side
+  const long pix_tiles = (long)((N + pl.BI - 1) / pl.BI) * ((H + pl.BH - 1) / pl.BH) * ((W + pl.BW - 1) / pl.BW);
+  if (pix_tiles >= (1l << 30)) return pl;
+  int units = (Cin / 64) * (aux ? 1 : Cout / pl.NB) * (pl.PT ? 3 : 1);
+  long sp = wgrad_splits(units, pix_tiles);
+  pl.part_floats = (size_t)sp * 9 * Cout * Cin;  // what a layer reserves: the row form never needs more
+  // 128 output channels: the form without an idle half, wherever 16 pixels of a tile are consecutive in one image.  Two chunks of
+  // input channels per CTA where that leaves two stages and as few splits as are reserved for, else one.
+  const size_t box = (size_t)pl.BI * (pl.BH + 2) * pl.BW * 128;
+  if (!aux && stride == 1 && Cout % 128 == 0 && pl.BW >= 4 && pl.BW * pl.BH % 16 == 0)
+    for (int cc = Cin % 128 == 0 ? 2 : 1; cc >= 1 && !pl.ROW; --cc) {
+      const int u = Cin / 64 / cc * (Cout / 128) * 3;
+      const long c = wgrad_splits(u, pix_tiles);
+      if (2 * (cc * box + 32768) > 232448 - 2048 || c > sp) continue;
+      pl.ROW = cc;
+      pl.NB = 128;
+      units = u;
+      sp = c;
+    }
+  size_t g_region = (size_t)(pl.GX ? 4 : 3) * 128 * pl.NB * 2;
+  if (g_region < 4096) g_region = 4096;
+  const size_t stage = pl.ROW ? pl.ROW * box + 32768
+                     : pl.PT ? (size_t)49152 + (pl.NB > 64 ? pl.NB / 64 : 1) * 16384 : (size_t)(pl.BH + 2) * pl.BW * 128 + g_region;
+  pl.stages = pl.PT && !pl.ROW ? (pl.NB > 64 ? 2 : 3) : (int)((232448 - 2048) / stage);
+  if (pl.stages > kMaxStages) pl.stages = kMaxStages;
+  if (pl.stages < 2) return pl;
+  pl.smem = (size_t)pl.stages * stage + 1024 + 1024;
+  if (pl.smem > 232448) return pl;
   pl.splits = (int)sp;
-  pl.grid = (int)(sp * blocks * groups);
-  pl.part_floats = (size_t)sp * 9 * Cout * Cin;
+  pl.grid = (int)(sp * units);
   pl.ok = 1;
   return pl;
 }
@@ -2288,6 +2444,19 @@ int launch_wgrad_kw(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& 
     attr_done = true;
   }
   nf_launch(conv_wgrad_kw_kernel<NB>, pl.grid, kThreads, pl.smem, mx, mg, p);
+  NF_LAUNCHED();
+  return NF_OK;
+}
+
+template <int CC>
+int launch_wgrad_row(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& mg, const WgParams& p) {
+  static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
+  bool& attr_done = attr_done_dev[current_device()];
+  if (!attr_done) {
+    NF_CUDA(cudaFuncSetAttribute(conv_wgrad_row_kernel<CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    attr_done = true;
+  }
+  nf_launch(conv_wgrad_row_kernel<CC>, pl.grid, kThreads, pl.smem, mx, mg, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2327,7 +2496,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
   if (pl.part_floats > part_floats) return NF_ENOWS;
   CUtensorMap mx, mg;
   const uint64_t dx[4] = {(uint64_t)Cin, (uint64_t)Win, (uint64_t)Hin, (uint64_t)N};
-  const uint32_t bx[4] = {64, (uint32_t)pl.BW, (uint32_t)(pl.PT ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
+  const uint32_t bx[4] = {64, (uint32_t)pl.BW, (uint32_t)(pl.PT && !pl.ROW ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
   const uint64_t dg[4] = {(uint64_t)Cout, (uint64_t)W, (uint64_t)H, (uint64_t)N};
   const uint32_t bg[4] = {(uint32_t)(pl.NB > 64 ? 64 : pl.NB), (uint32_t)pl.BW, (uint32_t)pl.BH, (uint32_t)pl.BI};
   int rc;
@@ -2338,9 +2507,11 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
   p.tiles_w = (W + pl.BW - 1) / pl.BW; p.tiles_h = (H + pl.BH - 1) / pl.BH; p.pix_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w;
   p.stride = stride; p.BI = pl.BI;
   p.tg = tile_grid(1, p.tiles_w, p.tiles_h);
-  p.ci_chunks = Cin / 64; p.co_chunks = aux ? 1 : Cout / pl.NB; p.splits = pl.splits; p.part = part; p.status = status;
+  p.ci_chunks = pl.ROW ? Cin / 64 / pl.ROW : Cin / 64; p.co_chunks = aux ? 1 : Cout / pl.NB; p.splits = pl.splits; p.part = part; p.status = status;
   p.stages = pl.stages;
-  if (pl.GX)
+  if (pl.ROW)
+    rc = pl.ROW == 2 ? launch_wgrad_row<2>(pl, mx, mg, p) : launch_wgrad_row<1>(pl, mx, mg, p);
+  else if (pl.GX)
     rc = pl.NB == 32 ? launch_wgrad_gx<32>(pl, mx, mg, p) : launch_wgrad_gx<16>(pl, mx, mg, p);
   else if (pl.PT)
     rc = pl.NB == 256 ? launch_wgrad<256, 1>(pl, mx, mg, p) : pl.NB == 128 ? launch_wgrad<128, 1>(pl, mx, mg, p)
