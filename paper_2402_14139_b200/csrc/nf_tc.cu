@@ -928,23 +928,33 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       const bool vcol = valid && (UF || w0 + we - 1 < p.W);
       const uint32_t tbase = tmem_base + ((uint32_t)(lg * 32) << 16) + acc * kAccStride;
       bf16* gdst = EPI == 1 ? p.out + (((size_t)n * p.H + h0 + hh) * p.W + w0 + we - 1) * p.Cout : nullptr;
+      // 16 output channels at a time; the next 16 are on their way from tensor memory while these are added and stored
+      uint32_t t0[2][16], t1[2][16], t2[2][16];
+      auto fetch = [&](int q, uint32_t (&a0)[16], uint32_t (&a1)[16], uint32_t (&a2)[16]) {
+        if constexpr (UF) {
+          ptx::tmem_ld16(tbase + q * 16, a1);
+        } else {
+          ptx::tmem_ld16(tbase + (MIR ? 2 * G : 0) + q * 16, a0);  // group feeding the pixel on the left
+          ptx::tmem_ld16(tbase + G + q * 16, a1);
+          ptx::tmem_ld16(tbase + (MIR ? 0 : 2 * G) + q * 16, a2);  // group feeding the pixel on the right
+        }
+      };
+      fetch(0, t0[0], t1[0], t2[0]);
 #pragma unroll
-      for (int q = 0; q < G / 16; ++q) {     // 16 output channels at a time
-        uint32_t v0[16], v1[16], v2[16];
+      for (int q = 0; q < G / 16; ++q) {
+        uint32_t (&v0)[16] = t0[q & 1];
+        uint32_t (&v1)[16] = t1[q & 1];
+        uint32_t (&v2)[16] = t2[q & 1];
+        ptx::tmem_ld_wait();
+        if (q + 1 < G / 16) fetch(q + 1, t0[(q + 1) & 1], t1[(q + 1) & 1], t2[(q + 1) & 1]);
         uint32_t w[8];
         if constexpr (UF) {
-          ptx::tmem_ld16(tbase + q * 16, v1);
-          ptx::tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v1[2 * e]), __uint_as_float(v1[2 * e + 1]));
             w[e] = *reinterpret_cast<const uint32_t*>(&b2);
           }
         } else {
-        ptx::tmem_ld16(tbase + (MIR ? 2 * G : 0) + q * 16, v0);  // group feeding the pixel on the left
-        ptx::tmem_ld16(tbase + G + q * 16, v1);
-        ptx::tmem_ld16(tbase + (MIR ? 0 : 2 * G) + q * 16, v2);  // group feeding the pixel on the right
-        ptx::tmem_ld_wait();
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           float o[2];
