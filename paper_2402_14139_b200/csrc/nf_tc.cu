@@ -1427,6 +1427,7 @@ struct WgParams {
   int N, H, W, Cin, Cout;
   int BW, BH, tiles_w, tiles_h, pix_tiles, ci_chunks, co_chunks, splits, stages, stride, BI;
   TileGrid tg;
+  int dy_shift;     // row form: the column tap moves the gradient (as in conv_wgrad_kw_kernel) instead of the activation
   float* part;      // [splits][9][Cout][Cin]
   int32_t* status;
 };
@@ -1723,7 +1724,8 @@ conv_wgrad_kw_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 // A CTA owns one column tap kw, 128 output channels and CC chunks of 64 input channels:
 //   A (M = 128) = the gradient tile of 128 output channels (two MN-major atoms),
 //   B (N = 192) = the three row taps of ONE activation box (rows h0 - 1 .. h0 + BH, columns shifted by kw - 1) as consecutive
-//                 64-channel atoms one image row apart,
+//                 64-channel atoms one image row apart (or the box unshifted and the gradient shifted by 1 - kw, the same sum over
+//                 the activation's pixels),
 // so an instruction per 16 pixels and chunk yields three taps x 64 x 128 with no idle half: the forms with the activation on the M
 // side stack taps 0 | 1 and 2 | nothing and waste a quarter of the tensor pipe, and the per-tap one fetches each pixel three times
 // (112 KB of shared memory fill per 128 pixels and 3 x 64 x 256 products; here 72 KB for the same with CC = 2).  Tiles of BI images
@@ -1784,10 +1786,10 @@ conv_wgrad_row_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         uint8_t* st = smem + (size_t)rg.s * stage_bytes;
         ptx::mbar_expect_tx(fb, (uint32_t)stage_bytes);
 #pragma unroll
-        for (int a = 0; a < 2; ++a) ptx::tma_load_4d(st + a * 16384, &tm_dy, fb, coc * 128 + a * 64, w0, h0, n);
+        for (int a = 0; a < 2; ++a) ptx::tma_load_4d(st + a * 16384, &tm_dy, fb, coc * 128 + a * 64, w0 - (p.dy_shift ? kw - 1 : 0), h0, n);
 #pragma unroll
         for (int c = 0; c < CC; ++c)
-          ptx::tma_load_4d(st + 32768 + c * box_bytes, &tm_x, fb, (cic * CC + c) * 64, w0 + kw - 1, h0 - 1, n);
+          ptx::tma_load_4d(st + 32768 + c * box_bytes, &tm_x, fb, (cic * CC + c) * 64, w0 + (p.dy_shift ? 0 : kw - 1), h0 - 1, n);
       }
     }
     __syncwarp();
@@ -2416,20 +2418,26 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
   if (pix_tiles >= (1l << 30)) return pl;
   int units = (Cin / 64) * (aux ? 1 : Cout / pl.NB) * (pl.PT ? 3 : 1);
   long sp = wgrad_splits(units, pix_tiles);
-  pl.part_floats = (size_t)sp * 9 * Cout * Cin;  // what a layer reserves: the row form never needs more
-  // 128 output channels: the form without an idle half, wherever 16 pixels of a tile are consecutive in one image.  Two chunks of
-  // input channels per CTA where that leaves two stages and as few splits as are reserved for, else one.
+  pl.part_floats = (size_t)sp * 9 * Cout * Cin;
+  // 128 output channels: the form without an idle half, wherever 16 pixels of a tile are consecutive in one image.  The splits are
+  // those of the other forms, so that every sum runs over the same pixels in the same order and the bits stay what they were; of one
+  // or two chunks of input channels per CTA the one whose CTAs fill their waves better (two on near ties: less to fetch).
   const size_t box = (size_t)pl.BI * (pl.BH + 2) * pl.BW * 128;
-  if (!aux && stride == 1 && Cout % 128 == 0 && pl.BW >= 4 && pl.BW * pl.BH % 16 == 0)
-    for (int cc = Cin % 128 == 0 ? 2 : 1; cc >= 1 && !pl.ROW; --cc) {
-      const int u = Cin / 64 / cc * (Cout / 128) * 3;
-      const long c = wgrad_splits(u, pix_tiles);
-      if (2 * (cc * box + 32768) > 232448 - 2048 || c > sp) continue;
-      pl.ROW = cc;
-      pl.NB = 128;
-      units = u;
-      sp = c;
+  if (!aux && stride == 1 && Cout % 128 == 0 && pl.BW >= 4 && pl.BW * pl.BH % 16 == 0) {
+    // single-image tiles with one chunk only: the form above has as little to fetch and fills its wave (64 -> 128 channels at 32x32)
+    double best = pl.PT || Cin % 128 == 0 ? 0.0 : 0.75;
+    for (int cc = Cin % 128 == 0 ? 2 : 1; cc >= 1; --cc) {
+      if (2 * (cc * box + 32768) > 232448 - 2048) continue;  // two stages have to fit
+      const long u = Cin / 64 / cc * (Cout / 128) * 3, ctas = u * sp, waves = (ctas + sm_count() - 1) / sm_count();
+      const double eff = (double)ctas / (double)(waves * sm_count());
+      if (eff > best + 0.1) {
+        best = eff;
+        pl.ROW = cc;
+        pl.NB = 128;
+        units = (int)u;
+      }
     }
+  }
   size_t g_region = (size_t)(pl.GX ? 4 : 3) * 128 * pl.NB * 2;
   if (g_region < 4096) g_region = 4096;
   const size_t stage = pl.ROW ? pl.ROW * box + 32768
@@ -2519,6 +2527,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
   p.tg = tile_grid(1, p.tiles_w, p.tiles_h);
   p.ci_chunks = pl.ROW ? Cin / 64 / pl.ROW : Cin / 64; p.co_chunks = aux ? 1 : Cout / pl.NB; p.splits = pl.splits; p.part = part; p.status = status;
   p.stages = pl.stages;
+  p.dy_shift = !pl.PT;
   if (pl.ROW)
     rc = pl.ROW == 2 ? launch_wgrad_row<2>(pl, mx, mg, p) : launch_wgrad_row<1>(pl, mx, mg, p);
   else if (pl.GX)
