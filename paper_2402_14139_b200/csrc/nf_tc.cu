@@ -13,6 +13,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <utility>
 
 #include "nf_ptx.cuh"
 #include "nf_tc.h"
@@ -87,7 +88,7 @@ struct FwdParams {
   int BW, BH, tiles_w, tiles_h, n_tiles, total_tiles, kchunks, stages;
   int stride, BI;     // PT mode: conv stride and images per tile (BW*BH*BI = 128)
   TileGrid tg;
-  int stats;
+  int stats, yslots;  // yslots: buffers for the tiles of y2
   float* red;         // [grid / n_tiles * parts][2][Cout] channel partials
   int32_t* status;    // device status word
   const float* bias;  // EPI 1: per-channel bias added before the ReLU
@@ -99,7 +100,7 @@ struct FwdParams {
 };
 
 struct TcPlan {
-  int ok, BW, BH, BI, PT, BN, KC, RW, SEG, stages, grid, parts;
+  int ok, BW, BH, BI, PT, BN, KC, RW, SEG, stages, grid, parts, yslots;
   size_t smem;
 };
 
@@ -142,6 +143,10 @@ __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& ta
 // PT  : 1 = one TMA box per tap: stride-2 convolutions (the box is gathered with element stride 2, so the
 //       three row taps cannot share a box), feature maps smaller than a tile, where a tile spans BI whole
 //       images (8x8x2, 4x4x8, 2x2x32), and maps that no tile divides; p.H, p.W are the OUTPUT sizes.
+//       2 (HN) = tiles of several images for narrow auxiliary convolutions: the box's dimensions run (channel, column, image, row),
+//       so that a row tap is a constant offset for all images and THREE boxes per chunk serve the nine taps, in one stage with
+//       all the weights.  The per-tap form is bound by its TMA rows (nine boxes of 128) and L2 fill: 512 channels, 8 filters,
+//       8602 maps of 8x8 NNN.
 // RW  : 1 = all nine weight tiles of the CTA's channel tile stay resident in shared memory for the whole
 //       kernel (single 64-channel K chunk, 9*BN*128 bytes); the pipeline then carries activations only.
 // SEG : 1 (PT, forward only) = a new accumulator every kSegSteps k-steps, the segments added in fp32 by the epilogue.  The tensor
@@ -156,16 +161,18 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr int kARow = KC * 2;  // bytes of one pixel row of the activation box
   constexpr uint32_t kALayout = KC == 64 ? 2 : KC == 32 ? 4 : 6;
-  const int a_bytes = PT ? 128 * kARow : (p.BH + 2) * p.BW * kARow;
+  constexpr bool HN = PT == 2;
+  const int a_box = (p.BH + 2) * p.BW * p.BI * kARow;  // HN: one of the three column-shifted boxes, a multiple of 1024
+  const int a_bytes = HN ? 3 * a_box : PT ? 128 * kARow : a_box;
   const int a_stride = (a_bytes + 1023) & ~1023;  // keeps the weight tiles 1024-byte aligned
-  constexpr int b_bytes = RW ? 0 : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
+  constexpr int b_bytes = RW ? 0 : HN ? 9 * (BMN ? (BN / 64) * KC * 128 : BN * 128) : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
   constexpr int w_bytes = RW ? 9 * BN * 128 : 0;  // resident weights [kw][kh][BN][64]
   const int stage_bytes = a_stride + b_bytes;
   constexpr int kSub = EPI == 0 ? BN / 64 : 0;  // 64-channel sub-tiles of the output staging
   uint8_t* wres = smem + (size_t)p.stages * stage_bytes;
   uint8_t* stg = wres + w_bytes;
   uint8_t* ybuf = stg + kSub * 16384;  // stats 2: the y2 tile of the tile in the epilogue (kSub sub-tiles)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(stg + (p.stats == 2 ? 2 : 1) * kSub * 16384);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(stg + (p.stats == 2 ? 1 + p.yslots : 1) * kSub * 16384);
   uint64_t* full = bars;
   uint64_t* empty = bars + kMaxStages;
   uint64_t* tfull = bars + 2 * kMaxStages;
@@ -173,8 +180,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   uint64_t* tempty = tfull + kAccs;
   uint64_t* wfull = tempty + kAccs;
   uint64_t* yfull = wfull + 1;
-  uint64_t* yempty = yfull + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(yempty + 1);
+  uint64_t* yempty = yfull + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(yempty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* epi_go = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
@@ -190,8 +197,10 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       ptx::mbar_init(&tempty[a], 128);
     }
     ptx::mbar_init(wfull, 1);
-    ptx::mbar_init(yfull, 1);
-    ptx::mbar_init(yempty, 128);
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&yfull[i], 1);
+      ptx::mbar_init(&yempty[i], 128);
+    }
     *abort_flag = 0;
     ptx::fence_mbar_init();
     ptx::prefetch_tmap(&tm_x);
@@ -230,12 +239,22 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         const int co0 = at.nt * BN, w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
         for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
-          for (int tap = 0; tap < (PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+          for (int tap = 0; tap < (HN ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
             if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) { ok = false; break; }
             uint64_t* fb = &full[rg.s];
             uint8_t* a_s = smem + (size_t)rg.s * stage_bytes;
             ptx::mbar_expect_tx(fb, (uint32_t)(a_bytes + b_bytes));
-            if constexpr (PT) {
+            if constexpr (HN) {
+#pragma unroll
+              for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(a_s + kw * a_box, &tm_x, fb, ck * KC, w0 + kw - 1, n, h0 - 1);
+              if constexpr (BMN) {
+#pragma unroll
+                for (int hf = 0; hf < BN / 64; ++hf)  // [half][kh][kw][KC rows of f][64 channels]
+                  ptx::tma_load_4d(a_s + a_stride + hf * 9 * KC * 128, &tm_w, fb, co0 + hf * 64, 0, 0, 0);
+              } else {
+                ptx::tma_load_4d(a_s + a_stride, &tm_w, fb, ck * 64, co0, 0, 0);  // [kh][kw][BN][64]
+              }
+            } else if constexpr (PT) {
               const int kh = tap / 3, kw = tap % 3;
               ptx::tma_load_4d(a_s, &tm_x, fb, ck * KC, p.stride * w0 + kw - 1, p.stride * h0 + kh - 1, n);
               if constexpr (BMN) {
@@ -258,13 +277,14 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           }
         }
         if constexpr (EPI == 0) {
-          // the y2 tile of this output tile goes out after its operand loads: the single buffer is free once the epilogue
-          // has finished the statistics of the previous tile, which it does while this tile is being multiplied
+          // the y2 tile of this output tile goes out after its operand loads: its buffer is free once the epilogue has finished
+          // the statistics of the previous tile (of the one before with two buffers), which it does while this tile is multiplied
           if (ok && p.stats == 2) {
-            if (!ptx::mbar_wait(yempty, (ptl & 1) ^ 1, abort_flag)) break;
-            ptx::mbar_expect_tx(yfull, (uint32_t)(kSub * 16384));
+            const uint32_t ys = p.yslots == 2 ? ptl & 1 : 0, yph = p.yslots == 2 ? (ptl >> 1) & 1 : ptl & 1;
+            if (!ptx::mbar_wait(&yempty[ys], yph ^ 1, abort_flag)) break;
+            ptx::mbar_expect_tx(&yfull[ys], (uint32_t)(kSub * 16384));
 #pragma unroll
-            for (int sb = 0; sb < kSub; ++sb) ptx::tma_load_4d(ybuf + sb * 16384, &p.tm_y2, yfull, co0 + sb * 64, w0, h0, n);
+            for (int sb = 0; sb < kSub; ++sb) ptx::tma_load_4d(ybuf + (ys * kSub + sb) * 16384, &p.tm_y2, &yfull[ys], co0 + sb * 64, w0, h0, n);
           }
         }
       }
@@ -275,8 +295,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     constexpr uint32_t idesc = ptx::idesc_bf16(128, BN, 0, BMN);
     // descriptors differ only in their 14-bit address field: constant upper parts, address added per use
     const uint64_t a_hi = ptx::sdesc(0, 16, 8 * kARow, kALayout);
-    const uint64_t b_hi = BMN ? ptx::sdesc(0, (PT ? 1 : 3) * KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
-    const uint32_t a_row16 = (uint32_t)(p.BW * kARow) >> 4;  // one image row of the box, in 16-byte units
+    const uint64_t b_hi = BMN ? ptx::sdesc(0, (HN ? 9 : PT ? 1 : 3) * KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
+    const uint32_t a_row16 = (uint32_t)((HN ? p.BI : 1) * p.BW * kARow) >> 4;  // one image row of the box, in 16-byte units
     if (ptx::elect_one()) {
       Ring rg;
       uint32_t tl = 0;
@@ -284,13 +304,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if constexpr (RW) {
         if (blockIdx.x < p.total_tiles) ok = ptx::mbar_wait(wfull, 0, abort_flag);
       }
-      const int steps = (PT ? 9 : 3) * p.kchunks;
+      const int steps = (HN ? 1 : PT ? 9 : 3) * p.kchunks;
       for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
         uint32_t acc = 0, d = 0, accumulate = 0;
         int step = 0;
         for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
-          for (int tap = 0; tap < (PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+          for (int tap = 0; tap < (HN ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
             if (step == 0 || (SEG && step % kSegSteps == 0)) {
               acc = tl % kAccs;
               if (!ptx::mbar_wait(&tempty[acc], ((tl / kAccs) & 1) ^ 1, abort_flag)) { ok = false; break; }
@@ -304,6 +324,18 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             const uint32_t a_base = ptx::smem_u32(smem) + rg.s * stage_bytes;
             const uint32_t a16 = a_base >> 4;
             const uint32_t b16 = RW ? (ptx::smem_u32(wres) + tap * 3 * BN * 128) >> 4 : (a_base + a_stride) >> 4;
+            if constexpr (HN) {  // all nine taps of the chunk, in the per-tap form's order
+              const uint32_t box16 = (uint32_t)a_box >> 4;
+#pragma unroll
+              for (int t9 = 0; t9 < 9; ++t9)
+#pragma unroll
+                for (int k = 0; k < KC / 16; ++k) {
+                  const uint64_t ad = a_hi | (uint64_t)(a16 + (t9 % 3) * box16 + (t9 / 3) * a_row16 + k * 2);
+                  const uint64_t bd = b_hi | (uint64_t)(BMN ? b16 + (((8 - t9) * KC * 128 + k * 16 * 128) >> 4) : b16 + ((t9 * BN * 128 + k * 32) >> 4));
+                  ptx::mma_f16(d, ad, bd, idesc, accumulate);
+                  accumulate = 1;
+                }
+            } else
 #pragma unroll
             for (int kh = 0; kh < (PT ? 1 : 3); ++kh)
 #pragma unroll
@@ -329,7 +361,9 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     const int r = lg * 32 + lane;     // row of the tile = pixel (r % BW, r / BW)
     constexpr int kRowsPer = BN >= 128 ? 128 : 64;  // rows each thread sums for its channel
     const int sc = et % BN, shalf = et / BN;        // stats: channel and row half of this thread
-    const int rw = r % p.BW, rh = (r / p.BW) % p.BH;  // place of the thread's pixel in its tile
+    // place of the thread's pixel in its tile; HN: rows of the accumulator run over (row, image, column)
+    const int rw = r % p.BW, rh = HN ? r / (p.BW * p.BI) : (r / p.BW) % p.BH;
+    const int sr = HN ? (((r / p.BW) % p.BI) * p.BH + rh) * p.BW + rw : r;  // its row of the staging tile (image, row, column)
     uint32_t sg = 0;                                  // SEG: segments taken so far
     float ssum = 0.f, ssq = 0.f;
     float ssum2 = 0.f, ssq2 = 0.f;                  // BN = 256: the thread's second channel, sc + 128
@@ -373,7 +407,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 32, v);
           ptx::tmem_ld_wait();
         }
-        uint8_t* sub = stg + ((j * 32) / 64) * 16384 + r * 128;
+        uint8_t* sub = stg + ((j * 32) / 64) * 16384 + sr * 128;
         const int u0 = ((j * 32) % 64) / 8;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -396,7 +430,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             for (int e = 0; e < 4; ++e)
               w[e] = bn_relu2(w[e], __ldg(reinterpret_cast<const float2*>(ps) + e), __ldg(reinterpret_cast<const float2*>(ph) + e));
           }
-          *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (r & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
+          *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (sr & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
         }
       }
       if constexpr (!SEG) {
@@ -412,7 +446,9 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
       if (p.stats == 2) {
         // sums of dz and dz*y2 (the last step turns them into sum dz*xhat = invstd * (sum dz*y2 - mu * sum dz))
-        ptx::mbar_wait(yfull, tl & 1, abort_flag);
+        const uint32_t ys = p.yslots == 2 ? tl & 1 : 0;
+        const uint8_t* yb = ybuf + ys * kSub * 16384;
+        ptx::mbar_wait(&yfull[ys], p.yslots == 2 ? (tl >> 1) & 1 : tl & 1, abort_flag);
         const int coff = (sc / 64) * 16384 + (sc % 8) * 2;
         const int u = (sc % 64) / 8;
         const int rb = shalf * kRowsPer;
@@ -421,19 +457,19 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           const int row = rb + rr;
           const int off = coff + row * 128 + ((u ^ (row & 7)) * 16);
           const float d = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(stg + off));
-          const float yv = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(ybuf + off));
+          const float yv = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(yb + off));
           const float dz = fmaf(yv, bsc, bsh) > 0.f ? d : 0.f;
           ssum += dz;
           ssq = fmaf(dz, yv, ssq);
           if constexpr (BN == 256) {
             const float d2 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(stg + 2 * 16384 + off));
-            const float y2 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(ybuf + 2 * 16384 + off));
+            const float y2 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(yb + 2 * 16384 + off));
             const float dz2 = fmaf(y2, bsc2, bsh2) > 0.f ? d2 : 0.f;
             ssum2 += dz2;
             ssq2 = fmaf(dz2, y2, ssq2);
           }
         }
-        ptx::mbar_arrive(yempty);
+        ptx::mbar_arrive(&yempty[ys]);
       } else if (p.stats) {
         const uint8_t* col = stg + (sc / 64) * 16384 + (sc % 8) * 2;
         const int u = (sc % 64) / 8;
@@ -472,7 +508,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const int et = threadIdx.x - 64;
       const int lg = warp & 3;
       const int r = lg * 32 + lane;
-      const int rw = r % p.BW, rh = (r / p.BW) % p.BH, img = r / (p.BW * p.BH);  // place of the thread's pixel in its tile
+      // place of the thread's pixel in its tile
+      const int rw = r % p.BW, rh = HN ? r / (p.BW * p.BI) : (r / p.BW) % p.BH, img = HN ? (r / p.BW) % p.BI : r / (p.BW * p.BH);
       uint32_t sg = 0;
       uint32_t tl = 0;
       for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
@@ -2004,7 +2041,10 @@ EncodeTiledFn encode_fn() {
 }
 
 // bf16 tensor, 4 dims (innermost first), zero fill outside; the swizzle span equals the inner box (32/64/128 bytes)
-int make_map4(CUtensorMap* m, const void* base, const uint64_t dims[4], const uint32_t box[4], int spatial_stride = 1) {
+// rows_last: the map's dimensions run (channel, column, image, row) instead of (channel, column, row, image); dims and box stay in
+// the latter order.
+int make_map4(CUtensorMap* m, const void* base, const uint64_t dims[4], const uint32_t box[4], int spatial_stride = 1,
+              bool rows_last = false) {
   const CUtensorMapSwizzle sw = box[0] * 2 >= 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                 : box[0] * 2 == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
   EncodeTiledFn fn = encode_fn();
@@ -2015,6 +2055,11 @@ int make_map4(CUtensorMap* m, const void* base, const uint64_t dims[4], const ui
   const cuuint32_t ss = (cuuint32_t)spatial_stride;
   cuuint32_t bx[4] = {box[0], box[1] * ss, box[2] * ss, box[3]};
   cuuint32_t es[4] = {1, ss, ss, 1};
+  if (rows_last) {
+    std::swap(gdim[2], gdim[3]);
+    std::swap(gstr[1], gstr[2]);
+    std::swap(bx[2], bx[3]);
+  }
   const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), gdim, gstr, bx, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -2093,12 +2138,24 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   pl.BN = epi != 1 ? (Cout % 128 == 0 ? 128 : 64) : (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64);
   if (epi == 0 && pl.PT && !pl.SEG && Cout % 256 == 0) pl.BN = 256;  // per-tap form: weights of one tap and 256 channels are 32 KB a stage
   pl.KC = epi == 2 ? (Cin <= 16 ? 16 : Cin <= 32 ? 32 : 64) : 64;
-  const size_t a_stride = pl.PT ? (size_t)128 * pl.KC * 2 : ((size_t)(pl.BH + 2) * pl.BW * pl.KC * 2 + 1023) & ~(size_t)1023;
+  size_t a_stride = pl.PT ? (size_t)128 * pl.KC * 2 : ((size_t)(pl.BH + 2) * pl.BW * pl.KC * 2 + 1023) & ~(size_t)1023;
   pl.RW = (!pl.PT && epi != 2 && Cin == 64 && pl.BN <= 64) ? 1 : 0;  // weights resident in shared memory
-  const size_t b_stage = pl.RW ? 0 : pl.PT ? (epi == 2 ? (size_t)(pl.BN / 64) * pl.KC * 128 : (size_t)pl.BN * 128)
+  size_t b_stage = pl.RW ? 0 : pl.PT ? (epi == 2 ? (size_t)(pl.BN / 64) * pl.KC * 128 : (size_t)pl.BN * 128)
                                            : epi == 2 ? (size_t)(pl.BN / 64) * 3 * pl.KC * 128 : (size_t)3 * pl.BN * 128;
+  pl.yslots = ybuf ? 1 : 0;
+  // narrow auxiliary convolutions on several images per tile: three boxes per chunk where the swizzle allows it and two stages (and,
+  // for the gradient, two y2 tiles) fit; maps of one row gain nothing
+  if (pl.PT && stride == 1 && !pl.SEG && pl.BI > 1 && pl.BH > 1 && pl.BI * pl.BW % 8 == 0 && (epi == 1 ? pl.BN <= 32 : epi == 2 && pl.KC == 16)) {
+    const size_t a3 = (size_t)3 * (pl.BH + 2) * pl.BW * pl.BI * pl.KC * 2, b9 = (size_t)9 * (epi == 2 ? pl.BN / 64 * pl.KC : pl.BN) * 128;
+    if (a3 % 3072 == 0 && 2 * (a3 + b9) + (epi == 2 ? (size_t)pl.BN / 64 * 16384 * 3 : 0) + 2048 <= 232448) {
+      pl.PT = 2;
+      a_stride = a3;
+      b_stage = b9;
+      pl.yslots *= 2;
+    }
+  }
   const size_t stage = ((a_stride + 1023) & ~(size_t)1023) + b_stage;
-  const size_t fixed = (size_t)(epi != 1 ? pl.BN / 64 : 0) * 16384 * (ybuf ? 2 : 1) + (pl.RW ? (size_t)9 * pl.BN * 128 : 0) + 1024 + 1024;
+  const size_t fixed = (size_t)(epi != 1 ? pl.BN / 64 : 0) * 16384 * (1 + pl.yslots) + (pl.RW ? (size_t)9 * pl.BN * 128 : 0) + 1024 + 1024;
   int st = (int)((232448 - fixed) / stage);
   if (st > kMaxStages) st = kMaxStages;
   if (st < 2) return pl;
@@ -2298,16 +2355,17 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   const TcPlan pl = plan_fwd(H, W, Cin, Cout, N, epi, stride, stats == 2);
   if (!pl.ok) return NF_EUNSUPPORTED;
   CUtensorMap mx, mw, my;
+  const bool hn = pl.PT == 2;
   const uint64_t dx[4] = {(uint64_t)Cin, (uint64_t)Win, (uint64_t)Hin, (uint64_t)N};
-  const uint32_t bx[4] = {(uint32_t)pl.KC, (uint32_t)pl.BW, (uint32_t)(pl.PT ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
+  const uint32_t bx[4] = {(uint32_t)pl.KC, (uint32_t)pl.BW, (uint32_t)(pl.PT == 1 ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
   // forward: weights [kh][kw][Cout][Cin] -> box of BN rows x 64 ci for three kh; input gradient: weights
   // [kh][kw][F][Cout] -> box of KC rows of f x 64 c for three kh
   const uint64_t dw[4] = {(uint64_t)(epi == 2 ? Cout : Cin), (uint64_t)(epi == 2 ? Cin : Cout), 3, 3};
-  const uint32_t bw[4] = {64, (uint32_t)(epi == 2 ? pl.KC : pl.BN), 1, (uint32_t)(pl.PT ? 1 : 3)};
+  const uint32_t bw[4] = {64, (uint32_t)(epi == 2 ? pl.KC : pl.BN), hn ? 3u : 1u, (uint32_t)(pl.PT == 1 ? 1 : 3)};
   const uint64_t dy[4] = {(uint64_t)Cout, (uint64_t)W, (uint64_t)H, (uint64_t)N};
   const uint32_t by[4] = {64, (uint32_t)pl.BW, (uint32_t)pl.BH, (uint32_t)pl.BI};
   int rc;
-  if ((rc = make_map4(&mx, x, dx, bx, stride)) != NF_OK) return rc;
+  if ((rc = make_map4(&mx, x, dx, bx, stride, hn)) != NF_OK) return rc;
   if ((rc = make_map4(&mw, w, dw, bw)) != NF_OK) return rc;
   if (epi != 1) {
     if ((rc = make_map4(&my, y, dy, by)) != NF_OK) return rc;
@@ -2322,6 +2380,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   p.stride = stride; p.BI = pl.BI;
   p.tg = tile_grid(p.n_tiles, p.tiles_w, p.tiles_h);
   p.kchunks = epi == 2 ? 1 : Cin / 64; p.stages = pl.stages; p.stats = stats; p.red = red; p.status = status;
+  p.yslots = pl.yslots;
   p.tm_y2 = my;
   if (stats == 0 && bn) {
     p.bn_scale = bn->scale; p.bn_shift = bn->shift;
@@ -2348,6 +2407,10 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     if (epi == 0) return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
     return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p)
                        : pl.BN == 32 ? launch_fwd<32, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
+  }
+  if (pl.PT == 2) {
+    if (epi == 1) return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 2>(pl, mx, mw, my, p) : launch_fwd<32, 1, 64, 0, 2>(pl, mx, mw, my, p);
+    return pl.BN == 128 ? launch_fwd<128, 0, 16, 1, 2>(pl, mx, mw, my, p) : launch_fwd<64, 0, 16, 1, 2>(pl, mx, mw, my, p);
   }
   if (pl.PT) {  // per-tap boxes: stride 2, or several small images per tile
     if (epi == 0)
