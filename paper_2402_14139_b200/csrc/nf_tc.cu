@@ -83,6 +83,9 @@ struct Ring {
   }
 };
 
+// a second group of four epilogue warps in the input gradient of tiles of several images
+constexpr int fwd_threads(int epi, int pt) { return epi == 0 && pt == 2 ? kThreads + 128 : kThreads; }
+
 struct FwdParams {
   int N, H, W, Cin, Cout;
   int BW, BH, tiles_w, tiles_h, n_tiles, total_tiles, kchunks, stages;
@@ -146,7 +149,7 @@ __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& ta
 //       2 (HN) = tiles of several images for narrow auxiliary convolutions: the box's dimensions run (channel, column, image, row),
 //       so that a row tap is a constant offset for all images and THREE boxes per chunk serve the nine taps, in one stage with
 //       all the weights.  The per-tap form is bound by its TMA rows (nine boxes of 128) and L2 fill: 512 channels, 8 filters,
-//       8602 maps of 8x8 NNN.
+//       8602 maps of 8x8, forward 352 -> 297 us; input gradient of a pooled 256-channel layer at 16x16 198 -> 126 us.
 // RW  : 1 = all nine weight tiles of the CTA's channel tile stay resident in shared memory for the whole
 //       kernel (single 64-channel K chunk, 9*BN*128 bytes); the pipeline then carries activations only.
 // SEG : 1 (PT, forward only) = a new accumulator every kSegSteps k-steps, the segments added in fp32 by the epilogue.  The tensor
@@ -154,25 +157,27 @@ __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& ta
 //       off the nearest value, against 0.016 % of an fp32 chain.  Maps that no tile divides had such chains (they ran on the CUDA
 //       cores), and their layers are small enough for that to show; a segment's 192 products keep the error below theirs.
 template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(fwd_threads(EPI, PT), 1)
 conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                    const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ FwdParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr int kARow = KC * 2;  // bytes of one pixel row of the activation box
   constexpr uint32_t kALayout = KC == 64 ? 2 : KC == 32 ? 4 : 6;
-  constexpr bool HN = PT == 2;
+  constexpr bool HN = PT == 2, SG = HN && EPI == 0;  // SG: the sums of stats 2 are taken by a warp group of their own
   const int a_box = (p.BH + 2) * p.BW * p.BI * kARow;  // HN: one of the three column-shifted boxes, a multiple of 1024
   const int a_bytes = HN ? 3 * a_box : PT ? 128 * kARow : a_box;
   const int a_stride = (a_bytes + 1023) & ~1023;  // keeps the weight tiles 1024-byte aligned
-  constexpr int b_bytes = RW ? 0 : HN ? 9 * (BMN ? (BN / 64) * KC * 128 : BN * 128) : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
-  constexpr int w_bytes = RW ? 9 * BN * 128 : 0;  // resident weights [kw][kh][BN][64]
+  static_assert(!HN || RW == BMN, "forward: weights in the stages; input gradient: resident");
+  constexpr int b_bytes = RW ? 0 : HN ? 9 * BN * 128 : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
+  constexpr int w_bytes = !RW ? 0 : BMN ? 9 * (BN / 64) * KC * 128 : 9 * BN * 128;  // resident weights [kw][kh][BN][64] (BMN: [half][kh][kw][KC][64])
   const int stage_bytes = a_stride + b_bytes;
   constexpr int kSub = EPI == 0 ? BN / 64 : 0;  // 64-channel sub-tiles of the output staging
   uint8_t* wres = smem + (size_t)p.stages * stage_bytes;
   uint8_t* stg = wres + w_bytes;
-  uint8_t* ybuf = stg + kSub * 16384;  // stats 2: the y2 tile of the tile in the epilogue (kSub sub-tiles)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(stg + (p.stats == 2 ? 1 + p.yslots : 1) * kSub * 16384);
+  constexpr int kStg = SG ? 2 : 1;              // staging tiles
+  uint8_t* ybuf = stg + kStg * kSub * 16384;  // stats 2: the y2 tile of the tile in the epilogue (kSub sub-tiles)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(ybuf + (p.stats == 2 ? p.yslots : 0) * kSub * 16384);
   uint64_t* full = bars;
   uint64_t* empty = bars + kMaxStages;
   uint64_t* tfull = bars + 2 * kMaxStages;
@@ -181,7 +186,9 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   uint64_t* wfull = tempty + kAccs;
   uint64_t* yfull = wfull + 1;
   uint64_t* yempty = yfull + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(yempty + 2);
+  uint64_t* sfull = yempty + 2;  // SG: staging tile written / its sums taken
+  uint64_t* sfree = sfull + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sfree + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* epi_go = reinterpret_cast<volatile int*>(tmem_slot + 2);
 
@@ -200,6 +207,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&yfull[i], 1);
       ptx::mbar_init(&yempty[i], 128);
+      ptx::mbar_init(&sfull[i], 128);
+      ptx::mbar_init(&sfree[i], 128);
     }
     *abort_flag = 0;
     ptx::fence_mbar_init();
@@ -227,8 +236,14 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if constexpr (RW) {
         if (blockIdx.x < p.total_tiles) {
           ptx::mbar_expect_tx(wfull, (uint32_t)w_bytes);
+          if constexpr (BMN) {
 #pragma unroll
-          for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(wres + kw * 3 * BN * 128, &tm_w, wfull, 0, (blockIdx.x % p.n_tiles) * BN, kw, 0);
+            for (int hf = 0; hf < BN / 64; ++hf)
+              ptx::tma_load_4d(wres + hf * 9 * KC * 128, &tm_w, wfull, (blockIdx.x % p.n_tiles) * BN + hf * 64, 0, 0, 0);
+          } else {
+#pragma unroll
+            for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(wres + kw * 3 * BN * 128, &tm_w, wfull, 0, (blockIdx.x % p.n_tiles) * BN, kw, 0);
+          }
         }
       }
       Ring rg;
@@ -247,11 +262,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             if constexpr (HN) {
 #pragma unroll
               for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(a_s + kw * a_box, &tm_x, fb, ck * KC, w0 + kw - 1, n, h0 - 1);
-              if constexpr (BMN) {
-#pragma unroll
-                for (int hf = 0; hf < BN / 64; ++hf)  // [half][kh][kw][KC rows of f][64 channels]
-                  ptx::tma_load_4d(a_s + a_stride + hf * 9 * KC * 128, &tm_w, fb, co0 + hf * 64, 0, 0, 0);
-              } else {
+              if constexpr (!RW) {
                 ptx::tma_load_4d(a_s + a_stride, &tm_w, fb, ck * 64, co0, 0, 0);  // [kh][kw][BN][64]
               }
             } else if constexpr (PT) {
@@ -379,7 +390,39 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         bsh2 = p.bn_shift[ch + 128];
       }
     }
-    for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
+    const bool sums = SG && warp >= 6;
+    if constexpr (SG) {
+      if (sums && p.stats == 2) {
+        // sums of (dz, dz * y2), one channel per thread in row order as below, while the other group stages the next tile (that
+        // work in one group took 8000 cycles per 128 x 128 tile whose products take 600)
+        const int st = threadIdx.x - 192, c = st % BN, half = st / BN;
+        const float fsc = p.bn_scale[my_nt * BN + c], fsh = p.bn_shift[my_nt * BN + c];
+        for (int t = blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
+          const uint32_t bsel = tl & 1, ph = (tl >> 1) & 1;
+          if (!ptx::mbar_wait(&yfull[bsel], ph, abort_flag) || !ptx::mbar_wait(&sfull[bsel], ph, abort_flag)) break;
+          const uint8_t* dcol = stg + bsel * kSub * 16384 + (c / 64) * 16384 + (c % 8) * 2 + half * kRowsPer * 128;
+          const uint8_t* ycol = ybuf + bsel * kSub * 16384 + (c / 64) * 16384 + (c % 8) * 2 + half * kRowsPer * 128;
+          const int u = (c % 64) / 8;
+#pragma unroll 16
+          for (int row = 0; row < kRowsPer; ++row) {
+            const int off = row * 128 + ((u ^ (row & 7)) * 16);
+            const float d = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(dcol + off));
+            const float yv = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(ycol + off));
+            const float dz = fmaf(yv, fsc, fsh) > 0.f ? d : 0.f;
+            ssum += dz;
+            ssq = fmaf(dz, yv, ssq);
+          }
+          ptx::mbar_arrive(&yempty[bsel]);
+          ptx::mbar_arrive(&sfree[bsel]);
+        }
+        const int ch = my_nt * BN + c;
+        ssq = (float)((double)p.bn_invstd[ch] * ((double)ssq - (double)p.bn_mu[ch] * (double)ssum));
+        const size_t row = (size_t)(blockIdx.x / p.n_tiles) * (128 / BN) + half;
+        p.red[(row * 2 + 0) * p.Cout + ch] = ssum;
+        p.red[(row * 2 + 1) * p.Cout + ch] = ssq;
+      }
+    }
+    for (int t = sums ? p.total_tiles : blockIdx.x; t < p.total_tiles; t += gridDim.x, ++tl) {
       const TileAt at = tile_at(t, p.tg);
       const int nt = at.nt, w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
       const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
@@ -390,8 +433,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         ptx::mbar_wait(&tfull[acc], aph, abort_flag);  // sets the abort flag itself when it gives up
         ptx::tc_fence_after();
       }
+      uint8_t* const stile = stg + (SG ? (tl & 1) * kSub * 16384 : 0);
+      if constexpr (SG) {
+        if (p.stats == 2) ptx::mbar_wait(&sfree[tl & 1], ((tl >> 1) & 1) ^ 1, abort_flag);
+      }
       if (et == 0) {
-        ptx::tma_store_wait_read();  // the previous tile's store has finished reading the staging tile
+        // the last store out of this staging tile has finished reading it
+        if constexpr (SG) ptx::tma_store_wait_read_but_one(); else ptx::tma_store_wait_read();
         *epi_go = *abort_flag ? 0 : 1;  // one thread decides for all 128, so nobody is left alone at a barrier
       }
       ptx::named_barrier(1, 128);
@@ -407,7 +455,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 32, v);
           ptx::tmem_ld_wait();
         }
-        uint8_t* sub = stg + ((j * 32) / 64) * 16384 + sr * 128;
+        uint8_t* sub = stile + ((j * 32) / 64) * 16384 + sr * 128;
         const int u0 = ((j * 32) % 64) / 8;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -441,8 +489,12 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       ptx::named_barrier(1, 128);
       if (et == 0) {
 #pragma unroll
-        for (int sb = 0; sb < kSub; ++sb) ptx::tma_store_4d(&tm_y, stg + sb * 16384, nt * BN + sb * 64, w0, h0, n);
+        for (int sb = 0; sb < kSub; ++sb) ptx::tma_store_4d(&tm_y, stile + sb * 16384, nt * BN + sb * 64, w0, h0, n);
         ptx::tma_store_commit();
+      }
+      if constexpr (SG) {
+        if (p.stats == 2) ptx::mbar_arrive(&sfull[tl & 1]);
+        continue;
       }
       if (p.stats == 2) {
         // sums of dz and dz*y2 (the last step turns them into sum dz*xhat = invstd * (sum dz*y2 - mu * sum dz))
@@ -489,7 +541,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       }
     }
     if (et == 0) ptx::tma_store_wait_all();
-    if (p.stats) {
+    if (!SG && p.stats) {
       constexpr int parts = 128 / BN > 0 ? 128 / BN : 1;
       const size_t b = (size_t)(blockIdx.x / p.n_tiles) * parts + shalf;  // the CTAs of one pixel range fill one row of partials
       if (p.stats == 2) {
@@ -2143,19 +2195,23 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   size_t b_stage = pl.RW ? 0 : pl.PT ? (epi == 2 ? (size_t)(pl.BN / 64) * pl.KC * 128 : (size_t)pl.BN * 128)
                                            : epi == 2 ? (size_t)(pl.BN / 64) * 3 * pl.KC * 128 : (size_t)3 * pl.BN * 128;
   pl.yslots = ybuf ? 1 : 0;
+  size_t extra = pl.RW ? (size_t)9 * pl.BN * 128 : 0;
   // narrow auxiliary convolutions on several images per tile: three boxes per chunk where the swizzle allows it and two stages (and,
   // for the gradient, two y2 tiles) fit; maps of one row gain nothing
   if (pl.PT && stride == 1 && !pl.SEG && pl.BI > 1 && pl.BH > 1 && pl.BI * pl.BW % 8 == 0 && (epi == 1 ? pl.BN <= 32 : epi == 2 && pl.KC == 16)) {
     const size_t a3 = (size_t)3 * (pl.BH + 2) * pl.BW * pl.BI * pl.KC * 2, b9 = (size_t)9 * (epi == 2 ? pl.BN / 64 * pl.KC : pl.BN) * 128;
-    if (a3 % 3072 == 0 && 2 * (a3 + b9) + (epi == 2 ? (size_t)pl.BN / 64 * 16384 * 3 : 0) + 2048 <= 232448) {
+    const size_t staged = epi == 2 ? (size_t)pl.BN / 64 * 16384 : 0;  // two output tiles, two of y2
+    if (a3 % 3072 == 0 && 2 * a3 + (epi == 2 ? 1 : 2) * b9 + 4 * staged + 2048 <= 232448) {
       pl.PT = 2;
+      pl.RW = epi == 2;
       a_stride = a3;
-      b_stage = b9;
+      b_stage = epi == 2 ? 0 : b9;
       pl.yslots *= 2;
+      extra = staged + (epi == 2 ? b9 : 0);
     }
   }
   const size_t stage = ((a_stride + 1023) & ~(size_t)1023) + b_stage;
-  const size_t fixed = (size_t)(epi != 1 ? pl.BN / 64 : 0) * 16384 * (1 + pl.yslots) + (pl.RW ? (size_t)9 * pl.BN * 128 : 0) + 1024 + 1024;
+  const size_t fixed = (size_t)(epi != 1 ? pl.BN / 64 : 0) * 16384 * (1 + pl.yslots) + extra + 1024 + 1024;
   int st = (int)((232448 - fixed) / stage);
   if (st > kMaxStages) st = kMaxStages;
   if (st < 2) return pl;
@@ -2182,7 +2238,7 @@ int launch_fwd(const TcPlan& pl, const CUtensorMap& mx, const CUtensorMap& mw, c
     NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, pl.grid, kThreads, pl.smem, mx, mw, my, p);
+  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, pl.grid, fwd_threads(EPI, PT), pl.smem, mx, mw, my, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2410,7 +2466,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   }
   if (pl.PT == 2) {
     if (epi == 1) return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 2>(pl, mx, mw, my, p) : launch_fwd<32, 1, 64, 0, 2>(pl, mx, mw, my, p);
-    return pl.BN == 128 ? launch_fwd<128, 0, 16, 1, 2>(pl, mx, mw, my, p) : launch_fwd<64, 0, 16, 1, 2>(pl, mx, mw, my, p);
+    return pl.BN == 128 ? launch_fwd<128, 0, 16, 1, 2, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 16, 1, 2, 1>(pl, mx, mw, my, p);
   }
   if (pl.PT) {  // per-tap boxes: stride 2, or several small images per tile
     if (epi == 0)
