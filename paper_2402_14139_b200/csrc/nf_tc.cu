@@ -172,7 +172,10 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   constexpr int b_bytes = RW ? 0 : HN ? 9 * BN * 128 : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
   constexpr int w_bytes = !RW ? 0 : BMN ? 9 * (BN / 64) * KC * 128 : 9 * BN * 128;  // resident weights [kw][kh][BN][64] (BMN: [half][kh][kw][KC][64])
   const int stage_bytes = a_stride + b_bytes;
-  constexpr int kSub = EPI == 0 ? BN / 64 : 0;  // 64-channel sub-tiles of the output staging
+  // 256 channels leave through staging (and y2) tiles of 128, one half after the other: with 32 KB instead of 64 the ring gets four
+  // stages of 48 KB for three, three for two beside y2 tiles (a stage is multiplied in 512 cycles, a fill takes over 1000)
+  constexpr int kHalf = BN == 256 ? 2 : 1;
+  constexpr int kSub = EPI == 0 ? BN / 64 / kHalf : 0;  // 64-channel sub-tiles of the output staging
   uint8_t* wres = smem + (size_t)p.stages * stage_bytes;
   uint8_t* stg = wres + w_bytes;
   constexpr int kStg = SG ? 2 : 1;              // staging tiles
@@ -290,7 +293,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         if constexpr (EPI == 0) {
           // the y2 tile of this output tile goes out after its operand loads: its buffer is free once the epilogue has finished
           // the statistics of the previous tile (of the one before with two buffers), which it does while this tile is multiplied
-          if (ok && p.stats == 2) {
+          if (kHalf == 1 && ok && p.stats == 2) {
             const uint32_t ys = p.yslots == 2 ? ptl & 1 : 0, yph = p.yslots == 2 ? (ptl >> 1) & 1 : ptl & 1;
             if (!ptx::mbar_wait(&yempty[ys], yph ^ 1, abort_flag)) break;
             ptx::mbar_expect_tx(&yfull[ys], (uint32_t)(kSub * 16384));
@@ -433,112 +436,119 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         ptx::mbar_wait(&tfull[acc], aph, abort_flag);  // sets the abort flag itself when it gives up
         ptx::tc_fence_after();
       }
-      uint8_t* const stile = stg + (SG ? (tl & 1) * kSub * 16384 : 0);
-      if constexpr (SG) {
-        if (p.stats == 2) ptx::mbar_wait(&sfree[tl & 1], ((tl >> 1) & 1) ^ 1, abort_flag);
-      }
-      if (et == 0) {
-        // the last store out of this staging tile has finished reading it
-        if constexpr (SG) ptx::tma_store_wait_read_but_one(); else ptx::tma_store_wait_read();
-        *epi_go = *abort_flag ? 0 : 1;  // one thread decides for all 128, so nobody is left alone at a barrier
-      }
-      ptx::named_barrier(1, 128);
-      if (!*epi_go) break;
-      const bool inside = w0 + rw < p.W && h0 + rh < p.H;  // a pixel over the edge is staged as zero: it adds nothing to the sums
+      bool go = true;
 #pragma unroll
-      for (int j = 0; j < BN / 32; ++j) {
-        uint32_t v[32];
-        if constexpr (SEG) {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(seg[j * 32 + e]);
-        } else {
-          ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + j * 32, v);
-          ptx::tmem_ld_wait();
+      for (int hf = 0; hf < kHalf; ++hf) {
+        const int ch0 = nt * BN + hf * 128;  // first channel of the half
+        uint8_t* const stile = stg + (SG ? (tl & 1) * kSub * 16384 : 0);
+        if constexpr (SG) {
+          if (p.stats == 2) ptx::mbar_wait(&sfree[tl & 1], ((tl >> 1) & 1) ^ 1, abort_flag);
         }
-        uint8_t* sub = stile + ((j * 32) / 64) * 16384 + sr * 128;
-        const int u0 = ((j * 32) % 64) / 8;
+        if (et == 0) {
+          // the last store out of this staging tile has finished reading it
+          if constexpr (SG) ptx::tma_store_wait_read_but_one(); else ptx::tma_store_wait_read();
+          *epi_go = *abort_flag ? 0 : 1;  // one thread decides for all 128, so nobody is left alone at a barrier
+        }
+        ptx::named_barrier(1, 128);
+        if (!*epi_go) {
+          go = false;
+          break;
+        }
+        if constexpr (kHalf == 2) {
+          if (et == 0 && p.stats == 2) {  // every thread has passed the last half's sums
+            ptx::mbar_expect_tx(yfull, (uint32_t)(kSub * 16384));
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          uint32_t w[4];
+            for (int sb = 0; sb < kSub; ++sb) ptx::tma_load_4d(ybuf + sb * 16384, &p.tm_y2, yfull, ch0 + sb * 64, w0, h0, n);
+          }
+        }
+        const bool inside = w0 + rw < p.W && h0 + rh < p.H;  // a pixel over the edge is staged as zero: it adds nothing to the sums
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            float o0 = __uint_as_float(v[q * 8 + 2 * e]), o1 = __uint_as_float(v[q * 8 + 2 * e + 1]);
-            if (p.bias) {  // wide aux forward: bias and ReLU before the value is rounded for storage
-              const float* bch = p.bias + nt * BN + j * 32 + q * 8 + 2 * e;
-              o0 = fmaxf(o0 + __ldg(bch), 0.f);
-              o1 = fmaxf(o1 + __ldg(bch + 1), 0.f);
+        for (int j = 0; j < BN / kHalf / 32; ++j) {
+          uint32_t v[32];
+          if constexpr (SEG) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(seg[j * 32 + e]);
+          } else {
+            ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + hf * 128 + j * 32, v);
+            ptx::tmem_ld_wait();
+          }
+          uint8_t* sub = stile + ((j * 32) / 64) * 16384 + sr * 128;
+          const int u0 = ((j * 32) % 64) / 8;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              float o0 = __uint_as_float(v[q * 8 + 2 * e]), o1 = __uint_as_float(v[q * 8 + 2 * e + 1]);
+              if (p.bias) {  // wide aux forward: bias and ReLU before the value is rounded for storage
+                const float* bch = p.bias + ch0 + j * 32 + q * 8 + 2 * e;
+                o0 = fmaxf(o0 + __ldg(bch), 0.f);
+                o1 = fmaxf(o1 + __ldg(bch + 1), 0.f);
+              }
+              const __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
+              w[e] = *reinterpret_cast<const uint32_t*>(&b2);
             }
-            const __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
-            w[e] = *reinterpret_cast<const uint32_t*>(&b2);
-          }
-          if constexpr (POST) {
-            const float* ps = p.bn_scale + nt * BN + j * 32 + q * 8;
-            const float* ph = p.bn_shift + nt * BN + j * 32 + q * 8;
+            if constexpr (POST) {
+              const float* ps = p.bn_scale + ch0 + j * 32 + q * 8;
+              const float* ph = p.bn_shift + ch0 + j * 32 + q * 8;
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-              w[e] = bn_relu2(w[e], __ldg(reinterpret_cast<const float2*>(ps) + e), __ldg(reinterpret_cast<const float2*>(ph) + e));
+              for (int e = 0; e < 4; ++e)
+                w[e] = bn_relu2(w[e], __ldg(reinterpret_cast<const float2*>(ps) + e), __ldg(reinterpret_cast<const float2*>(ph) + e));
+            }
+            *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (sr & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
           }
-          *reinterpret_cast<uint4*>(sub + (((u0 + q) ^ (sr & 7)) * 16)) = inside ? make_uint4(w[0], w[1], w[2], w[3]) : make_uint4(0u, 0u, 0u, 0u);
         }
-      }
-      if constexpr (!SEG) {
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(&tempty[acc]);
-      }
-      ptx::fence_async_smem();
-      ptx::named_barrier(1, 128);
-      if (et == 0) {
+        if (!SEG && hf == kHalf - 1) {
+          ptx::tc_fence_before();
+          ptx::mbar_arrive(&tempty[acc]);
+        }
+        ptx::fence_async_smem();
+        ptx::named_barrier(1, 128);
+        if (et == 0) {
 #pragma unroll
-        for (int sb = 0; sb < kSub; ++sb) ptx::tma_store_4d(&tm_y, stile + sb * 16384, nt * BN + sb * 64, w0, h0, n);
-        ptx::tma_store_commit();
-      }
-      if constexpr (SG) {
-        if (p.stats == 2) ptx::mbar_arrive(&sfull[tl & 1]);
-        continue;
-      }
-      if (p.stats == 2) {
-        // sums of dz and dz*y2 (the last step turns them into sum dz*xhat = invstd * (sum dz*y2 - mu * sum dz))
-        const uint32_t ys = p.yslots == 2 ? tl & 1 : 0;
-        const uint8_t* yb = ybuf + ys * kSub * 16384;
-        ptx::mbar_wait(&yfull[ys], p.yslots == 2 ? (tl >> 1) & 1 : tl & 1, abort_flag);
-        const int coff = (sc / 64) * 16384 + (sc % 8) * 2;
-        const int u = (sc % 64) / 8;
-        const int rb = shalf * kRowsPer;
-#pragma unroll 8
-        for (int rr = 0; rr < kRowsPer; ++rr) {
-          const int row = rb + rr;
-          const int off = coff + row * 128 + ((u ^ (row & 7)) * 16);
-          const float d = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(stg + off));
-          const float yv = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(yb + off));
-          const float dz = fmaf(yv, bsc, bsh) > 0.f ? d : 0.f;
-          ssum += dz;
-          ssq = fmaf(dz, yv, ssq);
-          if constexpr (BN == 256) {
-            const float d2 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(stg + 2 * 16384 + off));
-            const float y2 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(yb + 2 * 16384 + off));
-            const float dz2 = fmaf(y2, bsc2, bsh2) > 0.f ? d2 : 0.f;
-            ssum2 += dz2;
-            ssq2 = fmaf(dz2, y2, ssq2);
-          }
+          for (int sb = 0; sb < kSub; ++sb) ptx::tma_store_4d(&tm_y, stile + sb * 16384, ch0 + sb * 64, w0, h0, n);
+          ptx::tma_store_commit();
         }
-        ptx::mbar_arrive(&yempty[ys]);
-      } else if (p.stats) {
-        const uint8_t* col = stg + (sc / 64) * 16384 + (sc % 8) * 2;
-        const int u = (sc % 64) / 8;
-        const int rb = shalf * kRowsPer;
+        if constexpr (SG) {
+          if (p.stats == 2) ptx::mbar_arrive(&sfull[tl & 1]);
+          continue;
+        }
+        if (p.stats == 2) {
+          // sums of dz and dz*y2 (the last step turns them into sum dz*xhat = invstd * (sum dz*y2 - mu * sum dz))
+          const uint32_t ys = p.yslots == 2 ? tl & 1 : 0;
+          const uint8_t* yb = ybuf + ys * kSub * 16384;
+          ptx::mbar_wait(&yfull[ys], kHalf == 2 ? hf : p.yslots == 2 ? (tl >> 1) & 1 : tl & 1, abort_flag);
+          const float csc = hf ? bsc2 : bsc, csh = hf ? bsh2 : bsh;
+          float &sum = hf ? ssum2 : ssum, &sq = hf ? ssq2 : ssq;
+          const int coff = (sc / 64) * 16384 + (sc % 8) * 2;
+          const int u = (sc % 64) / 8;
+          const int rb = shalf * kRowsPer;
 #pragma unroll 8
-        for (int rr = 0; rr < kRowsPer; ++rr) {
-          const int row = rb + rr;
-          const float v = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(col + row * 128 + ((u ^ (row & 7)) * 16)));
-          ssum += v;
-          ssq = fmaf(v, v, ssq);
-          if constexpr (BN == 256) {
-            const float v2 = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(col + 2 * 16384 + row * 128 + ((u ^ (row & 7)) * 16)));
-            ssum2 += v2;
-            ssq2 = fmaf(v2, v2, ssq2);
+          for (int rr = 0; rr < kRowsPer; ++rr) {
+            const int row = rb + rr;
+            const int off = coff + row * 128 + ((u ^ (row & 7)) * 16);
+            const float d = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(stg + off));
+            const float yv = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(yb + off));
+            const float dz = fmaf(yv, csc, csh) > 0.f ? d : 0.f;
+            sum += dz;
+            sq = fmaf(dz, yv, sq);
+          }
+          ptx::mbar_arrive(&yempty[ys]);
+        } else if (p.stats) {
+          float &sum = hf ? ssum2 : ssum, &sq = hf ? ssq2 : ssq;
+          const uint8_t* col = stg + (sc / 64) * 16384 + (sc % 8) * 2;
+          const int u = (sc % 64) / 8;
+          const int rb = shalf * kRowsPer;
+#pragma unroll 8
+          for (int rr = 0; rr < kRowsPer; ++rr) {
+            const int row = rb + rr;
+            const float v = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(col + row * 128 + ((u ^ (row & 7)) * 16)));
+            sum += v;
+            sq = fmaf(v, v, sq);
           }
         }
       }
+      if (!go) break;
     }
     if (et == 0) ptx::tma_store_wait_all();
     if (!SG && p.stats) {
@@ -2211,7 +2221,7 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
     }
   }
   const size_t stage = ((a_stride + 1023) & ~(size_t)1023) + b_stage;
-  const size_t fixed = (size_t)(epi != 1 ? pl.BN / 64 : 0) * 16384 * (1 + pl.yslots) + extra + 1024 + 1024;
+  const size_t fixed = (size_t)(epi != 1 ? (pl.BN == 256 ? 2 : pl.BN / 64) : 0) * 16384 * (1 + pl.yslots) + extra + 1024 + 1024;
   int st = (int)((232448 - fixed) / stage);
   if (st > kMaxStages) st = kMaxStages;
   if (st < 2) return pl;
