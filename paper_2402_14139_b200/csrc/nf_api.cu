@@ -364,6 +364,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   trace_begin(0);
   if (L->fam[0]) {
     NF_TRY(nf_tc_conv_fwd(L, x, nb));
+    if (!nb) NF_TRY(nf_k_channel_sums(dt, L->y, (size_t)N * Ho * Wo, Co, L->red, L->red_floats, &nb));
   } else {
     NF_TRY(nf_k_conv(dt, x, N, L->H, L->W, Ci, Wm, (long)Co * Ci, Ci, 1, 0, nullptr, 0, s, Co, L->y));
     NF_TRY(nf_k_channel_sums(dt, L->y, (size_t)N * Ho * Wo, Co, L->red, L->red_floats, &nb));

@@ -654,17 +654,18 @@ __global__ void unpad_grad_kernel(const float* __restrict__ gwpad, size_t rows, 
 
 // out[i] = sum over the splits of part[k][i]: eight chains (split k in chain k % 8) in index order, the chains added in order.  V
 // consecutive elements per thread (4: 16-byte loads); LN = 8: a thread per chain, for many splits of few elements (148 of
-// 36 864); LN = 1: one thread runs all chains, for fewer than 16 splits (at most two terms each) of many elements.
-template <int V, int LN>
+// 36 864); LN = 1: one thread runs all chains, for fewer than 16 splits (at most two terms each) of many elements.  A: type of the
+// chains (double: partials whose own error is below a rounding of the sum).
+template <int V, int LN, typename A>
 __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict__ part, int splits, size_t n, float* __restrict__ out) {
   nf_pdl_begin();
   constexpr int kCols = 256 / LN;
-  __shared__ float sm[LN][kCols * V];
+  __shared__ A sm[LN][kCols * V];
   const int tx = threadIdx.x % kCols, ty = threadIdx.x / kCols;
   const size_t i = ((size_t)blockIdx.x * kCols + tx) * V;
-  float s[V];
+  A s[V];
 #pragma unroll
-  for (int e = 0; e < V; ++e) s[e] = 0.f;
+  for (int e = 0; e < V; ++e) s[e] = 0;
   auto term = [&](int k, float(&v)[V]) {
     const float* src = part + (size_t)k * n + i;
     if constexpr (V == 4) {
@@ -688,11 +689,11 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
     for (int e = 0; e < V; ++e) sm[ty][tx * V + e] = s[e];
     __syncthreads();
     if (threadIdx.x < kCols * V) {  // one thread per element
-      float v = sm[0][threadIdx.x];
+      A v = sm[0][threadIdx.x];
 #pragma unroll
       for (int l = 1; l < LN; ++l) v += sm[l][threadIdx.x];
       const size_t o = (size_t)blockIdx.x * kCols * V + threadIdx.x;
-      if (o < n) out[o] = v;
+      if (o < n) out[o] = (float)v;
     }
   } else if (i < n) {
     const int heads = splits < 8 ? splits : 8;
@@ -704,12 +705,12 @@ __global__ void __launch_bounds__(256) sum_parts_kernel(const float* __restrict_
       for (int e = 0; e < V; ++e) w[e] = 0.f;
       if (k + 8 < splits) term(k + 8, w);
 #pragma unroll
-      for (int e = 0; e < V; ++e) s[e] += v[e] + w[e];
+      for (int e = 0; e < V; ++e) s[e] += (A)v[e] + (A)w[e];
     }
     if constexpr (V == 4) {
-      *reinterpret_cast<float4*>(out + i) = make_float4(s[0], s[1], s[2], s[3]);
+      *reinterpret_cast<float4*>(out + i) = make_float4((float)s[0], (float)s[1], (float)s[2], (float)s[3]);
     } else {
-      out[i] = s[0];
+      out[i] = (float)s[0];
     }
   }
 }
@@ -1940,15 +1941,21 @@ int nf_k_unpad_grad(const float* gwpad, size_t rows, int C, int Cp, float* gw) {
   return NF_OK;
 }
 
-int nf_k_sum_parts(const float* part, int splits, size_t n, float* out) {
+template <typename A>
+static void sum_parts(const float* part, int splits, size_t n, float* out) {
   const bool vec = n % 4 == 0 && (((uintptr_t)part | (uintptr_t)out) & 15) == 0;
   if (splits >= 16) {
-    if (vec) nf_launch(sum_parts_kernel<4, 8>, nblk(n, 128), 256, 0, part, splits, n, out);
-    else nf_launch(sum_parts_kernel<1, 8>, nblk(n, 32), 256, 0, part, splits, n, out);
+    if (vec) nf_launch(sum_parts_kernel<4, 8, A>, nblk(n, 128), 256, 0, part, splits, n, out);
+    else nf_launch(sum_parts_kernel<1, 8, A>, nblk(n, 32), 256, 0, part, splits, n, out);
   } else {
-    if (vec) nf_launch(sum_parts_kernel<4, 1>, nblk(n, 1024), 256, 0, part, splits, n, out);
-    else nf_launch(sum_parts_kernel<1, 1>, nblk(n, 256), 256, 0, part, splits, n, out);
+    if (vec) nf_launch(sum_parts_kernel<4, 1, A>, nblk(n, 1024), 256, 0, part, splits, n, out);
+    else nf_launch(sum_parts_kernel<1, 1, A>, nblk(n, 256), 256, 0, part, splits, n, out);
   }
+}
+
+int nf_k_sum_parts(const float* part, int splits, size_t n, float* out, bool fp64) {
+  if (fp64) sum_parts<double>(part, splits, n, out);
+  else sum_parts<float>(part, splits, n, out);
   NF_LAUNCHED();
   return NF_OK;
 }

@@ -128,8 +128,8 @@ int nf_k_conv_taps(int dtype, const void* x, int N, int H, int W, int Ci, const 
 int nf_k_wgrad_splits(int N, int Ho, int Ci, int Co);
 int nf_k_wgrad(int dtype, const void* x, int N, int H, int W, int Ci, const void* g, int Co, int stride,
                  float* part, size_t part_floats, float* dw);
-// out[i] = sum over k of part[k][i], i < n: the split partials of a weight gradient
-int nf_k_sum_parts(const float* part, int splits, size_t n, float* out);
+// out[i] = sum over k of part[k][i], i < n: the split partials of a weight gradient, added in fp32 or fp64
+int nf_k_sum_parts(const float* part, int splits, size_t n, float* out, bool fp64 = false);
 int nf_k_channel_blocks(size_t P, int C);
 int nf_k_channel_sums(int dtype, const void* src, size_t P, int C, float* red, size_t red_floats, int* nblocks);
 int nf_k_bn_finalize(const float* red, int nblocks, int C, double M, const float* gamma, const float* beta,

@@ -22,7 +22,6 @@ namespace {
 
 constexpr int kThreads = 192;  // warp 0: TMA producer, warp 1: MMA issuer + TMEM owner, warps 2-5: epilogue
 constexpr int kMaxStages = 8;
-constexpr int kSegSteps = 3;  // k-steps of 64 products per accumulator in the segmented forward
 // normalisation threads of the fused BatchNorm + aux forward: two groups of 128 that take the stages in turn.  A single group
 // was the slowest role of the kernel (busy 2350 of every 2450 cycles per tile while the issuer waited 520 on it: one warp per
 // scheduler cannot hide the latency of its load - arithmetic - store - fence chain).  Splitting the ten rows of ONE box over
@@ -90,6 +89,7 @@ struct FwdParams {
   int N, H, W, Cin, Cout;
   int BW, BH, tiles_w, tiles_h, n_tiles, total_tiles, kchunks, stages;
   int stride, BI;     // PT mode: conv stride and images per tile (BW*BH*BI = 128)
+  int seg_steps;      // SEG: k-steps per accumulator
   TileGrid tg;
   int stats, yslots;  // yslots: buffers for the tiles of y2
   float* red;         // [grid / n_tiles * parts][2][Cout] channel partials
@@ -152,10 +152,10 @@ __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& ta
 //       8602 maps of 8x8, forward 352 -> 297 us; input gradient of a pooled 256-channel layer at 16x16 198 -> 126 us.
 // RW  : 1 = all nine weight tiles of the CTA's channel tile stay resident in shared memory for the whole
 //       kernel (single 64-channel K chunk, 9*BN*128 bytes); the pipeline then carries activations only.
-// SEG : 1 (PT, forward only) = a new accumulator every kSegSteps k-steps, the segments added in fp32 by the epilogue.  The tensor
+// SEG : 1 (PT) = a new accumulator every seg_steps k-steps, the segments added in fp32 by the epilogue.  The tensor
 //       core's running sum drops low bits on every instruction: over 2304 products 0.07 % of the bf16 outputs came out one unit
 //       off the nearest value, against 0.016 % of an fp32 chain.  Maps that no tile divides had such chains (they ran on the CUDA
-//       cores), and their layers are small enough for that to show; a segment's 192 products keep the error below theirs.
+//       cores), and their layers are small enough for that to show; seg_steps (run_fwd) keeps the error below theirs.
 template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0>
 __global__ void __launch_bounds__(fwd_threads(EPI, PT), 1)
 conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
@@ -219,7 +219,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     ptx::prefetch_tmap(&tm_w);
     ptx::prefetch_tmap(&tm_y);
   }
-  static_assert(!SEG || (PT && !BMN && BN <= 128), "segmented accumulation: per-tap forward");
+  static_assert(!SEG || (PT == 1 && BN <= 128), "segmented accumulation: per-tap form");
   constexpr uint32_t kTmemCols = kAccs * BN < 32 ? 32 : kAccs * BN;
   if (warp == 1) {
     ptx::tmem_alloc(tmem_slot, kTmemCols);
@@ -318,14 +318,14 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if constexpr (RW) {
         if (blockIdx.x < p.total_tiles) ok = ptx::mbar_wait(wfull, 0, abort_flag);
       }
-      const int steps = (HN ? 1 : PT ? 9 : 3) * p.kchunks;
+      const int steps = (HN ? 1 : PT ? 9 : 3) * p.kchunks, seg = SEG ? p.seg_steps : steps;
       for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
         uint32_t acc = 0, d = 0, accumulate = 0;
-        int step = 0;
+        int step = 0, in_seg = 0;  // in_seg: k-steps of the segment so far
         for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
           for (int tap = 0; tap < (HN ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
-            if (step == 0 || (SEG && step % kSegSteps == 0)) {
+            if (in_seg == 0) {
               acc = tl % kAccs;
               if (!ptx::mbar_wait(&tempty[acc], ((tl / kAccs) & 1) ^ 1, abort_flag)) { ok = false; break; }
               ++tl;
@@ -333,6 +333,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
               accumulate = 0;
             }
             ++step;
+            ++in_seg;
             if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
             ptx::tc_fence_after();
             const uint32_t a_base = ptx::smem_u32(smem) + rg.s * stage_bytes;
@@ -361,7 +362,10 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
                 accumulate = 1;
               }
             ptx::mma_commit(&empty[rg.s]);
-            if (step == steps || (SEG && step % kSegSteps == 0)) ptx::mma_commit(&tfull[acc]);
+            if (step == steps || in_seg == seg) {
+              ptx::mma_commit(&tfull[acc]);
+              in_seg = 0;
+            }
           }
         }
       }
@@ -431,7 +435,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
       float seg[SEG ? BN : 1];
       if constexpr (SEG) {
-        add_segments<BN>(tmem_base + ((uint32_t)(lg * 32) << 16), (9 * p.kchunks + kSegSteps - 1) / kSegSteps, sg, tfull, tempty, abort_flag, seg);
+        add_segments<BN>(tmem_base + ((uint32_t)(lg * 32) << 16), (9 * p.kchunks + p.seg_steps - 1) / p.seg_steps, sg, tfull, tempty, abort_flag, seg);
       } else {
         ptx::mbar_wait(&tfull[acc], aph, abort_flag);  // sets the abort flag itself when it gives up
         ptx::tc_fence_after();
@@ -580,7 +584,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         const uint32_t acc = tl & 1, aph = (tl >> 1) & 1;
         float seg[SEG ? BN : 1];
         if constexpr (SEG) {
-          add_segments<BN>(tmem_base + ((uint32_t)(lg * 32) << 16), (9 * p.kchunks + kSegSteps - 1) / kSegSteps, sg, tfull, tempty, abort_flag, seg);
+          add_segments<BN>(tmem_base + ((uint32_t)(lg * 32) << 16), (9 * p.kchunks + p.seg_steps - 1) / p.seg_steps, sg, tfull, tempty, abort_flag, seg);
         } else {
           ptx::mbar_wait(&tfull[acc], aph, abort_flag);
           ptx::tc_fence_after();
@@ -1533,12 +1537,23 @@ struct WgParams {
 
 // NB = width of the output-gradient tile in channels (64: main conv, one 64-channel chunk per CTA;
 // 16/32/64: aux conv with F <= NB filters, rows of 2*NB bytes with the matching TMA swizzle).
-// Per-tap form (S2 is always 1): stride-2 convolutions, and feature maps smaller than a tile where a tile
+// Per-tap form: stride-2 convolutions, and feature maps smaller than a tile where a tile
 // spans BI whole images.  The shifted activation tiles are gathered by TMA, with element stride 2 for
 // stride 2, one 128-pixel tile per tap; a CTA then owns one kernel row kh (grid dimension) with its three column
 // taps: taps (kh,0) and (kh,1) stacked in one instruction, tap (kh,2) in a second, half-empty one.
-template <int NB, int S2>
-__global__ void __launch_bounds__(kThreads, 1)
+// SEG = 1, 2 (maps that no tile divides, NB <= 64): a new pair of accumulators every SEG instructions of 16 pixels, added outside the
+// tensor core, two segments to one term of a compensated fp32 sum, so that the error is one segment's and not the whole pixel
+// range's.  The running sum of the tensor core loses about 2^-27 per instruction, always towards zero: over the 80 instructions of a
+// CTA's range the weight gradient of 256 -> 256 channels on 61 maps of 14x14 was off by 1.9e-6 of its size, the auxiliary one by
+// 5.5e-7, where the fp32 chains that such maps had before gave 8.5e-7 and 6.6e-8.  A thread holds one row's 64 sums and 64
+// corrections: warps 0-3 the first accumulator of the pair, warps 4 and 5 the filled half of the second; warps 6 and 7 produce
+// and issue (with 256 threads all of that stays in registers).  The sums bound this form: that stage of two layers 281 -> 342 us,
+// the two gradients now off by 1.1e-7 and 6.0e-8.
+constexpr int kSegSets = 4;
+constexpr int wgrad_threads(int seg) { return seg ? 256 : kThreads; }
+
+template <int NB, int SEG>
+__global__ void __launch_bounds__(wgrad_threads(SEG), 1)
 conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dy, const WgParams p) {
   constexpr int kAtoms = NB > 64 ? NB / 64 : 1;                // 64-channel atoms of the dy tile (NB = 128, 256: main conv only)
   constexpr int kBRow = (NB > 64 ? 64 : NB) * 2;               // bytes of one pixel row of one atom
@@ -1546,7 +1561,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   constexpr int kBTile = 128 * kBRow;                          // one atom
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  static_assert(S2 == 1, "stride 1 on tileable maps uses conv_wgrad_kw_kernel");
+  static_assert(!SEG || NB <= 64, "a thread holds the sums of one accumulator");
   constexpr int kStages = NB > 64 ? 2 : 3;
   constexpr int kJobs = 2;  // instructions (accumulators) per 16 pixels
   constexpr int copy_bytes = 16384;  // one 128-pixel tap tile
@@ -1556,12 +1571,15 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   uint64_t* full = bars;
   uint64_t* empty = bars + kStages;
   uint64_t* done = bars + 2 * kStages;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  uint64_t* tfull = done + 1;    // SEG: pair of accumulators complete / taken
+  uint64_t* tempty = tfull + kSegSets;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + kSegSets);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  constexpr uint32_t kNeed = kJobs * NB;
+  constexpr uint32_t kNeed = kJobs * NB * (SEG ? kSegSets : 1);
   constexpr uint32_t kCols = kNeed <= 32 ? 32 : kNeed <= 64 ? 64 : kNeed <= 128 ? 128 : kNeed <= 256 ? 256 : 512;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kProducer = SEG ? 6 : 0, kIssuer = SEG ? 7 : 1;
   const int blocks = p.ci_chunks * p.co_chunks;
   const int blk = blockIdx.x % blocks;
   const int rest = blockIdx.x / blocks;
@@ -1576,12 +1594,16 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       ptx::mbar_init(&empty[s], 1);
     }
     ptx::mbar_init(done, 1);
+    for (int a = 0; a < kSegSets; ++a) {
+      ptx::mbar_init(&tfull[a], 1);
+      ptx::mbar_init(&tempty[a], 192);
+    }
     *abort_flag = 0;
     ptx::fence_mbar_init();
     ptx::prefetch_tmap(&tm_x);
     ptx::prefetch_tmap(&tm_dy);
   }
-  if (warp == 1) {
+  if (warp == kIssuer) {
     ptx::tmem_alloc(tmem_slot, kCols);
     ptx::tmem_relinquish();
   }
@@ -1591,7 +1613,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   const uint32_t tmem_base = *tmem_slot;
   nf_pdl_begin();  // everything above touches only this CTA and overlaps the previous kernel
 
-  if (warp == 0) {
+  if (warp == kProducer) {
     if (ptx::elect_one()) {  // producer and issuer: one thread runs the whole loop, as in the forward kernels
       Ring rg;
       for (int t = t0; t < t1; ++t, rg.next(kStages)) {
@@ -1609,7 +1631,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
       }
     }
     __syncwarp();
-  } else if (warp == 1) {
+  } else if (warp == kIssuer) {
     constexpr uint32_t idesc = ptx::idesc_bf16(128, NB, 1, 1);
     // descriptors differ only in the address field; the second stacked chunk sits one tap tile further
     const uint64_t a_copy_hi = ptx::sdesc(0, copy_bytes, 1024, 2);
@@ -1618,7 +1640,8 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     if (ptx::elect_one()) {
       Ring rg;
       bool ok = true;
-      for (int t = t0; t < t1; ++t, rg.next(kStages)) {
+      uint32_t sg = 0;  // SEG: segments started
+      for (int t = t0; ok && t < t1; ++t, rg.next(kStages)) {
         if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint32_t xb = ptx::smem_u32(smem) + rg.s * stage_bytes;
@@ -1627,16 +1650,72 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         for (int k = 0; k < 8; ++k) {
           const uint32_t k16 = k * 128;  // 16 pixels x 128 bytes, in 16-byte units
           const uint64_t bd = b_hi | (uint64_t)(g16 + k * kBRow);
-          const uint32_t acc = t > t0 || k != 0;
+          uint32_t acc = t > t0 || k != 0, d = tmem_base;
+          if constexpr (SEG) {
+            if (k % SEG == 0) {
+              if (!ptx::mbar_wait(&tempty[sg % kSegSets], ((sg / kSegSets) & 1) ^ 1, abort_flag)) { ok = false; break; }
+              ptx::tc_fence_after();
+            }
+            d += (sg % kSegSets) * kJobs * NB;
+            acc = k % SEG != 0;
+          }
           // taps (kh,0) and (kh,1): second chunk one tile further; tap (kh,2): rows 64..127 unused
-          ptx::mma_f16(tmem_base, a_copy_hi | (uint64_t)(x16 + k16), bd, idesc, acc);
-          ptx::mma_f16(tmem_base + NB, a_copy_hi | (uint64_t)(x16 + 2 * copy16 + k16), bd, idesc, acc);
+          ptx::mma_f16(d, a_copy_hi | (uint64_t)(x16 + k16), bd, idesc, acc);
+          ptx::mma_f16(d + NB, a_copy_hi | (uint64_t)(x16 + 2 * copy16 + k16), bd, idesc, acc);
+          if constexpr (SEG) {
+            if (k % SEG == SEG - 1) {
+              if (k == 7) ptx::mma_commit(&empty[rg.s]);  // before the last arrival that somebody waits for
+              ptx::mma_commit(&tfull[sg % kSegSets]);
+              ++sg;
+            }
+          }
         }
-        ptx::mma_commit(&empty[rg.s]);
+        if constexpr (!SEG) ptx::mma_commit(&empty[rg.s]);
       }
-      if (ok) ptx::mma_commit(done);
+      if (!SEG && ok) ptx::mma_commit(done);
     }
     __syncwarp();
+  } else if constexpr (SEG) {
+    // the sums of accumulator j over the segments; lane m of tensor memory = row m of the stacked (tap, ci) chunks
+    const int lg = warp & 3, m = lg * 32 + lane, j = warp >> 2;
+    const int tap = khg * 3 + (j == 0 ? (m < 64 ? 0 : 1) : 2);
+    float s[NB], c[NB];
+#pragma unroll
+    for (int e = 0; e < NB; ++e) s[e] = c[e] = 0.f;
+    const int pairs = (t1 - t0) * (8 / SEG / 2);
+    const uint32_t row = tmem_base + ((uint32_t)(lg * 32) << 16) + j * NB;
+#pragma unroll 1
+    for (int i = 0; i < pairs; ++i) {
+      const uint32_t a0 = 2 * i % kSegSets, ph = (2 * i / kSegSets) & 1;  // both sets of a pair are in the same round
+      ptx::mbar_wait(&tfull[a0], ph, abort_flag);  // sets the abort flag itself when it gives up
+      ptx::mbar_wait(&tfull[a0 + 1], ph, abort_flag);
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int q = 0; q < NB / 16; ++q) {
+        uint32_t u[16], v[16];
+        ptx::tmem_ld16(row + a0 * kJobs * NB + q * 16, u);
+        ptx::tmem_ld16(row + (a0 + 1) * kJobs * NB + q * 16, v);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {  // Kahan's sum
+          float &se = s[q * 16 + e], &ce = c[q * 16 + e];
+          const float y = (__uint_as_float(u[e]) + __uint_as_float(v[e])) - ce, t = se + y;
+          ce = fmaxf((t - se) - y, -1e32f);  // NaN after an infinite t: the sum stays infinite (a true correction is below 2^104)
+          se = t;
+        }
+      }
+      ptx::tc_fence_before();
+      ptx::mbar_arrive(&tempty[a0]);
+      ptx::mbar_arrive(&tempty[a0 + 1]);
+    }
+    if (!*abort_flag) {
+      const size_t plane = (size_t)p.Cout * p.Cin, pitch = p.Cin;
+      float* dst = p.part + ((size_t)sp * 9 + tap) * plane + (size_t)(coc * NB) * p.Cin + cic * 64 + (m & 63);
+      const int co_left = p.Cout - coc * NB;
+#pragma unroll
+      for (int e = 0; e < NB; ++e, dst += pitch)
+        if (e < co_left) *dst = s[e];
+    }
   } else {
     // epilogue: after the last MMA, lane m of tensor memory = row m of the stacked (tap, ci) chunks
     const int lg = warp & 3, m = lg * 32 + lane;
@@ -1674,7 +1753,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     const unsigned long long tt = ptx::globaltimer();
     while (ptx::globaltimer() - tt < 2000000ull) __nanosleep(1000);
   }
-  if (warp == 1) {
+  if (warp == kIssuer) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, kCols);
   }
@@ -2179,12 +2258,18 @@ bool pick_tile(int N, int H, int W, int* BW, int* BH, int* BI) {
   return false;
 }
 // Whether a convolution whose result is rounded for storage (forward, input gradient) goes to the tensor cores.  Maps that tile
-// exactly always do; the others from 8192 output pixels on (64 tiles).  Below that a layer's gradients hang on a few thousand ReLU
-// decisions, and an output one bfloat16 unit off moves them by up to several per cent in the next step; the CUDA-core kernels
-// give the same bits as they always have there.  The weight gradients stay in fp32 and always run here.
+// exactly always do; the others, in segments, from 8192 output pixels on (64 tiles).  Below that a layer's gradients hang on a few
+// thousand ReLU decisions, and an output that is rounded the other way moves them by up to several per cent in the next step; the
+// CUDA-core kernels give the same bits as they always have there.  The line is drawn by that, not by speed: just below it the
+// tensor cores would be several times faster.  The weight gradients stay in fp32, decide nothing and always run here.
 bool tc_size_ok(int N, int H, int W) {
   int BW, BH, BI;
   return pick_tile(N, H, W, &BW, &BH, &BI) || (long)N * H * W >= 8192;
+}
+
+bool tiles_exactly(int H, int W) {
+  int BW, BH, BI;
+  return pick_tile(1, H, W, &BW, &BH, &BI);
 }
 
 // ybuf = 1 reserves the y2 tile of the fused BatchNorm-backward sums (as large as the output staging)
@@ -2195,7 +2280,7 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   if (epi == 0 ? (Cout % 64 != 0) : epi == 1 ? (Cout > 64) : false) return pl;
   const bool exact = pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
   pl.PT = (stride == 2 || pl.BI > 1 || !exact) ? 1 : 0;
-  pl.SEG = !exact && epi != 2;  // the input gradient is rounded but decides nothing
+  pl.SEG = !exact;  // maps that no tile divides
   if (epi == 0 && Cout % 256 == 0) pl.PT = 1;  // 256-wide instructions need the per-tap form (one tap of weights per stage)
   pl.BN = epi != 1 ? (Cout % 128 == 0 ? 128 : 64) : (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64);
   if (epi == 0 && pl.PT && !pl.SEG && Cout % 256 == 0) pl.BN = 256;  // per-tap form: weights of one tap and 256 channels are 32 KB a stage
@@ -2264,8 +2349,10 @@ int fold_group(int Cout, int epi) { return epi != 1 ? 64 : (Cout <= 16 ? 16 : Co
 // at most a third (32, 48, 64, ...: the zero-filled loads and clipped stores of TMA make the overhang harmless)
 bool fold_width_ok(int W) { return W % 14 == 0 || (W >= 28 && ((W + 13) / 14) * 14 * 3 <= W * 4); }
 
-bool fold_ok(int H, int W, int Cin, int Cout, int epi, int stride, int stats = 0, size_t extra_smem = 0) {
-  if (stride != 1 || H % 8) return false;
+// Maps that no 128-pixel tile divides (56 x 56, 40 x 40) stay with the segmented sums in a layer; the stand-alone forward (any_map)
+// takes the folded kernel there too, as it always has.
+bool fold_ok(int H, int W, int Cin, int Cout, int epi, int stride, int stats = 0, size_t extra_smem = 0, bool any_map = false) {
+  if (stride != 1 || H % 8 || !(any_map || tiles_exactly(H, W))) return false;
   if (epi == 2 && W % 14 && W % 16 == 0 && (stats >= 2 || Cout == 64)) return Cin <= 32 && Cin % 8 == 0 && Cout % 64 == 0;
   if (epi == 2 ? W % 14 != 0 : !fold_width_ok(W)) return false;
   // the plain aux forward (no fused normalisation: extra_smem == 0) stays on the generic kernel for ragged widths: with 64
@@ -2412,9 +2499,9 @@ int run_fold(int N, int H, int W, int Cin, int Cout, const void* x, const void* 
 // H, W are the INPUT size; stride 2 halves them (rounding up) for the output.
 int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const void* w, void* y, int stats, float* red,
             size_t red_floats, int32_t* status, int* nb, int epi = 0, const float* bias = nullptr, int stride = 1,
-            const BnBwdIn* bn = nullptr) {
+            const BnBwdIn* bn = nullptr, bool any_map = false) {
   const int H = (Hin - 1) / stride + 1, W = (Win - 1) / stride + 1;
-  if (fold_ok(H, W, Cin, Cout, epi, stride, stats))
+  if (fold_ok(H, W, Cin, Cout, epi, stride, stats, 0, any_map))
     return run_fold(N, H, W, Cin, Cout, x, w, y, stats, red, red_floats, status, nb, epi, bias, bn);
   if (stats > 2) return NF_EUNSUPPORTED;  // the two-pass input gradient exists in the folded kernel only
   if (stats == 2 && (!bn || epi == 1)) return NF_EINVAL;
@@ -2445,7 +2532,12 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   p.total_tiles = ((N + pl.BI - 1) / pl.BI) * p.tiles_h * p.tiles_w * p.n_tiles;
   p.stride = stride; p.BI = pl.BI;
   p.tg = tile_grid(p.n_tiles, p.tiles_w, p.tiles_h);
-  p.kchunks = epi == 2 ? 1 : Cin / 64; p.stages = pl.stages; p.stats = stats; p.red = red; p.status = status;
+  p.kchunks = epi == 2 ? 1 : Cin / 64;
+  // An fp32 chain over 64 channels has only 576 roundings, one over 16 or 32 filters 144 or 288: segments of 64 (16 filters: 48)
+  // products there, of 192 from 128 channels on.  Share of outputs off the nearest bf16 value, chain -> segments: 64 channels
+  // 0.0078 -> 0.0064 %, 128 0.0118 -> 0.0105 %, 512 0.022 -> 0.012 %.
+  p.seg_steps = pl.KC == 16 ? 3 : pl.KC == 32 ? 2 : p.kchunks == 1 ? 1 : 3;
+  p.stages = pl.stages; p.stats = stats; p.red = red; p.status = status;
   p.yslots = pl.yslots;
   p.tm_y2 = my;
   if (stats == 0 && bn) {
@@ -2471,6 +2563,12 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   }
   if (pl.SEG) {  // maps that no tile divides
     if (epi == 0) return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
+    if (epi == 2 && pl.BN == 128)
+      return pl.KC == 16 ? launch_fwd<128, 0, 16, 1, 1, 0, 1>(pl, mx, mw, my, p)
+                         : pl.KC == 32 ? launch_fwd<128, 0, 32, 1, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<128, 0, 64, 1, 1, 0, 1>(pl, mx, mw, my, p);
+    if (epi == 2)
+      return pl.KC == 16 ? launch_fwd<64, 0, 16, 1, 1, 0, 1>(pl, mx, mw, my, p)
+                         : pl.KC == 32 ? launch_fwd<64, 0, 32, 1, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 1, 1, 0, 1>(pl, mx, mw, my, p);
     return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p)
                        : pl.BN == 32 ? launch_fwd<32, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
   }
@@ -2508,7 +2606,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
 }
 
 struct WgPlan {
-  int ok, exact, BW, BH, BI, PT, NB, GX, ROW, splits, grid, stages;  // ROW: input-channel chunks per CTA of the row kernel, or 0
+  int ok, exact, BW, BH, BI, PT, SEG, NB, GX, ROW, splits, grid, stages;  // ROW: input-channel chunks per CTA of the row kernel, or 0
   size_t smem, part_floats;
 };
 
@@ -2541,7 +2639,9 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
   pl.exact = pick_tile(N, H, W, &pl.BW, &pl.BH, &pl.BI);
   pl.PT = (stride == 2 || pl.BI > 1 || !pl.exact) ? 1 : 0;
   pl.NB = aux ? (Cout <= 16 ? 16 : Cout <= 32 ? 32 : 64) : 64;
-  if (!aux && pl.PT) pl.NB = Cout % 256 == 0 ? 256 : Cout % 128 == 0 ? 128 : 64;  // per-tap form: as wide an instruction as Cout allows
+  // maps that no tile divides: segments of 32 pixels, of 16 below 8192 pixels, where the chains to compare with are shorter
+  pl.SEG = pl.exact ? 0 : (long)N * H * W < 8192 ? 1 : 2;
+  if (!aux && pl.PT && !pl.SEG) pl.NB = Cout % 256 == 0 ? 256 : Cout % 128 == 0 ? 128 : 64;  // per-tap form: as wide an instruction as Cout allows
   pl.GX = (aux && !pl.PT && pl.NB <= 32) ? 1 : 0;  // few filters: one instruction per 16 pixels with the gradient on the M side
   const long pix_tiles = (long)((N + pl.BI - 1) / pl.BI) * ((H + pl.BH - 1) / pl.BH) * ((W + pl.BW - 1) / pl.BW);
   if (pix_tiles >= (1l << 30)) return pl;
@@ -2552,7 +2652,7 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
   // those of the other forms, so that every sum runs over the same pixels in the same order and the bits stay what they were; of one
   // or two chunks of input channels per CTA the one whose CTAs fill their waves better (two on near ties: less to fetch).
   const size_t box = (size_t)pl.BI * (pl.BH + 2) * pl.BW * 128;
-  if (!aux && stride == 1 && Cout % 128 == 0 && pl.BW >= 4 && pl.BW * pl.BH % 16 == 0) {
+  if (!aux && !pl.SEG && stride == 1 && Cout % 128 == 0 && pl.BW >= 4 && pl.BW * pl.BH % 16 == 0) {
     // single-image tiles with one chunk only: the form above has as little to fetch and fills its wave (64 -> 128 channels at 32x32)
     double best = pl.PT || Cin % 128 == 0 ? 0.0 : 0.75;
     for (int cc = Cin % 128 == 0 ? 2 : 1; cc >= 1; --cc) {
@@ -2621,15 +2721,15 @@ int launch_wgrad_gx(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& 
   return NF_OK;
 }
 
-template <int NB, int S2 = 0>
+template <int NB, int SEG>
 int launch_wgrad(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& mg, const WgParams& p) {
   static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
   bool& attr_done = attr_done_dev[current_device()];
   if (!attr_done) {
-    NF_CUDA(cudaFuncSetAttribute(conv_wgrad_tc_kernel<NB, S2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    NF_CUDA(cudaFuncSetAttribute(conv_wgrad_tc_kernel<NB, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_wgrad_tc_kernel<NB, S2>, pl.grid, kThreads, pl.smem, mx, mg, p);
+  nf_launch(conv_wgrad_tc_kernel<NB, SEG>, pl.grid, wgrad_threads(SEG), pl.smem, mx, mg, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2661,15 +2761,19 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
     rc = pl.ROW == 2 ? launch_wgrad_row<2>(pl, mx, mg, p) : launch_wgrad_row<1>(pl, mx, mg, p);
   else if (pl.GX)
     rc = pl.NB == 32 ? launch_wgrad_gx<32>(pl, mx, mg, p) : launch_wgrad_gx<16>(pl, mx, mg, p);
+  else if (pl.SEG == 1)
+    rc = pl.NB == 64 ? launch_wgrad<64, 1>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 1>(pl, mx, mg, p) : launch_wgrad<16, 1>(pl, mx, mg, p);
+  else if (pl.SEG)
+    rc = pl.NB == 64 ? launch_wgrad<64, 2>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 2>(pl, mx, mg, p) : launch_wgrad<16, 2>(pl, mx, mg, p);
   else if (pl.PT)
-    rc = pl.NB == 256 ? launch_wgrad<256, 1>(pl, mx, mg, p) : pl.NB == 128 ? launch_wgrad<128, 1>(pl, mx, mg, p)
-       : pl.NB == 64 ? launch_wgrad<64, 1>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 1>(pl, mx, mg, p) : launch_wgrad<16, 1>(pl, mx, mg, p);
+    rc = pl.NB == 256 ? launch_wgrad<256, 0>(pl, mx, mg, p) : pl.NB == 128 ? launch_wgrad<128, 0>(pl, mx, mg, p)
+       : pl.NB == 64 ? launch_wgrad<64, 0>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 0>(pl, mx, mg, p) : launch_wgrad<16, 0>(pl, mx, mg, p);
   else
     rc = pl.NB == 64 ? launch_wgrad_kw<64>(pl, mx, mg, p)
                      : pl.NB == 32 ? launch_wgrad_kw<32>(pl, mx, mg, p) : launch_wgrad_kw<16>(pl, mx, mg, p);
   if (rc != NF_OK) return rc;
   const size_t n = (size_t)9 * Cout * Cin;
-  return nf_k_sum_parts(part, pl.splits, n, dw);
+  return nf_k_sum_parts(part, pl.splits, n, dw, pl.SEG != 0);
 }
 
 }  // namespace
@@ -2740,16 +2844,17 @@ static int main_conv_operands(nf_layer* L, const void* x, int count, const void*
   return NF_OK;
 }
 
+// On maps that no tile divides the statistics (and in the input gradient the BatchNorm-backward sums) are left to the passes of the
+// CUDA-core path: the fused sums run in chains of a CTA's whole pixel range, the second ones in the form sum(dz*y) - mu*sum(dz),
+// which cost a factor of up to 5 in the error of a normalised activation's rounding and of 2 to 30 in that of sum(dz*xhat).
 int nf_tc_conv_fwd(nf_layer* L, const void* x, int& nb) {
-  if (L->cin_pad) {
-    const void *xin, *win;
-    int Cin;
-    const int rc = main_conv_operands(L, x, L->o.N, &xin, &win, &Cin);
-    if (rc != NF_OK) return rc;
-    return run_fwd(L->o.N, L->H, L->W, Cin, L->Cout, xin, win, L->y, 1, L->red, L->red_floats, L->status, &nb, 0, nullptr, L->o.stride);
-  }
-  return run_fwd(L->o.N, L->H, L->W, L->Cin, L->Cout, x, L->shadow + L->off[NF_P_W], L->y, 1, L->red, L->red_floats,
-                 L->status, &nb, 0, nullptr, L->o.stride);
+  const void *xin, *win;
+  int Cin;
+  const int rc = main_conv_operands(L, x, L->o.N, &xin, &win, &Cin);
+  if (rc != NF_OK) return rc;
+  nb = 0;
+  return run_fwd(L->o.N, L->H, L->W, Cin, L->Cout, xin, win, L->y, tiles_exactly(L->Ho, L->Wo), L->red, L->red_floats, L->status, &nb, 0,
+                 nullptr, L->o.stride);
 }
 
 int nf_tc_conv_fwd_eval(nf_layer* L, const void* x, int count, void* act) {
@@ -2854,7 +2959,7 @@ int nf_tc_aux_dgrad(nf_layer* L, int* bn_nb) {
   const int epi = wide ? 0 : 2;
   // Without a pool (and without a shortcut) da has the shape of y, and the kernel that produces it also reduces
   // (dz, dz*xhat) per channel while it holds the tile: the BatchNorm backward then needs no reduction pass.
-  if (!L->o.maxpool && !L->skip) {
+  if (!L->o.maxpool && !L->skip && tiles_exactly(L->Ha, L->Wa)) {
     const BnBwdIn bn{L->y, L->scale, L->shift, L->mu, L->invstd};
     bool fits;
     if (fold_ok(L->Ha, L->Wa, L->F, L->Cout, epi, 1, 2)) {
@@ -2899,11 +3004,12 @@ int nf_tc_op_status_ptr(int32_t** out) {
 }
 
 int nf_tc_conv3x3_forward(const void* x, const void* w, int N, int H, int W, int Cin, int Cout, int stride, void* y) {
-  if (!tc_size_ok(N, (H - 1) / stride + 1, (W - 1) / stride + 1)) return NF_EUNSUPPORTED;
+  const int Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
+  if (!tc_size_ok(N, Ho, Wo) && !fold_ok(Ho, Wo, Cin, Cout, 0, stride, 0, 0, true)) return NF_EUNSUPPORTED;
   int32_t* st = nullptr;
   if (nf_tc_op_status_ptr(&st) != NF_OK) return NF_ECUDA;
   int nb = 0;
-  return run_fwd(N, H, W, Cin, Cout, x, w, y, 0, nullptr, 0, st, &nb, 0, nullptr, stride);
+  return run_fwd(N, H, W, Cin, Cout, x, w, y, 0, nullptr, 0, st, &nb, 0, nullptr, stride, nullptr, true);
 }
 
 int nf_tc_conv3x3_wgrad(const void* x, const void* g, int N, int H, int W, int Cin, int Cout, int stride, float* part,

@@ -6,7 +6,8 @@
 void nf_tc_select(nf_layer* L);
 // Floats of split-K scratch the tensor-core weight gradient needs (0 if unused).
 size_t nf_tc_scratch_floats(const nf_layer* L);
-// y = conv(x) in bf16 plus per-CTA channel partials (sum, sum of squares) in L->red; nb = partial count.
+// y = conv(x) in bf16 plus per-CTA channel partials (sum, sum of squares) in L->red; nb = partial count, 0 where the kernel takes
+// no statistics (maps that no tile divides).
 int nf_tc_conv_fwd(nf_layer* L, const void* x, int& nb);
 // Same convolution for `count` samples without statistics (cache-filling forward): y, or, with act, straight to act = ReLU(y * scale +
 // shift) with the layer's current coefficients.
@@ -40,7 +41,7 @@ int nf_tc_bn_aux_fwd(nf_layer* L, void* act_out);
 // Aux conv weight gradient on tensor cores: grad(Wa) = wgrad(a, L->dh).
 int nf_tc_aux_wgrad(nf_layer* L, const void* a);
 // Aux conv input gradient on tensor cores: L->da = dgrad(L->dh, Wa) in bf16.  Where the kernel can also reduce
-// the BatchNorm-backward sums (no pool, folded-tap shape) it leaves *bn_nb > 0 partial blocks in L->red
+// the BatchNorm-backward sums (no pool, maps that tile) it leaves *bn_nb > 0 partial blocks in L->red
 // ([block][2][Cout]: sum dz, sum dz*xhat); otherwise *bn_nb = 0.
 int nf_tc_aux_dgrad(nf_layer* L, int* bn_nb);
 // Self-check of the bounded wait: one small CTA waits limit_ns on a barrier nobody arrives at; *waited_ns_dev (device)
