@@ -156,7 +156,7 @@ void nf_block_destroy(nf_block* block);
  * every layer runs conv, BatchNorm with its RUNNING statistics, ReLU and pool, so a sample's
  * cached row does not depend on its batch-mates.  No parameter changes.
  * x: device [count][H][W][Cin] of the first layer; out: device [count][Ha][Wa][Cout] of the
- * last layer.  count must be in [1, N] of the block's layers (call repeatedly to cover a
+ * last layer; it may overlap x.  count must be in [1, N] of the block's layers (call repeatedly to cover a
  * dataset); nf_block_cache uses count = N. */
 int nf_block_cache(nf_block* block, const void* x, void* out);
 int nf_block_cache_n(nf_block* block, const void* x, void* out, int count);
@@ -236,7 +236,8 @@ int nf_layer_stored_tensor(nf_layer* layer, int which, void** dev_ptr, size_t* b
  *   act_out = x_{n+1} for `count` samples (device, [count][Ha][Wa][Cout]; NULL keeps it in the workspace),
  *   logits_out = z_{n+1} (device float [count][classes]; may be NULL),
  *   pred_out = arg-max class per sample, first maximum (device int32 [count]).
- * count must be in [1, N].  Feed act_out to the next layer's nf_layer_predict to evaluate deeper exits. */
+ * count must be in [1, N].  Feed act_out to the next layer's nf_layer_predict to evaluate deeper exits.
+ * act_out may overlap x (evaluation in place). */
 int nf_layer_predict(nf_layer* layer, const void* x, int count, void* act_out, float* logits_out, int32_t* pred_out);
 
 /* Validation accuracy of an exit: *count += #{i < n : a[i] == b[i]} (device int32 arrays, device 64-bit counter that

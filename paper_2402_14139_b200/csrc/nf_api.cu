@@ -638,7 +638,14 @@ static int layer_eval_forward(nf_layer* L, const void* in, int count, void* dst)
   NF_TRY(nf_k_bn_eval_coeffs(L->Cout, L->val + L->off[NF_P_GAMMA], L->val + L->off[NF_P_BETA], L->o.bn_eps, L->rmean, L->rvar,
                                L->scale, L->shift));
   if (L->fam[0]) {
-    const bool fused = !L->o.maxpool && !L->skip;  // the convolution normalises in its epilogue: y is neither written nor read
+    // The convolution normalises in its epilogue and writes dst itself (y is neither written nor read), unless dst shares memory with
+    // the input: a block writes its tile while others still load the rows beside it.  Then y is formed first, as with a pool.  A
+    // padded input has been copied before the convolution starts.
+    const size_t es = nf_esize(dt);
+    const char *in0 = (const char*)in, *in1 = in0 + (size_t)count * L->H * L->W * L->Cin * es;
+    const char *out0 = (const char*)dst, *out1 = out0 + (size_t)count * L->Ha * L->Wa * L->Cout * es;
+    const bool shared = !L->cin_pad && in0 < out1 && out0 < in1;
+    const bool fused = !L->o.maxpool && !L->skip && !shared;
     NF_TRY(nf_tc_conv_fwd_eval(L, in, count, fused ? dst : nullptr));
     if (fused) return NF_OK;
   } else {
