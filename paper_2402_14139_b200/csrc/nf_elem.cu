@@ -2,6 +2,7 @@
 // the linear + softmax cross-entropy head, momentum SGD and the cache gather.  Storage fp32 or
 // bf16, arithmetic fp32, cross-block sums finished in fp64 in a fixed order (deterministic).
 #include <algorithm>
+#include <type_traits>
 #include "nf_internal.h"
 #include "nf_ldst.cuh"
 
@@ -808,6 +809,37 @@ template <> struct Vec8<float> {
   }
 };
 
+// The totals of one pixel range: out[k*C + c] = sum over the range's chains of value k at channel c, sm[k*8 + c%8][base + chain*C8 + c/8],
+// by the range's thr threads (lt: the thread among them).  TREE (fp32, a range per block): in fp64, the 256 / C8 chains sixteen at a
+// time; one serial fp32 sum over 128 chains of two pixels was less exact than the generic kernel's 16 chains of 16 (16 channels, 8
+// images of 32x32: sum(dz*xhat) off by 1.3e-7 against 7.4e-8).  bf16 keeps the serial order, on which bits hang.
+template <bool TREE>
+__device__ __forceinline__ void range_totals(const float (*sm)[256], int base, int lt, int thr, int C8, int planes, bool on, float* out) {
+  const int C = C8 * 8;
+  if constexpr (TREE) {
+    __shared__ double part[256];
+    if (planes > 16) {
+      const int o = lt % (2 * C), q0 = lt / (2 * C) * 16, c = o % C;
+      double s = 0.0;
+      for (int q = q0; q < q0 + 16; ++q) s += (double)sm[o / C * 8 + c % 8][q * C8 + c / 8];
+      part[lt] = s;
+      __syncthreads();
+      if (lt < 2 * C) {
+        for (int j = 1; j < planes / 16; ++j) s += part[j * 2 * C + lt];
+        if (on) out[lt] = (float)s;
+      }
+      return;
+    }
+  }
+  if (!on) return;
+  for (int t = lt; t < 2 * C; t += thr) {  // value k = t / C of channel c = t % C, one thread each
+    const int k = t / C, c = t % C, gg = c / 8, i = c % 8;
+    std::conditional_t<TREE, double, float> s = 0;
+    for (int q = 0; q < planes; ++q) s += sm[k * 8 + i][base + q * C8 + gg];
+    out[t] = (float)s;
+  }
+}
+
 // out = ReLU(y*scale+shift); grid-stride over (pixel, channel group)
 __global__ void __launch_bounds__(256) bn_apply_vec_kernel(const uint4* __restrict__ y, int C8, const float* __restrict__ scale,
                                                            const float* __restrict__ shift, size_t total8,
@@ -916,7 +948,7 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const T* __restr
         for (int i = 0; i < 8; ++i) {
           const float dz = MODE == 2 || fmaf(yv[i], sc[i], sh[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
           a[i] += dz;
-          b[i] = MODE == 1 ? fmaf(dz * (yv[i] - m[i]), is[i], b[i]) : fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
+          b[i] = MODE == 1 || (MODE == 0 && sizeof(T) == 4) ? fmaf(dz * (yv[i] - m[i]), is[i], b[i]) : fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
           dv[i] = dz;
         }
         if (MODE == 1 && dz_out) st8(dz_out + (q * C8 + g) * 8, dv);
@@ -929,15 +961,7 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const T* __restr
     sm[8 + i][threadIdx.x] = b[i];
   }
   __syncthreads();
-  // value k = t / C of channel c = t % C, one thread each, for every range of the block
-  const int base = threadIdx.x / thr * thr;
-  if (rng < ranges)
-    for (int t = lt; t < 2 * C; t += thr) {
-      const int k = t / C, c = t % C, gg = c / 8, i = c % 8;
-      float s = 0.f;
-      for (int q = 0; q < planes; ++q) s += sm[k * 8 + i][base + q * C8 + gg];
-      red[((size_t)rng * 2 + k) * C + c] = s;
-    }
+  range_totals<sizeof(T) == 4 && MODE != 1>(sm, threadIdx.x / thr * thr, lt, thr, C8, planes, rng < ranges, red + (size_t)rng * 2 * C);
 }
 
 // dy = scale * (dz - sum(dz)/M - xhat * sum(dz*xhat)/M)
@@ -992,7 +1016,10 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec_kernel(const uint4* __re
 // Same result with per-thread constants: when 256 % C8 == 0 a thread keeps its 8 channels over the whole
 // grid-stride loop, and dy = s*dz + k1*y + k0 with k1 = -s*m2*invstd, k0 = s*(m2*invstd*mu - m1),
 // m1 = sum(dz)/M, m2 = sum(dz*xhat)/M: five instructions per element.
-template <typename T, int MODE>
+// FORM 0: that.  k1*y and k0 cancel where |mu| is large against sigma (fp32, |mu| = 30 sigma: four times the error in a channel's
+// sum of dy), so it is for bf16 without a shortcut, whose rounding hides that.  FORM 1: dy = s*dz + (k1*(y - mu) - s*m1).
+// FORM 2: the generic kernel's form term by term.
+template <typename T, int MODE, int FORM>
 __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const T* __restrict__ y, const T* __restrict__ da, int C8,
                                                                 const float* __restrict__ scale, const float* __restrict__ shift,
                                                                 const float* __restrict__ mu, const float* __restrict__ invstd,
@@ -1006,8 +1033,10 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const T* __restr
     const float s = scale[c0 + i], m1 = sdz[c0 + i] * invM, m2 = sdzx[c0 + i] * invM, is = invstd[c0 + i];
     A[i] = s;
     B[i] = shift[c0 + i];
-    if constexpr (MODE == 1) {  // the generic kernel's form, term by term
+    if constexpr (FORM == 2) {
       M1[i] = mu[c0 + i]; IS[i] = is; K1[i] = sdzx[c0 + i]; K0[i] = sdz[c0 + i];
+    } else if constexpr (FORM == 1) {
+      M1[i] = mu[c0 + i]; K1[i] = -s * m2 * is; K0[i] = -s * m1;
     } else {
       K1[i] = -s * m2 * is;
       K0[i] = s * (m2 * is * mu[c0 + i] - m1);
@@ -1034,9 +1063,11 @@ __global__ void __launch_bounds__(256) bn_bwd_apply_vec2_kernel(const T* __restr
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const float dz = MODE == 2 || fmaf(yv[i], A[i], B[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
-          if constexpr (MODE == 1) {
+          if constexpr (FORM == 2) {
             const float xh = (yv[i] - M1[i]) * IS[i];
             o[i] = A[i] * (dz - K0[i] * invM - xh * K1[i] * invM);
+          } else if constexpr (FORM == 1) {
+            o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i] - M1[i], K0[i]));
           } else {
             o[i] = fmaf(A[i], dz, fmaf(K1[i], yv[i], K0[i]));
           }
@@ -1058,36 +1089,30 @@ __global__ void __launch_bounds__(256) channel_sums_vec_kernel(const T* __restri
 #pragma unroll
   for (int i = 0; i < 8; ++i) a[i] = b[i] = 0.f;
   const size_t p0 = P * blockIdx.x / gridDim.x, p1 = P * (blockIdx.x + 1) / gridDim.x;
-  if (pl < planes)
-    for (size_t p = p0 + pl; p < p1; p += 4 * (size_t)planes) {  // four loads in flight, added in index order
-      Vec8<T> q[4];
+  for (size_t p = p0 + pl; p < p1; p += 4 * (size_t)planes) {  // four loads in flight, added in index order
+    Vec8<T> q[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (p + (size_t)u * planes < p1) q[u].load(src, (p + (size_t)u * planes) * C8 + g);
+    for (int u = 0; u < 4; ++u)
+      if (p + (size_t)u * planes < p1) q[u].load(src, (p + (size_t)u * planes) * C8 + g);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (p + (size_t)u * planes < p1) {
-          float v[8];
-          q[u].get(v);
+    for (int u = 0; u < 4; ++u)
+      if (p + (size_t)u * planes < p1) {
+        float v[8];
+        q[u].get(v);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            a[i] += v[i];
-            b[i] = fmaf(v[i], v[i], b[i]);
-          }
+        for (int i = 0; i < 8; ++i) {
+          a[i] += v[i];
+          b[i] = fmaf(v[i], v[i], b[i]);
         }
-    }
+      }
+  }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     sm[i][threadIdx.x] = a[i];
     sm[8 + i][threadIdx.x] = b[i];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < 2 * C; t += 256) {
-    const int k = t / C, c = t % C, gg = c / 8, i = c % 8;
-    float s = 0.f;
-    for (int q = 0; q < planes; ++q) s += sm[k * 8 + i][q * C8 + gg];
-    red[((size_t)blockIdx.x * 2 + k) * C + c] = s;
-  }
+  range_totals<sizeof(T) == 4>(sm, 0, threadIdx.x, 256, C8, planes, true, red + (size_t)blockIdx.x * 2 * C);
 }
 
 
@@ -1885,10 +1910,12 @@ int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, i
   const size_t total = (size_t)N * Ho * Wo * C;
   const float invM = (float)(1.0 / M);
   if (vec2_ok(C, pool)) {
-#define NF_APPLY(T, M)                                                                                                                       \
-  nf_launch(bn_bwd_apply_vec2_kernel<T, M>, vec_blocks(total / 8), 256, 0, (const T*)y, (const T*)da, C / 8, scale, shift, mu, invstd, sdz, sdzx, \
+#define NF_APPLY(T, M, FM)                                                                                                                       \
+  nf_launch(bn_bwd_apply_vec2_kernel<T, M, FM>, vec_blocks(total / 8), 256, 0, (const T*)y, (const T*)da, C / 8, scale, shift, mu, invstd, sdz, sdzx, \
             invM, total / 8, (T*)dy, (const T*)skip)
-    DISPATCH(dtype, (skip ? NF_APPLY(float, 1) : NF_APPLY(float, 0)), (skip ? NF_APPLY(bf16, 1) : NF_APPLY(bf16, 0)));
+    // form 0 in bf16 up to 1024 channels: where it has always been
+    DISPATCH(dtype, (skip ? NF_APPLY(float, 1, 2) : NF_APPLY(float, 0, 1)),
+             (skip ? NF_APPLY(bf16, 1, 2) : C <= 1024 ? NF_APPLY(bf16, 0, 0) : NF_APPLY(bf16, 0, 1)));
 #undef NF_APPLY
     NF_LAUNCHED();
     return NF_OK;
@@ -2022,8 +2049,8 @@ int nf_k_bn_plain_bwd_apply(int dtype, const void* y, const void* dz, size_t P, 
   if (!vec2_ok(C, 0)) return NF_EUNSUPPORTED;
   const size_t n8 = P * C / 8;
   const float invM = (float)(1.0 / M);
-  DISPATCH(dtype, (nf_launch(bn_bwd_apply_vec2_kernel<float, 2>, vec_blocks(n8), 256, 0, (const float*)y, (const float*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx, invM, n8, (float*)dy, nullptr)),
-           (nf_launch(bn_bwd_apply_vec2_kernel<bf16, 2>, vec_blocks(n8), 256, 0, (const bf16*)y, (const bf16*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx, invM, n8, (bf16*)dy, nullptr)));
+  DISPATCH(dtype, (nf_launch(bn_bwd_apply_vec2_kernel<float, 2, 1>, vec_blocks(n8), 256, 0, (const float*)y, (const float*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx, invM, n8, (float*)dy, nullptr)),
+           (nf_launch(bn_bwd_apply_vec2_kernel<bf16, 2, 1>, vec_blocks(n8), 256, 0, (const bf16*)y, (const bf16*)dz, C / 8, scale, mu, mu, invstd, sdz, sdzx, invM, n8, (bf16*)dy, nullptr)));
   NF_LAUNCHED();
   return NF_OK;
 }
