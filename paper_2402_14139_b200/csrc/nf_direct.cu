@@ -1,6 +1,8 @@
 // Generic CUDA-core kernels of the local-layer step: any shape, fp32 or bf16 storage, fp32
 // accumulation, deterministic reductions (fixed-order partials, no floating-point atomics).
 // They carry the fp32 configuration and every shape the tensor-core kernels do not cover.
+#include <algorithm>
+
 #include "nf_internal.h"
 #include "nf_ldst.cuh"
 
@@ -23,7 +25,8 @@ struct ConvArgs {
   const float* bias;
   long ws_tap, ws_co, ws_ci;
   int H, W, Ci, Co, Ho, Wo, stride, taps, flip, relu;
-  uint32_t P;  // output pixels
+  uint32_t P;     // output pixels of the launch
+  uint32_t row0;  // the first one's row, where a launch takes some rows of one image (else 0)
 };
 
 // WCO: 1 = eight consecutive output channels of the weights are contiguous, 0 = eight input channels.  VEC: rows of eight are
@@ -41,7 +44,7 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
   const T* __restrict__ w = reinterpret_cast<const T*>(a.w);
   const int t = threadIdx.x, tc = t % (CO / TC), tp = t / (CO / TC);
   const uint32_t p0 = blockIdx.x * PX;
-  const int co0 = blockIdx.y * CO, pad = a.taps == 9 ? 1 : 0;
+  const int co0 = (blockIdx.y + gridDim.y * blockIdx.z) * CO, pad = a.taps == 9 ? 1 : 0;
 
   int xi[kXN], xj[kXN];   // input row and column of the unit's pixel at tap (0, 0)
   size_t xb[kXN];         // its image's first element; pixels past the end: marked by a row far outside
@@ -49,8 +52,8 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
   for (int u = 0; u < kXN; ++u) {
     const int e = t + u * kThr;
     const uint32_t p = p0 + e / (CK / 8);
-    const uint32_t r = p / a.Wo, n = r / a.Ho;
-    xj[u] = (int)(p - r * a.Wo) * a.stride - pad;
+    const uint32_t q = p / a.Wo, r = q + a.row0, n = r / a.Ho;
+    xj[u] = (int)(p - q * a.Wo) * a.stride - pad;
     xi[u] = p < a.P && e < kXU ? (int)(r - n * a.Ho) * a.stride - pad : -1000000;
     xb[u] = (size_t)n * a.H * a.W * a.Ci;
   }
@@ -193,7 +196,8 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
 
 template <typename T, int PX, int CO, int CK, int TP, int TC, int SPB>
 int launch_direct(const ConvArgs& a) {
-  const dim3 grid((unsigned)((a.P + PX - 1) / PX), (unsigned)((a.Co + CO - 1) / CO));
+  const unsigned cols = (unsigned)((a.Co + CO - 1) / CO), y = cols < 65535 ? cols : 65535;
+  const dim3 grid((unsigned)((a.P + PX - 1) / PX), y, (cols + y - 1) / y);  // channel tiles beyond Co do nothing
   const int thr = (PX / TP) * (CO / TC);
   const bool wco = a.ws_co == 1 && a.ws_ci != 1;
   const bool vec = a.Ci % 8 == 0 && (((uintptr_t)a.x | (uintptr_t)a.w) & 15) == 0 && (wco ? a.Co % 8 == 0 && a.ws_ci % 8 == 0 : a.ws_ci == 1 && a.ws_co % 8 == 0) &&
@@ -426,16 +430,26 @@ int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void*
     NF_LAUNCHED();
     return NF_OK;
   }
+  if ((long)N * Ho * ((Wo + 15) / 16) * ((Co + 15) / 16) > 0x7fffffffL) return NF_EUNSUPPORTED;
   return nf_k_conv_taps(dtype, x, N, H, W, Ci, w, 9, ws_tap, ws_co, ws_ci, flip, bias, relu, stride, Co, y);
 }
 
 int nf_k_conv_taps(int dtype, const void* x, int N, int H, int W, int Ci, const void* w, int taps, long ws_tap, long ws_co, long ws_ci,
                    int flip, const float* bias, int relu, int stride, int Co, void* y) {
   const int Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
-  const long P = (long)N * Ho * Wo;
-  if (P <= 0 || P > 0x7fffff00L || (Co + 15) / 16 > 65535) return NF_EUNSUPPORTED;
-  const ConvArgs a{x, w, y, bias, ws_tap, ws_co, ws_ci, H, W, Ci, Co, Ho, Wo, stride, taps, flip, relu, (uint32_t)P};
-  return dtype == NF_F32 ? run_direct<float>(a) : run_direct<bf16>(a);
+  // A launch numbers its pixels in 32 bits: as many images as that holds, or rows of one image where that is more.
+  constexpr long kMaxPixels = 0x7fffffffL;
+  const long map = (long)Ho * Wo, imgs = std::max(1L, kMaxPixels / map), rows = map > kMaxPixels ? kMaxPixels / Wo : Ho;
+  const size_t es = nf_esize(dtype);
+  for (long n0 = 0; n0 < N; n0 += imgs)
+    for (long r0 = 0; r0 < Ho; r0 += rows) {
+      const long P = std::min(imgs, N - n0) * std::min(rows, Ho - r0) * Wo;
+      const ConvArgs a{(const char*)x + (size_t)n0 * H * W * Ci * es, w, (char*)y + (size_t)(n0 * map + r0 * Wo) * Co * es, bias, ws_tap, ws_co, ws_ci,
+                       H, W, Ci, Co, Ho, Wo, stride, taps, flip, relu, (uint32_t)P, (uint32_t)r0};
+      const int rc = dtype == NF_F32 ? run_direct<float>(a) : run_direct<bf16>(a);
+      if (rc != NF_OK) return rc;
+    }
+  return NF_OK;
 }
 
 int nf_k_wgrad_splits(int N, int Ho, int Ci, int Co) {

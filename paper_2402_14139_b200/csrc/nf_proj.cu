@@ -80,12 +80,12 @@ __global__ void proj_bwd_apply_kernel(const T* __restrict__ ys, const T* __restr
 // 64 -> 128 channels and 32 768 pixels.)
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x, const T* __restrict__ dys, int H, int W, int Ci, int Co,
-                                                         int Ho, int Wo, uint32_t P, int stride, int splits, float* __restrict__ part) {
+                                                         int Ho, int Wo, size_t P, int stride, int splits, float* __restrict__ part) {
   nf_pdl_begin();
   __shared__ __align__(16) float xs[2][32][64];
   __shared__ __align__(16) float gs[2][32][64];
   const int ci0 = blockIdx.x * 64, co0 = blockIdx.y * 64, sp = blockIdx.z, t = threadIdx.x;
-  const uint32_t p0 = (uint32_t)((size_t)P * sp / splits), p1 = (uint32_t)((size_t)P * (sp + 1) / splits);
+  const size_t p0 = P * sp / splits, p1 = P * (sp + 1) / splits;
   const int q = t >> 3, c = (t & 7) * 8;  // the thread's pixel and channels of a step
   const int ti = (t >> 4) * 4, to = (t & 15) * 4;
   float xr[8], gr[8];
@@ -99,12 +99,19 @@ __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x
       for (int e = 0; e < 8 && c0 + e < C; ++e) v[e] = ldf(src, c0 + e);
     }
   };
-  auto fetch = [&](uint32_t pb) {
-    const uint32_t p = pb + q;
+  auto fetch = [&](size_t pb) {
+    const size_t p = pb + q;
     if (p < p1) {
-      const uint32_t r = p / Wo, n = r / Ho;
-      row(x + (((size_t)n * H + (size_t)(r - n * Ho) * stride) * W + (size_t)(p - r * Wo) * stride) * Ci, ci0 + c, Ci, xr);
-      row(dys + (size_t)p * Co, co0 + c, Co, gr);
+      size_t r = 0, n = 0;
+      if (P <= 0xffffffffull) {  // 32-bit divisions where they do
+        r = (uint32_t)p / (uint32_t)Wo;
+        n = (uint32_t)r / (uint32_t)Ho;
+      } else {
+        r = p / Wo;
+        n = r / Ho;
+      }
+      row(x + ((n * H + (r - n * Ho) * stride) * W + (p - r * Wo) * stride) * Ci, ci0 + c, Ci, xr);
+      row(dys + p * Co, co0 + c, Co, gr);
     } else {
 #pragma unroll
       for (int e = 0; e < 8; ++e) xr[e] = gr[e] = 0.f;
@@ -126,7 +133,7 @@ __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x
   put(0);
   __syncthreads();
   int b = 0;
-  for (uint32_t pb = p0; pb < p1; pb += 32) {
+  for (size_t pb = p0; pb < p1; pb += 32) {
     const bool more = pb + 32 < p1;
     if (more) fetch(pb + 32);
 #pragma unroll 8
@@ -390,11 +397,10 @@ int nf_proj_backward(nf_proj* P, const void* xb, const void* dz, float lr) {
   } else if (rc != NF_OK) {
     return rc;
   }
-  if (pix > 0x7fffffffu) return NF_EUNSUPPORTED;
   const dim3 grid((P->Cin + 63) / 64, (C + 63) / 64, P->splits);
   const bool vec = P->Cin % 8 == 0 && C % 8 == 0;
 #define PROJ_WGRAD(T, V)                                                                                                              \
-  nf_launch(proj_wgrad_kernel<T, V>, grid, 256, 0, (const T*)xb, (const T*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo, (uint32_t)pix, 2, \
+  nf_launch(proj_wgrad_kernel<T, V>, grid, 256, 0, (const T*)xb, (const T*)P->dys, P->H, P->W, P->Cin, C, P->Ho, P->Wo, pix, 2, \
             P->splits, P->wpart)
   PROJ_DISPATCH(P->dtype, (vec ? PROJ_WGRAD(float, 1) : PROJ_WGRAD(float, 0)), (vec ? PROJ_WGRAD(bf16, 1) : PROJ_WGRAD(bf16, 0)));
 #undef PROJ_WGRAD
