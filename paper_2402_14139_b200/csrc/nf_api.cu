@@ -428,7 +428,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     if (rc == NF_EUNSUPPORTED) {
       NF_TRY(nf_k_fc_ce(L->p, labels, N, D, K, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->logits, L->dlogits,
                         L->dp, L->lossn, L->status, L->o.loss, n_scale));
-      rc = nf_k_fc_wgrad(L->p, L->dlogits, L->lossn, N, D, K, g + L->off[NF_P_WF], g + L->off[NF_P_BF], loss_out, L->status, n_scale);
+      rc = nf_head_batch_sums(L->p, L->dlogits, L->lossn, N, D, K, g + L->off[NF_P_WF], g + L->off[NF_P_BF], loss_out, L->status, n_scale);
     }
     if (rc != NF_OK) return rc;
   }

@@ -501,48 +501,6 @@ __global__ void __launch_bounds__(256) fc_predict_kernel(const float* __restrict
   if (t == 0) pred[n] = bi[0];
 }
 
-// one block per class k: gWf[k][:] = sum_n dlogits[n][k] p[n][:], gbf[k]; block 0 also reduces the loss
-__global__ void __launch_bounds__(256) fc_wgrad_kernel(const float* __restrict__ p, const float* __restrict__ dl,
-                                                       const float* __restrict__ lossn, int N, int D, int K,
-                                                       float* __restrict__ gWf, float* __restrict__ gbf,
-                                                       float* __restrict__ loss_out, int32_t* status, int n_scale) {
-  nf_pdl_begin();
-  // Sums over the batch run as four interleaved chains (samples n % 4) that are combined in a fixed order, and the
-  // two scalar sums are spread over a warp: the serial chains of one load per sample were pure latency.
-  const int k = blockIdx.x, t = threadIdx.x;
-  for (int d = t; d < D; d += 256) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    int n = 0;
-    for (; n + 3 < N; n += 4) {
-      s0 = fmaf(dl[(size_t)n * K + k], p[(size_t)n * D + d], s0);
-      s1 = fmaf(dl[(size_t)(n + 1) * K + k], p[(size_t)(n + 1) * D + d], s1);
-      s2 = fmaf(dl[(size_t)(n + 2) * K + k], p[(size_t)(n + 2) * D + d], s2);
-      s3 = fmaf(dl[(size_t)(n + 3) * K + k], p[(size_t)(n + 3) * D + d], s3);
-    }
-    for (; n < N; ++n) s0 = fmaf(dl[(size_t)n * K + k], p[(size_t)n * D + d], s0);
-    gWf[(size_t)k * D + d] = (s0 + s1) + (s2 + s3);
-  }
-  const int warp = t >> 5, lane = t & 31;
-  if (warp == 7) {  // gbf[k]: lane sums over n = lane, lane + 32, ..., then a fixed butterfly
-    float s = 0.f;
-    for (int n = lane; n < N; n += 32) s += dl[(size_t)n * K + k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) gbf[k] = s;
-  }
-  if (k == 0 && warp == 6) {
-    double s = 0.0;
-    for (int n = lane; n < N; n += 32) s += (double)lossn[n];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      const float L = (float)(s / (double)n_scale);
-      *loss_out = L;
-      if (!isfinite(L)) atomicOr(status, NF_ENONFINITE);
-    }
-  }
-}
-
 // dh[n,i,j,f] = 1[h>0] * sum over bins containing (i,j) of dp[n][f*4+bin] / |bin|
 template <typename T>
 __global__ void dh_kernel(const T* __restrict__ h, const float* __restrict__ dp, int Ha, int Wa, int F, size_t total,
@@ -1793,13 +1751,6 @@ int nf_k_fc_predict(const float* p, int N, int D, int K, const float* Wf, const 
   const size_t smem = (size_t)D * sizeof(float);
   if (smem > 40000) return NF_EUNSUPPORTED;
   nf_launch(fc_predict_kernel, N, 256, smem, p, D, K, Wf, bf, logits, pred);
-  NF_LAUNCHED();
-  return NF_OK;
-}
-
-int nf_k_fc_wgrad(const float* p, const float* dlogits, const float* lossn, int N, int D, int K, float* gWf,
-                    float* gbf, float* loss_out, int32_t* status, int n_scale) {
-  nf_launch(fc_wgrad_kernel, K, 256, 0, p, dlogits, lossn, N, D, K, gWf, gbf, loss_out, status, n_scale);
   NF_LAUNCHED();
   return NF_OK;
 }

@@ -177,6 +177,9 @@ struct NfHeadIo {
 };
 int nf_head_sample_mode(int dtype, int N, int Ha, int Wa, int F, int K);
 int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, int F, int K, int loss_kind, int n_scale);
+// its second kernel alone, after nf_k_fc_ce: gWf, gbf and the mean loss
+int nf_head_batch_sums(const float* p, const float* dlogits, const float* lossn, int N, int D, int K, float* gWf, float* gbf, float* loss_out,
+                       int32_t* status, int n_scale);
 // small-batch head (nf_head_small.cu): class-sliced forward + backward of the linear layer and the loss; 0 floats = not covered
 size_t nf_head_small_scratch_floats(int N, int D, int K);
 // whether that head takes the sizes, and its summation order: classes per slice, slices, ranges the slices' shares are folded in
@@ -189,8 +192,6 @@ int nf_k_bn_finalize_tot(const double* tot, int C, double M, const float* gamma,
                            float* scale, float* shift, float* mu, float* invstd, float* rmean, float* rvar);
 int nf_k_bn_bwd_finalize_tot(const double* tot, int C, int world, float* sdz, float* sdzx, float* ggamma, float* gbeta);
 int nf_k_fc_predict(const float* p, int N, int D, int K, const float* Wf, const float* bf, float* logits, int32_t* pred);
-int nf_k_fc_wgrad(const float* p, const float* dlogits, const float* lossn, int N, int D, int K, float* gWf,
-                    float* gbf, float* loss_out, int32_t* status, int n_scale);
 int nf_k_dh(int dtype, const void* h, const float* dp, int N, int Ha, int Wa, int F, void* dh);
 int nf_k_sum_partials(const float* red, int nblocks, int C, float* out);
 int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
