@@ -1534,8 +1534,10 @@ __global__ void __launch_bounds__(256, 2) bn_bwd_apply_pool_vec_kernel(const uin
 inline bool vec_ok(int dtype, int C, int pool) { return dtype == NF_BF16 && C % 8 == 0 && C <= 1024 && !pool; }
 // either storage type: a thread keeps its eight channels over its whole loop
 inline bool vec2_ok(int C, int pool) { return C % 8 == 0 && C <= 2048 && 256 % (C / 8) == 0 && !pool; }
+// eight items per thread, fewer where that leaves SMs idle
 inline int vec_blocks(size_t work_items) {
-  size_t b = (work_items + 256 * 8 - 1) / (256 * 8);
+  const size_t one = (work_items + 255) / 256;
+  size_t b = std::max((work_items + 256 * 8 - 1) / (256 * 8), std::min(one, (size_t)296));
   if (b < 1) b = 1;
   if (b > 148 * 16) b = 148 * 16;
   return (int)b;
@@ -1704,7 +1706,8 @@ int nf_k_dh_fast(const void* h, const float* dp, int N, int Ha, int Wa, int F, v
 
 int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* p) {
   if ((long)((Ha + 1) / 2) * ((Wa + 1) / 2) <= 16) {  // tiny maps (late blocks train at thousands of samples): a thread per output
-    if (dtype == NF_BF16 && F % 8 == 0) {
+    // (bf16: 32 outputs per thread where one each would not fit the chip at once, or is one pixel; one image of 7 x 7: 15 against 6 us)
+    if (dtype == NF_BF16 && F % 8 == 0 && ((size_t)N * 4 * F > (size_t)148 * 2048 || Ha * Wa <= 4)) {
       const size_t groups = (size_t)N * (F / 8);
       nf_launch(avgpool_small_vec_kernel, nblk(groups, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, groups, (float4*)p);
       NF_LAUNCHED();
