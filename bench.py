@@ -29,21 +29,6 @@ METRIC = "local-layer train-step images/s (bf16)"
 FALLBACK_PEAKS = dict(hbm_gbs=6650.0, bf16_tflops=1590.0, bf16_tflops_sustained=1400.0)
 
 
-# DRAM bytes per image (read + write) of the kernels behind each traced op on the c4 layers 64->64 at 224x224,
-# from one ncu capture of the batch-24 case (profiles/ncu_full_c4s_conv_bn_kernels.md); every tensor is streamed
-# once, so traffic grows in proportion to the batch.  Valid for the kernels as captured; None elsewhere.
-NCU_TRAFFIC_C4_BYTES_PER_IMAGE = dict(conv_fwd=(154.31 + 107.70) * 1e6 / 24, wgrad=(324.60 + 3.75) * 1e6 / 24,
-                                      # aux forward with the fused BatchNorm + ReLU: reads y, writes a, the sign mask and the
-                                      # pooling partials (h is not stored)
-                                      aux_fwd=(154.21 + 115.70) * 1e6 / 24,
-                                      # second pass of the aux input gradient: reads dh and y, writes dy; the finalize kernel < 1 MB
-                                      bn_bwd=(192.74 + 108.21) * 1e6 / 24,
-                                      # dh from the mask + aux weight gradient; the two small partial-sum kernels move < 1 MB
-                                      aux_wgrad=(2.45 + 0.01 + 201.43 + 3.72) * 1e6 / 24,
-                                      # first pass of the input gradient (dh and y read, sums only)
-                                      aux_dgrad=(192.74 + 5.13) * 1e6 / 24)
-
-
 def load_peaks():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
@@ -140,19 +125,20 @@ def op_model(l, N, classes, es, fam):
     fused = len(fam) > 4 and fam[4] == "fused"   # BatchNorm + ReLU applied inside the aux forward kernel
     masked = len(fam) > 5 and fam[5] == "mask"   # h never stored: pooled in the aux forward's epilogue, sign bits kept
     two_pass = len(fam) > 6 and fam[6] == "two-pass"   # da never stored: the input gradient runs once for the sums, once for dy
+    head_dh = len(fam) > 8 and fam[8] == "head"        # the head's kernel reads h and writes dh
     return dict(conv_fwd=(tc(0), fl["conv_fwd"], es * (nx + ny)),          # read x, write y
                 wgrad=(tc(1), fl["wgrad"], es * (nx + ny)),                # read x and dy
                 # read a, write h; fused: read y, write a and h
                 aux_fwd=(tc(2), fl["aux_fwd"], es * ((ny if fused else 0) + na + (0 if masked else nh))),
-                # h -> dh (from the sign mask: dh written only); a, dh -> gWa
-                aux_wgrad=(tc(3), fl["aux_bwd"] / 2, es * ((2 if masked else 3) * nh + na)),
+                # h -> dh (from the sign mask: dh written only; where the head does it: nothing here); a, dh -> gWa
+                aux_wgrad=(tc(3), fl["aux_bwd"] / 2, es * ((2 if masked else 1 if head_dh else 3) * nh + na)),
                 # dh -> da (two-pass: dh and y read, sums only)
-                aux_dgrad=(tc(3), fl["aux_bwd"] / 2, es * (nh + (ny if two_pass else na))),
+                aux_dgrad=(tc(7 if len(fam) > 7 else 3), fl["aux_bwd"] / 2, es * (nh + (ny if two_pass else na))),
                 # read y, write a; fused: only the statistics are finished here (partial sums in, coefficients out)
                 bn_fwd=("hbm", None, 4 * 2 * l["Cout"] * 1184 if fused else es * (ny + na)),
                 # read y and da, write dy; two-pass: the second run of the input gradient reads dh and y and writes dy
                 bn_bwd=("hbm", None, es * (nh + 2 * ny) if two_pass else es * (2 * ny + na)),
-                head=("hbm", None, es * nh + 4 * N * (8 * l["F"] + 2 * classes)),
+                head=("hbm", None, es * (2 if head_dh else 1) * nh + 4 * N * (8 * l["F"] + 2 * classes)),
                 sgd=("hbm", None, 18 * nparam))                            # theta, v read+write (fp32), g read, bf16 copy write
 
 
@@ -276,7 +262,7 @@ def run_ours(args, rank, world):
     ms, e2e_s = max_over_ranks([ms, e2e_s], world, "cuda")
 
     peaks, peak_src = load_peaks()
-    fam = [[L.kernel_family(k) for k in range(7)] for L in layers]
+    fam = [[L.kernel_family(k) for k in range(9)] for L in layers]
     clocks = sampler.summary()
     # Which measured bf16 peak the tensor kernels are held against: the timed region and the per-op pass last a fraction
     # of a second each, so unless the sampled SM clock has already dropped well below its maximum these are burst
@@ -285,9 +271,7 @@ def run_ours(args, rank, world):
     tkey = "bf16_tflops" if burst else "bf16_tflops_sustained"
     kernels = kernel_table(trace, ls, N, wl["classes"], es, fam, peaks, tkey)
     best = kernels[0]
-    traffic = None
-    if wl["name"] in ("c4", "c4s") and best["layer"] in (0, 1) and best["op"] in NCU_TRAFFIC_C4_BYTES_PER_IMAGE:
-        traffic = round(NCU_TRAFFIC_C4_BYTES_PER_IMAGE[best["op"]] * N)
+    traffic = None  # measured DRAM bytes: none, the kernels have changed since the last capture
     roof = dict(bound=best["bound"], achieved=best["achieved"], peak=best["peak"], unit=best["unit"],
                 frac=best["frac"], traffic=traffic, kernel=f'{best["op"]}[layer {best["layer"]}]',
                 peak_source=f"{peak_src} ({'burst' if burst else 'sustained'} bf16 figure)" if best["bound"] != "hbm" else peak_src)

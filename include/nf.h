@@ -377,14 +377,16 @@ int nf_selftest_bounded_wait(unsigned long long limit_ns, unsigned long long* wa
 long long nf_launch_count(void);
 
 /* Name of the kernel family a configured layer uses for op 0 = main forward,
- * 1 = main weight gradient, 2 = aux forward, 3 = aux backward: "tcgen05" or "cuda-core".
+ * 1 = main weight gradient, 2 = aux forward, 3 = aux weight gradient, 7 = aux input gradient: "tcgen05" or "cuda-core".
  * op 4: "fused" when the BatchNorm + ReLU pass of the step runs inside the aux forward kernel
  * (which then also writes act_out), "separate" otherwise.
  * op 5: "mask" when that kernel also pools the aux output h in its epilogue and keeps only one sign bit per element of it
  * (Eq. 2's F_n applied before h ever reaches memory), "stored" when h is written and pooled by separate kernels.
  * op 6: "two-pass" when the aux input gradient runs twice -- once to reduce the BatchNorm-backward sums, once more to write
  * the gradient at the conv output directly -- so that the gradient at the activation (NF_T_DA) is never stored and no
- * separate BatchNorm-backward pass runs; "stored" otherwise. */
+ * separate BatchNorm-backward pass runs; "stored" otherwise.
+ * op 8: "head" when the kernel of the head writes the gradient at h too, "separate" when kernels of its own do (of a layer with
+ * a workspace). */
 const char* nf_layer_kernel_family(const nf_layer* layer, int op);
 
 const char* nf_strerror(int status);

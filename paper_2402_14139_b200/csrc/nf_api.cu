@@ -341,6 +341,14 @@ int nf_layer_get_param(nf_layer* L, int which, float* host, size_t n) {
     if (rc_ != NF_OK) return rc_; \
   } while (0)
 
+// nf_head_sample_mode for a layer: 2 only where h is stored and the sums of dh over each sample fit the reduction scratch
+static int layer_head_mode(const nf_layer* L, bool h_masked) {
+  const int N = L->o.N, F = L->F, K = L->classes;
+  if (L->o.aux_pool != NF_POOL_AVG || nf_head_is_large(N, 4 * F, K)) return 0;
+  const int mode = nf_head_sample_mode(L->o.dtype, N, L->Ha, L->Wa, F, K);
+  return mode == 2 && (h_masked || (size_t)N * F > L->red_floats) ? 1 : mode;
+}
+
 // The whole step (phase < 0, world = 1), or one of the four phases of the data-parallel step: 0 = conv forward and
 // the rank's per-channel sums; 1 = normalise with the statistics of the whole batch ... aux input gradient and the
 // rank's BatchNorm-backward sums; 2 = BatchNorm backward with the sums of the whole batch, weight gradient; 3 = update.
@@ -399,8 +407,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   // h_masked: the aux forward left pooling partials (L->wpart) and a sign mask (in L->h) instead of h
   const bool h_masked = fused_bn_aux && nf_tc_aux_pool_fused(L);
   // heads of ordinary size: one block per sample does all of it, and writes dh where the sample's h fits its shared memory
-  int sample_mode = L->o.aux_pool == NF_POOL_AVG && !nf_head_is_large(N, D, K) ? nf_head_sample_mode(dt, N, Ha, Wa, F, K) : 0;
-  if (sample_mode == 2 && (h_masked || (size_t)N * F > L->red_floats)) sample_mode = 1;
+  const int sample_mode = layer_head_mode(L, h_masked);
   if (sample_mode == 2 || (h_masked && sample_mode)) {  // pooled by the head itself
   } else if (h_masked) {
     NF_TRY(nf_k_pool_finish(L->wpart, N, Ha / 8, Wa / 14, F, 1.f / (float)((Ha / 2) * (Wa / 2)), L->p));
@@ -958,10 +965,12 @@ int nf_set_stream(void* s) {
 long long nf_launch_count(void) { return g_nf_launches; }
 
 const char* nf_layer_kernel_family(const nf_layer* L, int op) {
-  if (!L || op < 0 || op > 6) return "";
+  if (!L || op < 0 || op > 8) return "";
   if (op == 4) return nf_tc_bn_aux_fused(L) && !L->skip ? "fused" : "separate";
   if (op == 5) return nf_tc_bn_aux_fused(L) && !L->skip && nf_tc_aux_pool_fused(L) ? "mask" : "stored";
   if (op == 6) return nf_tc_dgrad_two_pass(L) && !L->skip && !L->skip_grad ? "two-pass" : "stored";
+  if (op == 7) return L->dgrad_tc ? "tcgen05" : "cuda-core";
+  if (op == 8) return layer_head_mode(L, nf_tc_bn_aux_fused(L) && !L->skip && nf_tc_aux_pool_fused(L)) == 2 ? "head" : "separate";
   return L->fam[op] ? "tcgen05" : "cuda-core";
 }
 
