@@ -119,7 +119,7 @@ static inline void nf_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t
 static inline size_t nf_align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 static inline size_t nf_esize(int dtype) { return dtype == NF_F32 ? 4 : 2; }
 
-// ---- generic CUDA-core kernels (nf_k_kernels.cu): any shape, fp32 or bf16 storage, fp32 accumulate
+// ---- generic CUDA-core kernels (nf_direct.cu, nf_elem.cu): any shape, fp32 or bf16 storage, fp32 accumulate
 int nf_k_conv(int dtype, const void* x, int N, int H, int W, int Ci, const void* w, long ws_tap, long ws_co,
                 long ws_ci, int flip, const float* bias, int relu, int stride, int Co, void* y);
 // the general form: taps = 9 (3x3, pad 1) or 1 (1x1, no pad)

@@ -36,7 +36,8 @@ constexpr int kFoldThreads = 320;  // folded-tap forward: producer, MMA issuer a
 // (about four tiles per HBM round trip) whatever else it did; with five the loads run as far ahead as the operand stages.
 constexpr int kYSlots = 5;
 
-// Division by a number that is fixed for a launch, as a multiplication (exact for dividends below 2^31).  The role loops decode
+// Division by a number that is fixed for a launch, as a multiplication by a rounded-up reciprocal (Granlund and Montgomery, Division by
+// Invariant Integers using Multiplication, 1994; exact for dividends below 2^31).  The role loops decode
 // a tile number per tile; a 32-bit division by a run-time value costs a single thread about 100 cycles of dependent instructions.
 struct FDiv {
   uint32_t d, mul, shift;
@@ -1247,8 +1248,8 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 }
 
 // ---------------------------------------------------------------- aux input gradient, 256 pixels per instruction
-// The narrow input gradient da = dh (*) Wa^T (K = F <= 32 per tap) is bound by the NUMBER of its K = 16 instructions, each of
-// which holds the tensor pipe for about the same time whatever its shape.  With the pixels on the M side an instruction covers
+// The narrow input gradient da = dh (*) Wa^T (K = F <= 32 per tap) is bound by the NUMBER of its K = 16 instructions: up to 64 columns
+// an instruction takes about 40 cycles, the time to read its operands, whatever its width.  With the pixels on the M side an instruction covers
 // 128 of them; here the operands are swapped: A = the mirrored weight tile of a tap, [64 output channels] x [16 f] (M = 64,
 // MN-major as stored), B = 256 pixels x [16 f] of the dh box (N = 256, K-major), so the nine taps of a 256-pixel tile are nine
 // instructions instead of eighteen.  A tile is 8 columns x 32 rows; ONE 10 x 34-pixel box feeds all taps (a tap is a start
@@ -2038,7 +2039,7 @@ conv_wgrad_row_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 }
 
 // ---------------------------------------------------------------- weight gradient, stride 1, few filters: gradient on the M side
-// An instruction holds the tensor pipe for about the same time whatever its shape, so for the auxiliary conv
+// An instruction of up to 64 columns takes about 40 cycles whatever its width, one of 192 takes 96, so for the auxiliary conv
 // (F <= 32 filters) the fewest instructions win.  Here the roles of conv_wgrad_kw_kernel are swapped:
 //   A (M = 4 * NB rows) = the three column-shifted gradient tiles as consecutive MN-major atoms (kw, f) plus one unused atom,
 //   B (N = 192)         = the three row taps of the activation box as consecutive 64-channel atoms (kh, ci),
@@ -2769,8 +2770,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
     rc = pl.NB == 256 ? launch_wgrad<256, 0>(pl, mx, mg, p) : pl.NB == 128 ? launch_wgrad<128, 0>(pl, mx, mg, p)
        : pl.NB == 64 ? launch_wgrad<64, 0>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 0>(pl, mx, mg, p) : launch_wgrad<16, 0>(pl, mx, mg, p);
   else
-    rc = pl.NB == 64 ? launch_wgrad_kw<64>(pl, mx, mg, p)
-                     : pl.NB == 32 ? launch_wgrad_kw<32>(pl, mx, mg, p) : launch_wgrad_kw<16>(pl, mx, mg, p);
+    rc = launch_wgrad_kw<64>(pl, mx, mg, p);  // up to 32 filters take the form above
   if (rc != NF_OK) return rc;
   const size_t n = (size_t)9 * Cout * Cin;
   return nf_k_sum_parts(part, pl.splits, n, dw, pl.SEG != 0);
@@ -2825,11 +2825,11 @@ size_t nf_tc_red_floats(const nf_layer* L) {
   if (L->fam[3]) need = (size_t)sm_count() * 8 * 2 * L->Cout;  // input-gradient kernel with the fused BatchNorm-backward sums
   if (!L->fam[0]) return need;
   const TcPlan pl = plan_fwd(L->Ho, L->Wo, L->cin_pad ? L->cin_pad : L->Cin, L->Cout, L->o.N, 0, L->o.stride);
-  const size_t fwd = (size_t)sm_count() * (pl.parts < 8 ? 8 : pl.parts) * 2 * L->Cout;  // the folded kernel writes 8 partials per CTA
+  const size_t fwd = (size_t)sm_count() * (pl.parts < 8 ? 8 : pl.parts) * 2 * L->Cout;  // room for 8 partials per CTA; the folded kernel writes 2
   return fwd > need ? fwd : need;
 }
 
-// input and operand weights of the main conv: the caller's, or their 64-channel zero-padded copies (refreshed here)
+// input and operand weights of the main conv: the caller's, or their zero-padded copies of 16 or 64 channels (refreshed here)
 static int main_conv_operands(nf_layer* L, const void* x, int count, const void** xin, const void** win, int* Cin) {
   *xin = x;
   *win = L->shadow + L->off[NF_P_W];
