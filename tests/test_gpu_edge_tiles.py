@@ -1,5 +1,5 @@
 """Edges of the tiles and of the dispatch rules: the weight gradient with 128 output channels on the M side, first layers over 16
-padded channels, the CUDA-core convolutions and the per-sample and large-batch heads.  Tolerances are those of parity_util.TOL."""
+padded channels, the CUDA-core convolutions and the per-sample heads (the large-batch ones: test_gpu_large_heads.py).  Tolerances are those of parity_util.TOL."""
 import pytest
 
 from tests import parity_util as pu
@@ -19,7 +19,7 @@ BF16 = [
     dict(N=3, Cin=3, Cout=64, H=28, W=28, F=8, classes=10, stride=1, pool=False),
     dict(N=9, Cin=4, Cout=64, H=32, W=32, F=16, classes=10, stride=1, pool=True),
     dict(N=2, Cin=3, Cout=64, H=64, W=128, F=16, classes=10, stride=1, pool=False),
-    # a class count and batch on each side of the heads' boundaries
+    # per-sample heads: few classes, many, one sample
     dict(N=63, Cin=64, Cout=64, H=8, W=8, F=12, classes=3, stride=1, pool=False),
     dict(N=130, Cin=64, Cout=64, H=8, W=8, F=40, classes=101, stride=1, pool=False),
     dict(N=1, Cin=64, Cout=64, H=8, W=16, F=8, classes=10, stride=1, pool=False),

@@ -56,3 +56,51 @@ def test_evaluation_in_place(ci):
     assert G.status() == 0
     blk.close()
     G.close()
+
+
+FORMS = [  # (config, count): every instantiation that normalises in the convolution's epilogue, and the stride-2 ones
+    (dict(N=9, Cin=64, Cout=64, H=32, W=32, F=16, classes=10, stride=1, pool=False), 7),     # folded column taps
+    (dict(N=6, Cin=3, Cout=64, H=32, W=32, F=16, classes=10, stride=1, pool=False), 5),      # folded, input padded to 16 channels
+    (dict(N=12, Cin=64, Cout=64, H=16, W=16, F=16, classes=10, stride=1, pool=False), 9),    # resident weights
+    (dict(N=9, Cin=64, Cout=128, H=16, W=16, F=16, classes=10, stride=1, pool=False), 8),    # three boxes per chunk, 128 channels
+    (dict(N=9, Cin=128, Cout=64, H=16, W=16, F=16, classes=10, stride=1, pool=False), 8),    # the same, 64 channels
+    (dict(N=11, Cin=64, Cout=256, H=8, W=8, F=16, classes=10, stride=1, pool=False), 9),     # 256 channels in two halves
+    (dict(N=11, Cin=64, Cout=128, H=8, W=8, F=16, classes=10, stride=1, pool=False), 9),     # per tap, 128 channels
+    (dict(N=11, Cin=64, Cout=64, H=16, W=16, F=16, classes=10, stride=2, pool=False), 9),    # per tap, 64 channels
+    (dict(N=45, Cin=64, Cout=128, H=14, W=14, F=16, classes=10, stride=1, pool=False), 43),  # segments, 128 channels
+    (dict(N=12, Cin=64, Cout=64, H=28, W=28, F=16, classes=10, stride=1, pool=False), 11),   # segments, 64 channels
+    (dict(N=45, Cin=64, Cout=256, H=14, W=14, F=16, classes=10, stride=1, pool=False), 11),  # fewer than 8192 pixels of a batch that has them
+]
+
+
+@pytest.mark.parametrize("ci", range(len(FORMS)))
+def test_every_form_of_the_evaluating_convolution(ci):
+    """predict and cache with running statistics against the checker, for fewer samples than the batch size; rows beyond are left alone."""
+    import torch
+    from paper_2402_14139_b200 import nf
+    nf.lib()
+    nf.nf_set_stream(None)
+    c, count = FORMS[ci]
+    P, x, rm, rv, G = _layer(nf, c, 0x4E46F100 + ci)
+    assert G.kernel_family(0) == "tcgen05"
+    O = pu.oracle_layer(c, P, store_bf16=True)
+    O.set(rmean=rm, rvar=rv)
+    act_o, logits_o, _ = O.predict(x[:count])
+    xd = pu.to_device_nhwc(torch, x[:count], 1)
+    act, cache = G.new_act(), G.new_act()
+    act.fill_(7.0)
+    cache.fill_(7.0)
+    logits, pred = torch.zeros((count, c["classes"]), device="cuda"), torch.zeros(count, dtype=torch.int32, device="cuda")
+    G.predict(xd, pred, act_out=act, logits_out=logits, count=count)
+    blk = nf.Block([G])
+    blk.cache(xd, cache, count=count)
+    torch.cuda.synchronize()
+    assert G.status() == 0
+    # stored twice in bf16 on both sides: a unit of 2^-8 of the value where the roundings of y fall on different sides
+    err = np.abs(pu.from_device_nhwc(act)[:count] - act_o)
+    assert (err <= 2.0 ** -7 * np.abs(act_o) + 2.0 ** -8 * np.abs(act_o).max()).all()
+    assert (err > 2.0 ** -9 * np.abs(act_o).max()).mean() <= 0.01
+    assert np.abs(logits.cpu().numpy() - logits_o).max() <= pu.TOL[1]["t"] * np.abs(logits_o).max()
+    assert torch.equal(cache, act) and bool((act[count:] == 7.0).all())
+    blk.close()
+    G.close()
