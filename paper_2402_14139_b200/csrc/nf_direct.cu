@@ -29,6 +29,18 @@ struct ConvArgs {
   uint32_t row0;  // the first one's row, where a launch takes some rows of one image (else 0)
 };
 
+template <int T> __device__ __forceinline__ void ld_tile(const float* p, float (&v)[T]) {
+  if constexpr (T == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else if constexpr (T == 2) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    v[0] = q.x; v[1] = q.y;
+  } else {
+    v[0] = *p;
+  }
+}
+
 // WCO: 1 = eight consecutive output channels of the weights are contiguous, 0 = eight input channels.  VEC: rows of eight are
 // whole and aligned; otherwise elements are fetched one by one.
 template <typename T, int PX, int CO, int CK, int TP, int TC, int SPB, int WCO, int VEC>
@@ -36,10 +48,12 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
   nf_pdl_begin();
   constexpr int kThr = (PX / TP) * (CO / TC), kXU = PX * CK / 8, kWU = CO * CK / 8;  // units of eight values per step
   constexpr int kXN = (kXU + kThr - 1) / kThr, kWN = (kWU + kThr - 1) / kThr;
+  constexpr int kW0 = kThr >= kXU + kWU ? kXU : 0;  // first thread that fetches weights: others than fetch pixels where there are enough
   // column q of row c is kept at q ^ (8 * (c / 8)) (mod the row): the transposing stores then hit different banks
   constexpr int kXM = PX >= 32 ? 24 : 8, kWM = CO >= 32 ? 24 : 8;
-  __shared__ __align__(16) float xs[2][SPB][CK][PX];
-  __shared__ __align__(16) float ws[2][SPB][CK][CO];
+  constexpr int kBuf = SPB == 9 ? 1 : 2;  // nine taps: one buffer, the next chunk waits in registers
+  __shared__ __align__(16) float xs[kBuf][SPB][CK][PX];
+  __shared__ __align__(16) float ws[kBuf][SPB][CK][CO];
   const T* __restrict__ x = reinterpret_cast<const T*>(a.x);
   const T* __restrict__ w = reinterpret_cast<const T*>(a.w);
   const int t = threadIdx.x, tc = t % (CO / TC), tp = t / (CO / TC);
@@ -78,11 +92,11 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
     const size_t tb = (size_t)(a.flip ? 8 - tap : tap) * a.ws_tap;
 #pragma unroll
     for (int u = 0; u < kWN; ++u) {
-      const int e = t + u * kThr;
+      const int e = t - kW0 + u * kThr;
       const int ci = c0 + (WCO ? e / (CO / 8) : (e % (CK / 8)) * 8), co = co0 + (WCO ? (e % (CO / 8)) * 8 : e / (CK / 8));
 #pragma unroll
       for (int q = 0; q < 8; ++q) wr[u][q] = 0.f;
-      if (e < kWU && ci < a.Ci && co < a.Co) {
+      if (e >= 0 && e < kWU && ci < a.Ci && co < a.Co) {
         const T* src = w + tb + (size_t)co * a.ws_co + (size_t)ci * a.ws_ci;
         if constexpr (VEC) {
           ld8(src, wr[u]);
@@ -104,8 +118,8 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
     }
 #pragma unroll
     for (int u = 0; u < kWN; ++u) {
-      const int e = t + u * kThr;
-      if (e < kWU) {
+      const int e = t - kW0 + u * kThr;
+      if (e >= 0 && e < kWU) {
         if constexpr (WCO) {
           const int c = e / (CO / 8), q0 = (e % (CO / 8)) * 8;
           float* dst = &ws[c][q0 ^ (c & ~7 & kWM)];
@@ -142,37 +156,55 @@ __global__ void __launch_bounds__((PX / TP) * (CO / TC)) conv_direct_kernel(cons
     if (more)
 #pragma unroll
       for (int i = 0; i < SPB; ++i) fetch(nc, nt + i, xr_[i], wr_[i]);
+    if constexpr (SPB == 9) {
+      // eight channels of operands on their way at once: alone on its SM, a block of this small tile otherwise waits for shared memory
+      // on every channel; the larger tiles hide that with other warps and are faster as the compiler orders them
 #pragma unroll 1
-    for (int st = 0; st < SPB; ++st)
+      for (int st = 0; st < SPB; ++st)
+#pragma unroll 1
+        for (int c = 0; c < CK; c += 8) {
+          float xv[8][TP], wv[8][TC];
+          const int sx = (tp * TP) ^ (c & kXM), sw = (tc * TC) ^ (c & kWM);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            ld_tile<TP>(&xs[b][st][c + u][sx], xv[u]);
+            ld_tile<TC>(&ws[b][st][c + u][sw], wv[u]);
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int i = 0; i < TP; ++i)
+#pragma unroll
+              for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(xv[u][i], wv[u][j], acc[i][j]);
+        }
+    } else {
+#pragma unroll 1
+      for (int st = 0; st < SPB; ++st)
 #pragma unroll 8
-      for (int c = 0; c < CK; ++c) {
-        float xv[TP], wv[TC];
-        const float* xp = &xs[b][st][c][(tp * TP) ^ (c & ~7 & kXM)];
-        const float* wp = &ws[b][st][c][(tc * TC) ^ (c & ~7 & kWM)];
-        if constexpr (TP == 4) {
-          const float4 v = *reinterpret_cast<const float4*>(xp);
-          xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
-        } else {
-          const float2 v = *reinterpret_cast<const float2*>(xp);
-          xv[0] = v.x; xv[1] = v.y;
-        }
-        if constexpr (TC == 4) {
-          const float4 v = *reinterpret_cast<const float4*>(wp);
-          wv[0] = v.x; wv[1] = v.y; wv[2] = v.z; wv[3] = v.w;
-        } else {
-          const float2 v = *reinterpret_cast<const float2*>(wp);
-          wv[0] = v.x; wv[1] = v.y;
-        }
+        for (int c = 0; c < CK; ++c) {
+          float xv[TP], wv[TC];
+          const float* xp = &xs[b][st][c][(tp * TP) ^ (c & ~7 & kXM)];
+          const float* wp = &ws[b][st][c][(tc * TC) ^ (c & ~7 & kWM)];
+          ld_tile<TP>(xp, xv);
+          ld_tile<TC>(wp, wv);
 #pragma unroll
-        for (int i = 0; i < TP; ++i)
+          for (int i = 0; i < TP; ++i)
 #pragma unroll
-          for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
-      }
+            for (int j = 0; j < TC; ++j) acc[i][j] = fmaf(xv[i], wv[j], acc[i][j]);
+        }
+    }
     if (!more) break;
+    if constexpr (kBuf == 1) {
+      __syncthreads();
 #pragma unroll
-    for (int i = 0; i < SPB; ++i) put(xs[b ^ 1][i], ws[b ^ 1][i], xr_[i], wr_[i]);
-    __syncthreads();
-    b ^= 1;
+      for (int i = 0; i < SPB; ++i) put(xs[0][i], ws[0][i], xr_[i], wr_[i]);
+      __syncthreads();
+    } else {
+#pragma unroll
+      for (int i = 0; i < SPB; ++i) put(xs[b ^ 1][i], ws[b ^ 1][i], xr_[i], wr_[i]);
+      __syncthreads();
+      b ^= 1;
+    }
     c0 = nc;
     tap = nt;
   }
@@ -216,12 +248,15 @@ template <typename T>
 int run_direct(const ConvArgs& a) {
   // Few output channels: 64 x 16 tiles; with at most 16 input channels (chunks of 16: the same chain, half the shared memory work)
   // a step is so short that the trip to L2 shows, so three taps share one (16 -> 8 channels on 8 images of 32x32: 10.7 -> 6 us)
-  if (a.Co <= 16) {
-    if (a.Ci > 16) return launch_direct<T, 64, 16, 32, 2, 2, 1>(a);
+  if (a.Co <= 16 && a.Ci <= 16)
     return a.taps == 9 ? launch_direct<T, 64, 16, 16, 2, 2, 3>(a) : launch_direct<T, 64, 16, 16, 2, 2, 1>(a);
-  }
-  // 64 x 64 tiles from one block per SM on (148): below that, four times as many blocks of 32 x 32 finish sooner
-  const long big = (long)((a.P + 63) / 64) * ((a.Co + 63) / 64);
+  // 64 x 64 tiles from one block per SM on (148): below that, four times as many blocks of 32 x 32 finish sooner.  Where even those
+  // (or blocks of 64 x 16) leave SMs idle, 16 x 16 with all nine taps per step, a chain of a ninth as many trips to L2: evaluation of one
+  // image, 512 channels at 7x7 382 -> 225 us, 256 at 14x14 213 -> 139 (229 and 152 with a block per 16 pixels of a row, one output
+  // per thread, as all sizes once had)
+  const long big = (long)((a.P + 63) / 64) * ((a.Co + 63) / 64), mid = a.Co <= 16 ? (a.P + 63) / 64 : (long)((a.P + 31) / 32) * ((a.Co + 31) / 32);
+  if (mid < 148) return a.taps == 9 ? launch_direct<T, 16, 16, 32, 2, 1, 9>(a) : launch_direct<T, 16, 16, 32, 2, 1, 1>(a);
+  if (a.Co <= 16) return launch_direct<T, 64, 16, 32, 2, 2, 1>(a);
   if (big >= 148) return launch_direct<T, 64, 64, 32, 4, 4, 1>(a);
   return launch_direct<T, 32, 32, 32, 2, 2, 1>(a);
 }
