@@ -1534,10 +1534,8 @@ __global__ void __launch_bounds__(256, 2) bn_bwd_apply_pool_vec_kernel(const uin
 inline bool vec_ok(int dtype, int C, int pool) { return dtype == NF_BF16 && C % 8 == 0 && C <= 1024 && !pool; }
 // either storage type: a thread keeps its eight channels over its whole loop
 inline bool vec2_ok(int C, int pool) { return C % 8 == 0 && C <= 2048 && 256 % (C / 8) == 0 && !pool; }
-// eight items per thread, fewer where that leaves SMs idle
 inline int vec_blocks(size_t work_items) {
-  const size_t one = (work_items + 255) / 256;
-  size_t b = std::max((work_items + 256 * 8 - 1) / (256 * 8), std::min(one, (size_t)296));
+  size_t b = (work_items + 256 * 8 - 1) / (256 * 8);
   if (b < 1) b = 1;
   if (b > 148 * 16) b = 148 * 16;
   return (int)b;
