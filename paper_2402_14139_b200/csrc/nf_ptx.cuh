@@ -82,6 +82,14 @@ __device__ __forceinline__ void tma_store_wait_read_but_one() { asm volatile("cp
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Gives a shared-memory buffer that TMA filled and that this thread has read with ordinary loads back to the thread that refills it.
+// The fence orders those loads before the next copy's writes, which go through the async proxy; the arrival alone does not: without
+// it a refill overtook the last loads of a tile (BatchNorm-backward sums of 64 channels at 32x32 off by 1e-4 in one step out of ten).
+__device__ __forceinline__ void mbar_release_read(uint64_t* bar) {
+  fence_async_smem();
+  mbar_arrive(bar);
+}
+
 // ---- tensor memory
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {  // whole warp
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)), "r"(ncols) : "memory");

@@ -420,7 +420,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             ssum += dz;
             ssq = fmaf(dz, yv, ssq);
           }
-          ptx::mbar_arrive(&yempty[bsel]);
+          ptx::mbar_release_read(&yempty[bsel]);
           ptx::mbar_arrive(&sfree[bsel]);
         }
         const int ch = my_nt * BN + c;
@@ -538,7 +538,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             sum += dz;
             sq = fmaf(dz, yv, sq);
           }
-          ptx::mbar_arrive(&yempty[ys]);
+          ptx::mbar_release_read(&yempty[ys]);
         } else if (p.stats) {
           float &sum = hf ? ssum2 : ssum, &sq = hf ? ssq2 : ssq;
           const uint8_t* col = stg + (sc / 64) * 16384 + (sc % 8) * 2;
@@ -1172,7 +1172,7 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             }
             *reinterpret_cast<uint4*>(stg_g + off) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
           }
-          ptx::mbar_arrive(&yempty[slot]);
+          ptx::mbar_release_read(&yempty[slot]);
           ptx::fence_async_smem();
           ptx::named_barrier(1 + grp, 128);
         }
@@ -1204,7 +1204,7 @@ conv_fwd_fold_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
               s2[2 * e + 1] = fmaf(z1, y1, s2[2 * e + 1]);
             }
           }
-          ptx::mbar_arrive(&yempty[slot]);
+          ptx::mbar_release_read(&yempty[slot]);
         } else if (p.stats == 1) {
 #pragma unroll
           for (int rr = 0; rr < kStatIters; ++rr) {
@@ -1467,7 +1467,7 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
           }
           *reinterpret_cast<uint4*>(stg_g + off) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
         }
-        ptx::mbar_arrive(&yempty[slot]);
+        ptx::mbar_release_read(&yempty[slot]);
         ptx::fence_async_smem();
         ptx::named_barrier(1 + grp, 128);
       }
@@ -1498,7 +1498,7 @@ aux_dgrad_wide_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             s2[2 * e + 1] = fmaf(z1, y1, s2[2 * e + 1]);
           }
         }
-        ptx::mbar_arrive(&yempty[slot]);
+        ptx::mbar_release_read(&yempty[slot]);
       }
     }
     if (et == 0) ptx::tma_store_wait_all();
