@@ -640,7 +640,13 @@ int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, in
   else
     rc = F == 8 ? run_sample<bf16, 1>(a, smem, stage) : F == 16 ? run_sample<bf16, 2>(a, smem, stage)
        : F == 32 ? run_sample<bf16, 4>(a, smem, stage) : run_sample<bf16, 8>(a, smem, stage);
-  if (rc != NF_OK) return rc;
+  return rc;
+}
+
+int nf_head_sample_sums(const NfHeadIo& io, int N, int F, int K, int n_scale) {
+  int KS, S, parts;
+  const int D = 4 * F;
+  const bool sliced = nf_head_slice_order(N, D, K, &KS, &S, &parts);
   const int DT = (D + 63) / 64, FT = io.dh ? (F + 31) / 32 : 0;
   const int KT = sliced ? (K + 3) / 4 : K;
   nf_launch(sliced ? head_batch_kernel<true> : head_batch_kernel<false>, (unsigned)(KT * DT + FT + 1), 256, 0, io.p, io.dlogits, io.lossn, io.bred, N, D,

@@ -17,6 +17,13 @@ typedef __nv_bfloat16 bf16;
 // fp32 value, fp32 momentum, fp32 gradient, bf16 copy of the value.
 enum { NF_NPARAM = 7 };
 
+// A side stream with the event that orders it against the stream it is forked off; owned by a layer or a block.
+struct NfLane {
+  cudaStream_t s;                      // NULL: could not be had, everything stays in one stream
+  cudaEvent_t e;
+  int dev;                             // the device it belongs to
+};
+
 struct nf_layer {
   // description
   int Cin, Cout, H, W, F, classes;  // F = aux filters as the kernels see them: the caller's count rounded up to a
@@ -71,16 +78,26 @@ struct nf_layer {
   void* xpad;                          // [N][H][W][cin_pad] (bf16)
   bf16* wpad;                          // [9][Cout][cin_pad] operand copy of W, zero beyond Cin
   float* gwpad;                        // [9][Cout][cin_pad] weight gradient over the padded channels
+  NfLane lane;                         // for the parts of a step that nothing in the rest of it waits for
+  size_t ws_total;                     // bytes of the bound workspace
 };
 
 struct nf_block {
   int n;
   nf_layer** layers;
+  NfLane lane[2];                      // where layers' steps go on while the next layer's forward pass runs
 };
 
 // launch bookkeeping (nf_api.cu)
 extern cudaStream_t g_nf_stream;
 extern long long g_nf_launches;
+// Where the calling thread's launches go: the caller's stream (nf_set_stream), or inside a step a side stream forked off it.
+struct NfRoute {
+  cudaStream_t aside;  // NULL: the caller's stream
+  bool plain;          // the next launch follows a wait for another stream: it starts when all it depends on has ended
+};
+extern __thread NfRoute t_nf_route;
+static inline cudaStream_t nf_stream() { return t_nf_route.aside ? t_nf_route.aside : g_nf_stream; }
 int nf_cuda_check(cudaError_t e, const char* what);
 #define NF_CUDA(x)                                        \
   do {                                                    \
@@ -107,12 +124,13 @@ static inline void nf_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = g_nf_stream;
+  cfg.stream = nf_stream();
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = t_nf_route.plain ? 0 : 1;
+  t_nf_route.plain = false;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // an error stays as the last error, which NF_LAUNCHED reads
 }
 
@@ -177,6 +195,8 @@ struct NfHeadIo {
 };
 int nf_head_sample_mode(int dtype, int N, int Ha, int Wa, int F, int K);
 int nf_head_sample_step(const NfHeadIo& io, int dtype, int N, int Ha, int Wa, int F, int K, int loss_kind, int n_scale);
+// the sums over the batch behind it: gWf, gbf, the mean loss and (with dh) the aux bias gradient
+int nf_head_sample_sums(const NfHeadIo& io, int N, int F, int K, int n_scale);
 // its second kernel alone, after nf_k_fc_ce: gWf, gbf and the mean loss
 int nf_head_batch_sums(const float* p, const float* dlogits, const float* lossn, int N, int D, int K, float* gWf, float* gbf, float* loss_out,
                        int32_t* status, int n_scale);

@@ -1,0 +1,135 @@
+"""nf_block_step runs what a layer does behind its forward pass beside the next layers; nf_layer_step runs the auxiliary gradients beside
+the rest.  Neither may change a bit against the same layers stepped one after the other, whatever the caller's buffers share."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = {
+    "bf16": [(3, 64, 32, 32, False), (64, 64, 32, 32, False), (64, 128, 32, 16, True), (128, 128, 16, 16, False)],
+    "f32": [(3, 8, 16, 4, False), (8, 8, 16, 4, False), (8, 8, 16, 8, True)],
+    "same": [(64, 64, 16, 16, False)] * 5,
+}
+
+
+def _block(kind, N, seed, host_io=0):
+    import torch
+    from paper_2402_14139_b200 import nf
+    nf.nf_set_stream(torch.cuda.current_stream())
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    layers = []
+    for i, (Cin, Cout, S, F, pool) in enumerate(SHAPES[kind]):
+        L = nf.Layer(Cin, Cout, S, S, F, 10, N, maxpool=pool, dtype=nf.NF_F32 if kind == "f32" else nf.NF_BF16, host_io=host_io if i == 0 else 0)
+        for name, fan in (("W", 9 * Cin), ("Wa", 9 * Cout), ("Wf", 4 * F)):
+            L.set_param(name, (torch.randn(L.shapes[name], generator=gen, device="cuda") * (2.0 / fan) ** 0.5).cpu().numpy())
+        layers.append(L)
+    Cin, _, S, _, _ = SHAPES[kind][0]
+    x = torch.randn((N, S, S, Cin), generator=gen, device="cuda").to(layers[0].tdtype)
+    y = torch.randint(0, 10, (N,), generator=gen, device="cuda", dtype=torch.int32)
+    return nf, layers, nf.Block(layers), x, y
+
+
+def _state(layers):
+    return [L.get_param(k, kind) for L in layers for k in ("W", "gamma", "Wa", "ba", "Wf", "bf") for kind in (0, 0x200)] + \
+        [L.get_param("rmean") for L in layers]
+
+
+def _one_by_one(layers, x, y, loss, acts, steps):
+    for _ in range(steps):
+        cur = x
+        for i, L in enumerate(layers):
+            L.step(cur, y, 0.05, loss[i:i + 1], acts[i])
+            cur = acts[i]
+
+
+def _same(a, b):
+    assert all((p == q).all() for p, q in zip(a, b))
+
+
+@pytest.mark.parametrize("how", ["step", "graph", "other stream", "host"])
+@pytest.mark.parametrize("kind,N", [("bf16", 96), ("bf16", 7), ("f32", 8), ("same", 40)])
+def test_block_step_has_the_bits_of_single_steps(kind, N, how):
+    import torch
+    nf, ref, _, x, y = _block(kind, N, 3)
+    loss = torch.zeros(len(ref), device="cuda")
+    acts = [L.new_act() for L in ref]
+    _one_by_one(ref, x, y, loss, acts, 3)
+    nf, layers, block, x, y = _block(kind, N, 3, 2 if how == "host" else 0)
+    got, act = torch.zeros(len(ref), device="cuda"), layers[-1].new_act()
+    if how == "graph":
+        block.step(x, y, 0.05, got, act)
+        g = block.capture(x, y, 0.05, got, act)
+        for _ in range(2):
+            g.replay()
+    elif how == "host":
+        xh, yh, got = x.cpu().pin_memory(), y.cpu().pin_memory(), got.cpu().pin_memory()
+        for _ in range(3):
+            block.step_host_next(xh, yh, 0.05, got, xh, yh)
+    else:
+        s = torch.cuda.Stream() if how == "other stream" else torch.cuda.current_stream()
+        s.wait_stream(torch.cuda.current_stream())
+        nf.nf_set_stream(s)
+        for _ in range(3):
+            block.step(x, y, 0.05, got, act)
+        torch.cuda.current_stream().wait_stream(s)
+        nf.nf_set_stream(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert torch.equal(got.cuda(), loss)
+    assert how == "host" or torch.equal(act, acts[-1])
+    _same(_state(layers), _state(ref))
+    assert all(L.status() == 0 for L in layers)
+
+
+def test_buffers_that_share_memory_keep_the_order_of_one_stream():
+    """act_out in the input's place, and a shortcut that is a view of an earlier layer's buffer: single steps of the same calls agree."""
+    import torch
+    N = 40
+    nf, ref, _, x, y = _block("same", N, 5)
+    loss, acts = torch.zeros(len(ref), device="cuda"), [L.new_act() for L in ref]
+    for c in range(2):
+        ref[3].set_skip(ref[0].stored("dy") if c else None)
+        xr = x.clone()
+        cur = xr
+        for i, L in enumerate(ref):
+            out = xr if i == len(ref) - 1 else acts[i]
+            L.step(cur, y, 0.05, loss[i:i + 1], out)
+            cur = out
+    nf, layers, block, x, y = _block("same", N, 5)
+    got = torch.zeros(len(ref), device="cuda")
+    for c in range(2):
+        layers[3].set_skip(layers[0].stored("dy") if c else None)
+        xb = x.clone()
+        block.step(xb, y, 0.05, got, xb)
+    torch.cuda.synchronize()
+    assert torch.equal(xb, xr) and torch.equal(got, loss)
+    _same(_state(layers), _state(ref))
+
+
+def test_a_call_that_fails_half_way_leaves_the_stream_in_order():
+    import torch
+    nf, layers, block, x, y = _block("bf16", 16, 7)
+    act = torch.empty(layers[-1].new_act().numel() + 8, dtype=torch.bfloat16, device="cuda")
+    loss = torch.zeros(len(layers), device="cuda")
+    with pytest.raises(nf.NfError):        # the last layer refuses its output's address; the ones before it have run
+        block.step(x, y, 0.05, loss, act[1:])
+    first = [loss.clone() for _ in range(1)]
+    block.step(x, y, 0.05, loss, act)      # no update was made by the first call
+    torch.cuda.synchronize()
+    assert torch.equal(first[0][:-1], loss[:-1])
+
+
+def test_lanes_of_many_layers_come_and_go():
+    """More layers than streams are kept for; the ones that get a used stream step as the first ones did."""
+    import torch
+    nf, layers, block, x, y = _block("f32", 8, 9)
+    loss = torch.zeros(len(layers), device="cuda")
+    block.step(x, y, 0.05, loss)
+    want = _state(layers)
+    for _ in range(3):
+        many = [_block("f32", 8, 9) for _ in range(12)]
+        for _, ls, b, xx, yy in many:
+            b.step(xx, yy, 0.05, torch.zeros(len(ls), device="cuda"))
+        for _, ls, b, _, _ in many:
+            _same(_state(ls), want)
+            b.close()
+            for L in ls:
+                L.close()
