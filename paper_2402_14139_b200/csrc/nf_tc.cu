@@ -17,6 +17,7 @@
 
 #include "nf_ptx.cuh"
 #include "nf_tc.h"
+#include "nf_tiles.cuh"
 
 namespace {
 
@@ -35,42 +36,6 @@ constexpr int kFoldThreads = 320;  // folded-tap forward: producer, MMA issuer a
 // load latency plus epilogue time, so with the earlier two slots per epilogue group the kernel ran at the pace of these loads
 // (about four tiles per HBM round trip) whatever else it did; with five the loads run as far ahead as the operand stages.
 constexpr int kYSlots = 5;
-
-// Division by a number that is fixed for a launch, as a multiplication by a rounded-up reciprocal (Granlund and Montgomery, Division by
-// Invariant Integers using Multiplication, 1994; exact for dividends below 2^31).  The role loops decode
-// a tile number per tile; a 32-bit division by a run-time value costs a single thread about 100 cycles of dependent instructions.
-struct FDiv {
-  uint32_t d, mul, shift;
-};
-FDiv fdiv_of(uint32_t d) {
-  FDiv f{d, 0, 0};
-  if (d == 1) return f;
-  uint32_t lg = 0;
-  while ((1ull << lg) < d) ++lg;
-  f.mul = (uint32_t)(((1ull << (31 + lg)) + d - 1) / d);
-  f.shift = lg - 1;
-  return f;
-}
-__device__ __forceinline__ uint32_t fdiv(uint32_t n, const FDiv& f, uint32_t* rem) {
-  const uint32_t q = f.d == 1 ? n : __umulhi(n, f.mul) >> f.shift;
-  *rem = n - q * f.d;
-  return q;
-}
-
-// First pixel and image (group) of pixel tile m: tiles run along the width, then the height, then the images
-struct TileGrid {
-  FDiv nt, tw, th;  // channel tiles, tile columns, tile rows
-};
-TileGrid tile_grid(int n_tiles, int tiles_w, int tiles_h) { return {fdiv_of(n_tiles), fdiv_of(tiles_w), fdiv_of(tiles_h)}; }
-struct TileAt {
-  uint32_t nt, w, h, n;
-};
-__device__ __forceinline__ TileAt tile_at(uint32_t t, const TileGrid& g) {
-  TileAt a;
-  const uint32_t m = fdiv(t, g.nt, &a.nt), r = fdiv(m, g.tw, &a.w);
-  a.n = fdiv(r, g.th, &a.h);
-  return a;
-}
 
 // Position in a ring of `stages` buffers: index and the parity a waiter for "full" expects in this round
 struct Ring {
@@ -2858,6 +2823,7 @@ int nf_tc_conv_fwd(nf_layer* L, const void* x, int& nb) {
 }
 
 int nf_tc_conv_fwd_eval(nf_layer* L, const void* x, int count, void* act) {
+  if (act && nf_first_eval_ok(L, x, count, act)) return nf_first_eval(L, x, count, act);
   int nb = 0, Cin;
   const void *xin, *win;
   const int rc = main_conv_operands(L, x, count, &xin, &win, &Cin);
@@ -2991,6 +2957,17 @@ size_t nf_tc_conv3x3_wgrad_scratch_floats(int N, int H, int W, int Cin, int Cout
   const int Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
   const WgPlan pl = plan_wgrad(Ho, Wo, Cin, Cout, N, 0, stride);
   return standalone_wgrad_ok(N, Ho, Wo, Cin, Cout, pl) ? pl.part_floats : 0;
+}
+
+int nf_tc_sm_count() { return sm_count(); }
+int nf_tc_tile(int H, int W, int* BW, int* BH) {
+  int BI;
+  return pick_tile(1, H, W, BW, BH, &BI) && BI == 1;
+}
+int nf_tc_out_map(CUtensorMap* m, void* base, int N, int H, int W, int C, int BW, int BH) {
+  const uint64_t d[4] = {(uint64_t)C, (uint64_t)W, (uint64_t)H, (uint64_t)N};
+  const uint32_t b[4] = {64, (uint32_t)BW, (uint32_t)BH, 1};
+  return make_map4(m, base, d, b);
 }
 
 static __device__ int32_t g_op_status;  // status word of the stand-alone operations (one per device that loads the library)

@@ -52,3 +52,12 @@ int nf_tc_bounded_wait_probe(unsigned long long limit_ns, unsigned long long* wa
 // writes L->dy = BatchNorm-backward(da) with da formed again inside the kernel; M = elements per channel of the whole batch.
 bool nf_tc_dgrad_two_pass(const nf_layer* L);
 int nf_tc_aux_dgrad_dy(nf_layer* L, double M);
+// What nf_first.cu shares with the other tensor-core kernels: SM count, the 128-pixel tile of one image that divides a map (0: none) and
+// the map of a [N][H][W][C] tensor for stores of such tiles, 64 channels at a time.
+struct CUtensorMap_st;
+int nf_tc_sm_count();
+int nf_tc_tile(int H, int W, int* BW, int* BH);
+int nf_tc_out_map(CUtensorMap_st* m, void* base, int N, int H, int W, int C, int BW, int BH);
+// First layer in evaluation (nf_first.cu): act = ReLU(conv(x) * scale + shift) of `count` RGB images, from the images as they are.
+bool nf_first_eval_ok(const nf_layer* L, const void* x, int count, const void* act);
+int nf_first_eval(nf_layer* L, const void* x, int count, void* act);
