@@ -48,8 +48,8 @@ struct Ring {
   }
 };
 
-// a second group of four epilogue warps in the input gradient of tiles of several images
-constexpr int fwd_threads(int epi, int pt) { return epi == 0 && pt == 2 ? kThreads + 128 : kThreads; }
+// a second group of four epilogue warps in the input gradient of tiles of several images, and for 256 channels without sums
+constexpr int fwd_threads(int epi, int pt, int ns = 0) { return (epi == 0 && pt == 2) || ns ? kThreads + 128 : kThreads; }
 
 struct FwdParams {
   int N, H, W, Cin, Cout;
@@ -69,7 +69,7 @@ struct FwdParams {
 };
 
 struct TcPlan {
-  int ok, BW, BH, BI, PT, BN, KC, RW, SEG, stages, grid, parts, yslots;
+  int ok, BW, BH, BI, PT, BN, KC, RW, SEG, SB, NS, stages, grid, parts, yslots;
   size_t smem;
 };
 
@@ -122,8 +122,16 @@ __device__ __forceinline__ void add_segments(uint32_t tbase, int n, uint32_t& ta
 //       core's running sum drops low bits on every instruction: over 2304 products 0.07 % of the bf16 outputs came out one unit
 //       off the nearest value, against 0.016 % of an fp32 chain.  Maps that no tile divides had such chains (they ran on the CUDA
 //       cores), and their layers are small enough for that to show; seg_steps (run_fwd) keeps the error below theirs.
-template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0>
-__global__ void __launch_bounds__(fwd_threads(EPI, PT), 1)
+// SB  : 1 (PT 0) = ONE box per chunk for the nine taps.  A tile is 8 columns x 16 rows, its box has a column more on either side, and an
+//       image row of the tile is one 8-row group of the operand: a tap is a start address kh rows and kw pixels into the box, the groups
+//       lie 10 pixels apart (the swizzle is a function of the address, so TMA and the tensor core agree wherever a tap starts).  The
+//       products come in the order of the three-box form, so every bit stays.  For tiles of several images it gained nothing: there
+//       the narrow instructions are the limit (512 channels, 8 filters, 8x8: 264 us with three boxes, 264 to 281 with one).
+// NS  : 1 (EPI 0, no sums) = two epilogue groups with a staging tile of 64 channels each.  256 channels: they take the quarters of a
+//       tile in turn; 64 and 128: every second tile.  One group was the slowest role: 16 000 to 20 000 cycles for a tile of 256
+//       channels whose products take 9200 with 128 input channels (evaluation, 1777 maps of 16x16: 257 -> 190 us).
+template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0, int SB = 0, int NS = 0>
+__global__ void __launch_bounds__(fwd_threads(EPI, PT, NS), 1)
 conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                    const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ FwdParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -131,12 +139,16 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   constexpr int kARow = KC * 2;  // bytes of one pixel row of the activation box
   constexpr uint32_t kALayout = KC == 64 ? 2 : KC == 32 ? 4 : 6;
   constexpr bool HN = PT == 2, SG = HN && EPI == 0;  // SG: the sums of stats 2 are taken by a warp group of their own
-  const int a_box = (p.BH + 2) * p.BW * p.BI * kARow;  // HN: one of the three column-shifted boxes, a multiple of 1024
-  const int a_bytes = HN ? 3 * a_box : PT ? 128 * kARow : a_box;
+  const int a_box = (p.BH + 2) * (SB ? 10 : p.BW) * p.BI * kARow;  // HN: one of the three column-shifted boxes, a multiple of 1024
+  const int a_bytes = SB ? a_box : HN ? 3 * a_box : PT ? 128 * kARow : a_box;
   const int a_stride = (a_bytes + 1023) & ~1023;  // keeps the weight tiles 1024-byte aligned
   static_assert(!HN || RW == BMN, "forward: weights in the stages; input gradient: resident");
-  constexpr int b_bytes = RW ? 0 : HN ? 9 * BN * 128 : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
-  constexpr int w_bytes = !RW ? 0 : BMN ? 9 * (BN / 64) * KC * 128 : 9 * BN * 128;  // resident weights [kw][kh][BN][64] (BMN: [half][kh][kw][KC][64])
+  static_assert(!SB || (PT == 0 && !SEG && (!BMN || RW)), "one box: tiles of one image; input gradient: weights resident");
+  static_assert(!NS || (EPI == 0 && !SEG && PT != 2), "two groups: no sums");
+  constexpr bool NINE = HN || SB;  // all nine taps of a chunk in one stage
+  constexpr int b_bytes = RW ? 0 : NINE ? 9 * BN * 128 : PT ? (BMN ? (BN / 64) * KC * 128 : BN * 128) : BMN ? (BN / 64) * 3 * KC * 128 : 3 * BN * 128;
+  // resident weights [kw][kh][BN][64] (SB: [chunk][kh][kw][BN][64], BMN: [half][kh][kw][KC][64])
+  const int w_bytes = !RW ? 0 : BMN ? 9 * (BN / 64) * KC * 128 : (SB ? p.kchunks : 1) * 9 * BN * 128;
   const int stage_bytes = a_stride + b_bytes;
   // 256 channels leave through staging (and y2) tiles of 128, one half after the other: with 32 KB instead of 64 the ring gets four
   // stages of 48 KB for three, three for two beside y2 tiles (a stage is multiplied in 512 cycles, a fill takes over 1000)
@@ -145,7 +157,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   uint8_t* wres = smem + (size_t)p.stages * stage_bytes;
   uint8_t* stg = wres + w_bytes;
   constexpr int kStg = SG ? 2 : 1;              // staging tiles
-  uint8_t* ybuf = stg + kStg * kSub * 16384;  // stats 2: the y2 tile of the tile in the epilogue (kSub sub-tiles)
+  uint8_t* ybuf = stg + (NS ? 2 : kStg * kSub) * 16384;  // stats 2: the y2 tile of the tile in the epilogue (kSub sub-tiles)
   uint64_t* bars = reinterpret_cast<uint64_t*>(ybuf + (p.stats == 2 ? p.yslots : 0) * kSub * 16384);
   uint64_t* full = bars;
   uint64_t* empty = bars + kMaxStages;
@@ -170,7 +182,7 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     }
     for (int a = 0; a < (int)kAccs; ++a) {
       ptx::mbar_init(&tfull[a], 1);
-      ptx::mbar_init(&tempty[a], 128);
+      ptx::mbar_init(&tempty[a], NS && BN == 256 ? 256 : 128);
     }
     ptx::mbar_init(wfull, 1);
     for (int i = 0; i < 2; ++i) {
@@ -209,6 +221,8 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
 #pragma unroll
             for (int hf = 0; hf < BN / 64; ++hf)
               ptx::tma_load_4d(wres + hf * 9 * KC * 128, &tm_w, wfull, (blockIdx.x % p.n_tiles) * BN + hf * 64, 0, 0, 0);
+          } else if constexpr (SB) {
+            for (int ck = 0; ck < p.kchunks; ++ck) ptx::tma_load_4d(wres + ck * 9 * BN * 128, &tm_w, wfull, ck * 64, 0, 0, 0);
           } else {
 #pragma unroll
             for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(wres + kw * 3 * BN * 128, &tm_w, wfull, 0, (blockIdx.x % p.n_tiles) * BN, kw, 0);
@@ -223,14 +237,18 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         const int co0 = at.nt * BN, w0 = at.w * p.BW, h0 = at.h * p.BH, n = at.n * p.BI;
         for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
-          for (int tap = 0; tap < (HN ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+          for (int tap = 0; tap < (NINE ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
             if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) { ok = false; break; }
             uint64_t* fb = &full[rg.s];
             uint8_t* a_s = smem + (size_t)rg.s * stage_bytes;
             ptx::mbar_expect_tx(fb, (uint32_t)(a_bytes + b_bytes));
-            if constexpr (HN) {
+            if constexpr (NINE) {
+              if constexpr (SB) {
+                ptx::tma_load_4d(a_s, &tm_x, fb, ck * KC, w0 - 1, h0 - 1, n);
+              } else {
 #pragma unroll
-              for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(a_s + kw * a_box, &tm_x, fb, ck * KC, w0 + kw - 1, n, h0 - 1);
+                for (int kw = 0; kw < 3; ++kw) ptx::tma_load_4d(a_s + kw * a_box, &tm_x, fb, ck * KC, w0 + kw - 1, n, h0 - 1);
+              }
               if constexpr (!RW) {
                 ptx::tma_load_4d(a_s + a_stride, &tm_w, fb, ck * 64, co0, 0, 0);  // [kh][kw][BN][64]
               }
@@ -274,9 +292,9 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     // ---------------- MMA issuer (one thread, as above)
     constexpr uint32_t idesc = ptx::idesc_bf16(128, BN, 0, BMN);
     // descriptors differ only in their 14-bit address field: constant upper parts, address added per use
-    const uint64_t a_hi = ptx::sdesc(0, 16, 8 * kARow, kALayout);
-    const uint64_t b_hi = BMN ? ptx::sdesc(0, (HN ? 9 : PT ? 1 : 3) * KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
-    const uint32_t a_row16 = (uint32_t)((HN ? p.BI : 1) * p.BW * kARow) >> 4;  // one image row of the box, in 16-byte units
+    const uint64_t a_hi = ptx::sdesc(0, 16, (SB ? 10 : 8) * kARow, kALayout);
+    const uint64_t b_hi = BMN ? ptx::sdesc(0, (NINE ? 9 : PT ? 1 : 3) * KC * 128, 1024, 2) : ptx::sdesc(0, 16, 1024, 2);
+    const uint32_t a_row16 = (uint32_t)((HN ? p.BI : 1) * (SB ? 10 : p.BW) * kARow) >> 4;  // one image row of the box, in 16-byte units
     if (ptx::elect_one()) {
       Ring rg;
       uint32_t tl = 0;
@@ -284,13 +302,13 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if constexpr (RW) {
         if (blockIdx.x < p.total_tiles) ok = ptx::mbar_wait(wfull, 0, abort_flag);
       }
-      const int steps = (HN ? 1 : PT ? 9 : 3) * p.kchunks, seg = SEG ? p.seg_steps : steps;
+      const int steps = (NINE ? 1 : PT ? 9 : 3) * p.kchunks, seg = SEG ? p.seg_steps : steps;
       for (int t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
         uint32_t acc = 0, d = 0, accumulate = 0;
         int step = 0, in_seg = 0;  // in_seg: k-steps of the segment so far
         for (int ck = 0; ok && ck < p.kchunks; ++ck) {
 #pragma unroll
-          for (int tap = 0; tap < (HN ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
+          for (int tap = 0; tap < (NINE ? 1 : PT ? 9 : 3); ++tap, rg.next(p.stages)) {
             if (in_seg == 0) {
               acc = tl % kAccs;
               if (!ptx::mbar_wait(&tempty[acc], ((tl / kAccs) & 1) ^ 1, abort_flag)) { ok = false; break; }
@@ -304,15 +322,16 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
             ptx::tc_fence_after();
             const uint32_t a_base = ptx::smem_u32(smem) + rg.s * stage_bytes;
             const uint32_t a16 = a_base >> 4;
-            const uint32_t b16 = RW ? (ptx::smem_u32(wres) + tap * 3 * BN * 128) >> 4 : (a_base + a_stride) >> 4;
-            if constexpr (HN) {  // all nine taps of the chunk, in the per-tap form's order
-              const uint32_t box16 = (uint32_t)a_box >> 4;
+            const uint32_t b16 = RW ? (ptx::smem_u32(wres) + (SB && !BMN ? ck * 9 : tap * 3) * BN * 128) >> 4 : (a_base + a_stride) >> 4;
+            if constexpr (NINE) {  // all nine taps of the chunk, in the order of the per-tap form (HN) or of the three-box form
+              const uint32_t col16 = SB ? kARow >> 4 : (uint32_t)a_box >> 4;  // one column tap on
 #pragma unroll
               for (int t9 = 0; t9 < 9; ++t9)
 #pragma unroll
                 for (int k = 0; k < KC / 16; ++k) {
-                  const uint64_t ad = a_hi | (uint64_t)(a16 + (t9 % 3) * box16 + (t9 / 3) * a_row16 + k * 2);
-                  const uint64_t bd = b_hi | (uint64_t)(BMN ? b16 + (((8 - t9) * KC * 128 + k * 16 * 128) >> 4) : b16 + ((t9 * BN * 128 + k * 32) >> 4));
+                  const int kh = HN ? t9 / 3 : t9 % 3, kw = HN ? t9 % 3 : t9 / 3, tw = kh * 3 + kw;
+                  const uint64_t ad = a_hi | (uint64_t)(a16 + kw * col16 + kh * a_row16 + k * 2);
+                  const uint64_t bd = b_hi | (uint64_t)(BMN ? b16 + (((8 - tw) * KC * 128 + k * 16 * 128) >> 4) : b16 + ((tw * BN * 128 + k * 32) >> 4));
                   ptx::mma_f16(d, ad, bd, idesc, accumulate);
                   accumulate = 1;
                 }
@@ -339,7 +358,78 @@ conv_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     __syncwarp();
   } else {
     // ---------------- epilogue: 128 threads, thread <-> output pixel (TMEM lane)
-    if constexpr (EPI == 0) {
+    if constexpr (NS) {
+      const int grp = warp >= 6 ? 1 : 0, et = (threadIdx.x - 64) & 127, lg = warp & 3, r = lg * 32 + lane;
+      const bool affine = POST, biased = !POST && p.bias;
+      uint8_t* const stile = stg + grp * 16384;
+      constexpr bool kShare = BN == 256;  // both groups work on every tile
+      constexpr int kQ = kShare ? 2 : BN / 64;
+      uint32_t tl = kShare ? 0 : grp;
+      bool go = true;
+      for (int t = blockIdx.x + tl * gridDim.x; go && t < p.total_tiles; t += (kShare ? 1 : 2) * gridDim.x, tl += kShare ? 1 : 2) {
+        const TileAt at = tile_at(t, p.tg);
+        const uint32_t acc = tl & 1;
+        ptx::mbar_wait(&tfull[acc], (tl >> 1) & 1, abort_flag);  // sets the abort flag itself when it gives up
+        ptx::tc_fence_after();
+#pragma unroll
+        for (int qi = 0; qi < kQ; ++qi) {
+          const int cq = (kShare ? 2 * qi + grp : qi) * 64, ch0 = at.nt * BN + cq;  // first column and channel of these 64
+          if (et == 0) {
+            ptx::tma_store_wait_read();  // the last store out of this group's staging tile has finished reading it
+            epi_go[grp] = *abort_flag ? 0 : 1;
+          }
+          ptx::named_barrier(1 + grp, 128);
+          if (!epi_go[grp]) {
+            go = false;
+            break;
+          }
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            uint32_t v[32];
+            ptx::tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * BN + cq + j * 32, v);
+            ptx::tmem_ld_wait();
+            const float4* c0 = reinterpret_cast<const float4*>((POST ? p.bn_scale : p.bias) + ch0 + j * 32);
+            const float4* c1 = reinterpret_cast<const float4*>(p.bn_shift + ch0 + j * 32);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              uint32_t w[4];
+#pragma unroll
+              for (int e = 0; e < 4; e += 2) {
+                float o[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) o[i] = __uint_as_float(v[q * 8 + 2 * e + i]);
+                if (biased) {  // bias and ReLU before the value is rounded for storage
+                  const float4 b = __ldg(c0 + q * 2 + e / 2);
+                  o[0] = fmaxf(o[0] + b.x, 0.f); o[1] = fmaxf(o[1] + b.y, 0.f); o[2] = fmaxf(o[2] + b.z, 0.f); o[3] = fmaxf(o[3] + b.w, 0.f);
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                  const __nv_bfloat162 b2 = __floats2bfloat162_rn(o[2 * i], o[2 * i + 1]);
+                  w[e + i] = *reinterpret_cast<const uint32_t*>(&b2);
+                }
+                if (affine) {
+                  const float4 sc = __ldg(c0 + q * 2 + e / 2), sh = __ldg(c1 + q * 2 + e / 2);
+                  w[e] = bn_relu2(w[e], make_float2(sc.x, sc.y), make_float2(sh.x, sh.y));
+                  w[e + 1] = bn_relu2(w[e + 1], make_float2(sc.z, sc.w), make_float2(sh.z, sh.w));
+                }
+              }
+              *reinterpret_cast<uint4*>(stile + r * 128 + (((j * 4 + q) ^ (r & 7)) * 16)) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+          if (qi == kQ - 1) {
+            ptx::tc_fence_before();
+            ptx::mbar_arrive(&tempty[acc]);
+          }
+          ptx::fence_async_smem();
+          ptx::named_barrier(1 + grp, 128);
+          if (et == 0) {
+            ptx::tma_store_4d(&tm_y, stile, ch0, (int)at.w * p.BW, (int)at.h * p.BH, (int)at.n * p.BI);
+            ptx::tma_store_commit();
+          }
+        }
+      }
+      if (et == 0) ptx::tma_store_wait_all();
+    } else if constexpr (EPI == 0) {
     const int et = threadIdx.x - 64;
     const int lg = warp & 3;          // TMEM lane group this warp may read
     const int r = lg * 32 + lane;     // row of the tile = pixel (r % BW, r / BW)
@@ -2271,8 +2361,27 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
       extra = staged + (epi == 2 ? b9 : 0);
     }
   }
+  // Tiles of one image without sums over them.  64 aux filters: two epilogue groups, outputs through staging tiles (1904 maps of 32x32x64
+  // 242 -> 151 us, 64 maps 14.6 -> 11.1).  One box per chunk: up to 32 filters over several chunks (256 channels at 16x16, 1777 maps:
+  // 115 -> 107 us; with one chunk the box of a tile is too little to tell); and, with two epilogue groups, the input gradient (of a
+  // pooled layer or one with a shortcut), where the weights fit beside three stages (1904 maps of 32x32x64 158 -> 148 us).
+  const bool sumless = pl.PT == 0 && stride == 1 && (epi == 1 || (epi == 2 && !ybuf));
+  if (sumless && W % 8 == 0 && H % 16 == 0 && (epi == 2 || (Cin > 64 && Cout <= 32))) {
+    const size_t a1 = ((size_t)18 * 10 * pl.KC * 2 + 1023) & ~(size_t)1023, b9 = (size_t)9 * (epi == 2 ? pl.BN / 64 * pl.KC : pl.BN) * 128;
+    const size_t staged = epi == 2 || Cout == 64 ? 32768 : 0;
+    const bool resident = epi == 2 || Cin / 64 * b9 + staged + 4 * a1 + 2048 <= 232448;
+    if (resident ? b9 * (epi == 2 ? 1 : Cin / 64) + staged + 3 * a1 + 2048 <= 232448 : staged + 2 * (a1 + b9) + 2048 <= 232448) {
+      pl.SB = 1;
+      pl.BW = 8; pl.BH = 16;
+      pl.RW = resident;
+      a_stride = a1;
+      b_stage = resident ? 0 : b9;
+      extra = resident ? b9 * (epi == 2 ? 1 : Cin / 64) : 0;
+    }
+  }
+  pl.NS = sumless && !pl.SEG && (epi == 1 ? Cout == 64 : pl.SB);
   const size_t stage = ((a_stride + 1023) & ~(size_t)1023) + b_stage;
-  const size_t fixed = (size_t)(epi != 1 ? (pl.BN == 256 ? 2 : pl.BN / 64) : 0) * 16384 * (1 + pl.yslots) + extra + 1024 + 1024;
+  const size_t fixed = (size_t)(pl.NS ? 2 : epi != 1 ? (pl.BN == 256 ? 2 : pl.BN / 64) : 0) * 16384 * (1 + pl.yslots) + extra + 1024 + 1024;
   int st = (int)((232448 - fixed) / stage);
   if (st > kMaxStages) st = kMaxStages;
   if (st < 2) return pl;
@@ -2291,15 +2400,15 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   return pl;
 }
 
-template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0>
+template <int BN, int EPI, int KC = 64, int BMN = 0, int PT = 0, int RW = 0, int SEG = 0, int POST = 0, int SB = 0, int NS = 0>
 int launch_fwd(const TcPlan& pl, const CUtensorMap& mx, const CUtensorMap& mw, const CUtensorMap& my, const FwdParams& p) {
   static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
   bool& attr_done = attr_done_dev[current_device()];
   if (!attr_done) {
-    NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    NF_CUDA(cudaFuncSetAttribute(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST, SB, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST>, pl.grid, fwd_threads(EPI, PT), pl.smem, mx, mw, my, p);
+  nf_launch(conv_fwd_tc_kernel<BN, EPI, KC, BMN, PT, RW, SEG, POST, SB, NS>, pl.grid, fwd_threads(EPI, PT, NS), pl.smem, mx, mw, my, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2476,17 +2585,17 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
   CUtensorMap mx, mw, my;
   const bool hn = pl.PT == 2;
   const uint64_t dx[4] = {(uint64_t)Cin, (uint64_t)Win, (uint64_t)Hin, (uint64_t)N};
-  const uint32_t bx[4] = {(uint32_t)pl.KC, (uint32_t)pl.BW, (uint32_t)(pl.PT == 1 ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
+  const uint32_t bx[4] = {(uint32_t)pl.KC, (uint32_t)(pl.SB ? 10 : pl.BW), (uint32_t)(pl.PT == 1 ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
   // forward: weights [kh][kw][Cout][Cin] -> box of BN rows x 64 ci for three kh; input gradient: weights
   // [kh][kw][F][Cout] -> box of KC rows of f x 64 c for three kh
   const uint64_t dw[4] = {(uint64_t)(epi == 2 ? Cout : Cin), (uint64_t)(epi == 2 ? Cin : Cout), 3, 3};
-  const uint32_t bw[4] = {64, (uint32_t)(epi == 2 ? pl.KC : pl.BN), hn ? 3u : 1u, (uint32_t)(pl.PT == 1 ? 1 : 3)};
+  const uint32_t bw[4] = {64, (uint32_t)(epi == 2 ? pl.KC : pl.BN), hn || pl.SB ? 3u : 1u, (uint32_t)(pl.PT == 1 ? 1 : 3)};
   const uint64_t dy[4] = {(uint64_t)Cout, (uint64_t)W, (uint64_t)H, (uint64_t)N};
   const uint32_t by[4] = {64, (uint32_t)pl.BW, (uint32_t)pl.BH, (uint32_t)pl.BI};
   int rc;
   if ((rc = make_map4(&mx, x, dx, bx, stride, hn)) != NF_OK) return rc;
   if ((rc = make_map4(&mw, w, dw, bw)) != NF_OK) return rc;
-  if (epi != 1) {
+  if (epi != 1 || pl.NS) {
     if ((rc = make_map4(&my, y, dy, by)) != NF_OK) return rc;
   } else {
     my = mx;  // not used by this epilogue
@@ -2522,7 +2631,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     if (pl.SEG)
       return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 1, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 1, 1>(pl, mx, mw, my, p);
     if (pl.PT)
-      return pl.BN == 256 ? launch_fwd<256, 0, 64, 0, 1, 0, 0, 1>(pl, mx, mw, my, p)
+      return pl.BN == 256 ? launch_fwd<256, 0, 64, 0, 1, 0, 0, 1, 0, 1>(pl, mx, mw, my, p)
            : pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1, 0, 0, 1>(pl, mx, mw, my, p);
     if (pl.RW) return launch_fwd<64, 0, 64, 0, 0, 1, 0, 1>(pl, mx, mw, my, p);
     return pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 0, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
@@ -2538,13 +2647,28 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p)
                        : pl.BN == 32 ? launch_fwd<32, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
   }
+  if (pl.NS && epi == 1) {  // 64 filters: the outputs leave as a main convolution's do
+    if (pl.SB) return pl.RW ? launch_fwd<64, 0, 64, 0, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 0, 0, 0, 0, 1, 1>(pl, mx, mw, my, p);
+    return pl.RW ? launch_fwd<64, 0, 64, 0, 0, 1, 0, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 0, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
+  }
+  if (pl.SB && epi == 1) {
+    if (pl.BN == 16) return pl.RW ? launch_fwd<16, 1, 64, 0, 0, 1, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<16, 1, 64, 0, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
+    return pl.RW ? launch_fwd<32, 1, 64, 0, 0, 1, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<32, 1, 64, 0, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
+  }
+  if (pl.SB) {
+    if (pl.BN == 128)
+      return pl.KC == 16 ? launch_fwd<128, 0, 16, 1, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p)
+                         : pl.KC == 32 ? launch_fwd<128, 0, 32, 1, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p) : NF_EUNSUPPORTED;
+    return pl.KC == 16 ? launch_fwd<64, 0, 16, 1, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p)
+                       : pl.KC == 32 ? launch_fwd<64, 0, 32, 1, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 1, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p);
+  }
   if (pl.PT == 2) {
     if (epi == 1) return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 2>(pl, mx, mw, my, p) : launch_fwd<32, 1, 64, 0, 2>(pl, mx, mw, my, p);
     return pl.BN == 128 ? launch_fwd<128, 0, 16, 1, 2, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 16, 1, 2, 1>(pl, mx, mw, my, p);
   }
   if (pl.PT) {  // per-tap boxes: stride 2, or several small images per tile
     if (epi == 0)
-      return pl.BN == 256 ? launch_fwd<256, 0, 64, 0, 1>(pl, mx, mw, my, p)
+      return pl.BN == 256 ? (stats ? launch_fwd<256, 0, 64, 0, 1>(pl, mx, mw, my, p) : launch_fwd<256, 0, 64, 0, 1, 0, 0, 0, 0, 1>(pl, mx, mw, my, p))
                           : pl.BN == 128 ? launch_fwd<128, 0, 64, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 1>(pl, mx, mw, my, p);
     if (epi == 1)
       return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 1>(pl, mx, mw, my, p)

@@ -1,0 +1,60 @@
+"""Auxiliary forward and input gradient without sums over their tiles (one activation box per chunk, two epilogue groups) and the average
+pool in one pass: every instantiation, with tiles left over at the end of a block's range, against 64 bits from the step's own tensors."""
+import numpy as np
+import pytest
+
+from tests import parity_util as pu
+from tests.test_gpu_ragged_precision import _nhwc64
+
+pytestmark = pytest.mark.gpu
+
+
+def _c(N, Cout, H, W, F, pool=False):
+    return dict(N=N, Cin=64, Cout=Cout, H=H, W=W, F=F, classes=10, stride=1, pool=pool)
+
+
+CASES = [
+    # aux forward with 64 filters: two groups in turn, odd numbers of tiles per block; one chunk (resident weights) and two
+    _c(75, 64, 32, 32, 64), _c(41, 128, 32, 16, 64), _c(1, 64, 16, 8, 64),
+    # one box per chunk, weights resident / in the stages: 16 filters over four and eight chunks, 32 over two and four; 40 filters: in 64 columns
+    _c(77, 256, 16, 16, 16), _c(37, 512, 16, 16, 16), _c(77, 128, 16, 16, 32), _c(39, 256, 16, 16, 24), _c(21, 128, 16, 16, 40),
+    # pooled layers: input gradient of 16, 32 and 64 filters to 128 and 64 channels, one box, two groups
+    _c(77, 128, 32, 32, 16, True), _c(39, 128, 32, 32, 32, True), _c(150, 64, 64, 64, 64, True), _c(151, 64, 32, 16, 16, True), _c(75, 64, 32, 16, 32, True),
+    # average pool of many images: chains of one, two and eight pixels; 8x8 with 256 filters (a division at the end)
+    _c(1500, 64, 16, 16, 8), _c(300, 64, 32, 32, 16), _c(1000, 64, 32, 32, 64), _c(700, 64, 8, 8, 256), _c(170, 64, 20, 20, 8),
+]
+
+
+@pytest.mark.parametrize("ci", range(len(CASES)))
+def test_forms_without_sums(ci):
+    import torch
+    from paper_2402_14139_b200 import nf
+    nf.lib()
+    nf.nf_set_stream(None)
+    c = CASES[ci]
+    P, x, y = pu.seeded_case(c, 2600 + ci, bf16=True)
+    L = pu.gpu_layer(nf, c, P, nf.NF_BF16)
+    xd, act = pu.to_device_nhwc(torch, np.maximum(x, 0.0), 1), L.new_act()
+    for _ in range(2):
+        L.step(xd, torch.from_numpy(y).cuda(), 0.0, torch.zeros(1, device="cuda"), act)
+    torch.cuda.synchronize()
+    assert L.status() == 0
+    F = c["F"]
+    Wa = torch.from_numpy(np.ascontiguousarray(P["Wa"].transpose(2, 3, 0, 1).reshape(9, F, -1))).float().cuda()
+    h = (_nhwc64(torch, act, Wa, 1) + torch.from_numpy(P["ba"]).cuda().double()).clamp_min(0)
+
+    def rounded(got, exact, what):      # bf16 keeps 8 bits: half a unit is at most 2^-8 of a value; sums in fp32 add 2^-12 of the largest
+        lim = 2.0 ** -8 * exact.abs() + 2.0 ** -12 * exact.abs().max()
+        assert bool(((got.double() - exact).abs() <= lim).all()), what
+
+    if L.kernel_family(5) == "stored":
+        H = L.stored("h")[..., :F]
+        rounded(H, h, "h")
+        ha, wa = H.shape[1] // 2, H.shape[2] // 2
+        p64 = torch.stack([H[:, a * ha:(a + 1) * ha, b * wa:(b + 1) * wa].double().mean((1, 2)) for a in (0, 1) for b in (0, 1)], -1)
+        p = L.stored("p").view(c["N"], -1, 4)[:, :F]
+        # fp32 sums of up to 256 values of one sign: at most 256 half units of 2^-24 each
+        assert bool(((p.double() - p64).abs() <= 2.0 ** -16 * p64 + 1e-7).all()), "p"
+    if L.kernel_family(6) == "stored":
+        rounded(L.stored("da"), _nhwc64(torch, L.stored("dh")[..., :F], Wa.flip(0).permute(0, 2, 1).contiguous(), 1), "da")
+    L.close()
