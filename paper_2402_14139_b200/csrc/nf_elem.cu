@@ -1192,6 +1192,55 @@ __global__ void __launch_bounds__(256) avgpool_small_vec_kernel(const uint4* __r
   for (int c = 0; c < 8; ++c) p[e * 8 + c] = make_float4(o[0][c], o[1][c], o[2][c], o[3][c]);
 }
 
+// Average pool of even maps in one pass: a thread per (image, eight channels, bin), sixteen loads in flight.  The sums are those of the
+// kernels around it: M = 1, the bin's pixels in order; M > 1, `planes` chains of M pixels each, planes apart, the chains added in order.
+// Many images: 16x16 maps with 16 filters, 1777 of them, 37 + 3 -> 5 us (there half the threads of a block per bin had nothing to do and
+// sixteen added 128 sums one by one); 8x8 with 256, 6366 of them, 61 -> 45 (a thread for all four bins left a second wave nearly empty).
+template <int M>
+__global__ void __launch_bounds__(256) avgpool_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, int cnt, int planes,
+                                                          uint32_t bw_mul, bool divide, size_t total, float* __restrict__ p) {
+  nf_pdl_begin();
+  const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (e >= total) return;
+  const int bin = (int)(e & 3), g = (int)((e >> 2) % F8), bw = Wa / 2;
+  const size_t n = (e >> 2) / F8;
+  const uint4* hb = h + ((n * Ha + (bin & 2 ? Ha / 2 : 0)) * Wa + (bin & 1 ? bw : 0)) * F8 + g;
+  const int chains = M == 1 ? cnt : planes;
+  constexpr int B = 16 / M;
+  float s[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) s[c] = 0.f;
+#pragma unroll 1
+  for (int q0 = 0; q0 < chains; q0 += B) {
+    uint4 v[B][M];
+#pragma unroll
+    for (int u = 0; u < B; ++u)
+#pragma unroll
+      for (int r = 0; r < M; ++r) {
+        const uint32_t k = (uint32_t)(min(q0 + u, chains - 1) + r * planes), row = __umulhi(k, bw_mul);  // k / bw
+        v[u][r] = __ldg(hb + ((size_t)row * Wa + (k - row * bw)) * F8);
+      }
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      float a[8];
+      unpack8(v[u][0], a);
+#pragma unroll
+      for (int r = 1; r < M; ++r) {
+        float b[8];
+        unpack8(v[u][r], b);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) a[c] += b[c];
+      }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) s[c] = q0 + u < chains ? s[c] + a[c] : s[c];
+    }
+  }
+  float* o = p + (n * F8 + g) * 32 + bin;
+  const float inv = 1.f / (float)cnt;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) o[c * 4] = divide ? s[c] / (float)cnt : s[c] * inv;
+}
+
 // average pool, stage 1: partial bin sums over a slice of rows; part[(n*4+bin)*S + s][F]
 __global__ void __launch_bounds__(256) avgpool_part_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, int S,
                                                                float* __restrict__ part) {
@@ -1657,10 +1706,22 @@ int nf_k_avgpool_slices(int N, int Ha, int Wa) {
   return (int)S;
 }
 
+// k / bw as the upper half of k * ceil(2^32 / bw): exact for k * bw < 2^32
+static uint32_t recip(int bw) { return (uint32_t)((((uint64_t)1 << 32) + bw - 1) / bw); }
+
 int nf_k_avgpool_fast(const void* h, int N, int Ha, int Wa, int F, float* part, size_t part_floats, float* p) {
   if (F % 8 || 256 % (F / 8) || (Ha & 1) || (Wa & 1)) return NF_EUNSUPPORTED;
   if ((long)(Ha / 2) * (Wa / 2) <= 16) return NF_EUNSUPPORTED;  // tiny maps: the caller's generic path has a kernel for them
   const int S = nf_k_avgpool_slices(N, Ha, Wa);
+  // one pass where no slices are cut, the chains are whole and there are threads enough for their length
+  const int cnt = (Ha / 2) * (Wa / 2), planes = 256 / (F / 8), m = cnt <= planes ? 1 : cnt % planes ? 0 : cnt / planes;
+  const size_t total = (size_t)N * 4 * (F / 8);
+  if (S == 1 && Wa >= 4 && (m == 1 || m == 2 || m == 4 || m == 8) && cnt < 65536 && (cnt <= 64 || total >= 16384)) {
+    auto* k = m == 1 ? avgpool_vec_kernel<1> : m == 2 ? avgpool_vec_kernel<2> : m == 4 ? avgpool_vec_kernel<4> : avgpool_vec_kernel<8>;
+    nf_launch(k, nblk(total, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, cnt, planes, recip(Wa / 2), false, total, p);
+    NF_LAUNCHED();
+    return NF_OK;
+  }
   if ((size_t)N * 4 * S * F > part_floats) return NF_EUNSUPPORTED;
   nf_launch(avgpool_part_vec_kernel, N * 4 * S, 256, 0, (const uint4*)h, Ha, Wa, F / 8, S, part);
   NF_LAUNCHED();
@@ -1707,6 +1768,12 @@ int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* 
     // (bf16: 32 outputs per thread where one each would not fit the chip at once, or is one pixel; one image of 7 x 7: 15 against 6 us)
     if (dtype == NF_BF16 && F % 8 == 0 && ((size_t)N * 4 * F > (size_t)148 * 2048 || Ha * Wa <= 4)) {
       const size_t groups = (size_t)N * (F / 8);
+      if (Ha % 2 == 0 && Wa % 2 == 0 && Wa >= 4) {
+        nf_launch(avgpool_vec_kernel<1>, nblk(groups * 4, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, (Ha / 2) * (Wa / 2), 1, recip(Wa / 2), true,
+                  groups * 4, p);
+        NF_LAUNCHED();
+        return NF_OK;
+      }
       nf_launch(avgpool_small_vec_kernel, nblk(groups, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, groups, (float4*)p);
       NF_LAUNCHED();
       return NF_OK;
