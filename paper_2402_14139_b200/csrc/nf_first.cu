@@ -155,7 +155,14 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) first_eval_kernel(cons
     }
     __syncwarp();
   } else {
-    const int et = threadIdx.x - 128, lg = warp & 3, r = lg * 32 + lane;
+    // Accumulators are read as matrix fragments: a thread holds 16 channels of every eighth pixel, so that its coefficients stay in
+    // registers, and matrix stores write a pixel's 8 channels as 16 bytes.  With a thread per pixel the coefficients came from shared
+    // memory, 32 loads of 16 bytes per tile, and kept the load-store unit busy 82 % of the time.
+    const int et = threadIdx.x - 128, lg = warp & 3;
+    const int mrow = (lane & 7) + (lane >> 3 & 1) * 8, mchunk = lane >> 4;  // the row and 8-channel chunk this thread addresses
+    float4 cf[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) cf[i] = coef[i * 4 + (lane & 3)];  // channels 8 i + 2 (lane % 4) and the next
     uint32_t tl = 0;
     for (int t = blockIdx.x; t < p.total; t += gridDim.x, ++tl) {
       const TileAt at = tile_at(t, p.tg);
@@ -169,18 +176,24 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) first_eval_kernel(cons
       ptx::named_barrier(1, 128);
       if (!*epi_go) break;
       uint8_t* const out = stg + acc * kOut;
+      const uint32_t tbase = tmem_base + acc * 64, obase = ptx::smem_u32(out);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint32_t v[16], o[8];
-        ptx::tmem_ld16(tmem_base + ((uint32_t)(lg * 32) << 16) + acc * 64 + j * 16, v);
+      for (int hf = 0; hf < 2; ++hf) {  // 16 pixels of the warp's 32
+        const uint32_t px = (uint32_t)(lg * 32 + hf * 16 + mrow);
+        uint32_t v[4][8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ptx::tmem_ld_16x256b_x2(tbase + ((uint32_t)(lg * 32 + hf * 16) << 16) + j * 16, v[j]);
         ptx::tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {  // rounded for storage, as where y is stored, then normalised
-          const __nv_bfloat162 y = __floats2bfloat162_rn(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
-          o[e] = bn_relu2(*reinterpret_cast<const uint32_t*>(&y), coef[j * 8 + e]);
+        for (int j = 0; j < 4; ++j) {
+          uint32_t o[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {  // rounded for storage, as where y is stored, then normalised
+            const __nv_bfloat162 y = __floats2bfloat162_rn(__uint_as_float(v[j][2 * q]), __uint_as_float(v[j][2 * q + 1]));
+            o[q] = bn_relu2(*reinterpret_cast<const uint32_t*>(&y), cf[2 * j + q / 2]);
+          }
+          ptx::stmatrix_x4(obase + px * 128 + (((2 * j + mchunk) ^ (px & 7)) * 16), o[0], o[1], o[2], o[3]);
         }
-        *reinterpret_cast<uint4*>(out + r * 128 + (((2 * j) ^ (r & 7)) * 16)) = make_uint4(o[0], o[1], o[2], o[3]);
-        *reinterpret_cast<uint4*>(out + r * 128 + (((2 * j + 1) ^ (r & 7)) * 16)) = make_uint4(o[4], o[5], o[6], o[7]);
       }
       ptx::tc_fence_before();
       ptx::mbar_arrive(&tempty[acc]);
