@@ -502,7 +502,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   }
   // where the shape allows, the aux forward kernel normalises y on the way in and writes act_out itself
   const bool fused_bn_aux = nf_tc_bn_aux_fused(L) && !L->skip;
-  if (!fused_bn_aux) NF_TRY(nf_k_bn_apply(dt, L->y, N, Ho, Wo, Co, pool, L->scale, L->shift, act_out, L->skip));
+  if (!fused_bn_aux) NF_TRY(nf_k_bn_apply(dt, L->y, N, Ho, Wo, Co, pool, L->scale, L->shift, act_out, L->skip, L->dy));
   trace_end();
   if (!fused_bn_aux && tail) NF_TRY(tail->fork() == NF_OK ? tail->open() : NF_ECUDA);
   // Eq. 2: aux conv + ReLU, average pool to 2x2, linear; Eq. 3: softmax cross-entropy
@@ -600,7 +600,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     if (L->skip_grad) NF_TRY(nf_k_write_dz(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->skip, L->skip_grad));
   } else {
     NF_TRY(nf_k_bn_bwd_reduce(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->mu, L->invstd, L->red,
-                                L->red_floats, &nb, L->skip, L->skip_grad));
+                                L->red_floats, &nb, L->skip, L->skip_grad, L->dy));
   }
   if (!all) return nf_k_partial_totals(L->red, nb, Co, L->dptot + 2 * Co);
   }

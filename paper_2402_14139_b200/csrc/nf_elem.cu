@@ -1423,35 +1423,10 @@ __device__ __forceinline__ size_t win_base(size_t q, int Ho, int Wo, int C8) {  
   return ((n * Ho + 2 * ia) * Wo + 2 * ja) * C8;
 }
 
-__global__ void __launch_bounds__(256) bn_apply_pool_vec_kernel(const uint4* __restrict__ y, int Ho, int Wo, int C8,
-                                                                const float* __restrict__ scale, const float* __restrict__ shift,
-                                                                size_t total8, uint4* __restrict__ out) {
-  nf_pdl_begin();
-  const int c0 = (threadIdx.x % C8) * 8;
-  float A[8], B[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { A[i] = scale[c0 + i]; B[i] = shift[c0 + i]; }
-  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < total8; e += (size_t)gridDim.x * 256) {
-    const size_t b = win_base(div_small(e, C8), Ho, Wo, C8) + threadIdx.x % C8;  // 256 % C8 == 0: the chunk of a thread is fixed
-    const uint4 v4[4] = {__ldg(y + b), __ldg(y + b + C8), __ldg(y + b + (size_t)Wo * C8), __ldg(y + b + (size_t)Wo * C8 + C8)};
-    float best[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) best[i] = 0.f;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      float v[8];
-      unpack8(v4[d], v);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) best[i] = fmaxf(best[i], fmaf(v[i], A[i], B[i]));
-    }
-    out[e] = pack8(best);
-  }
-}
-
 // Which of the four window positions of a channel pair (packed bf16 y in w[0..3]) receives the gradient: all-ones halves in keep[d]
-// where position d is the first maximum, in scan order, of the bf16-rounded ReLU outputs and that maximum is positive.  Two channels
+// where position d is the first maximum, in scan order, of the bf16-rounded ReLU outputs and that maximum is positive; returns that maximum.  Two channels
 // per instruction from the conversion on: with one channel at a time the two kernels below were bound by these instructions.
-__device__ __forceinline__ void pool_winner2(const uint32_t (&w)[4], float A0, float A1, float B0, float B1, uint32_t (&keep)[4]) {
+__device__ __forceinline__ __nv_bfloat162 pool_winner2(const uint32_t (&w)[4], float A0, float A1, float B0, float B1, uint32_t (&keep)[4]) {
   __nv_bfloat162 r[4];
 #pragma unroll
   for (int d = 0; d < 4; ++d) {
@@ -1467,13 +1442,61 @@ __device__ __forceinline__ void pool_winner2(const uint32_t (&w)[4], float A0, f
   keep[1] = pos & e1 & ~e0;
   keep[2] = pos & e2 & ~(e0 | e1);
   keep[3] = pos & ~(e0 | e1 | e2);
+  return m;
 }
 
-__global__ void __launch_bounds__(256, 2) bn_bwd_reduce_pool_vec_kernel(const uint4* __restrict__ y, const uint4* __restrict__ da,
-                                                                     size_t Pq, int Ho, int Wo, int C8,
-                                                                     const float* __restrict__ scale, const float* __restrict__ shift,
-                                                                     const float* __restrict__ mu, const float* __restrict__ invstd,
-                                                                     float* __restrict__ red) {
+// BatchNorm + ReLU + 2x2 max-pool.  WIN: a step also keeps, per window and channel, the y that its backward pass will want (the winner's,
+// or where nothing is positive the first one, whose own test then says so): a quarter of y, so that the sums of the backward pass need
+// not read y again and find the winners once more.  1904 maps of 64x64x64: this kernel 200 -> 234 us, the sums 264 -> 96.
+template <bool WIN>
+__global__ void __launch_bounds__(256) bn_apply_pool_vec_kernel(const uint4* __restrict__ y, int Ho, int Wo, int C8,
+                                                                const float* __restrict__ scale,
+                                                                const float* __restrict__ shift,
+                                                                size_t total8, uint4* __restrict__ out, uint4* __restrict__ ywin) {
+  nf_pdl_begin();
+  const int c0 = (threadIdx.x % C8) * 8;
+  float A[8], B[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { A[i] = scale[c0 + i]; B[i] = shift[c0 + i]; }
+  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < total8; e += (size_t)gridDim.x * 256) {
+    const size_t b = win_base(div_small(e, C8), Ho, Wo, C8) + threadIdx.x % C8;  // 256 % C8 == 0: the chunk of a thread is fixed
+    const uint4 v4[4] = {__ldg(y + b), __ldg(y + b + C8), __ldg(y + b + (size_t)Wo * C8), __ldg(y + b + (size_t)Wo * C8 + C8)};
+    if constexpr (WIN) {
+      const uint32_t* yw = reinterpret_cast<const uint32_t*>(v4);  // [window position][channel pair]
+      uint32_t o[4], w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t p[4] = {yw[i], yw[4 + i], yw[8 + i], yw[12 + i]};
+        uint32_t k[4];
+        const __nv_bfloat162 m = pool_winner2(p, A[2 * i], A[2 * i + 1], B[2 * i], B[2 * i + 1], k);
+        const __nv_bfloat162 z = __hmax2(m, __floats2bfloat162_rn(0.f, 0.f));  // NaN counts as zero, as in fmaxf
+        o[i] = *reinterpret_cast<const uint32_t*>(&z);
+        w[i] = (p[1] & k[1]) | (p[2] & k[2]) | (p[3] & k[3]) | (p[0] & ~(k[1] | k[2] | k[3]));
+      }
+      out[e] = make_uint4(o[0], o[1], o[2], o[3]);
+      ywin[e] = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+      float best[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) best[i] = 0.f;
+#pragma unroll
+      for (int d = 0; d < 4; ++d) {
+        float v[8];
+        unpack8(v4[d], v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) best[i] = fmaxf(best[i], fmaf(v[i], A[i], B[i]));
+      }
+      out[e] = pack8(best);
+    }
+  }
+}
+
+// Partial sums of (dz, dz*xhat) of a pooled layer from the winners that its forward pass kept: ywin and da have the pooled shape.  The
+// ranges, chains and order are those of the kernels that read y itself.
+__global__ void __launch_bounds__(256) bn_bwd_reduce_win_vec_kernel(const uint4* __restrict__ ywin, const uint4* __restrict__ da, size_t Pq,
+                                                                    int C8, const float* __restrict__ scale,
+                                                                    const float* __restrict__ shift, const float* __restrict__ mu,
+                                                                    const float* __restrict__ invstd, float* __restrict__ red) {
   nf_pdl_begin();
   __shared__ float sm[16][256];
   const int C = C8 * 8;
@@ -1486,33 +1509,33 @@ __global__ void __launch_bounds__(256, 2) bn_bwd_reduce_pool_vec_kernel(const ui
     a[i] = 0.f; b[i] = 0.f;
   }
   const size_t q0 = Pq * blockIdx.x / gridDim.x, q1 = Pq * (blockIdx.x + 1) / gridDim.x;
-  // the next window's five loads fly while this one is worked on (one window at a time: 547 us for 1.25 GB)
-  uint4 nx[5];
-  auto fetch = [&](size_t q) {
-    const size_t bb = win_base(q, Ho, Wo, C8) + g;
-    nx[0] = __ldg(y + bb);
-    nx[1] = __ldg(y + bb + C8);
-    nx[2] = __ldg(y + bb + (size_t)Wo * C8);
-    nx[3] = __ldg(y + bb + (size_t)Wo * C8 + C8);
-    nx[4] = __ldg(da + q * C8 + g);
-  };
-  if (q0 + pl < q1) fetch(q0 + pl);
-  for (size_t q = q0 + pl; q < q1; q += planes) {
-    const uint4 v4[5] = {nx[0], nx[1], nx[2], nx[3], nx[4]};
-    if (q + planes < q1) fetch(q + planes);
-    const uint32_t* yw = reinterpret_cast<const uint32_t*>(v4);  // [window position][channel pair]
+  constexpr int kU = 4;  // windows in flight, added in index order
+  for (size_t q = q0 + pl; q < q1; q += (size_t)kU * planes) {
+    uint4 yv[kU], dv[kU];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint32_t w[4] = {yw[i], yw[4 + i], yw[8 + i], yw[12 + i]};
-      uint32_t k[4];
-      pool_winner2(w, A[2 * i], A[2 * i + 1], B[2 * i], B[2 * i + 1], k);
-      const uint32_t dd = yw[16 + i] & (k[0] | k[1] | k[2] | k[3]);
-      const uint32_t yy = (w[0] & k[0]) | (w[1] & k[1]) | (w[2] & k[2]) | (w[3] & k[3]);
-      const float d0 = __uint_as_float(dd << 16), d1 = __uint_as_float(dd & 0xffff0000u);
-      a[2 * i] += d0;
-      a[2 * i + 1] += d1;
-      b[2 * i] = fmaf(d0, (__uint_as_float(yy << 16) - m[2 * i]) * is[2 * i], b[2 * i]);
-      b[2 * i + 1] = fmaf(d1, (__uint_as_float(yy & 0xffff0000u) - m[2 * i + 1]) * is[2 * i + 1], b[2 * i + 1]);
+    for (int u = 0; u < kU; ++u) {
+      const size_t e = q + (size_t)u * planes;
+      if (e < q1) {
+        yv[u] = __ldg(ywin + e * C8 + g);
+        dv[u] = __ldg(da + e * C8 + g);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      if (q + (size_t)u * planes >= q1) break;
+      const uint32_t yw[4] = {yv[u].x, yv[u].y, yv[u].z, yv[u].w}, dw[4] = {dv[u].x, dv[u].y, dv[u].z, dv[u].w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float z0 = fmaf(__uint_as_float(yw[i] << 16), A[2 * i], B[2 * i]), z1 = fmaf(__uint_as_float(yw[i] & 0xffff0000u), A[2 * i + 1], B[2 * i + 1]);
+        const __nv_bfloat162 r = __floats2bfloat162_rn(z0, z1);
+        const uint32_t pos = __hgt2_mask(r, __floats2bfloat162_rn(0.f, 0.f));
+        const uint32_t dd = dw[i] & pos, yy = yw[i] & pos;
+        const float d0 = __uint_as_float(dd << 16), d1 = __uint_as_float(dd & 0xffff0000u);
+        a[2 * i] += d0;
+        a[2 * i + 1] += d1;
+        b[2 * i] = fmaf(d0, (__uint_as_float(yy << 16) - m[2 * i]) * is[2 * i], b[2 * i]);
+        b[2 * i + 1] = fmaf(d1, (__uint_as_float(yy & 0xffff0000u) - m[2 * i + 1]) * is[2 * i + 1], b[2 * i + 1]);
+      }
     }
   }
 #pragma unroll
@@ -1662,7 +1685,7 @@ int nf_k_bn_eval_coeffs(int C, const float* gamma, const float* beta, float eps,
 }
 
 int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int pool, const float* scale,
-                    const float* shift, void* out, const void* skip) {
+                    const float* shift, void* out, const void* skip, void* ywin) {
   const size_t total = (size_t)N * (pool ? Ho / 2 : Ho) * (pool ? Wo / 2 : Wo) * C;
   if (vec2_ok(C, pool)) {
 #define NF_APPLY(T, M) \
@@ -1680,8 +1703,8 @@ int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int po
     return NF_OK;
   }
   if (pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    nf_launch(bn_apply_pool_vec_kernel, vec_blocks(total / 8), 256, 0, (const uint4*)y, Ho, Wo, C / 8, scale, shift, total / 8,
-                                                                            (uint4*)out);
+    nf_launch(ywin ? bn_apply_pool_vec_kernel<true> : bn_apply_pool_vec_kernel<false>, vec_blocks(total / 8), 256, 0, (const uint4*)y, Ho, Wo, C / 8,
+              scale, shift, total / 8, (uint4*)out, (uint4*)ywin);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1869,7 +1892,7 @@ int nf_k_sum_partials(const float* red, int nblocks, int C, float* out) {
 
 int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
                          const float* scale, const float* shift, const float* mu, const float* invstd, float* red,
-                         size_t red_floats, int* nblocks, const void* skip, void* dz_out) {
+                         size_t red_floats, int* nblocks, const void* skip, void* dz_out, const void* ywin) {
   const size_t P = (size_t)N * Ho * Wo;
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
@@ -1879,8 +1902,8 @@ int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, 
     if (rc != NF_OK) return rc;
   }
   if (!skip && pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
-    nf_launch(bn_bwd_reduce_pool_vec_kernel, nb, 256, 0, (const uint4*)y, (const uint4*)da, P / 4, Ho, Wo, C / 8, scale, shift, mu,
-                                                              invstd, red);
+    if (!ywin) return NF_EINVAL;
+    nf_launch(bn_bwd_reduce_win_vec_kernel, nb, 256, 0, (const uint4*)ywin, (const uint4*)da, P / 4, C / 8, scale, shift, mu, invstd, red);
     NF_LAUNCHED();
     *nblocks = nb;
     return NF_OK;

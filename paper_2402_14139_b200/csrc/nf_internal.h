@@ -156,7 +156,7 @@ int nf_k_bn_finalize(const float* red, int nblocks, int C, double M, const float
 int nf_k_bn_eval_coeffs(int C, const float* gamma, const float* beta, float eps, const float* rmean,
                           const float* rvar, float* scale, float* shift);
 int nf_k_bn_apply(int dtype, const void* y, int N, int Ho, int Wo, int C, int pool, const float* scale,
-                    const float* shift, void* out, const void* skip = nullptr);
+                    const float* shift, void* out, const void* skip = nullptr, void* ywin = nullptr);  // ywin: see nf_k_bn_bwd_reduce
 int nf_k_avgpool_slices(int N, int Ha, int Wa);
 int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* p);
 // bf16 fast paths (F % 8 == 0, even Ha and Wa); NF_EUNSUPPORTED means "use the generic kernel"
@@ -216,7 +216,8 @@ int nf_k_dh(int dtype, const void* h, const float* dp, int N, int Ha, int Wa, in
 int nf_k_sum_partials(const float* red, int nblocks, int C, float* out);
 int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
                          const float* scale, const float* shift, const float* mu, const float* invstd, float* red,
-                         size_t red_floats, int* nblocks, const void* skip = nullptr, void* dz_out = nullptr);  // dz_out: dz is written too
+                         size_t red_floats, int* nblocks, const void* skip = nullptr, void* dz_out = nullptr,  // dz_out: dz is written too
+                         const void* ywin = nullptr);  // pooled layers: what nf_k_bn_apply left there, [N][Ho/2][Wo/2][C]
 int nf_k_bn_bwd_finalize(const float* red, int nblocks, int C, float* sdz, float* sdzx, float* ggamma,
                            float* gbeta);
 int nf_k_bn_bwd_apply(int dtype, const void* y, const void* da, int N, int Ho, int Wo, int C, int pool,
