@@ -1605,10 +1605,14 @@ struct WgParams {
 // corrections: warps 0-3 the first accumulator of the pair, warps 4 and 5 the filled half of the second; warps 6 and 7 produce
 // and issue (with 256 threads all of that stays in registers).  The sums bound this form: that stage of two layers 281 -> 342 us,
 // the two gradients now off by 1.1e-7 and 6.0e-8.
+// HB = 1 (maps 8 pixels wide, stride 1, no segments): the three column taps are one box of ten columns.  An image row of the tile is one
+// group of eight pixels, groups lie ten pixels apart, and the second stacked tap starts one pixel further.  Same products in the same
+// order as three boxes, 24 KB a tile for 52: the auxiliary gradient of 512 channels, 8 filters, 8602 maps of 8x8, which the fill of shared
+// memory bound, 384 -> 324 us.
 constexpr int kSegSets = 4;
 constexpr int wgrad_threads(int seg) { return seg ? 256 : kThreads; }
 
-template <int NB, int SEG>
+template <int NB, int SEG, int HB>
 __global__ void __launch_bounds__(wgrad_threads(SEG), 1)
 conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dy, const WgParams p) {
   constexpr int kAtoms = NB > 64 ? NB / 64 : 1;                // 64-channel atoms of the dy tile (NB = 128, 256: main conv only)
@@ -1618,10 +1622,12 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   static_assert(!SEG || NB <= 64, "a thread holds the sums of one accumulator");
-  constexpr int kStages = NB > 64 ? 2 : 3;
+  static_assert(!HB || (!SEG && NB <= 64), "one box: no segments");
+  constexpr int kStages = NB > 64 ? 2 : HB ? 5 : 3;
   constexpr int kJobs = 2;  // instructions (accumulators) per 16 pixels
-  constexpr int copy_bytes = 16384;  // one 128-pixel tap tile
-  const int stage_bytes = 3 * copy_bytes + kAtoms * 16384;  // a dy atom always gets 16 KB so the unused rows read by the
+  constexpr int copy_bytes = HB ? 128 : 16384;  // from one column tap to the next: one pixel of the box, or a 128-pixel tile
+  constexpr int x_bytes = HB ? 160 * 128 : 3 * copy_bytes;
+  const int stage_bytes = x_bytes + kAtoms * 16384;  // a dy atom always gets 16 KB so the unused rows read by the
                                                             // half-empty last instruction stay inside the stage
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)kStages * stage_bytes);
   uint64_t* full = bars;
@@ -1678,19 +1684,19 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         if (!ptx::mbar_wait(&empty[rg.s], rg.ph ^ 1, abort_flag)) break;
         uint64_t* fb = &full[rg.s];
         uint8_t* st = smem + (size_t)rg.s * stage_bytes;
-        ptx::mbar_expect_tx(fb, (uint32_t)(3 * copy_bytes + kAtoms * kBTile));
+        ptx::mbar_expect_tx(fb, (uint32_t)(x_bytes + kAtoms * kBTile));
 #pragma unroll
-        for (int kw = 0; kw < 3; ++kw)
+        for (int kw = 0; kw < (HB ? 1 : 3); ++kw)
           ptx::tma_load_4d(st + kw * copy_bytes, &tm_x, fb, cic * 64, p.stride * w0 + kw - 1, p.stride * h0 + khg - 1, n);
 #pragma unroll
-        for (int a = 0; a < kAtoms; ++a) ptx::tma_load_4d(st + 3 * copy_bytes + a * 16384, &tm_dy, fb, coc * NB + a * 64, w0, h0, n);
+        for (int a = 0; a < kAtoms; ++a) ptx::tma_load_4d(st + x_bytes + a * 16384, &tm_dy, fb, coc * NB + a * 64, w0, h0, n);
       }
     }
     __syncwarp();
   } else if (warp == kIssuer) {
     constexpr uint32_t idesc = ptx::idesc_bf16(128, NB, 1, 1);
     // descriptors differ only in the address field; the second stacked chunk sits one tap tile further
-    const uint64_t a_copy_hi = ptx::sdesc(0, copy_bytes, 1024, 2);
+    const uint64_t a_copy_hi = ptx::sdesc(0, copy_bytes, HB ? 1280 : 1024, 2);
     const uint64_t b_hi = ptx::sdesc(0, 16384, 8 * kBRow, kBLayout);  // next 64-channel atom: 16 KB further
     constexpr uint32_t copy16 = (uint32_t)copy_bytes >> 4;
     if (ptx::elect_one()) {
@@ -1701,10 +1707,10 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         if (!ptx::mbar_wait(&full[rg.s], rg.ph, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint32_t xb = ptx::smem_u32(smem) + rg.s * stage_bytes;
-        const uint32_t x16 = xb >> 4, g16 = (xb + 3 * copy_bytes) >> 4;
+        const uint32_t x16 = xb >> 4, g16 = (xb + x_bytes) >> 4;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const uint32_t k16 = k * 128;  // 16 pixels x 128 bytes, in 16-byte units
+          const uint32_t k16 = k * (HB ? 160 : 128);  // 16 pixels (HB: two rows of the box) x 128 bytes, in 16-byte units
           const uint64_t bd = b_hi | (uint64_t)(g16 + k * kBRow);
           uint32_t acc = t > t0 || k != 0, d = tmem_base;
           if constexpr (SEG) {
@@ -2696,7 +2702,7 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
 }
 
 struct WgPlan {
-  int ok, exact, BW, BH, BI, PT, SEG, NB, GX, ROW, splits, grid, stages;  // ROW: input-channel chunks per CTA of the row kernel, or 0
+  int ok, exact, BW, BH, BI, PT, SEG, NB, GX, ROW, HB, splits, grid, stages;  // ROW: input-channel chunks per CTA of the row kernel, or 0
   size_t smem, part_floats;
 };
 
@@ -2757,11 +2763,13 @@ WgPlan plan_wgrad(int H, int W, int Cin, int Cout, int N, int aux = 0, int strid
       }
     }
   }
+  pl.HB = aux && stride == 1 && pl.PT && !pl.SEG && !pl.ROW && pl.BW == 8 && W == 8;  // (a main convolution there takes the row form)
   size_t g_region = (size_t)(pl.GX ? 4 : 3) * 128 * pl.NB * 2;
   if (g_region < 4096) g_region = 4096;
   const size_t stage = pl.ROW ? pl.ROW * box + 32768
+                     : pl.HB ? (size_t)20480 + 16384
                      : pl.PT ? (size_t)49152 + (pl.NB > 64 ? pl.NB / 64 : 1) * 16384 : (size_t)(pl.BH + 2) * pl.BW * 128 + g_region;
-  pl.stages = pl.PT && !pl.ROW ? (pl.NB > 64 ? 2 : 3) : (int)((232448 - 2048) / stage);
+  pl.stages = pl.PT && !pl.ROW ? (pl.NB > 64 ? 2 : pl.HB ? 5 : 3) : (int)((232448 - 2048) / stage);
   if (pl.stages > kMaxStages) pl.stages = kMaxStages;
   if (pl.stages < 2) return pl;
   pl.smem = (size_t)pl.stages * stage + 1024 + 1024;
@@ -2811,15 +2819,15 @@ int launch_wgrad_gx(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& 
   return NF_OK;
 }
 
-template <int NB, int SEG>
+template <int NB, int SEG, int HB = 0>
 int launch_wgrad(const WgPlan& pl, const CUtensorMap& mx, const CUtensorMap& mg, const WgParams& p) {
   static bool attr_done_dev[kMaxDevices];  // function attributes belong to a device's context: set once per device
   bool& attr_done = attr_done_dev[current_device()];
   if (!attr_done) {
-    NF_CUDA(cudaFuncSetAttribute(conv_wgrad_tc_kernel<NB, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
+    NF_CUDA(cudaFuncSetAttribute(conv_wgrad_tc_kernel<NB, SEG, HB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448));
     attr_done = true;
   }
-  nf_launch(conv_wgrad_tc_kernel<NB, SEG>, pl.grid, wgrad_threads(SEG), pl.smem, mx, mg, p);
+  nf_launch(conv_wgrad_tc_kernel<NB, SEG, HB>, pl.grid, wgrad_threads(SEG), pl.smem, mx, mg, p);
   NF_LAUNCHED();
   return NF_OK;
 }
@@ -2833,7 +2841,7 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
   if (pl.part_floats > part_floats) return NF_ENOWS;
   CUtensorMap mx, mg;
   const uint64_t dx[4] = {(uint64_t)Cin, (uint64_t)Win, (uint64_t)Hin, (uint64_t)N};
-  const uint32_t bx[4] = {64, (uint32_t)pl.BW, (uint32_t)(pl.PT && !pl.ROW ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
+  const uint32_t bx[4] = {64, (uint32_t)(pl.HB ? 10 : pl.BW), (uint32_t)(pl.PT && !pl.ROW ? pl.BH : pl.BH + 2), (uint32_t)pl.BI};
   const uint64_t dg[4] = {(uint64_t)Cout, (uint64_t)W, (uint64_t)H, (uint64_t)N};
   const uint32_t bg[4] = {(uint32_t)(pl.NB > 64 ? 64 : pl.NB), (uint32_t)pl.BW, (uint32_t)pl.BH, (uint32_t)pl.BI};
   int rc;
@@ -2855,6 +2863,8 @@ int run_wgrad(int N, int Hin, int Win, int Cin, int Cout, const void* x, const v
     rc = pl.NB == 64 ? launch_wgrad<64, 1>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 1>(pl, mx, mg, p) : launch_wgrad<16, 1>(pl, mx, mg, p);
   else if (pl.SEG)
     rc = pl.NB == 64 ? launch_wgrad<64, 2>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 2>(pl, mx, mg, p) : launch_wgrad<16, 2>(pl, mx, mg, p);
+  else if (pl.HB)
+    rc = pl.NB == 64 ? launch_wgrad<64, 0, 1>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 0, 1>(pl, mx, mg, p) : launch_wgrad<16, 0, 1>(pl, mx, mg, p);
   else if (pl.PT)
     rc = pl.NB == 256 ? launch_wgrad<256, 0>(pl, mx, mg, p) : pl.NB == 128 ? launch_wgrad<128, 0>(pl, mx, mg, p)
        : pl.NB == 64 ? launch_wgrad<64, 0>(pl, mx, mg, p) : pl.NB == 32 ? launch_wgrad<32, 0>(pl, mx, mg, p) : launch_wgrad<16, 0>(pl, mx, mg, p);

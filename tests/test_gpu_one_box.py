@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from tests import parity_util as pu
-from tests.test_gpu_ragged_precision import _nhwc64
+from tests.test_gpu_ragged_precision import _nhwc64, _wgrad64
 
 pytestmark = pytest.mark.gpu
 
@@ -20,6 +20,8 @@ CASES = [
     _c(77, 256, 16, 16, 16), _c(37, 512, 16, 16, 16), _c(77, 128, 16, 16, 32), _c(39, 256, 16, 16, 24), _c(21, 128, 16, 16, 40),
     # pooled layers: input gradient of 16, 32 and 64 filters to 128 and 64 channels, one box, two groups
     _c(77, 128, 32, 32, 16, True), _c(39, 128, 32, 32, 32, True), _c(150, 64, 64, 64, 64, True), _c(151, 64, 32, 16, 16, True), _c(75, 64, 32, 16, 32, True),
+    # maps 8 pixels wide: weight gradient of 16, 32 and 64 filters from one box per tile, the last tile short of images
+    _c(75, 128, 8, 8, 16), _c(2, 64, 8, 8, 32), _c(77, 64, 4, 8, 64), _c(1203, 64, 8, 8, 8),
     # average pool of many images: chains of one, two and eight pixels; 8x8 with 256 filters (a division at the end)
     _c(1500, 64, 16, 16, 8), _c(300, 64, 32, 32, 16), _c(1000, 64, 32, 32, 64), _c(700, 64, 8, 8, 256), _c(170, 64, 20, 20, 8),
 ]
@@ -57,4 +59,9 @@ def test_forms_without_sums(ci):
         assert bool(((p.double() - p64).abs() <= 2.0 ** -16 * p64 + 1e-7).all()), "p"
     if L.kernel_family(6) == "stored":
         rounded(L.stored("da"), _nhwc64(torch, L.stored("dh")[..., :F], Wa.flip(0).permute(0, 2, 1).contiguous(), 1), "da")
+    if L.kernel_family(3) == "tcgen05" and not c["pool"]:
+        g64 = _wgrad64(torch, act, L.stored("dh")[..., :F], 1).cpu().numpy()
+        g = np.ascontiguousarray(L.get_param("Wa", nf.NF_K_GRAD).transpose(2, 3, 0, 1)).reshape(g64.shape)
+        # exact products; the running sum of the tensor core loses 2^-27 per instruction, a few hundred of them per range
+        assert np.sqrt(((g - g64) ** 2).sum() / (g64 ** 2).sum()) <= 1e-5, "gWa"
     L.close()
