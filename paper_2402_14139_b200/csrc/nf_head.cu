@@ -8,6 +8,7 @@
 #include <algorithm>
 
 #include "nf_internal.h"
+#include "nf_ldst.cuh"
 
 namespace {
 
@@ -16,7 +17,8 @@ namespace {
 // two buffers: the next step's loads fly while this one is multiplied, one barrier of two warps per step.  Operands whose
 // contiguous index is aligned are fetched four values at a time.  A thread's 64 products per four 16-byte reads keep the FMA pipes
 // ahead of shared memory; with 256 threads of 4 x 4 or 2 x 4 outputs the reads and barriers set the pace (the head of
-// 6366 images with 1024 inputs and 100 classes: 366 -> 309 us, three products).
+// 6366 images with 1024 inputs and 100 classes: 366 -> 309 us, three products).  Two columns share a packed multiply-add, which rounds each
+// as fmaf does (the three products 198 -> 188 us; what is left is the latency of the loads, a few warps per SM).
 
 // Fetches an HK x R tile (R rows of index i, HK of k) of `src` into registers and puts it to sm[k][i].
 template <int R, int HK>
@@ -68,11 +70,11 @@ __global__ void __launch_bounds__(64) head_gemm_kernel(const float* __restrict__
   const int k_lo = (int)((long)Kd * z / Z), k_hi = (int)((long)Kd * (z + 1) / Z);
   const bool va = (((uintptr_t)A & 15) == 0) && (sai == 1 ? sak % 4 == 0 : sak == 1 && sai % 4 == 0 && k_lo % 4 == 0);
   const bool vb = (((uintptr_t)B & 15) == 0) && (sbj == 1 ? sbk % 4 == 0 : sbk == 1 && sbj % 4 == 0 && k_lo % 4 == 0);
-  float acc[TM][8];
+  f32x2 acc[TM][4];  // columns 2v and 2v + 1
 #pragma unroll
   for (int a = 0; a < TM; ++a)
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0;
   HeadTile<BM, HK> ta;
   HeadTile<64, HK> tb;
   ta.fetch(A, sai, sak, va, i0, M, k_lo, k_hi);
@@ -89,7 +91,8 @@ __global__ void __launch_bounds__(64) head_gemm_kernel(const float* __restrict__
     }
 #pragma unroll 4
     for (int kk = 0; kk < HK; ++kk) {
-      float a[TM], b[8];
+      float a[TM];
+      f32x2 b[4];
 #pragma unroll
       for (int u = 0; u < TM; u += 4) {
         const float4 q = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM + u]);
@@ -97,13 +100,15 @@ __global__ void __launch_bounds__(64) head_gemm_kernel(const float* __restrict__
       }
 #pragma unroll
       for (int v = 0; v < 8; v += 4) {  // columns tx * 4 .. + 3 and 32 more
-        const float4 q = *reinterpret_cast<const float4*>(&Bs[buf][kk][v * 8 + tx * 4]);
-        b[v] = q.x; b[v + 1] = q.y; b[v + 2] = q.z; b[v + 3] = q.w;
+        const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][v * 8 + tx * 4]);
+        b[v / 2] = q.x; b[v / 2 + 1] = q.y;
       }
 #pragma unroll
-      for (int u = 0; u < TM; ++u)
+      for (int u = 0; u < TM; ++u) {
+        const f32x2 aa = nf_pack2(a[u], a[u]);
 #pragma unroll
-        for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+        for (int v = 0; v < 4; ++v) acc[u][v] = nf_fma2(aa, b[v], acc[u][v]);
+      }
     }
     if (more) {
       ta.put(As[buf ^ 1], sai);
@@ -117,16 +122,19 @@ __global__ void __launch_bounds__(64) head_gemm_kernel(const float* __restrict__
 #pragma unroll
   for (int u = 0; u < TM; ++u) {
     const int i = i0 + ty * TM + u;
+    float r[8];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) nf_unpack2(acc[u][v], r[2 * v], r[2 * v + 1]);
 #pragma unroll
     for (int v = 0; v < 8; v += 4) {
       const int j = j0 + v * 8 + tx * 4;
       float* o = out + (size_t)i * Nn + j;
       if (i < M && vo && j < Nn) {
-        *reinterpret_cast<float4*>(o) = make_float4(acc[u][v], acc[u][v + 1], acc[u][v + 2], acc[u][v + 3]);
+        *reinterpret_cast<float4*>(o) = make_float4(r[v], r[v + 1], r[v + 2], r[v + 3]);
       } else if (i < M) {
 #pragma unroll
         for (int w = 0; w < 4; ++w)
-          if (j + w < Nn) o[w] = acc[u][v + w];
+          if (j + w < Nn) o[w] = r[v + w];
       }
     }
   }

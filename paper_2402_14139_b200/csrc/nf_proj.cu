@@ -77,7 +77,7 @@ __global__ void proj_bwd_apply_kernel(const T* __restrict__ ys, const T* __restr
 // part[split][ci][co] = sum over the split's pixel range (ascending) of dys[pix][co] * x[n][s*i][s*j][ci].  Block: 64 x 64 channels,
 // a thread 4 x 4 of them, 32 pixels per step with the next step's loads in flight; both operands lie in shared memory as they
 // do in memory, a pixel's channels in a row.  (16 x 64 channels with 16-pixel steps and one output row per thread took 132 us on
-// 64 -> 128 channels and 32 768 pixels.)
+// 64 -> 128 channels and 32 768 pixels; packed multiply-adds 23.5 -> 23.)
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x, const T* __restrict__ dys, int H, int W, int Ci, int Co,
                                                          int Ho, int Wo, size_t P, int stride, int splits, float* __restrict__ part) {
@@ -124,11 +124,9 @@ __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x
       *reinterpret_cast<float4*>(&gs[b][q][c + e]) = make_float4(gr[e], gr[e + 1], gr[e + 2], gr[e + 3]);
     }
   };
-  float acc[4][4];
+  f32x2 acc[4][2];  // output channels 2j and 2j + 1
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = 0;
   fetch(p0);
   put(0);
   __syncthreads();
@@ -138,22 +136,29 @@ __global__ void __launch_bounds__(256) proj_wgrad_kernel(const T* __restrict__ x
     if (more) fetch(pb + 32);
 #pragma unroll 8
     for (int k = 0; k < 32; ++k) {
-      const float4 xv = *reinterpret_cast<const float4*>(&xs[b][k][ti]), gv = *reinterpret_cast<const float4*>(&gs[b][k][to]);
-      const float xa[4] = {xv.x, xv.y, xv.z, xv.w}, ga[4] = {gv.x, gv.y, gv.z, gv.w};
+      const float4 xv = *reinterpret_cast<const float4*>(&xs[b][k][ti]);
+      const ulonglong2 gv = *reinterpret_cast<const ulonglong2*>(&gs[b][k][to]);
+      const float xa[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(ga[j], xa[i], acc[i][j]);
+      for (int i = 0; i < 4; ++i) {
+        const f32x2 xx = nf_pack2(xa[i], xa[i]);
+        acc[i][0] = nf_fma2(gv.x, xx, acc[i][0]);
+        acc[i][1] = nf_fma2(gv.y, xx, acc[i][1]);
+      }
     }
     if (more) put(b ^ 1);
     __syncthreads();
     b ^= 1;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 4; ++i) {
+    float r[4];
+    nf_unpack2(acc[i][0], r[0], r[1]);
+    nf_unpack2(acc[i][1], r[2], r[3]);
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (ci0 + ti + i < Ci && co0 + to + j < Co) part[((size_t)sp * Ci + ci0 + ti + i) * Co + co0 + to + j] = acc[i][j];
+      if (ci0 + ti + i < Ci && co0 + to + j < Co) part[((size_t)sp * Ci + ci0 + ti + i) * Co + co0 + to + j] = r[j];
+  }
 }
 
 inline unsigned blocks_for(size_t n, int per) { return (unsigned)((n + per - 1) / per); }
