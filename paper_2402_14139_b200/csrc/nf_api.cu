@@ -537,6 +537,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
                       L->val + L->off[NF_P_BF], L->p, L->logits, L->dlogits, L->dp, L->lossn, L->status,
                       sample_mode == 2 ? L->dh : nullptr, (float*)L->parg, g + L->off[NF_P_WF], g + L->off[NF_P_BF], g + L->off[NF_P_BA], loss_out};
     NF_TRY(nf_head_sample_step(io, dt, N, Ha, Wa, F, K, L->o.loss, n_scale));
+    if (g_trace_on) NF_TRY(nf_head_sample_sums(io, N, F, K, n_scale));  // timed: nothing runs aside, and an operation is one group
   } else if (nf_head_is_large(N, D, K)) {  // late blocks: tens of thousands of samples, up to 1024 head inputs
     NF_TRY(nf_head_step(L->p, labels, N, D, K, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->logits, L->dlogits, L->dp,
                         L->lossn, L->status, L->o.loss, g + L->off[NF_P_WF], g + L->off[NF_P_BF], loss_out, L->wpart,
@@ -572,6 +573,11 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   }
   if (!dh_nb && sample_mode != 2) NF_TRY(nf_k_channel_sums(dt, L->dh, (size_t)N * Ha * Wa, F, L->red, L->red_floats, &dh_nb));
   if (dh_nb) NF_TRY(nf_k_sum_partials(L->red, dh_nb, F, g + L->off[NF_P_BA]));  // before the input gradient, which uses L->red too
+  auto aux_wgrad = [&]() {
+    if (L->fam[3]) return nf_tc_aux_wgrad(L, act_out);
+    return nf_k_wgrad(dt, act_out, N, Ha, Wa, Co, L->dh, F, 1, L->wpart, L->wpart_floats, g + L->off[NF_P_WA]);
+  };
+  if (g_trace_on) NF_TRY(aux_wgrad());
   NF_TRY(beside.fork());
   trace_end();
   // gradient at the aux input
@@ -583,16 +589,12 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     NF_TRY(nf_k_conv(dt, L->dh, N, Ha, Wa, F, Wx, (long)F * Co, 1, Co, 1, nullptr, 0, 1, Co, L->da));
   }
   trace_end();
-  NF_TRY(beside.open());
-  trace_begin(4);
-  if (sample_mode) NF_TRY(nf_head_sample_sums(io, N, F, K, n_scale));
-  if (L->fam[3]) {
-    NF_TRY(nf_tc_aux_wgrad(L, act_out));
-  } else {
-    NF_TRY(nf_k_wgrad(dt, act_out, N, Ha, Wa, Co, L->dh, F, 1, L->wpart, L->wpart_floats, g + L->off[NF_P_WA]));
+  if (!g_trace_on) {
+    NF_TRY(beside.open());
+    if (sample_mode) NF_TRY(nf_head_sample_sums(io, N, F, K, n_scale));
+    NF_TRY(aux_wgrad());
+    NF_TRY(beside.close());
   }
-  trace_end();
-  NF_TRY(beside.close());
   // back through pool / ReLU / BatchNorm; a trainable shortcut joined at the BatchNorm output gets the gradient dz at that sum
   trace_begin(5);
   if (bn_nb) {
