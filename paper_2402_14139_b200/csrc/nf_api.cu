@@ -476,7 +476,15 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   const void* Wx = dt == NF_F32 ? (const void*)(L->val + L->off[NF_P_WA]) : (const void*)(L->shadow + L->off[NF_P_WA]);
   float* g = L->grad;
   int nb = 0;
-  Aside beside(&L->lane, all);  // gradients of the auxiliary network, which nothing else in the step waits for
+  // The gradients of the auxiliary network, which nothing else in the step waits for, run beside the rest, unless the activation they read
+  // shares memory with what the rest writes: with dz, or with one of the layer's own tensors (then they come before those, and a pooled
+  // layer's winners lie in the activation buffer that such a call leaves unused).  Under timing they come first too: one group per operation.
+  const char *a0 = (const char*)act_out, *a1 = a0 + (size_t)N * Ha * Wa * Co * nf_esize(dt);
+  const bool own = a0 < L->ws + L->ws_total && L->ws < a1 && act_out != L->act && act_out != L->stage_act;
+  const char *z0 = (const char*)L->skip_grad, *z1 = z0 + (size_t)N * Ho * Wo * Co * nf_esize(dt);
+  const bool in_line = g_trace_on || own || (L->skip_grad && a0 < z1 && z0 < a1);
+  void* const ywin = own ? L->act : L->dy;
+  Aside beside(&L->lane, all && !in_line);
 
   // Eq. 1: conv, BatchNorm (batch statistics), ReLU, optional max-pool -> act_out
   if (all || phase == 0) {
@@ -502,7 +510,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   }
   // where the shape allows, the aux forward kernel normalises y on the way in and writes act_out itself
   const bool fused_bn_aux = nf_tc_bn_aux_fused(L) && !L->skip;
-  if (!fused_bn_aux) NF_TRY(nf_k_bn_apply(dt, L->y, N, Ho, Wo, Co, pool, L->scale, L->shift, act_out, L->skip, L->dy));
+  if (!fused_bn_aux) NF_TRY(nf_k_bn_apply(dt, L->y, N, Ho, Wo, Co, pool, L->scale, L->shift, act_out, L->skip, ywin));
   trace_end();
   if (!fused_bn_aux && tail) NF_TRY(tail->fork() == NF_OK ? tail->open() : NF_ECUDA);
   // Eq. 2: aux conv + ReLU, average pool to 2x2, linear; Eq. 3: softmax cross-entropy
@@ -537,7 +545,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
                       L->val + L->off[NF_P_BF], L->p, L->logits, L->dlogits, L->dp, L->lossn, L->status,
                       sample_mode == 2 ? L->dh : nullptr, (float*)L->parg, g + L->off[NF_P_WF], g + L->off[NF_P_BF], g + L->off[NF_P_BA], loss_out};
     NF_TRY(nf_head_sample_step(io, dt, N, Ha, Wa, F, K, L->o.loss, n_scale));
-    if (g_trace_on) NF_TRY(nf_head_sample_sums(io, N, F, K, n_scale));  // timed: nothing runs aside, and an operation is one group
+    if (in_line) NF_TRY(nf_head_sample_sums(io, N, F, K, n_scale));
   } else if (nf_head_is_large(N, D, K)) {  // late blocks: tens of thousands of samples, up to 1024 head inputs
     NF_TRY(nf_head_step(L->p, labels, N, D, K, L->val + L->off[NF_P_WF], L->val + L->off[NF_P_BF], L->logits, L->dlogits, L->dp,
                         L->lossn, L->status, L->o.loss, g + L->off[NF_P_WF], g + L->off[NF_P_BF], loss_out, L->wpart,
@@ -577,7 +585,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     if (L->fam[3]) return nf_tc_aux_wgrad(L, act_out);
     return nf_k_wgrad(dt, act_out, N, Ha, Wa, Co, L->dh, F, 1, L->wpart, L->wpart_floats, g + L->off[NF_P_WA]);
   };
-  if (g_trace_on) NF_TRY(aux_wgrad());
+  if (in_line) NF_TRY(aux_wgrad());
   NF_TRY(beside.fork());
   trace_end();
   // gradient at the aux input
@@ -589,7 +597,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     NF_TRY(nf_k_conv(dt, L->dh, N, Ha, Wa, F, Wx, (long)F * Co, 1, Co, 1, nullptr, 0, 1, Co, L->da));
   }
   trace_end();
-  if (!g_trace_on) {
+  if (!in_line) {
     NF_TRY(beside.open());
     if (sample_mode) NF_TRY(nf_head_sample_sums(io, N, F, K, n_scale));
     NF_TRY(aux_wgrad());
@@ -602,7 +610,7 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
     if (L->skip_grad) NF_TRY(nf_k_write_dz(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->skip, L->skip_grad));
   } else {
     NF_TRY(nf_k_bn_bwd_reduce(dt, L->y, L->da, N, Ho, Wo, Co, pool, L->scale, L->shift, L->mu, L->invstd, L->red,
-                                L->red_floats, &nb, L->skip, L->skip_grad, L->dy));
+                                L->red_floats, &nb, L->skip, L->skip_grad, ywin));
   }
   if (!all) return nf_k_partial_totals(L->red, nb, Co, L->dptot + 2 * Co);
   }

@@ -133,3 +133,30 @@ def test_lanes_of_many_layers_come_and_go():
             b.close()
             for L in ls:
                 L.close()
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("where", ["dy", "da", "dz"])
+def test_activation_in_a_buffer_that_the_step_writes_later(kind, where):
+    """act_out in the layer's own gradient buffers, or in the place of dz: the step reads it before it is written over."""
+    import torch
+    nf, ref, _, x, y = _block(kind, 24, 11)
+    nf, layers, _, _, _ = _block(kind, 24, 11)
+    loss, got = torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda")
+    cur = x
+    for R, L in zip(ref, layers):
+        act = R.new_act()
+        if where == "dz" and not L.maxpool:
+            dz = L.new_act()
+            L.set_skip_grad(dz)
+            R.set_skip_grad(R.new_act())
+            out = dz
+        else:
+            out = L.stored("dy" if where == "dz" else where).flatten()[:act.numel()]
+        for _ in range(2):
+            R.step(cur, y, 0.05, loss, act)
+            L.step(cur, y, 0.05, got, out)
+        assert torch.equal(loss, got)
+        cur = act
+    torch.cuda.synchronize()
+    _same(_state(layers), _state(ref))
