@@ -1203,11 +1203,12 @@ __global__ void __launch_bounds__(256) avgpool_small_vec_kernel(const uint4* __r
 // kernels around it: M = 1, the bin's pixels in order; M > 1, `planes` chains of M pixels each, planes apart, the chains added in order.
 // Many images: 16x16 maps with 16 filters, 1777 of them, 37 + 3 -> 5 us (there half the threads of a block per bin had nothing to do and
 // sixteen added 128 sums one by one); 8x8 with 256, 6366 of them, 61 -> 45 (a thread for all four bins left a second wave nearly empty).
+// Blocks of 64 threads, so that a few thousand of them reach every SM.
 template <int M>
-__global__ void __launch_bounds__(256) avgpool_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, int cnt, int planes,
+__global__ void __launch_bounds__(64) avgpool_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, int cnt, int planes,
                                                           uint32_t bw_mul, bool divide, size_t total, float* __restrict__ p) {
   nf_pdl_begin();
-  const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+  const size_t e = (size_t)blockIdx.x * 64 + threadIdx.x;
   if (e >= total) return;
   const int bin = (int)(e & 3), g = (int)((e >> 2) % F8), bw = Wa / 2;
   const size_t n = (e >> 2) / F8;
@@ -1746,9 +1747,9 @@ int nf_k_avgpool_fast(const void* h, int N, int Ha, int Wa, int F, float* part, 
   // one pass where no slices are cut, the chains are whole and there are threads enough for their length
   const int cnt = (Ha / 2) * (Wa / 2), planes = 256 / (F / 8), m = cnt <= planes ? 1 : cnt % planes ? 0 : cnt / planes;
   const size_t total = (size_t)N * 4 * (F / 8);
-  if (S == 1 && Wa >= 4 && (m == 1 || m == 2 || m == 4 || m == 8) && cnt < 65536 && (cnt <= 64 || total >= 16384)) {
+  if (S == 1 && Wa >= 4 && (m == 1 || m == 2 || m == 4 || m == 8) && cnt < 65536 && (m > 1 ? total >= 49152 : cnt <= 64 || total >= 16384)) {
     auto* k = m == 1 ? avgpool_vec_kernel<1> : m == 2 ? avgpool_vec_kernel<2> : m == 4 ? avgpool_vec_kernel<4> : avgpool_vec_kernel<8>;
-    nf_launch(k, nblk(total, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, cnt, planes, recip(Wa / 2), false, total, p);
+    nf_launch(k, nblk(total, 64), 64, 0, (const uint4*)h, Ha, Wa, F / 8, cnt, planes, recip(Wa / 2), false, total, p);
     NF_LAUNCHED();
     return NF_OK;
   }
@@ -1799,7 +1800,7 @@ int nf_k_avgpool(int dtype, const void* h, int N, int Ha, int Wa, int F, float* 
     if (dtype == NF_BF16 && F % 8 == 0 && ((size_t)N * 4 * F > (size_t)148 * 2048 || Ha * Wa <= 4)) {
       const size_t groups = (size_t)N * (F / 8);
       if (Ha % 2 == 0 && Wa % 2 == 0 && Wa >= 4) {
-        nf_launch(avgpool_vec_kernel<1>, nblk(groups * 4, 256), 256, 0, (const uint4*)h, Ha, Wa, F / 8, (Ha / 2) * (Wa / 2), 1, recip(Wa / 2), true,
+        nf_launch(avgpool_vec_kernel<1>, nblk(groups * 4, 64), 64, 0, (const uint4*)h, Ha, Wa, F / 8, (Ha / 2) * (Wa / 2), 1, recip(Wa / 2), true,
                   groups * 4, p);
         NF_LAUNCHED();
         return NF_OK;
