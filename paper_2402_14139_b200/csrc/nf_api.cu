@@ -66,12 +66,12 @@ int trace_flush() {
 
 // ---- side streams
 // Lanes of layers and blocks that are gone, for the next ones: making a stream and an event takes 90 us, a quarter of what preparing a
-// small layer takes.  At most kLanesKept; what comes back beyond that is destroyed.  A lane that a running capture has drawn in is not
-// given out before that capture has ended.
+// small layer takes.  At most kLanesKept idle ones; what comes back beyond that is destroyed.  A lane that a running capture has drawn in
+// is neither given out nor destroyed before that capture has ended, so there may be more for that long.
 constexpr int kLanesKept = 32;
 std::mutex g_lanes_mutex;
-NfLane g_lanes[kLanesKept];
-int g_lane_count = 0;
+NfLane* g_lanes = nullptr;
+int g_lane_count = 0, g_lane_room = 0;
 
 bool lane_idle(const NfLane& n) {  // of no capture
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -98,19 +98,34 @@ void lane_open(NfLane* n) {
   }
   if (!n->s) cudaGetLastError();  // not an error of the call: everything then runs in the caller's stream
 }
-void lane_close(NfLane* n) {
-  if (!n->s) return;
-  {
-    const std::lock_guard<std::mutex> lock(g_lanes_mutex);
-    if (g_lane_count < kLanesKept) {
-      g_lanes[g_lane_count++] = *n;
-      n->s = nullptr;
-      return;
-    }
-  }
+void lane_destroy(NfLane* n) {
   cudaEventDestroy(n->e);
   cudaStreamDestroy(n->s);
   n->s = nullptr;
+}
+void lane_close(NfLane* n) {
+  if (!n->s) return;
+  const std::lock_guard<std::mutex> lock(g_lanes_mutex);
+  if (g_lane_count == g_lane_room) {
+    NfLane* const more = (NfLane*)realloc(g_lanes, (g_lane_room + kLanesKept + 1) * sizeof(NfLane));
+    if (!more) {  // no room to keep it
+      if (lane_idle(*n)) lane_destroy(n);
+      n->s = nullptr;
+      return;
+    }
+    g_lanes = more;
+    g_lane_room += kLanesKept + 1;
+  }
+  g_lanes[g_lane_count++] = *n;
+  n->s = nullptr;
+  for (int i = 0; i < g_lane_count && g_lane_count > kLanesKept;) {
+    if (lane_idle(g_lanes[i])) {
+      lane_destroy(&g_lanes[i]);
+      g_lanes[i] = g_lanes[--g_lane_count];
+    } else {
+      ++i;
+    }
+  }
 }
 bool lane_usable(const NfLane* n) {
   int dev = -1;

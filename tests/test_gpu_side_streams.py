@@ -135,6 +135,35 @@ def test_lanes_of_many_layers_come_and_go():
                 L.close()
 
 
+def test_layers_that_go_while_a_capture_holds_their_lanes():
+    """More layers than lanes are kept for, closed before the capture that has stepped them ends: the graph is whole, and its replay does
+    what the same steps one after the other do."""
+    import torch
+    nf, ref, _, x, y = _block("f32", 8, 13)
+    loss, act = torch.zeros(1, device="cuda"), ref[0].new_act()
+    ref[0].step(x, y, 0.05, loss, act)
+    many = [_block("f32", 8, 13)[1][0] for _ in range(40)]
+    got, acts = torch.zeros(len(many), device="cuda"), [L.new_act() for L in many]
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        nf.nf_set_stream(torch.cuda.current_stream())
+        for i, L in enumerate(many):
+            L.step(x, y, 0.05, got[i:i + 1], acts[i])
+        grads = [L.dp_buffer(2) for L in many]
+        for L in many:          # the handles only: their memory stays
+            L.close()
+    nf.nf_set_stream(torch.cuda.current_stream())
+    g.replay()
+    torch.cuda.synchronize()
+    assert bool((got == loss).all()) and all(torch.equal(a, act) for a in acts)
+    assert all(torch.equal(v, ref[0].dp_buffer(2)) for v in grads)
+    _, fresh, block, x, y = _block("f32", 8, 13)    # and the lanes serve again
+    block.step(x, y, 0.05, torch.zeros(len(fresh), device="cuda"))
+    torch.cuda.synchronize()
+    assert torch.equal(fresh[0].dp_buffer(2), ref[0].dp_buffer(2))
+
+
 @pytest.mark.parametrize("kind", ["bf16", "f32"])
 @pytest.mark.parametrize("where", ["dy", "da", "dz"])
 def test_activation_in_a_buffer_that_the_step_writes_later(kind, where):
