@@ -73,10 +73,18 @@ std::mutex g_lanes_mutex;
 NfLane* g_lanes = nullptr;
 int g_lane_count = 0, g_lane_room = 0;
 
-bool lane_idle(const NfLane& n) {  // of no capture
+// The capture that a stream is part of: 0 for none, a number of its own for each, kNoCapture where it has failed or cannot be told.
+constexpr unsigned long long kNoCapture = ~0ull;
+unsigned long long capture_of(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(n.s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return kNoCapture;
+  }
+  return st == cudaStreamCaptureStatusNone ? 0 : st == cudaStreamCaptureStatusActive ? id : kNoCapture;
 }
+bool lane_idle(const NfLane& n) { return capture_of(n.s) == 0; }
 void lane_open(NfLane* n) {
   if (n->s) return;
   if (cudaGetDevice(&n->dev) == cudaSuccess) {
@@ -89,12 +97,15 @@ void lane_open(NfLane* n) {
           return;
         }
     }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // a capture that the calling thread has begun has no part in this
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (cudaStreamCreateWithFlags(&n->s, cudaStreamNonBlocking) != cudaSuccess) {
       n->s = nullptr;
     } else if (cudaEventCreateWithFlags(&n->e, cudaEventDisableTiming) != cudaSuccess) {
       cudaStreamDestroy(n->s);
       n->s = nullptr;
     }
+    cudaThreadExchangeStreamCaptureMode(&mode);
   }
   if (!n->s) cudaGetLastError();  // not an error of the call: everything then runs in the caller's stream
 }
@@ -127,9 +138,17 @@ void lane_close(NfLane* n) {
     }
   }
 }
-bool lane_usable(const NfLane* n) {
+// Whether work may go aside on the lane.  A capture that has drawn it in keeps it, until that capture ends, from calls on streams that are
+// not part of the same capture: those take another.
+bool lane_usable(NfLane* n) {
   int dev = -1;
-  return n->s && cudaGetDevice(&dev) == cudaSuccess && dev == n->dev && !g_trace_on;
+  if (g_trace_on || !n->s || cudaGetDevice(&dev) != cudaSuccess || dev != n->dev) return false;
+  const unsigned long long id = capture_of(n->s);
+  if (id != 0 && (id == kNoCapture || id != capture_of(nf_stream()))) {
+    lane_close(n);
+    lane_open(n);
+  }
+  return n->s != nullptr;
 }
 
 // Work beside the stream in use: fork() puts the lane's stream behind all that the stream has so far, open() sends the launches that

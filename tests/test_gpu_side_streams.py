@@ -164,6 +164,67 @@ def test_layers_that_go_while_a_capture_holds_their_lanes():
     assert torch.equal(fresh[0].dp_buffer(2), ref[0].dp_buffer(2))
 
 
+class _Recording:
+    """A capture of one stream, which others may run beside."""
+
+    def __init__(self, stream):
+        from cuda.bindings import runtime as rt
+        self.rt, self.stream = rt, stream
+        self._do("cudaStreamBeginCapture", stream.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal)
+
+    def _do(self, name, *args):
+        err, *out = getattr(self.rt, name)(*args)
+        assert err == self.rt.cudaError_t.cudaSuccess, (name, err)
+        return out[0] if len(out) == 1 else out
+
+    def end(self):
+        self.graph = self._do("cudaStreamEndCapture", self.stream.cuda_stream)
+
+    def replay(self):
+        self._do("cudaGraphLaunch", self._do("cudaGraphInstantiate", self.graph, 0), self.stream.cuda_stream)
+
+
+@pytest.mark.parametrize("call", ["block", "layers"])
+def test_an_ordinary_call_while_a_capture_holds_the_lanes(call):
+    """Handles that a capture on one stream has stepped, stepped on another stream before it ends, and in a capture of a third one: what is
+    recorded runs when its graph does, the ordinary step at once."""
+    import torch
+    nf, ref, _, x, y = _block("bf16", 24, 15)
+    loss, acts = torch.zeros(len(ref), device="cuda"), [L.new_act() for L in ref]
+    nf, layers, block, x, y = _block("bf16", 24, 15)
+    got, out = torch.zeros(len(ref), device="cuda"), [L.new_act() for L in layers]
+
+    def step(stream):
+        nf.nf_set_stream(stream)
+        if call == "block":
+            block.step(x, y, 0.05, got, out[-1])
+        else:
+            _one_by_one(layers, x, y, got, out, 1)
+
+    step(torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    s1, s2, s3 = (torch.cuda.Stream() for _ in range(3))
+    g = _Recording(s1)
+    step(s1)
+    step(s2)
+    h = _Recording(s3)
+    step(s3)
+    step(s1)
+    h.end()
+    g.end()
+    torch.cuda.synchronize()
+    nf.nf_set_stream(torch.cuda.current_stream())
+    _one_by_one(ref, x, y, loss, acts, 2)
+    _same(_state(layers), _state(ref))
+    for graph, steps in ((h, 1), (g, 2)):
+        graph.replay()
+        torch.cuda.synchronize()
+        _one_by_one(ref, x, y, loss, acts, steps)
+        _same(_state(layers), _state(ref))
+    assert torch.equal(got, loss) and torch.equal(out[-1], acts[-1])
+    assert all(L.status() == 0 for L in layers)
+
+
 @pytest.mark.parametrize("kind", ["bf16", "f32"])
 @pytest.mark.parametrize("where", ["dy", "da", "dz"])
 def test_activation_in_a_buffer_that_the_step_writes_later(kind, where):
