@@ -21,8 +21,9 @@
  *  - Calls enqueue work on the stream given to nf_set_stream (default stream 0) and
  *    return without synchronising unless stated.  Buffers must stay valid until the
  *    stream has passed the call.  A training step also uses side streams that its layer or
- *    block keeps; they start behind that stream and it waits for them before the call ends,
- *    so the order against other work is that of the one stream (captures included).
+ *    block keeps, of that stream's priority; they start behind that stream and it waits for
+ *    them before the call ends, so the order against other work is that of the one stream
+ *    (captures included).
  *  - Return value: NF_OK (0) or a negative nf_status.  Nothing throws, aborts or
  *    traps.  Conditions found on the device (bad label, non-finite loss, a bounded
  *    wait that ran out) are OR-ed into a per-layer status word read by nf_layer_status.

@@ -85,13 +85,19 @@ unsigned long long capture_of(cudaStream_t s) {
   return st == cudaStreamCaptureStatusNone ? 0 : st == cudaStreamCaptureStatusActive ? id : kNoCapture;
 }
 bool lane_idle(const NfLane& n) { return capture_of(n.s) == 0; }
+int priority_of(cudaStream_t s) {
+  int prio = 0;
+  if (cudaStreamGetPriority(s, &prio) != cudaSuccess) cudaGetLastError();
+  return prio;
+}
 void lane_open(NfLane* n) {
   if (n->s) return;
   if (cudaGetDevice(&n->dev) == cudaSuccess) {
+    n->prio = priority_of(nf_stream());
     {
       const std::lock_guard<std::mutex> lock(g_lanes_mutex);
       for (int i = 0; i < g_lane_count; ++i)
-        if (g_lanes[i].dev == n->dev && lane_idle(g_lanes[i])) {
+        if (g_lanes[i].dev == n->dev && g_lanes[i].prio == n->prio && lane_idle(g_lanes[i])) {
           *n = g_lanes[i];
           g_lanes[i] = g_lanes[--g_lane_count];
           return;
@@ -99,7 +105,7 @@ void lane_open(NfLane* n) {
     }
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // a capture that the calling thread has begun has no part in this
     cudaThreadExchangeStreamCaptureMode(&mode);
-    if (cudaStreamCreateWithFlags(&n->s, cudaStreamNonBlocking) != cudaSuccess) {
+    if (cudaStreamCreateWithPriority(&n->s, cudaStreamNonBlocking, n->prio) != cudaSuccess) {
       n->s = nullptr;
     } else if (cudaEventCreateWithFlags(&n->e, cudaEventDisableTiming) != cudaSuccess) {
       cudaStreamDestroy(n->s);
@@ -139,12 +145,12 @@ void lane_close(NfLane* n) {
   }
 }
 // Whether work may go aside on the lane.  A capture that has drawn it in keeps it, until that capture ends, from calls on streams that are
-// not part of the same capture: those take another.
+// not part of the same capture: those take another.  So do calls on a stream of another priority, whose work keeps that priority aside.
 bool lane_usable(NfLane* n) {
   int dev = -1;
   if (g_trace_on || !n->s || cudaGetDevice(&dev) != cudaSuccess || dev != n->dev) return false;
   const unsigned long long id = capture_of(n->s);
-  if (id != 0 && (id == kNoCapture || id != capture_of(nf_stream()))) {
+  if ((id != 0 && (id == kNoCapture || id != capture_of(nf_stream()))) || n->prio != priority_of(nf_stream())) {
     lane_close(n);
     lane_open(n);
   }

@@ -21,7 +21,7 @@ enum { NF_NPARAM = 7 };
 struct NfLane {
   cudaStream_t s;                      // NULL: could not be had, everything stays in one stream
   cudaEvent_t e;
-  int dev;                             // the device it belongs to
+  int dev, prio;                       // the device it belongs to, and the priority of the streams it serves
 };
 
 struct nf_layer {

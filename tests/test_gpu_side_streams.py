@@ -183,6 +183,13 @@ class _Recording:
     def replay(self):
         self._do("cudaGraphLaunch", self._do("cudaGraphInstantiate", self.graph, 0), self.stream.cuda_stream)
 
+    def kernel_priorities(self):
+        rt = self.rt
+        nodes = self._do("cudaGraphGetNodes", self.graph, self._do("cudaGraphGetNodes", self.graph)[1])[0]
+        kernels = [n for n in nodes if self._do("cudaGraphNodeGetType", n) == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel]
+        assert len(kernels) >= 10 * len(SHAPES["bf16"])
+        return {self._do("cudaGraphKernelNodeGetAttribute", n, rt.cudaLaunchAttributeID.cudaLaunchAttributePriority).priority for n in kernels}
+
 
 @pytest.mark.parametrize("call", ["block", "layers"])
 def test_an_ordinary_call_while_a_capture_holds_the_lanes(call):
@@ -223,6 +230,27 @@ def test_an_ordinary_call_while_a_capture_holds_the_lanes(call):
         _same(_state(layers), _state(ref))
     assert torch.equal(got, loss) and torch.equal(out[-1], acts[-1])
     assert all(L.status() == 0 for L in layers)
+
+
+@pytest.mark.parametrize("call", ["block", "layers"])
+def test_side_streams_have_the_priority_of_the_callers_stream(call):
+    """Every kernel that a step records has the priority of the stream that it was called on, as a step in one stream does."""
+    import torch
+    nf, layers, block, x, y = _block("bf16", 24, 17)
+    loss, acts = torch.zeros(len(layers), device="cuda"), [L.new_act() for L in layers]
+    block.step(x, y, 0.05, loss)
+    torch.cuda.synchronize()
+    for prio in (0, -1, 0):
+        s = torch.cuda.Stream(priority=prio)
+        rec = _Recording(s)
+        nf.nf_set_stream(s)
+        if call == "block":
+            block.step(x, y, 0.05, loss, acts[-1])
+        else:
+            _one_by_one(layers, x, y, loss, acts, 1)
+        rec.end()
+        nf.nf_set_stream(torch.cuda.current_stream())
+        assert rec.kernel_priorities() == {prio}
 
 
 @pytest.mark.parametrize("kind", ["bf16", "f32"])
