@@ -85,6 +85,11 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) first_eval_kernel(cons
     ptx::tmem_alloc(tmem_slot, 128);
     ptx::tmem_relinquish();
   }
+  // The block has its columns before it lets the next kernel's blocks in: those allocate theirs and hold them while they wait for this grid,
+  // and the wait for columns knows no limit.
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
   nf_pdl_begin();
   for (int i = threadIdx.x; i < 256; i += kThreads) {  // weights: row co, places 8c .. 8c+7
     const int co = i >> 2, c = i & 3;
@@ -102,9 +107,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) first_eval_kernel(cons
     coef[threadIdx.x] = make_float4(p.scale[c], p.scale[c + 1], p.shift[c], p.shift[c + 1]);
   }
   ptx::fence_async_smem();
-  ptx::tc_fence_before();
   __syncthreads();
-  ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp < 4) {
