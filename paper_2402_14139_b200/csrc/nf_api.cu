@@ -517,15 +517,17 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   float* g = L->grad;
   int nb = 0;
   // The gradients of the auxiliary network, which nothing else in the step waits for, run beside the rest, unless the activation they read
-  // shares memory with what the rest writes: with dz, or with one of the layer's own tensors (then they come before those, and a pooled
-  // layer's winners lie in the activation buffer that such a call leaves unused).  Under timing they come first too: one group per operation.
+  // shares memory with what the rest writes: with dz, or with one of the layer's own tensors (then they come before those).  Under timing
+  // they come first too: one group per operation.
   const char *a0 = (const char*)act_out, *a1 = a0 + (size_t)N * Ha * Wa * Co * nf_esize(dt);
   const bool own = a0 < L->ws + L->ws_total && L->ws < a1 && act_out != L->act && act_out != L->stage_act;
   const char *z0 = (const char*)L->skip_grad, *z1 = z0 + (size_t)N * Ho * Wo * Co * nf_esize(dt);
   // fp32 kernels of many pixels fill the chip by themselves: there two at once only get in each other's way (851 against 862 us at 512 000)
   const bool full = dt == NF_F32 && (size_t)N * Ha * Wa >= 131072;
   const bool in_line = g_trace_on || own || full || (L->skip_grad && a0 < z1 && z0 < a1);
-  void* const ywin = own ? L->act : L->dy;
+  // A pooled layer's winners lie in a quarter of dy until dy is written: the first one, or the last where the activation lies over the first.
+  const char *d0 = (const char*)L->dy, *d1 = d0 + (a1 - a0);
+  void* const ywin = (char*)L->dy + (pool && a0 < d1 && d0 < a1 ? 3 * (a1 - a0) : 0);
   Aside beside(&L->lane, all && !in_line);
 
   // Eq. 1: conv, BatchNorm (batch statistics), ReLU, optional max-pool -> act_out

@@ -278,3 +278,30 @@ def test_activation_in_a_buffer_that_the_step_writes_later(kind, where):
         cur = act
     torch.cuda.synchronize()
     _same(_state(layers), _state(ref))
+
+
+def _own_memory(L, name, bytes_on):
+    """An activation-shaped view of the layer's workspace, `bytes_on` bytes into one of its tensors."""
+    base = L.stored(name).data_ptr() - L.ws.data_ptr() + bytes_on
+    n = L.N * L.Ha * L.Wa * L.Cout
+    return L.ws[base:base + n * 2].view(L.tdtype).view(L.N, L.Ha, L.Wa, L.Cout)
+
+
+@pytest.mark.parametrize("name,quarters", [("da", 0.125), ("da", 0.5), ("da", 0.875), ("dy", 0), ("dy", 0.5), ("dy", 1), ("dy", 1.5), ("dy", 2.75), ("dy", 3)])
+def test_activation_of_a_pooled_layer_anywhere_in_its_own_gradients(name, quarters):
+    """act_out at any place in da (and on into the activation buffer behind it) or in dy: the winners that the layer keeps for its backward
+    pass lie elsewhere."""
+    import torch
+    nf, ref, _, _, y = _block("bf16", 24, 19)
+    nf, layers, _, _, _ = _block("bf16", 24, 19)
+    R, L = ref[2], layers[2]
+    assert L.maxpool
+    x = torch.randn((24, 32, 32, 64), generator=torch.Generator(device="cuda").manual_seed(19), device="cuda").clamp_min(0).bfloat16()
+    loss, got, act = torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda"), R.new_act()
+    out = _own_memory(L, name, int(quarters * act.numel() * 2))
+    for _ in range(2):
+        R.step(x, y, 0.05, loss, act)
+        L.step(x, y, 0.05, got, out)
+    torch.cuda.synchronize()
+    assert torch.equal(got, loss)
+    _same(_state(layers), _state(ref))
