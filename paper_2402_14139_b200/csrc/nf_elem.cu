@@ -1905,16 +1905,17 @@ int nf_k_bn_bwd_reduce(int dtype, const void* y, const void* da, int N, int Ho, 
   const int nb = nf_k_channel_blocks(P, C);
   if ((size_t)nb * 2 * C > red_floats) return NF_ENOWS;
   const bool vec = vec2_ok(C, pool);
-  if (dz_out && !(skip && vec)) {  // else the reduction below writes it
-    const int rc = nf_k_write_dz(dtype, y, da, N, Ho, Wo, C, pool, scale, shift, skip, dz_out);
-    if (rc != NF_OK) return rc;
-  }
   if (!skip && pool && vec_ok(dtype, C, 0) && 256 % (C / 8) == 0) {
     if (!ywin) return NF_EINVAL;
     nf_launch(bn_bwd_reduce_win_vec_kernel, nb, 256, 0, (const uint4*)ywin, (const uint4*)da, P / 4, C / 8, scale, shift, mu, invstd, red);
     NF_LAUNCHED();
     *nblocks = nb;
-    return NF_OK;
+    // behind the sums: dz may lie over the winners
+    return dz_out ? nf_k_write_dz(dtype, y, da, N, Ho, Wo, C, pool, scale, shift, skip, dz_out) : NF_OK;
+  }
+  if (dz_out && !(skip && vec)) {  // else the reduction below writes it
+    const int rc = nf_k_write_dz(dtype, y, da, N, Ho, Wo, C, pool, scale, shift, skip, dz_out);
+    if (rc != NF_OK) return rc;
   }
   if (vec) {
     // without a shortcut a range is a block's 256 / (C / 8) chains; with one, the generic kernel's (256 channels and chains)

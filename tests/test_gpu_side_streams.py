@@ -305,3 +305,20 @@ def test_activation_of_a_pooled_layer_anywhere_in_its_own_gradients(name, quarte
     torch.cuda.synchronize()
     assert torch.equal(got, loss)
     _same(_state(layers), _state(ref))
+
+
+def test_dz_of_a_pooled_layer_over_its_dy():
+    """dz written where dy goes later, over the winners of the forward pass: the sums and gradients are those of a dz elsewhere."""
+    import torch
+    nf, ref, _, _, y = _block("bf16", 24, 21)
+    nf, layers, _, _, _ = _block("bf16", 24, 21)
+    R, L = ref[2], layers[2]
+    x = torch.randn((24, 32, 32, 64), generator=torch.Generator(device="cuda").manual_seed(21), device="cuda").clamp_min(0).bfloat16()
+    loss, act = torch.zeros(1, device="cuda"), R.new_act()
+    R.set_skip_grad(torch.empty_like(L.stored("dy")))
+    L.set_skip_grad(L.stored("dy"))
+    for _ in range(2):
+        R.step(x, y, 0.05, loss, act)
+        L.step(x, y, 0.05, loss, act)
+    torch.cuda.synchronize()
+    _same(_state(layers), _state(ref))
