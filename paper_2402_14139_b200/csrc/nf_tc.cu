@@ -2374,7 +2374,7 @@ TcPlan plan_fwd(int H, int W, int Cin, int Cout, int N, int epi = 0, int stride 
   const bool sumless = pl.PT == 0 && stride == 1 && (epi == 1 || (epi == 2 && !ybuf));
   if (sumless && W % 8 == 0 && H % 16 == 0 && (epi == 2 || (Cin > 64 && Cout <= 32))) {
     const size_t a1 = ((size_t)18 * 10 * pl.KC * 2 + 1023) & ~(size_t)1023, b9 = (size_t)9 * (epi == 2 ? pl.BN / 64 * pl.KC : pl.BN) * 128;
-    const size_t staged = epi == 2 || Cout == 64 ? 32768 : 0;
+    const size_t staged = epi == 2 ? 32768 : 0;
     const bool resident = epi == 2 || Cin / 64 * b9 + staged + 4 * a1 + 2048 <= 232448;
     if (resident ? b9 * (epi == 2 ? 1 : Cin / 64) + staged + 3 * a1 + 2048 <= 232448 : staged + 2 * (a1 + b9) + 2048 <= 232448) {
       pl.SB = 1;
@@ -2653,10 +2653,8 @@ int run_fwd(int N, int Hin, int Win, int Cin, int Cout, const void* x, const voi
     return pl.BN == 16 ? launch_fwd<16, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p)
                        : pl.BN == 32 ? launch_fwd<32, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 1, 64, 0, 1, 0, 1>(pl, mx, mw, my, p);
   }
-  if (pl.NS && epi == 1) {  // 64 filters: the outputs leave as a main convolution's do
-    if (pl.SB) return pl.RW ? launch_fwd<64, 0, 64, 0, 0, 1, 0, 0, 1, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 0, 0, 0, 0, 1, 1>(pl, mx, mw, my, p);
+  if (pl.NS && epi == 1)  // 64 filters: the outputs leave as a main convolution's do
     return pl.RW ? launch_fwd<64, 0, 64, 0, 0, 1, 0, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<64, 0, 64, 0, 0, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
-  }
   if (pl.SB && epi == 1) {
     if (pl.BN == 16) return pl.RW ? launch_fwd<16, 1, 64, 0, 0, 1, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<16, 1, 64, 0, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
     return pl.RW ? launch_fwd<32, 1, 64, 0, 0, 1, 0, 0, 1>(pl, mx, mw, my, p) : launch_fwd<32, 1, 64, 0, 0, 0, 0, 0, 1>(pl, mx, mw, my, p);
