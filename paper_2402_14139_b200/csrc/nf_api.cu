@@ -490,7 +490,11 @@ int nf_layer_get_param(nf_layer* L, int which, float* host, size_t n) {
     if (rc_ != NF_OK) return rc_; \
   } while (0)
 
-// nf_head_sample_mode for a layer: 2 only where h is stored and the sums of dh over each sample fit the reduction scratch
+// nf_head_sample_mode for a layer: 2 only where h is stored, and not for large batches of few pixels or channels.  The line between is
+// drawn by the size of the layer's partial sums (N * F against red_floats, from 2368 * Cout / F images on where its blocks fill the chip),
+// not by room: the kernel's own sums lie elsewhere.  Past it, kernel of the head against separate pool, head and dh (us a step): bf16
+// 64 -> 64 with 64 filters, 8x8, 3000 images 435 to 362, 4x4, 6000 images 464 to 424, 16x16, 3000 and 6000 images 622 to 610 and 1147 to
+// 1167; 32 filters, 16x16, 6000 images 956 to 941; fp32 3 -> 16 with 8 filters, 32x32, 6000 images 8648 to 8791, 16x16, 20 000 8506 to 8337.
 static int layer_head_mode(const nf_layer* L, bool h_masked) {
   const int N = L->o.N, F = L->F, K = L->classes;
   if (L->o.aux_pool != NF_POOL_AVG || nf_head_is_large(N, 4 * F, K)) return 0;

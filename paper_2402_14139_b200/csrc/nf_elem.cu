@@ -882,50 +882,50 @@ __global__ void __launch_bounds__(256) bn_bwd_reduce_vec_kernel(const T* __restr
     sc[i] = scale[c0 + i]; sh[i] = shift[c0 + i]; m[i] = mu[c0 + i]; is[i] = invstd[c0 + i];
   }
   for (int blk = blockIdx.x; blk * (256 / thr) < ranges; blk += gridDim.x) {
-  const int rng = blk * (256 / thr) + threadIdx.x / thr;
-  float a[8], b[8];
+    const int rng = blk * (256 / thr) + threadIdx.x / thr;
+    float a[8], b[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] = b[i] = 0.f;
-  const size_t p0 = rng < ranges ? P * rng / ranges : P, p1 = rng < ranges ? P * (rng + 1) / ranges : P;
-  constexpr int kU = 4;
-  for (size_t p = p0 + pl; p < p1; p += (size_t)kU * planes) {
-    Vec8<T> yq[kU], dq[kU], sq[kU];
+    for (int i = 0; i < 8; ++i) a[i] = b[i] = 0.f;
+    const size_t p0 = rng < ranges ? P * rng / ranges : P, p1 = rng < ranges ? P * (rng + 1) / ranges : P;
+    constexpr int kU = 4;
+    for (size_t p = p0 + pl; p < p1; p += (size_t)kU * planes) {
+      Vec8<T> yq[kU], dq[kU], sq[kU];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const size_t q = p + (size_t)u * planes;
-      if (q < p1) {
-        yq[u].load(y, q * C8 + g);
-        dq[u].load(da, q * C8 + g);
-        if constexpr (MODE == 1) sq[u].load(skip, q * C8 + g);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const size_t q = p + (size_t)u * planes;
-      if (q < p1) {
-        float yv[8], dv[8], kv[8];
-        yq[u].get(yv);
-        dq[u].get(dv);
-        if constexpr (MODE == 1) sq[u].get(kv);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float dz = MODE == 2 || fmaf(yv[i], sc[i], sh[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
-          a[i] += dz;
-          b[i] = MODE == 1 || (MODE == 0 && sizeof(T) == 4) ? fmaf(dz * (yv[i] - m[i]), is[i], b[i]) : fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
-          dv[i] = dz;
+      for (int u = 0; u < kU; ++u) {
+        const size_t q = p + (size_t)u * planes;
+        if (q < p1) {
+          yq[u].load(y, q * C8 + g);
+          dq[u].load(da, q * C8 + g);
+          if constexpr (MODE == 1) sq[u].load(skip, q * C8 + g);
         }
-        if (MODE == 1 && dz_out) st8(dz_out + (q * C8 + g) * 8, dv);
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const size_t q = p + (size_t)u * planes;
+        if (q < p1) {
+          float yv[8], dv[8], kv[8];
+          yq[u].get(yv);
+          dq[u].get(dv);
+          if constexpr (MODE == 1) sq[u].get(kv);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float dz = MODE == 2 || fmaf(yv[i], sc[i], sh[i]) + (MODE == 1 ? kv[i] : 0.f) > 0.f ? dv[i] : 0.f;
+            a[i] += dz;
+            b[i] = MODE == 1 || (MODE == 0 && sizeof(T) == 4) ? fmaf(dz * (yv[i] - m[i]), is[i], b[i]) : fmaf(dz, (yv[i] - m[i]) * is[i], b[i]);
+            dv[i] = dz;
+          }
+          if (MODE == 1 && dz_out) st8(dz_out + (q * C8 + g) * 8, dv);
+        }
       }
     }
-  }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    sm[i][threadIdx.x] = a[i];
-    sm[8 + i][threadIdx.x] = b[i];
-  }
-  __syncthreads();
-  range_totals<sizeof(T) == 4 && MODE != 1>(sm, threadIdx.x / thr * thr, lt, thr, C8, planes, rng < ranges, red + (size_t)rng * 2 * C);
-  __syncthreads();  // the totals are read before the next ranges are stored
+    for (int i = 0; i < 8; ++i) {
+      sm[i][threadIdx.x] = a[i];
+      sm[8 + i][threadIdx.x] = b[i];
+    }
+    __syncthreads();
+    range_totals<sizeof(T) == 4 && MODE != 1>(sm, threadIdx.x / thr * thr, lt, thr, C8, planes, rng < ranges, red + (size_t)rng * 2 * C);
+    __syncthreads();  // the totals are read before the next ranges are stored
   }
 }
 
@@ -1432,8 +1432,9 @@ __device__ __forceinline__ size_t win_base(size_t q, int Ho, int Wo, int C8) {  
 }
 
 // Which of the four window positions of a channel pair (packed bf16 y in w[0..3]) receives the gradient: all-ones halves in keep[d]
-// where position d is the first maximum, in scan order, of the bf16-rounded ReLU outputs and that maximum is positive; returns that maximum.  Two channels
-// per instruction from the conversion on: with one channel at a time the two kernels below were bound by these instructions.
+// where position d is the first maximum, in scan order, of the bf16-rounded ReLU outputs and that maximum is positive; returns that
+// maximum.  Two channels per instruction from the conversion on: with one channel at a time the two kernels below were bound by these
+// instructions.
 __device__ __forceinline__ __nv_bfloat162 pool_winner2(const uint32_t (&w)[4], float A0, float A1, float B0, float B1, uint32_t (&keep)[4]) {
   __nv_bfloat162 r[4];
 #pragma unroll
@@ -1744,7 +1745,11 @@ int nf_k_avgpool_fast(const void* h, int N, int Ha, int Wa, int F, float* part, 
   if (F % 8 || 256 % (F / 8) || (Ha & 1) || (Wa & 1)) return NF_EUNSUPPORTED;
   if ((long)(Ha / 2) * (Wa / 2) <= 16) return NF_EUNSUPPORTED;  // tiny maps: the caller's generic path has a kernel for them
   const int S = nf_k_avgpool_slices(N, Ha, Wa);
-  // one pass where no slices are cut, the chains are whole and there are threads enough for their length
+  // One pass where no slices are cut, the chains are whole and there are threads enough for their length.  One pass against the two kernels
+  // behind it, in us, operands in L2 where they fit.  Chains of one pixel, up to 64 of them: 16x16x16, 8 images 4.9 / 4.6, 256 images 5.1 /
+  // 10.4, 4096 images 7.8 / 70.  More of them: 32x32x8, 1024 threads 17.5 / 16.2, 4096 18 / 38, 16 384 21 / 129; 20x20x16, 7.8 / 6.3, 7.9 /
+  // 14, 9.2 / 38: the line lies on the safe side.  Longer chains: 32x32x64, 32 768 threads 43 / 35, 49 152 50 / 49, 65 536 56 / 63, which
+  // draws the line; the others there (32x32x32 43 / 61, 16x16x64 13 / 25, 16x16x256 8.4 / 15) would gain from 16 384 on.
   const int cnt = (Ha / 2) * (Wa / 2), planes = 256 / (F / 8), m = cnt <= planes ? 1 : cnt % planes ? 0 : cnt / planes;
   const size_t total = (size_t)N * 4 * (F / 8);
   if (S == 1 && Wa >= 4 && (m == 1 || m == 2 || m == 4 || m == 8) && cnt < 65536 && (m > 1 ? total >= 49152 : cnt <= 64 || total >= 16384)) {
