@@ -29,6 +29,14 @@ def _reference(x, p):
     return (y * s + (p["beta"].double() - p["rmean"].double() * s)).clamp_min(0), y * s
 
 
+def _cache(nf, block, x, out, launches, count=None):
+    """Block.cache, with the number of its launches: 2 straight from the images (coefficients, convolution), 4 by way of padded copies of
+    the images and the weights."""
+    before = nf.nf_launch_count()
+    block.cache(x, out, count=count)
+    assert nf.nf_launch_count() - before == launches
+
+
 def _check(got, want, ys):
     # y and the result are rounded to 8 bits each: half a unit is at most 2^-8 of the value; 27 products in fp32 are far below that
     assert bool(((got.double() - want).abs() <= 2.0 ** -8 * (ys.abs() + want) + 1e-5).all())
@@ -39,7 +47,7 @@ def test_first_layer_against_64_bits(N, count, H, W):
     import torch
     nf, L, p, x = _layer(N, H, W, H + W)
     out = torch.full((N, H, W, 64), 7.0, dtype=torch.bfloat16, device="cuda")
-    nf.Block([L]).cache(x, out, count=count)
+    _cache(nf, nf.Block([L]), x, out, 2, count)
     _check(out[:count], *_reference(x[:count], p))
     assert bool((out[count:] == 7.0).all()) and L.status() == 0
 
@@ -49,7 +57,7 @@ def test_images_with_infinities_reach_their_neighbours_only():
     nf, L, p, x = _layer(2, 32, 32, 5)
     out, ref = (torch.empty((2, 32, 32, 64), dtype=torch.bfloat16, device="cuda") for _ in range(2))
     block = nf.Block([L])
-    block.cache(x, ref)
+    _cache(nf, block, x, ref, 2)
     for r, c in ((0, 0), (7, 15), (8, 16), (31, 31), (13, 30)):
         xi = x.clone()
         xi[1, r, c, 1] = float("inf")
@@ -67,5 +75,5 @@ def test_output_over_the_images(shift):
     want, ys = _reference(x, p)
     buf = torch.zeros(shift + 3 * 32 * 32 * 64, dtype=torch.bfloat16, device="cuda")
     buf[:x.numel()] = x.flatten()
-    nf.Block([L]).cache(buf[:x.numel()], buf[shift:])
+    _cache(nf, nf.Block([L]), buf[:x.numel()], buf[shift:], 4)
     _check(buf[shift:].view(3, 32, 32, 64), want, ys)

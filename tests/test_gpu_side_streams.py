@@ -41,18 +41,27 @@ def _one_by_one(layers, x, y, loss, acts, steps):
             cur = acts[i]
 
 
+def _in_one_stream(nf, layers, x, y, loss, acts, steps):
+    """The same with per-operation timing on, which keeps every launch of a step in the caller's stream."""
+    nf.nf_trace_enable(True)
+    try:
+        _one_by_one(layers, x, y, loss, acts, steps)
+    finally:
+        nf.nf_trace_enable(False)
+
+
 def _same(a, b):
     assert all((p == q).all() for p, q in zip(a, b))
 
 
-@pytest.mark.parametrize("how", ["step", "graph", "other stream", "host"])
+@pytest.mark.parametrize("how", ["step", "graph", "other stream", "host", "layers"])
 @pytest.mark.parametrize("kind,N", [("bf16", 96), ("bf16", 7), ("f32", 8), ("same", 40)])
-def test_block_step_has_the_bits_of_single_steps(kind, N, how):
+def test_steps_have_the_bits_of_one_stream(kind, N, how):
     import torch
     nf, ref, _, x, y = _block(kind, N, 3)
     loss = torch.zeros(len(ref), device="cuda")
     acts = [L.new_act() for L in ref]
-    _one_by_one(ref, x, y, loss, acts, 3)
+    _in_one_stream(nf, ref, x, y, loss, acts, 3)
     nf, layers, block, x, y = _block(kind, N, 3, 2 if how == "host" else 0)
     got, act = torch.zeros(len(ref), device="cuda"), layers[-1].new_act()
     if how == "graph":
@@ -60,6 +69,8 @@ def test_block_step_has_the_bits_of_single_steps(kind, N, how):
         g = block.capture(x, y, 0.05, got, act)
         for _ in range(2):
             g.replay()
+    elif how == "layers":
+        _one_by_one(layers, x, y, got, [L.new_act() for L in layers[:-1]] + [act], 3)
     elif how == "host":
         xh, yh, got = x.cpu().pin_memory(), y.cpu().pin_memory(), got.cpu().pin_memory()
         for _ in range(3):
@@ -111,10 +122,10 @@ def test_a_call_that_fails_half_way_leaves_the_stream_in_order():
     loss = torch.zeros(len(layers), device="cuda")
     with pytest.raises(nf.NfError):        # the last layer refuses its output's address; the ones before it have run
         block.step(x, y, 0.05, loss, act[1:])
-    first = [loss.clone() for _ in range(1)]
+    first = loss.clone()
     block.step(x, y, 0.05, loss, act)      # no update was made by the first call
     torch.cuda.synchronize()
-    assert torch.equal(first[0][:-1], loss[:-1])
+    assert torch.equal(first[:-1], loss[:-1])
 
 
 def test_lanes_of_many_layers_come_and_go():
