@@ -526,8 +526,10 @@ static int step_phases(nf_layer* L, const void* x, const int32_t* labels, float 
   const char *a0 = (const char*)act_out, *a1 = a0 + (size_t)N * Ha * Wa * Co * nf_esize(dt);
   const bool own = a0 < L->ws + L->ws_total && L->ws < a1 && act_out != L->act && act_out != L->stage_act;
   const char *z0 = (const char*)L->skip_grad, *z1 = z0 + (size_t)N * Ho * Wo * Co * nf_esize(dt);
-  // fp32 kernels of many pixels fill the chip by themselves: there two at once only get in each other's way (851 against 862 us at 512 000)
-  const bool full = dt == NF_F32 && (size_t)N * Ha * Wa >= 131072;
+  // fp32 kernels of many pixels fill the chip by themselves, and two at once can get in each other's way.  Aside against in line, in us:
+  // 3 -> 16 channels, 4 filters, 32x32, 131 072 pixels 291 / 308, 262 144 480 / 501, 393 216 683 / 681, 524 288 873 / 859, which draws the
+  // line; others would gain beyond it too (64 -> 64, 524 288 pixels: 6584 / 6648; 16 -> 32 at 16x16: 2588 / 2626; 8 -> 8 at 64x64: 1066 / 1080).
+  const bool full = dt == NF_F32 && (size_t)N * Ha * Wa >= 393216;
   const bool in_line = g_trace_on || own || full || (L->skip_grad && a0 < z1 && z0 < a1);
   // A pooled layer's winners lie in a quarter of dy until dy is written: the first one, or the last where the activation lies over the first.
   const char *d0 = (const char*)L->dy, *d1 = d0 + (a1 - a0);

@@ -55,7 +55,7 @@ def _same(a, b):
 
 
 @pytest.mark.parametrize("how", ["step", "graph", "other stream", "host", "layers"])
-@pytest.mark.parametrize("kind,N", [("bf16", 96), ("bf16", 7), ("f32", 8), ("same", 40)])
+@pytest.mark.parametrize("kind,N", [("bf16", 96), ("bf16", 7), ("f32", 8), ("f32", 1535), ("f32", 1536), ("same", 40)])
 def test_steps_have_the_bits_of_one_stream(kind, N, how):
     import torch
     nf, ref, _, x, y = _block(kind, N, 3)
