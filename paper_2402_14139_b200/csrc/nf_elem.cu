@@ -1203,7 +1203,7 @@ __global__ void __launch_bounds__(256) avgpool_small_vec_kernel(const uint4* __r
 // kernels around it: M = 1, the bin's pixels in order; M > 1, `planes` chains of M pixels each, planes apart, the chains added in order.
 // Many images: 16x16 maps with 16 filters, 1777 of them, 37 + 3 -> 5 us (there half the threads of a block per bin had nothing to do and
 // sixteen added 128 sums one by one); 8x8 with 256, 6366 of them, 61 -> 45 (a thread for all four bins left a second wave nearly empty).
-// Blocks of 64 threads, so that a few thousand of them reach every SM.
+// Blocks of 64 threads, so that a few thousand of them reach every SM (exits of two layers at 16x16, 1777 images: 891 -> 881 us).
 template <int M>
 __global__ void __launch_bounds__(64) avgpool_vec_kernel(const uint4* __restrict__ h, int Ha, int Wa, int F8, int cnt, int planes,
                                                           uint32_t bw_mul, bool divide, size_t total, float* __restrict__ p) {
