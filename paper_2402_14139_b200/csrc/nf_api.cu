@@ -13,6 +13,7 @@
 #include "nf_tc.h"
 
 cudaStream_t g_nf_stream = 0;
+static int g_nf_prio = 0;  // its priority
 long long g_nf_launches = 0;
 __thread NfRoute t_nf_route = {nullptr, false};
 static char g_nf_err[256] = "";
@@ -85,15 +86,10 @@ unsigned long long capture_of(cudaStream_t s) {
   return st == cudaStreamCaptureStatusNone ? 0 : st == cudaStreamCaptureStatusActive ? id : kNoCapture;
 }
 bool lane_idle(const NfLane& n) { return capture_of(n.s) == 0; }
-int priority_of(cudaStream_t s) {
-  int prio = 0;
-  if (cudaStreamGetPriority(s, &prio) != cudaSuccess) cudaGetLastError();
-  return prio;
-}
 void lane_open(NfLane* n) {
   if (n->s) return;
   if (cudaGetDevice(&n->dev) == cudaSuccess) {
-    n->prio = priority_of(nf_stream());
+    n->prio = g_nf_prio;
     {
       const std::lock_guard<std::mutex> lock(g_lanes_mutex);
       for (int i = 0; i < g_lane_count; ++i)
@@ -150,7 +146,7 @@ bool lane_usable(NfLane* n) {
   int dev = -1;
   if (g_trace_on || !n->s || cudaGetDevice(&dev) != cudaSuccess || dev != n->dev) return false;
   const unsigned long long id = capture_of(n->s);
-  if ((id != 0 && (id == kNoCapture || id != capture_of(nf_stream()))) || n->prio != priority_of(nf_stream())) {
+  if ((id != 0 && (id == kNoCapture || id != capture_of(nf_stream()))) || n->prio != g_nf_prio) {
     lane_close(n);
     lane_open(n);
   }
@@ -1177,6 +1173,8 @@ long long nf_max_batch(double slope, double intercept, double budget_bytes) {
 
 int nf_set_stream(void* s) {
   g_nf_stream = (cudaStream_t)s;
+  g_nf_prio = 0;
+  if (s && cudaStreamGetPriority(g_nf_stream, &g_nf_prio) != cudaSuccess) cudaGetLastError();  // once, not in every step
   return NF_OK;
 }
 
