@@ -7,7 +7,7 @@ A step = one pass of the whole hot path over one batch: every layer of the block
 step in turn (conv+BN+ReLU forward, aux head forward/backward, weight gradients, SGD update).
 The K timed steps are K replays of a CUDA graph recorded from nf_block_step (--no-graph launches the kernels one by
 one instead); the per-op table and the roofline come from the same K steps launched one by one right after, with events
-around each operation.  That keeps every step in one stream: nothing runs beside anything else, as it does in the timed steps.
+around each operation.  Those steps stay in one stream; in the timed ones a layer's kernels also run beside the next layer's.
 Multi-GPU: independent replicas, one process per GPU (the step has no exchange to shard over),
 timed as the max over ranks; value = images of all ranks / that time.
 """
